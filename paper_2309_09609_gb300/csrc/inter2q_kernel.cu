@@ -8,8 +8,8 @@
 // two halves hold two different queries: the word of query rows (a_i, b_i)
 // against residue d_j is (SM(a_i, d_j), SM(b_i, d_j)), a single entry of a
 // per-strip profile built for the query pair, read ready-made from shared
-// memory.  The cell update is the same biased packed update (Eq. 1-3), so a
-// word costs 4.5 ALU-pipe operations instead of 5.5.
+// memory.  The cell update is the same (packed_cell), so a word costs 3.5
+// ALU-pipe operations instead of 4.5.
 //
 // Queries are laid out in "query streams": the plan deals the batch's queries
 // to pairs of streams (longest first, each to the shorter stream), each query
@@ -65,15 +65,15 @@ __device__ __forceinline__ void cp_async8(void* smem_dst, const void* gmem_src) 
 // lane's subject -- as one wavefront: column c updates row k - c at step k,
 // so up to W cell updates of a step are independent.  A column loads its
 // profile words 4 rows at a time (one 16-byte read) when it enters a 4-row
-// block.  b[q] / o[q] hold (H'_c, F'_c) of columns 2q and 2q + 1 above / at
+// block.  b[q] / o[q] hold (H_c, F_c) of columns 2q and 2q + 1 above / at
 // the bottom of the strip.  A chunk runs as two wavefronts of four columns:
 // on the paper-shaped search that was 3% faster than one of eight (880
 // against 907 ms at 32 rows) and no slower than four of two.
-template <int T, int W, int C0, int G>
+template <int T, int W, int C0>
 __device__ __forceinline__ void q2_wave(uint32_t (&Hp)[T], uint32_t (&E)[T], uint32_t& hdiag,
                                        uint32_t& smax, const uint8_t* prof, int p16, const uint2 rr,
                                        const uint4* b, uint4* o, uint32_t GO2,
-                                       uint32_t NGE2, uint32_t MGO, uint32_t one) {
+                                       uint32_t NGE2) {
   constexpr int RB = Q2Shape<T>::RB;
   uint32_t cb[W];  // base(c) of each column's residue code
 #pragma unroll
@@ -103,10 +103,10 @@ __device__ __forceinline__ void q2_wave(uint32_t (&Hp)[T], uint32_t (&E)[T], uin
   hdiag = htop[W - 1];
 #pragma unroll
   for (int k = 0; k < T + W - 1; k++) {
-    uint32_t out[W];
+    uint32_t out[W], x[W];
 #pragma unroll
     for (int c = 0; c < W; c++) {
-      out[c] = 0u;
+      out[c] = x[c] = 0u;
       const int r = k - c;
       if (r < 0 || r >= T) continue;
       if ((r & 3) == 0) pw[c] = *(const uint4*)(prof + cb[c] + (r >> 2) * 128);
@@ -116,20 +116,20 @@ __device__ __forceinline__ void q2_wave(uint32_t (&Hp)[T], uint32_t (&E)[T], uin
         hd = hd0;
         hd0 = Hp[r];
       } else {
-        hd = r == 0 ? htop[c - 1] : last2[c - 1];  // H' of column c - 1, row r - 1
+        hd = r == 0 ? htop[c - 1] : last2[c - 1];  // H of column c - 1, row r - 1
       }
       uint32_t e = E[r];
-      out[c] = packed_cell<G>(hd, w, e, f[c], GO2, NGE2, MGO, one);
+      out[c] = packed_cell(hd, w, e, f[c], x[c], GO2, NGE2);
       E[r] = e;
       if (c == W - 1) Hp[r] = out[c];
       if (r == T - 1) bottom[c] = out[c];
     }
-    // S' over this step's cells (pairs through a three-input max)
+    // S over this step's cells (pairs through a three-input max)
     const int lo = k - (T - 1) > 0 ? k - (T - 1) : 0;
     const int hi = k < W - 1 ? k : W - 1;
     int c = lo;
-    for (; c + 1 <= hi; c += 2) smax = __vimax3_s16x2(smax, out[c], out[c + 1]);
-    if (c == hi) smax = __vmaxs2(smax, out[c]);
+    for (; c + 1 <= hi; c += 2) smax = __vimax3_s16x2(smax, x[c], x[c + 1]);
+    if (c == hi) smax = __vmaxs2(smax, x[c]);
 #pragma unroll
     for (int c2 = 0; c2 < W; c2++) {
       last2[c2] = last[c2];
@@ -141,7 +141,7 @@ __device__ __forceinline__ void q2_wave(uint32_t (&Hp)[T], uint32_t (&E)[T], uin
     o[q] = make_uint4(bottom[2 * q], f[2 * q], bottom[2 * q + 1], f[2 * q + 1]);
 }
 
-// The 16-bit S' of one half: recorded (or flagged for the int32 recompute
+// The 16-bit S of one half: recorded (or flagged for the int32 recompute
 // when it may have saturated) as the score of (query q, sorted subject sidx).
 __device__ __forceinline__ void q2_emit(const DbView& db, const SearchParams* __restrict__ P,
                                         SearchState* st, const Scratch& scr, int q, int sidx,
@@ -154,7 +154,7 @@ __device__ __forceinline__ void q2_emit(const DbView& db, const SearchParams* __
     else  // the list is full: mark the pair for the host's next recompute round
       P->scores[(int64_t)q * db.n + orig] = FLAG_SENTINEL;
   } else {
-    P->scores[(int64_t)q * db.n + orig] = sb - P->go;
+    P->scores[(int64_t)q * db.n + orig] = sb;
   }
 }
 
@@ -168,16 +168,15 @@ __device__ void q2_item(const DbView& db, const SearchParams* __restrict__ P, Se
   // this lane's 8 residues of chunk c: bytes [8h, 8h + 8) of its 16-byte vector
   const uint2* __restrict__ res = (const uint2*)(db.inter + db.goff[g]) + lane * 2 + h;
   uint4* bd = scr.inter_border + warp_id * scr.inter_stride_vec + lane;
-  uint32_t GO2, NGE2, MGO;  // (Go, Go), (-Ge, -Ge), -(Go, Go)
-  gap_words<G>(P, GO2, NGE2, MGO);
-  const uint32_t one = (uint32_t)P->one;
+  uint32_t GO2, NGE2;  // (Go, Go), (-Ge, -Ge)
+  gap_words<G>(P, GO2, NGE2);
   const int p16 = (lane & 7) * 16;
   const int nch = L / CHUNK;
   const int sidx = g * GROUP + 2 * lane + h;
   const int orig = db.perm[sidx];
   uint4* bring = (uint4*)(slice + Q2Shape<T>::BORDER_RING) + lane;  // [slot][pair][lane]
   uint2* rring = (uint2*)(slice + Q2Shape<T>::RES_RING) + lane;     // [slot][lane]
-  uint32_t smax = GO2;  // S' of S = 0, both halves
+  uint32_t smax = 0u;  // S, both halves
   for (int s = 0; s < sp.y; s++) {
     const int4 si = P->strips[sp.x + s];
     const int qa = si.x, qb = si.z;                // -1: no query in that half
@@ -211,13 +210,13 @@ __device__ void q2_item(const DbView& db, const SearchParams* __restrict__ P, Se
     uint32_t Hp[T], E[T];
 #pragma unroll
     for (int r = 0; r < T; r++) {
-      Hp[r] = GO2;   // H(i, 0) = 0
-      E[r] = 0u;     // E(i, 1) = -Go
+      Hp[r] = 0u;  // H(i, 0) = 0
+      E[r] = 0u;   // any E(i, 1) <= 0 gives the same H
     }
-    uint32_t hdiag = GO2;
+    uint32_t hdiag = 0u;
     const bool last = (s == sp.y - 1);
     // keep-mask of the bottom row: the halves whose query ends here store
-    // the empty row above the next query instead (H' = Go, F' = 0)
+    // the empty row above the next query instead (H = F = 0)
     const uint32_t keep = (enda ? 0u : 0x0000ffffu) | (endb ? 0u : 0xffff0000u);
     // staging ring as in the packed inter-task kernel; the first strip's
     // border is the row above the matrix, copied from the parameter block
@@ -250,15 +249,15 @@ __device__ void q2_item(const DbView& db, const SearchParams* __restrict__ P, Se
       const uint4 bv[4] = {bring[(slot * 4 + 0) * 32], bring[(slot * 4 + 1) * 32],
                            bring[(slot * 4 + 2) * 32], bring[(slot * 4 + 3) * 32]};
       uint4 ov[4];
-      q2_wave<T, 4, 0, G>(Hp, E, hdiag, smax, slice, p16, rr, bv, ov, GO2, NGE2, MGO, one);
-      q2_wave<T, 4, 4, G>(Hp, E, hdiag, smax, slice, p16, rr, bv + 2, ov + 2, GO2, NGE2, MGO, one);
+      q2_wave<T, 4, 0>(Hp, E, hdiag, smax, slice, p16, rr, bv, ov, GO2, NGE2);
+      q2_wave<T, 4, 4>(Hp, E, hdiag, smax, slice, p16, rr, bv + 2, ov + 2, GO2, NGE2);
       if (!last) {
         if (keep != 0xffffffffu) {  // uniform: some query ends in this strip
 #pragma unroll
           for (int q = 0; q < 4; q++) {
-            ov[q].x = (ov[q].x & keep) | (GO2 & ~keep);
+            ov[q].x &= keep;
             ov[q].y &= keep;
-            ov[q].z = (ov[q].z & keep) | (GO2 & ~keep);
+            ov[q].z &= keep;
             ov[q].w &= keep;
           }
         }
@@ -269,11 +268,11 @@ __device__ void q2_item(const DbView& db, const SearchParams* __restrict__ P, Se
     cp_async_wait<0>();
     if (enda) {
       q2_emit(db, P, st, scr, qa, sidx, orig, (int)(int16_t)(smax & 0xffffu));
-      smax = (smax & 0xffff0000u) | (GO2 & 0xffffu);
+      smax &= 0xffff0000u;
     }
     if (endb) {
       q2_emit(db, P, st, scr, qb, sidx, orig, (int)(int16_t)(smax >> 16));
-      smax = (smax & 0x0000ffffu) | (GO2 & 0xffff0000u);
+      smax &= 0x0000ffffu;
     }
   }
 }

@@ -42,18 +42,18 @@ __device__ __forceinline__ uint32_t profile_word(const uint4 (&va)[T / 16], cons
 
 
 // Four adjacent columns of T rows as a wavefront: at step k, column c
-// updates row k - c.  Column c's row r needs E' of column c - 1 at row r
-// (written one step earlier) and its H' at row r - 1 (two steps earlier), so
-// the up to four updates of a step are independent.  Hp[r] / E[r] hold H' / E'
+// updates row k - c.  Column c's row r needs E of column c - 1 at row r
+// (written one step earlier) and its H at row r - 1 (two steps earlier), so
+// the up to four updates of a step are independent.  Hp[r] / E[r] hold H / E
 // of the previous column on entry and of the fourth column on exit; b0, b1
-// are the border vectors (H'_c, F'_c) above the strip for columns 0,1 and 2,3;
+// are the border vectors (H_c, F_c) above the strip for columns 0,1 and 2,3;
 // o0, o1 receive the strip's bottom row in the same layout.
-template <int T, int G>
+template <int T>
 __device__ __forceinline__ void packed_quad(uint32_t (&Hp)[T], uint32_t (&E)[T], uint32_t& hdiag,
                                             uint32_t& smax, const uint8_t* slice, int p16,
                                             uint32_t wa, uint32_t wb, const uint4& b0,
                                             const uint4& b1, uint4& o0, uint4& o1, uint32_t GO2,
-                                            uint32_t NGE2, uint32_t MGO, uint32_t one) {
+                                            uint32_t NGE2) {
   constexpr int HALVES = T / 16;
   constexpr int W = 4;
   uint4 pa[W][HALVES], pb[W][HALVES];
@@ -67,14 +67,14 @@ __device__ __forceinline__ void packed_quad(uint32_t (&Hp)[T], uint32_t (&E)[T],
       pb[c][h] = *(const uint4*)(slice + (cb * HALVES + h) * 128 + p16);
     }
   }
-  const uint32_t htop[W] = {b0.x, b0.z, b1.x, b1.z};  // H' above the strip, per column
-  uint32_t f[W] = {b0.y, b0.w, b1.y, b1.w};           // F' of the strip's first row
+  const uint32_t htop[W] = {b0.x, b0.z, b1.x, b1.z};  // H above the strip, per column
+  uint32_t f[W] = {b0.y, b0.w, b1.y, b1.w};           // F of the strip's first row
   uint32_t last[W] = {0, 0, 0, 0}, last2[W] = {0, 0, 0, 0}, bottom[W] = {0, 0, 0, 0};
   uint32_t hd0 = hdiag;  // column 0's diagonal: previous column, previous row
   hdiag = htop[W - 1];
 #pragma unroll
   for (int k = 0; k < T + W - 1; k++) {
-    uint32_t out[W] = {0, 0, 0, 0};
+    uint32_t out[W] = {0, 0, 0, 0}, x[W] = {0, 0, 0, 0};
 #pragma unroll
     for (int c = 0; c < W; c++) {
       const int r = k - c;
@@ -84,20 +84,20 @@ __device__ __forceinline__ void packed_quad(uint32_t (&Hp)[T], uint32_t (&E)[T],
         hd = hd0;
         hd0 = Hp[r];
       } else {
-        hd = r == 0 ? htop[c - 1] : last2[c - 1];  // H' of column c - 1, row r - 1
+        hd = r == 0 ? htop[c - 1] : last2[c - 1];  // H of column c - 1, row r - 1
       }
       uint32_t e = E[r];
-      out[c] = packed_cell<G>(hd, profile_word<T>(pa[c], pb[c], r), e, f[c], GO2, NGE2, MGO, one);
+      out[c] = packed_cell(hd, profile_word<T>(pa[c], pb[c], r), e, f[c], x[c], GO2, NGE2);
       E[r] = e;
       if (c == W - 1) Hp[r] = out[c];
       if (r == T - 1) bottom[c] = out[c];
     }
-    // S' over this step's cells (pairs through a three-input max)
+    // S over this step's cells (pairs through a three-input max)
     const int lo = k - (T - 1) > 0 ? k - (T - 1) : 0;
     const int hi = k < W - 1 ? k : W - 1;
     int c = lo;
-    for (; c + 1 <= hi; c += 2) smax = __vimax3_s16x2(smax, out[c], out[c + 1]);
-    if (c == hi) smax = __vmaxs2(smax, out[c]);
+    for (; c + 1 <= hi; c += 2) smax = __vimax3_s16x2(smax, x[c], x[c + 1]);
+    if (c == hi) smax = __vmaxs2(smax, x[c]);
 #pragma unroll
     for (int c2 = 0; c2 < W; c2++) {
       last2[c2] = last[c2];
@@ -113,14 +113,13 @@ __device__ __forceinline__ void packed_quad(uint32_t (&Hp)[T], uint32_t (&E)[T],
 // k), with up to eight independent cell updates per step.  Each column holds
 // only the 16-row half of its profile row that its current rows need,
 // loaded when the column reaches row 0 and row 16, so eight columns take the
-// profile registers of four.  b[q] / o[q] hold (H'_c, F'_c) of columns 2q and
+// profile registers of four.  b[q] / o[q] hold (H_c, F_c) of columns 2q and
 // 2q + 1 above / at the bottom of the strip.
-template <int T, int G>
+template <int T>
 __device__ __forceinline__ void packed_oct(uint32_t (&Hp)[T], uint32_t (&E)[T], uint32_t& hdiag,
                                            uint32_t& smax, const uint8_t* slice, int p16,
                                            const uint4& rr, const uint4 (&b)[4], uint4 (&o)[4],
-                                           uint32_t GO2, uint32_t NGE2, uint32_t MGO,
-                                           uint32_t one) {
+                                           uint32_t GO2, uint32_t NGE2) {
   static_assert(T == 32, "the eight-column wavefront is for 32 rows");
   constexpr int HALVES = 2;
   constexpr int W = 8;
@@ -145,10 +144,10 @@ __device__ __forceinline__ void packed_oct(uint32_t (&Hp)[T], uint32_t (&E)[T], 
   hdiag = htop[W - 1];
 #pragma unroll
   for (int k = 0; k < T + W - 1; k++) {
-    uint32_t out[W];
+    uint32_t out[W], x[W];
 #pragma unroll
     for (int c = 0; c < W; c++) {
-      out[c] = 0u;
+      out[c] = x[c] = 0u;
       const int r = k - c;
       if (r < 0 || r >= T) continue;
       if ((r & 15) == 0) {  // this column enters a new 16-row half of its profile row
@@ -161,23 +160,23 @@ __device__ __forceinline__ void packed_oct(uint32_t (&Hp)[T], uint32_t (&E)[T], 
         hd = hd0;
         hd0 = Hp[r];
       } else {
-        hd = r == 0 ? htop[c - 1] : last2[c - 1];  // H' of column c - 1, row r - 1
+        hd = r == 0 ? htop[c - 1] : last2[c - 1];  // H of column c - 1, row r - 1
       }
       const int wq = (r >> 2) & 3;
       const uint32_t a32 = wq == 0 ? pa[c].x : wq == 1 ? pa[c].y : wq == 2 ? pa[c].z : pa[c].w;
       const uint32_t b32 = wq == 0 ? pb[c].x : wq == 1 ? pb[c].y : wq == 2 ? pb[c].z : pb[c].w;
       uint32_t e = E[r];
-      out[c] = packed_cell<G>(hd, prmt(a32, b32, sext_pair_sel(r & 3)), e, f[c], GO2, NGE2, MGO, one);
+      out[c] = packed_cell(hd, prmt(a32, b32, sext_pair_sel(r & 3)), e, f[c], x[c], GO2, NGE2);
       E[r] = e;
       if (c == W - 1) Hp[r] = out[c];
       if (r == T - 1) bottom[c] = out[c];
     }
-    // S' over this step's cells (pairs through a three-input max)
+    // S over this step's cells (pairs through a three-input max)
     const int lo = k - (T - 1) > 0 ? k - (T - 1) : 0;
     const int hi = k < W - 1 ? k : W - 1;
     int c = lo;
-    for (; c + 1 <= hi; c += 2) smax = __vimax3_s16x2(smax, out[c], out[c + 1]);
-    if (c == hi) smax = __vmaxs2(smax, out[c]);
+    for (; c + 1 <= hi; c += 2) smax = __vimax3_s16x2(smax, x[c], x[c + 1]);
+    if (c == hi) smax = __vmaxs2(smax, x[c]);
 #pragma unroll
     for (int c2 = 0; c2 < W; c2++) {
       last2[c2] = last[c2];
@@ -197,18 +196,15 @@ __device__ void inter_item(const DbView& db, const SearchParams* __restrict__ P,
   const uint8_t* __restrict__ qr = P->qres + P->qoff[q];
   const uint4* __restrict__ res = (const uint4*)(db.inter + db.goff[g]) + lane;
   uint4* bd = scr.inter_border + warp_id * scr.inter_stride_vec + lane;
-  const int go = P->go;
-  uint32_t GO2, NGE2, MGO;  // (Go, Go), (-Ge, -Ge), -(Go, Go)
-  gap_words<G>(P, GO2, NGE2, MGO);
-  const uint32_t ZERO2 = 0u;                                       // E' of E = -Go
-  const uint32_t one = (uint32_t)P->one;
+  uint32_t GO2, NGE2;  // (Go, Go), (-Ge, -Ge)
+  gap_words<G>(P, GO2, NGE2);
   const int p16 = (lane & 7) * 16;
   constexpr int HALVES = T / 16;
   const int nstrips = L > 0 ? (m + T - 1) / T : 0;
   const int nch = L / CHUNK;
   uint4* bring = (uint4*)(slice + InterProfile<T>::BORDER_RING) + lane;  // [slot][pair][lane]
   uint4* rring = (uint4*)(slice + InterProfile<T>::RES_RING) + lane;     // [slot][lane]
-  uint32_t smax = GO2;  // S' of S = 0
+  uint32_t smax = 0u;  // S, both subjects
   for (int s = 0; s < nstrips; s++) {
     __syncwarp();
     if (lane < NCODES) {  // code c = lane: T bytes, written to all 8 copies
@@ -237,14 +233,14 @@ __device__ void inter_item(const DbView& db, const SearchParams* __restrict__ P,
     uint32_t Hp[T], E[T];
 #pragma unroll
     for (int r = 0; r < T; r++) {
-      Hp[r] = GO2;    // H(i, 0) = 0
-      E[r] = ZERO2;   // E(i, 1) = -Go
+      Hp[r] = 0u;  // H(i, 0) = 0
+      E[r] = 0u;   // any E(i, 1) <= 0 gives the same H
     }
-    uint32_t hdiag = GO2;
+    uint32_t hdiag = 0u;
     const bool last = (s == nstrips - 1);
     // Staging ring of CRING chunks, copied with cp.async CRING - 1 chunks ahead
     // (commit group c = chunk c).  The first strip's border is the row above
-    // the matrix, (H, F) = (0, -Go) for every column: it is copied from the
+    // the matrix, (H, F) = (0, 0) for every column: it is copied from the
     // parameter block, so the compute loop has no branch on it.  A slot is
     // refilled only after the registers read from it were consumed.
     const uint4* bsrc = s == 0 ? (const uint4*)&P->init_border : bd;
@@ -277,7 +273,7 @@ __device__ void inter_item(const DbView& db, const SearchParams* __restrict__ P,
         const uint4 bv[4] = {bring[(slot * 4 + 0) * 32], bring[(slot * 4 + 1) * 32],
                              bring[(slot * 4 + 2) * 32], bring[(slot * 4 + 3) * 32]};
         uint4 ov[4];
-        packed_oct<T, G>(Hp, E, hdiag, smax, slice, p16, rr, bv, ov, GO2, NGE2, MGO, one);
+        packed_oct<T>(Hp, E, hdiag, smax, slice, p16, rr, bv, ov, GO2, NGE2);
         if (!last) {
 #pragma unroll
           for (int q = 0; q < 4; q++) bd[(c * 4 + q) * 32] = ov[q];
@@ -293,8 +289,7 @@ __device__ void inter_item(const DbView& db, const SearchParams* __restrict__ P,
         const uint4 b0 = bring[(slot * 4 + 2 * hq) * 32];
         const uint4 b1 = bring[(slot * 4 + 2 * hq + 1) * 32];
         uint4 o0, o1;
-        packed_quad<T, G>(Hp, E, hdiag, smax, slice, p16, wa, wb, b0, b1, o0, o1, GO2, NGE2, MGO,
-                       one);
+        packed_quad<T>(Hp, E, hdiag, smax, slice, p16, wa, wb, b0, b1, o0, o1, GO2, NGE2);
         if (!last) {
           bd[(c * 4 + 2 * hq) * 32] = o0;
           bd[(c * 4 + 2 * hq + 1) * 32] = o1;
@@ -317,7 +312,7 @@ __device__ void inter_item(const DbView& db, const SearchParams* __restrict__ P,
     const int sidx = base + half;
     const int orig = db.perm[sidx];
     if (orig < 0) continue;
-    const int sb = (int)(int16_t)(half ? (smax >> 16) : (smax & 0xffffu));  // S'
+    const int sb = (int)(int16_t)(half ? (smax >> 16) : (smax & 0xffffu));  // S
     if (sb >= P->sat_threshold) {
       const unsigned long long k = atomicAdd(&st->n_flags, 1ull);
       if ((int64_t)k < scr.flag_capacity)
@@ -325,7 +320,7 @@ __device__ void inter_item(const DbView& db, const SearchParams* __restrict__ P,
       else  // the list is full: mark the pair for the host's next recompute round
         P->scores[(int64_t)q * db.n + orig] = FLAG_SENTINEL;
     } else {
-      P->scores[(int64_t)q * db.n + orig] = sb - go;
+      P->scores[(int64_t)q * db.n + orig] = sb;
     }
   }
 }

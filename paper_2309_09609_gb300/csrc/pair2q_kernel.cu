@@ -6,8 +6,8 @@
 // per word).  Here a warp scores ONE long subject, and the halves hold two
 // query streams (the layout of inter2q_kernel.cu): the word of rows (a_i,
 // b_i) against residue d_j is (SM(a_i, d_j), SM(b_i, d_j)), read ready-made
-// from a profile built for the pass.  The cell update is the same biased
-// packed update (Eq. 1-3), 4.5 ALU-pipe operations per word instead of 5.5.
+// from a profile built for the pass.  The cell update is the same
+// (packed_cell), 3.5 ALU-pipe operations per word instead of 4.5.
 //
 // Intra-task parallelism (Section II-B): lane k owns one 32-row strip of each
 // stream per 1024-row pass, split into four quarters of 8 rows; quarter q of
@@ -20,7 +20,7 @@
 // lanes (or passes).  A lane whose strip starts a query in a half replaces
 // that half of its top border by the empty row above the matrix (H = 0,
 // F = -Go).  At the end of a pass the warp takes, per half, a segmented
-// maximum of S' over the lanes of each query (with the maximum carried from
+// maximum of S over the lanes of each query (with the maximum carried from
 // the previous pass), and the lane holding a query's last strip emits the
 // score.
 //
@@ -96,7 +96,7 @@ __device__ __forceinline__ void p2_profile(uint8_t* prof, const int8_t* __restri
   }
 }
 
-// The 16-bit S' of one half (biased by +Go): recorded, or flagged for the
+// The 16-bit S of one half: recorded, or flagged for the
 // int32 recompute when it may have saturated, as the score of (query q,
 // sorted subject sidx).
 __device__ __forceinline__ void p2_emit(const DbView& db, const SearchParams* __restrict__ P,
@@ -110,7 +110,7 @@ __device__ __forceinline__ void p2_emit(const DbView& db, const SearchParams* __
     else  // the list is full: mark the pair for the host's next recompute round
       P->scores[(int64_t)q * db.n + orig] = FLAG_SENTINEL;
   } else {
-    P->scores[(int64_t)q * db.n + orig] = sb - P->go;
+    P->scores[(int64_t)q * db.n + orig] = sb;
   }
 }
 
@@ -146,9 +146,8 @@ pair2q_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Sc
   for (int i = lane; i < P2_RING; i += 32) ring[i] = PAD_CODE;
   __syncthreads();
   uint2* hb = scr.pair_border + ((int64_t)blockIdx.x * P2_WARPS + wib) * scr.pair_stride;
-  uint32_t GO2, NGE2, MGO;  // (Go, Go), (-Ge, -Ge), -(Go, Go)
-  gap_words<G>(P, GO2, NGE2, MGO);
-  const uint32_t one = (uint32_t)P->one;
+  uint32_t GO2, NGE2;  // (Go, Go), (-Ge, -Ge)
+  gap_words<G>(P, GO2, NGE2);
   const uint32_t lane_off = (uint32_t)(lane * P2_LANE_BYTES);
   // lane 0 takes its top border from the scratch row, the others from the
   // lane above: x * is0 + y * not0 picks one word exactly (a product by 0 or
@@ -178,7 +177,7 @@ pair2q_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Sc
       for (int i = 0; i < 4; i++) w |= (uint32_t)(c + i < n ? d[c + i] : PAD_CODE) << (8 * i);
       *(uint32_t*)(ring + c % P2_RING) = w;
     };
-    uint32_t carry = GO2;  // per half: S' so far of the query that continues into the next pass
+    uint32_t carry = 0u;  // per half: S so far of the query that continues into the next pass
     for (int p = 0; p < npass; p++) {
       __syncthreads();  // every warp is done with the previous pass's profile
       p2_profile(prof, sm, P, sp, p);
@@ -195,30 +194,29 @@ pair2q_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Sc
         if (qa >= 0 && (si.y & 0x7fffffff) != 0) keep |= 0x0000ffffu;
         if (qb >= 0 && (si.w & 0x7fffffff) != 0) keep |= 0xffff0000u;
       }
-      const uint32_t gtop = GO2 & ~keep;  // (H', F') = (Go, 0) where a query starts
       if (n > 0) load_block(0);
       __syncthreads();
-      uint32_t smax = GO2;
+      uint32_t smax = 0u;
       if (n > 0) {  // uniform over the warp
         uint32_t Hp[32], E[32];
 #pragma unroll
         for (int r = 0; r < 32; r++) {
-          Hp[r] = GO2;  // H(i, 0) = 0
-          E[r] = 0u;    // E(i, 1) = -Go
+          Hp[r] = 0u;  // H(i, 0) = 0
+          E[r] = 0u;   // any E(i, 1) <= 0 gives the same H
         }
-        // quarter q's bottom-row H' one and two steps back, its F' one step back
+        // quarter q's bottom-row H one and two steps back, its F one step back
         uint32_t qh1[PQ], qh2[PQ], qf1[PQ];
         // profile offset of the code read at each of the last four steps (slot
         // t mod 4): quarter q at step t scores the column read at step t - q
         uint32_t A[PQ];
 #pragma unroll
         for (int q = 0; q < PQ; q++) {
-          qh1[q] = GO2;
-          qh2[q] = GO2;
+          qh1[q] = 0u;
+          qh2[q] = 0u;
           qf1[q] = 0u;
           A[q] = lane_off;
         }
-        uint32_t hdiag = GO2, out_h = GO2, out_f = 0u;
+        uint32_t hdiag = 0u, out_h = 0u, out_f = 0u;
         // steady state: lane 0's border of columns t .. t + 3, slot t mod 4
         uint2 bq[4] = {make_uint2(0u, 0u), make_uint2(0u, 0u), make_uint2(0u, 0u),
                        make_uint2(0u, 0u)};
@@ -258,8 +256,8 @@ pair2q_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Sc
           in_h = imad(bv.x, is0, imad(in_h, not0, 0u));
           in_f = imad(bv.y, is0, imad(in_f, not0, 0u));
           if constexpr (decltype(masked)::value) {
-            in_h = (in_h & keep) | gtop;  // H(0, j) = 0 above a query's first row
-            in_f &= keep;                 // F(1, j) = -Go
+            in_h &= keep;  // H(0, j) = 0 above a query's first row
+            in_f &= keep;  // any F(1, j) <= 0
           }
           const int c0 = t - PQ * lane;  // quarter 0's column
           A[U] = lane_off + (uint32_t)ring[pos + U] * P2_CODE_BYTES;
@@ -276,27 +274,28 @@ pair2q_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Sc
               const uint4 w0 = *(const uint4*)pw;
               const uint4 w1 = *(const uint4*)(pw + 16);
               const uint32_t w[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
-              uint32_t hd = q == 0 ? hdiag : qh2[q - 1];  // H' one row up, one column back
-              uint32_t f = q == 0 ? in_f : qf1[q - 1];    // F' of this quarter's first row
-              uint32_t hprev = 0;
+              uint32_t hd = q == 0 ? hdiag : qh2[q - 1];  // H one row up, one column back
+              uint32_t f = q == 0 ? in_f : qf1[q - 1];    // F of this quarter's first row
+              uint32_t xprev = 0;
 #pragma unroll
               for (int i = 0; i < 8; i++) {
                 const int r = 8 * q + i;
                 uint32_t e = E[r];
-                const uint32_t h = packed_cell<G>(hd, w[i], e, f, GO2, NGE2, MGO, one);
+                uint32_t x;
+                const uint32_t h = packed_cell(hd, w[i], e, f, x, GO2, NGE2);
                 hd = Hp[r];
                 Hp[r] = h;
                 E[r] = e;
                 if (i & 1)
-                  smax = __vimax3_s16x2(smax, hprev, h);
+                  smax = __vimax3_s16x2(smax, xprev, x);
                 else
-                  hprev = h;
+                  xprev = x;
               }
               nh[q] = Hp[8 * q + 7];
               nf[q] = f;
               if (q == PQ - 1 && lane == 31 && !last_pass) hb[col] = make_uint2(nh[q], f);
             } else if (col < 0) {
-              nh[q] = GO2;  // left of the matrix: H = 0
+              nh[q] = 0u;  // left of the matrix: H = 0
             }
           }
           hdiag = in_h;
@@ -347,7 +346,7 @@ pair2q_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Sc
         for (; t0 < steps; t0 += 4)
           block(t0, std::true_type{}, std::true_type{}, std::true_type{});
       }
-      // S' of each query over its lanes of this pass (and the previous passes)
+      // S of each query over its lanes of this pass (and the previous passes)
       int va = (int)(int16_t)(smax & 0xffffu), vb = (int)(int16_t)(smax >> 16);
       if (lane == 0) {
         if (keep & 0x0000ffffu) va = max(va, (int)(int16_t)(carry & 0xffffu));
@@ -360,8 +359,8 @@ pair2q_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Sc
         if (endb) p2_emit(db, P, st, scr, qb, sidx, orig, vb);
       }
       // what lane 31's queries carry into the next pass (nothing past an end)
-      const int ca = __shfl_sync(FULL, (enda || qa < 0) ? (int)(int16_t)(GO2 & 0xffffu) : va, 31);
-      const int cb = __shfl_sync(FULL, (endb || qb < 0) ? (int)(int16_t)(GO2 >> 16) : vb, 31);
+      const int ca = __shfl_sync(FULL, (enda || qa < 0) ? 0 : va, 31);
+      const int cb = __shfl_sync(FULL, (endb || qb < 0) ? 0 : vb, 31);
       carry = (uint32_t)(uint16_t)(int16_t)ca | ((uint32_t)(uint16_t)(int16_t)cb << 16);
     }
   }

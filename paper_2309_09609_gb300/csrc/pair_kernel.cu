@@ -21,7 +21,7 @@ namespace swgb {
 // updates column t - PQ*k - q at step t (Section II-B, intra-task
 // parallelism with neighbour border exchange):
 //   * quarter q needs the bottom row of quarter q - 1 at the same column
-//     (produced one step earlier) and its H' one column back (two steps
+//     (produced one step earlier) and its H one column back (two steps
 //     earlier), so the PQ quarter updates of a step are independent;
 //   * quarter 0 receives the bottom row of lane k - 1 (its quarter PQ - 1,
 //     one step earlier) by __shfl_up_sync; lane 0 reads the previous pass's
@@ -29,8 +29,7 @@ namespace swgb {
 //     c is read at step c and rewritten at step c + 32*PQ - 1).
 // Residues are staged in a per-warp shared-memory ring 128 columns ahead;
 // quarter 0 loads the profile row of its column (16 bytes per 16 rows) and
-// later quarters reuse its words.  Values carry the +Go bias of the inter-task kernel, and a
-// pair half whose S' reaches the threshold is recomputed in int32 like any
+// later quarters reuse its words.  A pair half whose S reaches the threshold is recomputed in int32 like any
 // other saturated pair.
 constexpr int PQ = 4;                      // quarters (independent chains) per lane
 constexpr int PHALF = NCODES * 32 * 16;    // int8 [code][lane][16 rows]: one 16-row half
@@ -79,10 +78,8 @@ pair_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Scra
   const int64_t total = PR == 32 ? first : first + (int64_t)(npairs - nwide) * P->pair_queries;
   if (total <= 0) return;  // uniform over the grid
   unsigned long long* counter = PR == 32 ? &st->pair_work32 : &st->pair_work;
-  const int go = P->go;
-  uint32_t GO2, NGE2, MGO;  // (Go, Go), (-Ge, -Ge), -(Go, Go)
-  gap_words<G>(P, GO2, NGE2, MGO);
-  const uint32_t one = (uint32_t)P->one;
+  uint32_t GO2, NGE2;  // (Go, Go), (-Ge, -Ge)
+  gap_words<G>(P, GO2, NGE2);
   constexpr int ROWS = 32 * PR;
   for (;;) {
     unsigned long long it = 0;
@@ -120,7 +117,7 @@ pair_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Scra
       *(uint32_t*)(ring0 + c % PRING) = w0;
       *(uint32_t*)(ring1 + c % PRING) = w1;
     };
-    uint32_t smax = GO2;
+    uint32_t smax = 0u;  // S, both subjects
     for (int p = 0; p < npass; p++) {
       __syncwarp();
       // this lane's PR rows, 16 at a time
@@ -132,21 +129,21 @@ pair_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Scra
         // the row above the matrix, for the first pass's steady-state steps
         // (lane 0 reads column j at step j; lane 31 rewrites it 127 steps later)
         if (p == 0)
-          for (int j = lane; j < n0; j += 32) hb[j] = make_uint2(GO2, 0u);
+          for (int j = lane; j < n0; j += 32) hb[j] = make_uint2(0u, 0u);
       }
       __syncwarp();
       uint32_t Hp[PR], E[PR];
 #pragma unroll
       for (int r = 0; r < PR; r++) {
-        Hp[r] = GO2;  // H(i, 0) = 0
-        E[r] = 0u;    // E(i, 1) = -Go
+        Hp[r] = 0u;  // H(i, 0) = 0
+        E[r] = 0u;   // any E(i, 1) <= 0 gives the same H
       }
-      // quarter q's bottom-row H' one and two steps back, its F' one step back
+      // quarter q's bottom-row H one and two steps back, its F one step back
       uint32_t qh1[PQ], qh2[PQ], qf1[PQ];
 #pragma unroll
       for (int k = 0; k < PQ; k++) {
-        qh1[k] = GO2;
-        qh2[k] = GO2;
+        qh1[k] = 0u;
+        qh2[k] = 0u;
         qf1[k] = 0u;
       }
       // profile vectors of the last four steps in slot (t mod 4): quarter q at
@@ -161,7 +158,7 @@ pair_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Scra
         VA2[k] = make_uint4(0u, 0u, 0u, 0u);
         VB2[k] = make_uint4(0u, 0u, 0u, 0u);
       }
-      uint32_t hdiag = GO2, out_h = GO2, out_f = 0u;
+      uint32_t hdiag = 0u, out_h = 0u, out_f = 0u;
       const bool last_pass = (p == npass - 1);
       const int steps = n0 + 32 * PQ - 1;
       // ring position of column t0 - PQ*lane; a multiple of 4, as is PRING
@@ -193,11 +190,11 @@ pair_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Scra
             const uint2 bv = hb[min(t, n0 - 1)];
             const bool from_scratch = p > 0 && t < n0;
             if (lane == 0) {
-              in_h = from_scratch ? bv.x : GO2;  // else H(0, j) = 0
-              in_f = from_scratch ? bv.y : 0u;   // else F(1, j) = -Go
+              in_h = from_scratch ? bv.x : 0u;  // else H(0, j) = 0
+              in_f = from_scratch ? bv.y : 0u;  // else any F(1, j) <= 0
             }
           } else {
-            // the first pass's row holds (H', F') = (Go, 0) here (filled
+            // the first pass's row holds (H, F) = (0, 0) here (filled
             // before the pass), so the value needs no test either
             const uint2 bv = hb[t];
             if (lane == 0) {
@@ -211,8 +208,8 @@ pair_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Scra
             in_h = v.x;
             in_f = v.y;
           } else {
-            in_h = GO2;  // H(0, j) = 0
-            in_f = 0u;   // F(1, j) = -Go
+            in_h = 0u;  // H(0, j) = 0
+            in_f = 0u;  // any F(1, j) <= 0
           }
         }
         const int ra = ring0[pos + U];
@@ -242,28 +239,29 @@ pair_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Scra
           nh[k] = qh1[k];
           nf[k] = qf1[k];
           if (active) {
-            uint32_t hd = k == 0 ? hdiag : qh2[k - 1];  // H' one row up, one column back
-            uint32_t f = k == 0 ? in_f : qf1[k - 1];    // F' of this quarter's first row
-            uint32_t hprev = 0;
+            uint32_t hd = k == 0 ? hdiag : qh2[k - 1];  // H one row up, one column back
+            uint32_t f = k == 0 ? in_f : qf1[k - 1];    // F of this quarter's first row
+            uint32_t xprev = 0;
 #pragma unroll
             for (int i = 0; i < PQR; i++) {
               const int r = k * PQR + i;
               uint32_t e = E[r];
-              const uint32_t h = packed_cell<G>(hd, prmt(wa[k][i >> 2], wb[k][i >> 2],
-                                                      sext_pair_sel(i & 3)), e, f, GO2, NGE2, MGO, one);
+              uint32_t x;
+              const uint32_t h = packed_cell(hd, prmt(wa[k][i >> 2], wb[k][i >> 2],
+                                                   sext_pair_sel(i & 3)), e, f, x, GO2, NGE2);
               hd = Hp[r];
               Hp[r] = h;
               E[r] = e;
               if (i & 1)
-                smax = __vimax3_s16x2(smax, hprev, h);
+                smax = __vimax3_s16x2(smax, xprev, x);
               else
-                hprev = h;
+                xprev = x;
             }
             nh[k] = Hp[k * PQR + PQR - 1];
             nf[k] = f;
             if (k == PQ - 1 && lane == 31 && !last_pass) hb[col] = make_uint2(nh[k], f);
           } else if (col < 0) {
-            nh[k] = GO2;  // left of the matrix: H = 0
+            nh[k] = 0u;  // left of the matrix: H = 0
           }
         }
         hdiag = in_h;
@@ -310,7 +308,7 @@ pair_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Scra
     for (int o = 16; o > 0; o >>= 1) smax = __vmaxs2(smax, __shfl_xor_sync(FULL, smax, o));
     if (lane < 2 && (lane == 0 || has1)) {
       const int sidx = lane ? s1 : s0;
-      const int sb = (int)(int16_t)(lane ? (smax >> 16) : (smax & 0xffffu));  // S'
+      const int sb = (int)(int16_t)(lane ? (smax >> 16) : (smax & 0xffffu));  // S
       const int orig = db.perm[sidx];
       if (orig >= 0) {
         if (sb >= P->sat_threshold) {
@@ -320,7 +318,7 @@ pair_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Scra
           else  // the list is full: mark the pair for the host's next recompute round
             P->scores[(int64_t)q * db.n + orig] = FLAG_SENTINEL;
         } else {
-          P->scores[(int64_t)q * db.n + orig] = sb - go;
+          P->scores[(int64_t)q * db.n + orig] = sb;
         }
       }
     }

@@ -53,7 +53,7 @@ struct DbView {
 // Kept in device memory (not kernel arguments) so that one captured CUDA graph
 // serves every batch: a new search only rewrites this block.
 struct SearchParams {
-  uint4 init_border;      // packed (H', F') of the row above the matrix: (Go, 0, Go, 0)
+  uint4 init_border;      // packed (H, F) of the row above the matrix: zeros
   const uint8_t* qres;    // concatenated query codes
   const int64_t* qoff;    // [nq]
   const int32_t* qlen;    // [nq]
@@ -86,8 +86,7 @@ struct SearchParams {
   int32_t g_first;        // first inter-task group (n_long / GROUP)
   int32_t go;             // Go = gap_open + gap_extend  (Eq. 2-3)
   int32_t ge;             // Ge = gap_extend
-  int32_t sat_threshold;  // packed path: S + Go >= this (32767 - max SM) is recomputed in int32
-  int32_t one;            // 1, read at run time so multiply-adds stay integer multiply-adds
+  int32_t sat_threshold;  // packed path: S >= this (32767 - max SM - Go) is recomputed in int32
   int8_t sm[NCODES * NCODES];  // SM(query code, subject code), PAD row/column = PAD_SCORE
 };
 
@@ -113,7 +112,7 @@ struct Scratch {
   int64_t intra_stride;       // int2 per warp
   int2* flags;                // saturated pairs: (query index, sorted subject index)
   int64_t flag_capacity;
-  uint2* pair_border;         // packed intra-task kernels, per warp: [column] (H', F') words;
+  uint2* pair_border;         // packed intra-task kernels, per warp: [column] (H, F) words;
                               // rows [0, pair_rows16) for pair_kernel<16>, the rest for <32>
   int64_t pair_stride;        // uint2 per warp
   int64_t pair_rows16;
