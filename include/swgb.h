@@ -96,9 +96,12 @@ int32_t sw_db_max_length(const sw_db* db);
 /* Tuning of the exact search; every field has a safe default (zero-init and
  * call sw_options_default).  None of them changes a score. */
 typedef struct {
-  int32_t rows_per_thread;   /* query rows per thread in the packed inter-task kernel: 16 or 32 */
-  int32_t warps_per_block;   /* 4 or 8 */
-  int32_t long_cutoff;       /* subjects longer than this use the intra-task kernel */
+  int32_t rows_per_thread;   /* 16 or 32, warps_per_block 1..8, inter_columns 4 or 8: shapes of an
+                                earlier one-query kernel; checked, and without effect (the
+                                lane-group kernel takes its shape from each query's length) */
+  int32_t warps_per_block;
+  int32_t long_cutoff;       /* subjects longer than this are the long subjects: with two or more
+                                queries, a kernel of their own may score them (two_query_long) */
   int32_t intra_rows;        /* query rows per lane in the int32 intra-task kernel: 8 or 16 */
   int32_t use_graph;         /* 1: capture the launch sequence in a CUDA graph */
   int32_t force_int32;       /* 1: all subjects through the int32 intra-task kernel */
@@ -106,25 +109,19 @@ typedef struct {
                                 kernel every group whose (query, group) work item would
                                 exceed a quarter of one warp's share of the search (load
                                 balance for few long queries); default 0 */
-  int32_t wide_min_len;      /* long subjects are scored 32 query rows per lane (1024-row
-                                passes, fewer instructions per cell, half the warps) instead
-                                of 16 (512-row passes) for queries of at least this many
-                                residues whose padded cost is lower that way ... default 0 */
-  int32_t wide_min_subject;  /* ... against subject pairs whose longer subject has at least
-                                this many residues, or against every pair when the search
-                                has fewer (pair, query) items than 16-row warps; default 4096 */
-  int32_t inter_columns;     /* subject columns per wavefront in the packed inter-task kernel
-                                with rows_per_thread 32: 4 or 8 (16 rows always use 4);
-                                default 8 */
-  int32_t overlap_kernels;   /* 1: the inter-task kernel runs alongside the pair kernels
-                                instead of after them, so its blocks take the SMs that their
-                                tails leave (lower latency for small searches); search_ms and
-                                pair_ms then overlap, both from the start; default 0 */
-  int32_t two_query;         /* inter-task scoring with two queries per 32-bit word against one
-                                subject per lane (no per-cell byte merge, 4.5 instead of 5.5
-                                ALU operations per word): 0 never, 1 when the plan's cost
-                                model expects it to be faster (default), 2 whenever a search
-                                has at least two queries */
+  int32_t wide_min_len;      /* >= 0, as wide_min_subject: without effect, as rows_per_thread */
+  int32_t wide_min_subject;
+  int32_t inter_columns;     /* see rows_per_thread */
+  int32_t overlap_kernels;   /* 1: when the long and the short subjects go to kernels of their
+                                own, the two run side by side instead of one after the other, so
+                                the second's blocks take the SMs that the first's tail leaves;
+                                search_ms and pair_ms then overlap, both from the start;
+                                default 0 */
+  int32_t two_query;         /* scoring of the short subjects with two queries per 32-bit word
+                                against one subject per lane (no per-cell byte merge, 3.5
+                                instead of 4.5 ALU operations per word): 0 never, 1 when the
+                                plan's cost model expects it to be faster than the lane groups
+                                (default), 2 whenever a search has at least two queries */
   int32_t two_query_rows;    /* query rows per strip of that kernel: 16, 24 or 32 (default) */
   int32_t two_query_pairs;   /* stream pairs of the two-query layouts, inter- and intra-task
                                 (0: the plan's choice, per layout; otherwise at most
@@ -145,27 +142,28 @@ void sw_options_default(sw_options* opt);
 /* Statistics of the last search run through a plan. */
 typedef struct {
   int64_t cells;             /* sum(query lengths) * sum(subject lengths) */
-  int64_t inter_items;       /* (query, group of 64 subjects) work items of the two-subject
-                                inter-task kernel (0 when the two-query kernel ran) */
+  int64_t inter_items;       /* (query, group of 64 short subjects) pairs scored with two
+                                subjects per word (0 when the two-query kernel ran) */
   int64_t intra_items;       /* (query, long subject) work items */
   int64_t recomputed_pairs;  /* pairs whose 16-bit score saturated, redone in int32 */
   int32_t overflow_rounds;   /* extra rounds of the int32 kernel that the last search ran
                                 because it had more saturated pairs than the plan's flag list
                                 holds (0 normally); their time is not in recompute_ms */
   int32_t kernels_launched;  /* kernels of this library launched by the search */
-  float search_ms;           /* device time of the inter-task search kernel (CUDA events) */
+  float search_ms;           /* device time of the short subjects' kernel (CUDA events) */
   float recompute_ms;        /* device time of the int32 intra-task kernel (CUDA events):
                                 the recompute of saturated pairs, or every pair when the
-                                packed path is off */
-  float pair_ms;             /* device time of the packed intra-task kernels, both widths,
-                                from their fork to their join (CUDA events) */
+                                packed path is off; 0 when no pair could saturate */
+  float pair_ms;             /* device time of the long subjects' kernel (CUDA events); when one
+                                launch scored all subjects, its time is split between
+                                pair_ms and search_ms by their cells */
   int32_t pad_;
-  int64_t inter_cells;       /* cells scored by the inter-task kernel */
+  int64_t inter_cells;       /* cells of the short subjects */
   int64_t inter2_items;      /* (stream pair, half group) items of the two-query inter-task
-                                kernel; 0 when the one-query kernel scored the short subjects */
+                                kernel; 0 when the lane groups scored the short subjects */
   int64_t pair2_items;       /* (stream pair, group of 12 long subjects) items of the two-query
-                                intra-task kernel; 0 when the subject-pair kernels scored the
-                                long subjects */
+                                intra-task kernel; 0 when the lane groups scored the long
+                                subjects */
 } sw_stats;
 
 /* Creates a search context for up to max_queries queries holding up to
@@ -185,28 +183,25 @@ sw_status sw_plan_create(sw_db* db, int32_t max_queries, int64_t max_query_resid
 void sw_plan_destroy(sw_plan* plan);
 
 /* Exact scores of every query against every subject (Eq. 1-3), the batched
- * path: six persistent launches, each taking its work longest first from its
- * own atomic counter.  First, for the subjects longer than opt.long_cutoff,
- * one of two packed intra-task layouts: two queries per 32-bit word against
- * one subject per warp, over (pair of query streams, group of 12 subjects)
- * items; or two subjects per word, over (pair of subjects, query) items, at
- * 32 and at 16 query rows per lane, two launches side by side on two streams
- * (opt.wide_min_len and opt.wide_min_subject split the items between them).
- * Then one of two packed inter-task layouts for the other subjects: two
- * queries per word against one subject per lane, over (pair of query
- * streams, half of a group of 64 subjects) items, or two subjects per word,
- * over (query, group of 64 subjects) items.  opt.two_query_long and
- * opt.two_query with a cost model choose each layout per search; a single
- * query always takes the two-subject ones; the kernels of the other layout
- * find no items.  Last the int32 intra-task kernel recomputes every pair
- * whose 16-bit score may have saturated (one block per pair; more saturated
- * pairs than opt.flag_capacity are recomputed in further rounds before the
- * call returns).  With gap penalties too large for 16 bits, or
- * opt.force_int32, every pair goes to the int32 kernel instead (one warp per
- * pair).  The packed kernels are compiled with the gap penalties as
- * constants for (10, 2) and (11, 1), and read them at run time otherwise.
- * The launch sequence is replayed from a CUDA graph (one per such gap
- * setting) when opt.use_graph is set.
+ * path: up to three persistent launches, each taking its work longest first.
+ * The subjects longer than opt.long_cutoff and the others are each scored
+ * either with two queries per 32-bit word -- the long ones against one subject
+ * per warp, over (pair of query streams, group of 12 subjects) items, the
+ * others against one subject per lane, over (pair of query streams, half of a
+ * group of 64 subjects) items -- or with two subjects per word on groups of 8
+ * to 32 lanes, over (query, subject pairs) items; both parts go in one launch
+ * when both take the latter.  opt.two_query_long and opt.two_query with a cost
+ * model choose per search; a single query always takes the lane groups.  Last
+ * the int32 intra-task kernel recomputes every pair whose 16-bit score may
+ * have saturated (one block per pair; more saturated pairs than
+ * opt.flag_capacity are recomputed in further rounds before the call returns);
+ * it is left out when the lengths and the matrix allow no such score.  With
+ * gap penalties too large for 16 bits, or opt.force_int32, every pair goes to
+ * the int32 kernel instead (one warp per pair).  The packed kernels are
+ * compiled with the gap penalties as constants for (10, 2) and (11, 1), and
+ * read them at run time otherwise.  Several launches are replayed from a CUDA
+ * graph (one per such gap setting and set of kernels) when opt.use_graph is
+ * set.
  *   queries:   concatenated query codes (sum(q_lengths) bytes), host or device.
  *   q_lengths: n_queries int32, host or device.
  *   scores:    n_queries x n_subjects int32, host or device, written in full.

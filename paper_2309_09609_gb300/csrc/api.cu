@@ -6,12 +6,10 @@
 //     short (inter-task) and long (intra-task) part follows Section III-A.
 //   * sw_plan_*: a reusable search context.  Its device memory is allocated
 //     once (the host-order scores buffer at the first search that needs it);
-//     per search only the query block, the query-stream strip table and a
-//     parameter block are copied, and the kernel sequence (reset counters;
-//     the two pair-kernel widths on two streams; the two inter-task kernels,
-//     of which the plan gives one the items; the int32 kernel for saturated
-//     pairs) is replayed from a CUDA graph, one per gap class.  A flag-list
-//     overflow is recomputed in further rounds after the graph.
+//     per search one block is copied (parameters, zeroed counters, queries and
+//     work tables) and the kernels it needs are launched, several of them
+//     from a CUDA graph (one per gap class and set of kernels).  A flag-list
+//     overflow is recomputed in further rounds after that.
 //   * sw_search: through a plan kept by the database.
 //   * sw_search_plain: the int32 baseline, one kernel launch per query.
 //   * sw_align: optimal alignments with traceback of selected pairs.
@@ -387,8 +385,9 @@ static constexpr int kPackedMaxGap = 16384;
 static constexpr double kAutoCutoffMinCells = 1e10;
 static constexpr int kMaxGap = 100000000;
 
+// *max_sm: the largest matrix entry (optional).
 static sw_status fill_scoring(SearchParams& P, int32_t gap_open, int32_t gap_extend,
-                              const int8_t* matrix, bool* packed_ok) {
+                              const int8_t* matrix, bool* packed_ok, int* max_sm = nullptr) {
   if (gap_open < 0 || gap_extend < 0 || gap_open > kMaxGap || gap_extend > kMaxGap)
     return sw_set_error(SW_EINVAL, "gap penalties must be in [0, %d]", kMaxGap);
   int8_t m[ALPHA * ALPHA];
@@ -411,58 +410,68 @@ static sw_status fill_scoring(SearchParams& P, int32_t gap_open, int32_t gap_ext
   P.sat_threshold = S16_LIMIT - maxsm - P.go;
   P.init_border = make_uint4(0u, 0u, 0u, 0u);
   *packed_ok = (P.go + P.ge) <= kPackedMaxGap;
+  if (max_sm) *max_sm = maxsm;
   return SW_OK;
 }
 
 // ---- plan ---------------------------------------------------------------------------------
+constexpr int MAX_SEGS = 3;  // segments of the lane-group kernel per query: one per group size
+
+// The upload block: parameters, state, then the tables, each on a 16-byte boundary.
+static constexpr size_t block_align(size_t bytes) { return (bytes + 15) & ~(size_t)15; }
+static constexpr size_t BLOCK_HEADER = block_align(sizeof(SearchParams)) + block_align(sizeof(SearchState));
+
+// The kernels of one search (bits of sw_plan::kernels): the two-query kernel
+// or the lane groups for the long subjects, the lane groups (for the short
+// subjects, or for all in one launch) or the two-query kernel for the short
+// ones, and the int32 kernel.
+enum { K_PAIR2 = 1, K_LANES_LONG = 2, K_LANES = 4, K_INTER2 = 8, K_INT32 = 16, K_SETS = 32 };
+
 struct sw_plan {
   sw_db* db = nullptr;
   int device = 0;           // the database's device, kept for plan_free
   sw_options opt{};
-  KernelConfig kc{};        // inter-task kernel
   KernelConfig kc2{};       // inter-task kernel, two queries per word
   KernelConfig ikc{};       // int32 intra-task kernel
   int32_t max_queries = 0;
   int64_t max_residues = 0;
   int32_t g_first = 0;      // first inter-task group under the cutoff
-  int32_t pair_blocks16 = 0;  // grid of pair_kernel<16>
-  int32_t pair_blocks32 = 0;  // grid of pair_kernel<32>
+  int32_t sms = 1;
   int32_t pair2_blocks = 0;   // grid of pair2q_kernel
-  // device buffers
-  uint8_t* qres = nullptr;
-  int64_t* qoff = nullptr;
-  int32_t* qlen = nullptr;
-  int32_t* qorder = nullptr;
-  int4* strips = nullptr;         // strip table of the two-query kernel
-  int2* spairs = nullptr;         // its stream pairs
-  int64_t strip_capacity = 0;
-  int32_t spair_capacity = 0;
+  int32_t lane_blocks = 0;    // grid of lane_kernel
+  // One device block and its pinned image hold what a search uploads, in one
+  // copy: the parameter block, the zeroed state, and the tables that follow
+  // (the query arrays, the lane-group segments, the stream pairs, the strip
+  // table, the residues), packed back to back.
+  uint8_t* block = nullptr;
+  uint8_t* block_h = nullptr;
+  size_t block_bytes = 0;
+  SearchParams* params = nullptr;   // in block
+  SearchState* state = nullptr;     // in block
+  SearchState* state_h = nullptr;   // pinned: the state a search left
+  // the tables while a search is planned
+  std::vector<int4> strips;         // strip tables of the two-query kernels
+  std::vector<int2> spairs;         // their stream pairs
+  std::vector<LaneSeg> segs;
   int32_t* scores_dev = nullptr;  // used when the caller's scores live on the host:
                                   // allocated by the first such search
   cudaStream_t stream = nullptr;  // the stream of the search in flight
-  SearchParams* params = nullptr;
-  SearchState* state = nullptr;
   Scratch scr{};
-  // pinned host staging
-  SearchParams* params_h = nullptr;
-  SearchState* state_h = nullptr;
-  uint8_t* qres_h = nullptr;
-  int64_t* qoff_h = nullptr;
-  int32_t* qlen_h = nullptr;
-  int32_t* qorder_h = nullptr;
-  int4* strips_h = nullptr;
-  int2* spairs_h = nullptr;
-  // graphs, one per gap class (the packed kernels are compiled per class)
-  cudaGraphExec_t graphs[GAP_CLASSES] = {};
-  int gclass = 0;  // gap class of the search being staged
+  // graphs, one per gap class (the packed kernels are compiled per class) and
+  // set of kernels
+  cudaGraphExec_t graphs[GAP_CLASSES][K_SETS] = {};
+  int gclass = 0;   // gap class of the search being staged ...
+  int kernels = 0;  // ... and its kernels
+  int lane_grid = 0;
   cudaEvent_t done = nullptr;
-  // before the pair kernel, before and after the inter-task kernel, after recompute
+  // before the long subjects' kernel, before and after the short subjects'
+  // kernel, after the recompute
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
-  // the two pair-kernel widths run on two streams: fork after the reset, join
-  // before the inter-task kernel
-  cudaStream_t side = nullptr, side2 = nullptr;
-  cudaEvent_t fork = nullptr, join = nullptr, join2 = nullptr;
-  cudaEvent_t ev_join = nullptr;  // overlap: after the pair and inter-task kernels
+  // overlap_kernels: the short subjects' kernel on a stream of its own
+  cudaStream_t side = nullptr;
+  cudaEvent_t fork = nullptr, join = nullptr;
+  cudaEvent_t ev_join = nullptr;  // overlap: after both
+  double long_share = 0;  // the long subjects' share of the cells (one launch for all)
   bool in_flight = false;
   sw_stats stats{};
   sw_stats pending{};
@@ -475,38 +484,24 @@ static void plan_free(sw_plan* p) {
   // the plan's own device: its database may already be gone (a garbage
   // collector can finalize the two in either order)
   cudaSetDevice(p->device);
-  for (auto& g : p->graphs)
-    if (g) cudaGraphExecDestroy(g);
+  for (auto& c : p->graphs)
+    for (auto& g : c)
+      if (g) cudaGraphExecDestroy(g);
   if (p->done) cudaEventDestroy(p->done);
   for (auto& e : p->ev)
     if (e) cudaEventDestroy(e);
   if (p->fork) cudaEventDestroy(p->fork);
   if (p->join) cudaEventDestroy(p->join);
-  if (p->join2) cudaEventDestroy(p->join2);
   if (p->ev_join) cudaEventDestroy(p->ev_join);
   if (p->side) cudaStreamDestroy(p->side);
-  if (p->side2) cudaStreamDestroy(p->side2);
-  cudaFree(p->qres);
-  cudaFree(p->qoff);
-  cudaFree(p->qlen);
-  cudaFree(p->qorder);
-  cudaFree(p->strips);
-  cudaFree(p->spairs);
+  cudaFree(p->block);
   cudaFree(p->scores_dev);
-  cudaFree(p->params);
-  cudaFree(p->state);
   cudaFree(p->scr.inter_border);
   cudaFree(p->scr.intra_border);
   cudaFree(p->scr.flags);
   cudaFree(p->scr.pair_border);
-  cudaFreeHost(p->params_h);
+  cudaFreeHost(p->block_h);
   cudaFreeHost(p->state_h);
-  cudaFreeHost(p->qres_h);
-  cudaFreeHost(p->qoff_h);
-  cudaFreeHost(p->qlen_h);
-  cudaFreeHost(p->qorder_h);
-  cudaFreeHost(p->strips_h);
-  cudaFreeHost(p->spairs_h);
   cudaSetDevice(cur);
   cudaGetLastError();  // a failed free or device switch leaves no stale error
   delete p;
@@ -562,19 +557,7 @@ extern "C" sw_status sw_plan_create(sw_db* db, int32_t max_queries, int64_t max_
 
   int dev_sms = 0;
   cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, db->device);
-  // eight columns per wavefront need 32 rows per thread; 16 rows use four
-  const int cols = o.rows_per_thread == 32 ? o.inter_columns : 4;
-  const int bps = inter_blocks_per_sm(o.rows_per_thread, cols, o.warps_per_block);
-  if (bps < 1) {
-    plan_free(p);
-    return sw_set_error(SW_ECUDA, "inter-task kernel cannot launch with %d warps (rows %d)",
-                        o.warps_per_block, o.rows_per_thread);
-  }
-  p->kc.variant = o.rows_per_thread;
-  p->kc.cols = cols;
-  p->kc.warps = o.warps_per_block;
-  p->kc.blocks = dev_sms * bps;
-  p->kc.smem = inter_smem_bytes(o.rows_per_thread, o.warps_per_block);
+  p->sms = dev_sms;
   // the two-query kernel: one block per SM, as many warps as its shared memory allows
   const int warps2 = inter2q_warps(o.two_query_rows);
   const int bps2 = inter2q_blocks_per_sm(o.two_query_rows, warps2);
@@ -584,13 +567,10 @@ extern "C" sw_status sw_plan_create(sw_db* db, int32_t max_queries, int64_t max_
                         o.two_query_rows);
   }
   p->kc2.variant = o.two_query_rows;
-  p->kc2.cols = 8;
   p->kc2.warps = warps2;
   p->kc2.blocks = dev_sms * bps2;
   p->kc2.smem = inter2q_smem_bytes(o.two_query_rows, warps2);
-  // the two inter-task kernels run one after the other and share the border scratch
-  const int64_t W = std::max<int64_t>((int64_t)p->kc.blocks * p->kc.warps,
-                                      (int64_t)p->kc2.blocks * p->kc2.warps);
+  const int64_t W = (int64_t)p->kc2.blocks * p->kc2.warps;
   // one block of INTRA_WARPS per SM: enough for the int32 items, and the
   // border scratch (one subject-length row per warp) stays bounded
   if (intra_blocks_per_sm(o.intra_rows) < 1) {
@@ -602,27 +582,26 @@ extern "C" sw_status sw_plan_create(sw_db* db, int32_t max_queries, int64_t max_
   p->ikc.blocks = dev_sms;
   p->ikc.smem = intra_smem_bytes(o.intra_rows);
   const int64_t WI = (int64_t)p->ikc.blocks * INTRA_WARPS;
-  const int pbps16 = pair_blocks_per_sm(16), pbps32 = pair_blocks_per_sm(32);
-  if (pbps16 < 1 || pbps32 < 1) {
+  const int lbps = lane_blocks_per_sm();
+  if (lbps < 1) {
     plan_free(p);
-    return sw_set_error(SW_ECUDA, "packed intra-task kernel cannot launch");
+    return sw_set_error(SW_ECUDA, "lane-group kernel cannot launch");
   }
-  p->pair_blocks16 = dev_sms * pbps16;
-  p->pair_blocks32 = dev_sms * pbps32;
+  p->lane_blocks = dev_sms * lbps;
   const int p2bps = pair2q_blocks_per_sm();
   if (p2bps < 1) {
     plan_free(p);
     return sw_set_error(SW_ECUDA, "two-query packed intra-task kernel cannot launch");
   }
   p->pair2_blocks = dev_sms * p2bps;
-  // the two widths may run at the same time, each on its own scratch rows;
-  // the two-query kernel runs instead of them and uses the first rows
-  const int64_t WP = std::max<int64_t>((int64_t)(p->pair_blocks16 + p->pair_blocks32) * PAIR_WARPS,
-                                       (int64_t)p->pair2_blocks * pair2q_warps());
-  p->scr.pair_rows16 = (int64_t)p->pair_blocks16 * PAIR_WARPS;
+  // border rows of the two-query intra-task kernel and of the lane-group
+  // kernel, which share them unless overlap_kernels runs them side by side
+  const int64_t rows2 = (int64_t)p->pair2_blocks * pair2q_warps();
+  const int64_t rowsl = (int64_t)p->lane_blocks * LANE_WARPS;
+  const int64_t WP = o.overlap_kernels ? rows2 + rowsl : std::max(rows2, rowsl);
+  p->scr.lane_row0 = o.overlap_kernels ? rows2 : 0;
 
   cudaError_t e = injected_fault("alloc") ? cudaErrorMemoryAllocation : cudaSuccess;
-  const int64_t nres = std::max<int64_t>(max_query_residues, 1);
   p->scr.inter_stride_vec = (int64_t)(L_inter / CHUNK) * 4 * 32;
   p->scr.intra_stride = std::max(v.max_len, 1);
   // (+4: the two-query pair kernel loads its border 4 columns ahead)
@@ -631,47 +610,42 @@ extern "C" sw_status sw_plan_create(sw_db* db, int32_t max_queries, int64_t max_
                             ? (int64_t)o.flag_capacity
                             : std::min<int64_t>((int64_t)max_queries * std::max<int64_t>(v.n, 1),
                                                 DEFAULT_FLAG_CAPACITY);
-  if (e == cudaSuccess) e = dalloc(&p->scr.pair_border, (size_t)(WP * p->scr.pair_stride));
-  if (e == cudaSuccess) e = dalloc(&p->qres, nres);
-  if (e == cudaSuccess) e = dalloc(&p->qoff, max_queries);
-  if (e == cudaSuccess) e = dalloc(&p->qlen, max_queries);
-  if (e == cudaSuccess) e = dalloc(&p->qorder, 2 * (size_t)max_queries);  // qorder, then qpair
   // strips of the two tables (the inter-task kernel's, at least 16 rows per
   // strip, and the intra-task kernel's, 32): every query padded to whole
   // strips (at least one), and as many empty halves at most; stream pairs:
   // one per two queries at most, per table
-  p->strip_capacity = 2 * (max_query_residues / 16 + 2 * (int64_t)max_queries) + 16;
-  p->spair_capacity = 2 * (max_queries / 2 + 1);
-  if (e == cudaSuccess) e = dalloc(&p->strips, (size_t)p->strip_capacity);
-  if (e == cudaSuccess) e = dalloc(&p->spairs, (size_t)p->spair_capacity);
-  if (e == cudaSuccess) e = dalloc(&p->params, 1);
-  if (e == cudaSuccess) e = dalloc(&p->state, 1);
+  p->strips.resize((size_t)(2 * (max_query_residues / 16 + 2 * (int64_t)max_queries) + 16));
+  p->spairs.resize((size_t)(2 * (max_queries / 2 + 1)));
+  p->segs.resize((size_t)MAX_SEGS * max_queries);
+  p->block_bytes = BLOCK_HEADER + block_align((size_t)max_queries * sizeof(int64_t)) +
+                   2 * block_align((size_t)max_queries * sizeof(int32_t)) +
+                   block_align(p->segs.size() * sizeof(LaneSeg)) +
+                   block_align(p->spairs.size() * sizeof(int2)) +
+                   block_align(p->strips.size() * sizeof(int4)) +
+                   block_align((size_t)std::max<int64_t>(max_query_residues, 1));
+  if (e == cudaSuccess) e = dalloc(&p->scr.pair_border, (size_t)(WP * p->scr.pair_stride));
+  if (e == cudaSuccess) e = dalloc(&p->block, p->block_bytes);
   if (e == cudaSuccess) e = dalloc(&p->scr.inter_border, (size_t)(W * std::max<int64_t>(p->scr.inter_stride_vec, 1)));
   if (e == cudaSuccess) e = dalloc(&p->scr.intra_border, (size_t)(WI * p->scr.intra_stride));
   if (e == cudaSuccess) e = dalloc(&p->scr.flags, (size_t)p->scr.flag_capacity);
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&p->params_h, sizeof(SearchParams));
+  if (e == cudaSuccess) e = cudaMallocHost((void**)&p->block_h, p->block_bytes);
   if (e == cudaSuccess) e = cudaMallocHost((void**)&p->state_h, sizeof(SearchState));
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&p->qres_h, nres);
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&p->qoff_h, sizeof(int64_t) * max_queries);
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&p->qlen_h, sizeof(int32_t) * max_queries);
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&p->qorder_h, sizeof(int32_t) * 2 * max_queries);
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&p->strips_h, sizeof(int4) * p->strip_capacity);
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&p->spairs_h, sizeof(int2) * p->spair_capacity);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->done, cudaEventDisableTiming);
   for (auto& ev : p->ev)
     if (e == cudaSuccess) e = cudaEventCreate(&ev);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->fork, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->join, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&p->side2, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->join2, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreate(&p->ev_join);
   if (e != cudaSuccess) {
     sw_status st = sw_set_cuda_error(e, "sw_plan_create: allocation");
     plan_free(p);
     return st;
   }
-  memset(p->params_h, 0, sizeof(SearchParams));
+  p->params = (SearchParams*)p->block;
+  p->state = (SearchState*)(p->block + block_align(sizeof(SearchParams)));
+  memset(p->block_h, 0, p->block_bytes);
+  memset(p->state_h, 0, sizeof(SearchState));
   *out = p;
   return SW_OK;
 }
@@ -681,62 +655,64 @@ extern "C" void sw_plan_destroy(sw_plan* plan) {
   plan_free(plan);
 }
 
-// The device work of one search: reset the counters, then the packed
-// intra-task kernel (long subjects), the inter-task kernel (the rest) and the
-// int32 intra-task kernel (saturated pairs, or everything when the packed path
-// is off).  Events around the kernels give their device time on the launching
-// stream.  Under stream capture an event record only orders the capture
-// unless it carries cudaEventRecordExternal, which makes it a real
-// event-record node of the graph; outside capture that flag is illegal.
+// The device work of one search, after the upload of its parameters and
+// zeroed counters: the kernel of the long subjects, that of the short ones
+// (or the lane-group kernel for both) and the int32 intra-task kernel
+// (saturated pairs, or everything when the packed path is off) -- those of
+// p->kernels, in launches of their own.  Events around the kernels give their
+// device time on the launching stream.  Under stream capture an event record
+// only orders the capture unless it carries cudaEventRecordExternal, which
+// makes it a real event-record node of the graph; outside capture that flag
+// is illegal.
 static cudaError_t record(cudaEvent_t ev, cudaStream_t s, bool capturing) {
   return capturing ? cudaEventRecordWithFlags(ev, s, cudaEventRecordExternal)
                    : cudaEventRecord(ev, s);
 }
 
 static cudaError_t enqueue_kernels(sw_plan* p, cudaStream_t s, bool capturing) {
-  cudaError_t e = cudaMemsetAsync(p->state, 0, sizeof(SearchState), s);
-  if (e == cudaSuccess) e = record(p->ev[0], s, capturing);
-  // pair_kernel<32> on the side stream, pair_kernel<16> on this one: the two
-  // persistent grids share the SMs as their blocks come and go, so their
-  // tails overlap.  Under capture the fork and join become graph edges.
-  if (e == cudaSuccess) e = cudaEventRecord(p->fork, s);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(p->side, p->fork, 0);
-  const int gc = p->gclass;
-  if (e == cudaSuccess) e = launch_pairs(32, gc, p->pair_blocks32, p->db->view, p->params, p->state, p->scr, p->side);
-  // the two-query intra-task kernel, when the plan chose it for this search
-  // (the subject-pair kernels then find no items and return at once)
-  if (e == cudaSuccess) e = launch_pair2q(gc, p->pair2_blocks, p->db->view, p->params, p->state, p->scr, p->side);
-  if (e == cudaSuccess) e = launch_pairs(16, gc, p->pair_blocks16, p->db->view, p->params, p->state, p->scr, s);
-  if (p->opt.overlap_kernels) {
-    // the inter-task kernel too, on a third stream and issued after the pair
-    // kernels: one of its blocks needs a whole SM's registers, so it starts on
-    // an SM when the pair blocks there run out of work, and no SM idles in
-    // their tails
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(p->side2, p->fork, 0);
-    if (e == cudaSuccess) e = launch_inter(p->kc, gc, p->db->view, p->params, p->state, p->scr, p->side2);
-    if (e == cudaSuccess) e = launch_inter2q(p->kc2, gc, p->db->view, p->params, p->state, p->scr, p->side2);
-    if (e == cudaSuccess) e = record(p->ev[2], p->side2, capturing);
-    if (e == cudaSuccess) e = cudaEventRecord(p->join2, p->side2);
+  const int gc = p->gclass, set = p->kernels;
+  const DbView& v = p->db->view;
+  // with a kernel for the long subjects and one for the short ones,
+  // overlap_kernels issues the latter on a second stream: one of its blocks
+  // needs a whole SM's shared memory, so it starts on an SM when the blocks
+  // there run out of work, and no SM idles in their tails
+  const bool is_long = set & (K_PAIR2 | K_LANES_LONG), is_short = set & (K_LANES | K_INTER2);
+  const bool overlap = p->opt.overlap_kernels && is_long && is_short;
+  cudaError_t e = record(p->ev[0], s, capturing);
+  if (e == cudaSuccess && overlap) e = cudaEventRecord(p->fork, s);
+  if (e == cudaSuccess && (set & K_PAIR2))
+    e = launch_pair2q(gc, p->pair2_blocks, v, p->params, p->state, p->scr, s);
+  if (e == cudaSuccess && (set & K_LANES_LONG))
+    e = launch_lanes(gc, p->lane_grid, v, p->params, p->state, p->scr, s);
+  cudaStream_t s2 = s;
+  if (overlap) {
+    s2 = p->side;
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s2, p->fork, 0);
   }
-  if (e == cudaSuccess) e = cudaEventRecord(p->join, p->side);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->join, 0);
-  if (e == cudaSuccess) e = record(p->ev[1], s, capturing);
-  if (p->opt.overlap_kernels) {
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->join2, 0);
+  if (e == cudaSuccess && is_long && is_short) e = record(p->ev[1], s, capturing);
+  if (e == cudaSuccess && (set & K_LANES))
+    e = launch_lanes(gc, p->lane_grid, v, p->params, p->state, p->scr, s2);
+  if (e == cudaSuccess && (set & K_INTER2))
+    e = launch_inter2q(p->kc2, gc, v, p->params, p->state, p->scr, s2);
+  if (e == cudaSuccess) e = record(p->ev[2], s2, capturing);
+  if (overlap) {
+    if (e == cudaSuccess) e = cudaEventRecord(p->join, s2);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(s, p->join, 0);
     if (e == cudaSuccess) e = record(p->ev_join, s, capturing);
-  } else {
-    if (e == cudaSuccess) e = launch_inter(p->kc, gc, p->db->view, p->params, p->state, p->scr, s);
-    if (e == cudaSuccess) e = launch_inter2q(p->kc2, gc, p->db->view, p->params, p->state, p->scr, s);
-    if (e == cudaSuccess) e = record(p->ev[2], s, capturing);
   }
-  if (e == cudaSuccess) e = launch_intra(p->ikc, p->db->view, p->params, p->state, p->scr, s);
-  if (e == cudaSuccess) e = record(p->ev[3], s, capturing);
+  if (set & K_INT32) {
+    if (e == cudaSuccess) e = launch_intra(p->ikc, v, p->params, p->state, p->scr, s);
+    if (e == cudaSuccess) e = record(p->ev[3], s, capturing);
+  }
   return e;
 }
 
 static cudaError_t run_kernels(sw_plan* p, cudaStream_t s) {
-  if (!p->opt.use_graph) return enqueue_kernels(p, s, false);
-  cudaGraphExec_t& graph = p->graphs[p->gclass];
+  // one kernel is launched as it is, on a grid of its size
+  const bool single = (p->kernels & (p->kernels - 1)) == 0;
+  if (!p->opt.use_graph || single) return enqueue_kernels(p, s, false);
+  p->lane_grid = p->lane_blocks;  // a graph serves searches of any size
+  cudaGraphExec_t& graph = p->graphs[p->gclass][p->kernels];
   if (!graph) {
     cudaStream_t cs;
     cudaError_t e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
@@ -909,14 +885,13 @@ static int32_t deal_streams(const HostBatch& hb, int32_t nq, int T, int32_t fixe
 
 // The short subjects' two-query layout (inter2q_kernel.cu): items are
 // (stream pair, half of a 64-subject group), the workers its warps.  Returns
-// K, or 0 when the one-query kernel should score the short subjects instead:
-// with option two_query = 1 the two-query layout must cost less than the
-// one-query kernel's 32-row strips, counting a two-query word at 0.9 of a
-// one-query word (measured 0.88 on the paper-shaped search, 20 queries, and
-// 0.93 on a search of two queries of 375 and 455 residues, where the
-// one-query kernel is then the faster).
+// the number of stream pairs, and in *cycles what the layout is expected to
+// take, in SM cycles: kQ2WordCycles per word row and scheduler, or, when one
+// item outlasts that, the longest item, whose warp shares its scheduler with
+// one other.
+static constexpr double kQ2WordCycles = 9.4, kQ2ItemCycles = 19;
 static int32_t plan_streams(sw_plan* p, const HostBatch& hb, int32_t nq, int32_t g_first,
-                            int64_t* n_strips) {
+                            int64_t* n_strips, double* cycles) {
   const int T = p->kc2.variant;
   const DbView& v = p->db->view;
   double glen_sum = 0;
@@ -924,12 +899,12 @@ static int32_t plan_streams(sw_plan* p, const HostBatch& hb, int32_t nq, int32_t
   const double glen_max = g_first < v.groups ? p->db->glen_h[g_first] : 0.0;
   const int32_t K = deal_streams(hb, nq, T, p->opt.two_query_pairs,
                                  (double)p->kc2.blocks * p->kc2.warps, 0.35, glen_max, glen_sum,
-                                 p->strips_h, p->spairs_h, 0, p->strip_capacity, n_strips);
-  if (K == 0) return 0;
-  const int64_t cost2 = *n_strips * T;  // words per column and half-group: strips x T rows
-  int64_t cost1 = 0;                    // rows per column and group
-  for (int32_t i = 0; i < nq; i++) cost1 += (hb.len[i] + 31) / 32 * 32;
-  if (p->opt.two_query == 1 && 2.0 * 0.9 * (double)cost2 >= (double)cost1) return 0;
+                                 p->strips.data(), p->spairs.data(), 0,
+                                 (int64_t)p->strips.size(), n_strips);
+  int64_t longest = 0;
+  for (int32_t k = 0; k < K; k++) longest = std::max<int64_t>(longest, p->spairs[(size_t)k].y);
+  *cycles = std::max(kQ2WordCycles * (double)(*n_strips * T) * 2 * glen_sum / (4.0 * p->sms),
+                     kQ2ItemCycles * (double)(longest * T) * glen_max);
   return K;
 }
 
@@ -938,15 +913,14 @@ static int32_t plan_streams(sw_plan* p, const HostBatch& hb, int32_t nq, int32_t
 // pair, group of PAIR2_GROUP long subjects), the workers its blocks, and the
 // largest item may be one worker's share (on the paper-shaped search's long
 // subjects, 1, 2, 4 and 8 stream pairs took 45.4, 35.6, 40.0 and 44.2 ms;
-// the rule picks 2 there, and 1 on the long-sequence workload).  Returns
-// K, or 0 when the subject-pair kernels (pair_kernel.cu) should score the
-// long subjects instead: with option two_query_long = 1 when the two-query
-// layout, whose passes are 1024 rows of each stream, costs more than those
-// kernels' passes of 512 or 1024 rows of each query against half as many
-// subject columns, counting a two-query word at 0.85 of a subject-pair word
-// of pair_kernel<32> and a word of pair_kernel<16> at 1.15.
+// the rule picks 2 there, and 1 on the long-sequence workload).  Returns the
+// number of stream pairs, and in *cycles what the layout is expected to take:
+// the passes' steps of 32 words, three warps to a scheduler, over as many
+// rounds of blocks as the items need, or the longest item.
+static constexpr double kP2WordCycles = 8.9;
 static int32_t plan_streams_long(sw_plan* p, const HostBatch& hb, int32_t nq, int64_t n_long,
-                                 int64_t first_strip, int32_t first_pair, int64_t* n_strips) {
+                                 int64_t first_strip, int32_t first_pair, int64_t* n_strips,
+                                 double* cycles) {
   *n_strips = 0;
   if (nq < 2 || n_long <= 0) return 0;
   const int32_t* clen = p->db->clen_h.data();
@@ -954,21 +928,142 @@ static int32_t plan_streams_long(sw_plan* p, const HostBatch& hb, int32_t nq, in
   for (int64_t s = 0; s < n_long; s += PAIR2_GROUP) len_sum += clen[s];
   const int32_t K = deal_streams(hb, nq, PAIR2_STRIP, p->opt.two_query_pairs,
                                  (double)p->pair2_blocks, 1.0, clen[0],
-                                 len_sum, p->strips_h + first_strip, p->spairs_h + first_pair,
-                                 first_strip, p->strip_capacity - first_strip, n_strips);
-  if (K == 0 || p->opt.two_query_long == 2) return K;
-  // words per column of a subject
-  double two = 0, one = 0;
+                                 len_sum, p->strips.data() + first_strip,
+                                 p->spairs.data() + first_pair, first_strip,
+                                 (int64_t)p->strips.size() - first_strip, n_strips);
+  const double groups = (double)((n_long + PAIR2_GROUP - 1) / PAIR2_GROUP);
+  const double step = 3 * 32 * kP2WordCycles;  // cycles per step of a block's three warps
+  double total = 0, longest = 0;
   for (int32_t k = 0; k < K; k++) {
-    const int64_t S = p->spairs_h[first_pair + k].y;
-    two += (double)((S + 31) / 32) * 32 * PAIR2_STRIP;
+    const double passes = (double)((p->spairs[(size_t)(first_pair + k)].y + 31) / 32);
+    total += passes * step * (len_sum + 127 * groups);
+    longest = std::max(longest, passes * step * ((double)clen[0] + 127));
   }
+  *cycles = std::max(total / p->sms, longest);
+  return K;
+}
+
+// The lane-group kernel's segments (lane_kernel.cu) for the subject pairs
+// [pair0, pair1): per query up to one per group size.  A (group size, rows)
+// shape costs, per subject pair, passes x (columns + LG) steps of
+// kLaneWordCycles x rows + kLaneStepCycles cycles of a scheduler on LG / 32 of a
+// warp; the cheapest shape is used, except where one item of it would take
+// longer than kLaneTail of the whole search: those subjects (a prefix, longest
+// first) go to a larger group, whose items are shorter.
+static constexpr double kLaneWordCycles = 9.3, kLaneStepCycles = 30;
+static constexpr double kLaneRowLatency = 14, kLaneStepLatency = 100;
+static constexpr double kLaneTail = 0.5;
+
+struct LaneCand {
+  int lg, pr, passes;
+  // cycles of one step of every pass: of a scheduler, and of a warp alone
+  double thr() const {
+    return kLaneWordCycles * (32.0 * (passes - 1) + pr) + kLaneStepCycles * passes;
+  }
+  double lat() const {
+    return kLaneRowLatency * (32.0 * (passes - 1) + pr) + kLaneStepLatency * passes;
+  }
+};
+
+static int lane_candidates(int32_t m, LaneCand* c) {
+  int n = 0;
+  for (int lg = 8; lg <= 32; lg *= 2) {
+    const int passes = lg == 32 ? std::max(1, (m + 1023) / 1024) : 1;
+    const int rows = (m - (passes - 1) * 1024 + lg - 1) / lg;  // per lane, last pass
+    if (rows > 32) continue;
+    c[n++] = LaneCand{lg, std::max(4, (rows + 3) / 4 * 4), passes};
+  }
+  return n;
+}
+
+static int64_t plan_lanes(sw_plan* p, const HostBatch& hb, int32_t nq, int64_t pair0, int64_t pair1,
+                          int32_t* n_segs, double* cycles) {
+  *n_segs = 0;
+  *cycles = 0;
+  if (nq <= 0 || pair0 >= pair1) return 0;
+  const sw_db* db = p->db;
+  const int64_t N = db->view.n;
+  auto pair_len = [&](int64_t i) { return (double)db->clen_h[(size_t)(2 * i)]; };
+  const double npairs = (double)(pair1 - pair0);
+  const double cols = 0.5 * (double)(db->cres_h[std::min(N, 2 * pair1)] - db->cres_h[2 * pair0]);
+  const double sched = 4.0 * p->sms;
+  double total = 0, warps = 0;
   for (int32_t i = 0; i < nq; i++) {
-    const int64_t m = hb.len[i];
-    one += pair_wide((int32_t)m) ? (double)((m + 1023) / 1024 * 1024) / 2
-                                 : 1.15 * (double)((m + 511) / 512 * 512) / 2;
+    LaneCand c[MAX_SEGS];
+    const int nc = lane_candidates(hb.len[i], c);
+    double best = 1e300, w = 0;
+    for (int k = 0; k < nc; k++) {
+      const double cost = c[k].thr() * c[k].lg / 32 * (cols + npairs * c[k].lg);
+      if (cost < best) best = cost, w = npairs * c[k].lg / 32;
+    }
+    total += best;
+    warps += w;
   }
-  return 0.85 * two < one ? K : 0;
+  const double t_all = total / sched;
+  const double share = std::min(4.0, std::max(1.0, warps / sched));
+  struct Seg { LaneSeg s; double t; };
+  std::vector<Seg> segs;
+  for (int32_t i = 0; i < nq; i++) {
+    const int32_t q = hb.order[i];
+    LaneCand c[MAX_SEGS];
+    const int nc = lane_candidates(hb.len[q], c);
+    double cost[MAX_SEGS];
+    int ord[MAX_SEGS];
+    for (int k = 0; k < nc; k++) {
+      cost[k] = c[k].thr() * c[k].lg / 32 * (cols + npairs * c[k].lg);
+      ord[k] = k;
+    }
+    std::sort(ord, ord + nc, [&](int a, int b) { return cost[a] < cost[b]; });
+    auto item = [&](const LaneCand& x, double len) {
+      return (len + x.lg) * std::max(x.lat(), share * x.thr());
+    };
+    int64_t at = pair0;
+    // longest subjects first: the shapes from the largest group to the cheapest
+    for (int k = nc - 1; k >= 0 && at < pair1; k--) {
+      const LaneCand& x = c[ord[k]];
+      int64_t end = pair1;
+      if (k > 0) {
+        // the subjects for which no cheaper shape is short enough, and this
+        // one is shorter than those
+        int64_t lo = at, hi = pair1;
+        auto wants = [&](int64_t j) {
+          for (int kk = 0; kk < k; kk++) {
+            const double t = item(c[ord[kk]], pair_len(j));
+            if (t <= kLaneTail * t_all || t <= item(x, pair_len(j))) return false;
+          }
+          return true;
+        };
+        while (lo < hi) {
+          const int64_t mid = (lo + hi) / 2;
+          if (wants(mid)) lo = mid + 1; else hi = mid;
+        }
+        end = lo;
+      }
+      if (end <= at) continue;
+      LaneSeg s{};
+      s.q = q;
+      s.lg = x.lg;
+      s.pr = x.pr;
+      s.passes = x.passes;
+      s.pair0 = (int32_t)at;
+      s.pair1 = (int32_t)end;
+      segs.push_back({s, item(x, pair_len(at))});
+      at = end;
+    }
+  }
+  std::stable_sort(segs.begin(), segs.end(), [](const Seg& a, const Seg& b) { return a.t > b.t; });
+  int64_t items = 0;
+  for (size_t i = 0; i < segs.size(); i++) {
+    LaneSeg& s = p->segs[i];
+    s = segs[i].s;
+    *cycles = std::max(*cycles, segs[i].t);
+    s.first = items;
+    const int64_t per = LANE_WARPS * 32 / s.lg;
+    items += (s.pair1 - s.pair0 + per - 1) / per;
+  }
+  *cycles = std::max(*cycles, t_all);
+  *n_segs = (int32_t)segs.size();
+  return items;
 }
 
 // The stream layout alone, for a given number of stream pairs (host only).
@@ -1013,14 +1108,14 @@ static sw_status plan_enqueue(sw_plan* p, const HostBatch& hb, int32_t nq, int32
   if (nq > p->max_queries || hb.total > p->max_residues)
     return sw_set_error(SW_EBUSY, "batch (%d queries, %lld residues) exceeds the plan (%d, %lld)",
                         nq, (long long)hb.total, p->max_queries, (long long)p->max_residues);
-  SearchParams& P = *p->params_h;
+  SearchParams& P = *(SearchParams*)p->block_h;
   bool packed_ok = true;
-  sw_status st = fill_scoring(P, gap_open, gap_extend, matrix, &packed_ok);
+  int max_sm = 0;
+  sw_status st = fill_scoring(P, gap_open, gap_extend, matrix, &packed_ok, &max_sm);
   if (st != SW_OK) return st;
   const DbView& v = p->db->view;
-  // packed: long subjects go to the packed intra-task kernel (subject pairs);
-  // otherwise (penalties too large for 16 bits, or forced) every subject
-  // goes to the int32 intra-task code
+  // packed: the 16-bit kernels score every pair; otherwise (penalties too
+  // large for 16 bits, or forced) every pair goes to the int32 intra-task code
   const bool packed = packed_ok && !p->opt.force_int32;
   int32_t gf = packed ? p->g_first : v.groups;
   const double total_cells = (double)hb.total * (double)p->db->residues;
@@ -1030,132 +1125,141 @@ static sw_status plan_enqueue(sw_plan* p, const HostBatch& hb, int32_t nq, int32
     // warp's share of the search go to the intra-task kernel instead, where
     // each subject is its own item.  Groups are sorted longest first.  Small
     // searches (a few milliseconds) are left alone.
-    const double warps = (double)p->kc.blocks * p->kc.warps;
+    const double warps = (double)p->kc2.blocks * p->kc2.warps;
     const double share = total_cells / warps;
     const int32_t mmax = hb.len[hb.order[0]];
     while (gf < v.groups && (double)GROUP * p->db->glen_h[gf] * mmax > 0.25 * share) gf++;
   }
   const int64_t n_long = std::min<int64_t>(v.n, (int64_t)gf * GROUP);
-  P.qres = p->qres;
-  P.qoff = p->qoff;
-  P.qlen = p->qlen;
-  P.qorder = p->qorder;
   P.scores = scores_dev;
   P.nq = nq;
   P.n_long = (int32_t)n_long;
   P.g_first = gf;
   P.n_intra_items = packed ? 0 : n_long * nq;
-  // the pair kernels' queries: those for pair_kernel<32>, then those for
-  // pair_kernel<16>, each longest first (none when the packed path is off)
-  int32_t* qpair_h = p->qorder_h + nq;
-  int32_t n32 = 0, n16 = 0;
-  auto wide = [&](int32_t m) { return m >= p->opt.wide_min_len && pair_wide(m); };
-  // subject pairs eligible for the wide kernel: those whose longer subject
-  // has at least wide_min_subject residues (a prefix: pairs are sorted
-  // longest first), or every pair when there are fewer (pair, query) items
-  // than narrow warps -- then each item runs nearly alone and fewer passes win
-  const int32_t npairs = packed ? (int32_t)((n_long + 1) / 2) : 0;
-  int32_t nwide = 0;
-  if ((int64_t)npairs * nq <= (int64_t)p->pair_blocks16 * PAIR_WARPS) {
-    nwide = npairs;
-  } else {
-    while (nwide < npairs && p->db->clen_h[2 * (size_t)nwide] >= p->opt.wide_min_subject) nwide++;
-  }
-  P.pair_queries = packed ? nq : 0;
-  P.n_wide_pairs = nwide;
-  if (packed) {
-    for (int32_t i = 0; i < nq; i++)
-      if (wide(hb.len[hb.order[i]])) qpair_h[n32++] = hb.order[i];
-    for (int32_t i = 0; i < nq; i++)
-      if (!wide(hb.len[hb.order[i]])) qpair_h[n32 + n16++] = hb.order[i];
-  }
-  P.qpair = p->qorder + nq;
-  P.nq_pair32 = n32;
-  P.nq_pair16 = n16;
-  P.n_inter_items = (int64_t)(v.groups - gf) * nq;
-  // two queries per word for the short subjects, when the plan's options and
-  // the cost model say so (the one-query kernel then has no items)
-  P.strips = p->strips;
-  P.spairs = p->spairs;
-  P.n_spairs = 0;
-  P.n_inter2_items = 0;
-  int64_t n_strips = 0;
-  if (packed && gf < v.groups && nq >= 2 && p->opt.two_query > 0) {
-    const int32_t K = plan_streams(p, hb, nq, gf, &n_strips);
-    if (K > 0) {
-      P.n_spairs = K;
-      P.n_inter2_items = (int64_t)K * 2 * (v.groups - gf);
-      P.n_inter_items = 0;
-    } else {
-      n_strips = 0;
+  P.n_spairs = P.n_spairs2 = 0;
+  P.n_inter2_items = P.n_pair2_items = P.n_lane_items = 0;
+  P.n_lane_segs = 0;
+  int64_t n_strips = 0, n_strips2 = 0;
+  int kernels = 0;
+  double long_share = 0;
+  if (packed && nq > 0 && v.n > 0) {
+    // Each part of the subjects -- the long ones, above the cutoff, and the
+    // short ones -- goes to a two-query kernel or to the lane groups, whichever
+    // is expected to finish it first (options two_query and two_query_long: 0
+    // never two queries, 2 always with two or more queries).
+    const int64_t npairs = (v.n + 1) / 2, long_pairs = std::min(npairs, (n_long + 1) / 2);
+    const bool has_long = n_long > 0, has_short = gf < v.groups;
+    int32_t n_segs = 0;
+    double t2 = 0, tl = 0;
+    bool two = false, two_long = false;
+    if (has_short && nq >= 2 && p->opt.two_query > 0) {
+      const int32_t K = plan_streams(p, hb, nq, gf, &n_strips, &t2);
+      if (K > 0 && p->opt.two_query == 1) plan_lanes(p, hb, nq, long_pairs, npairs, &n_segs, &tl);
+      two = K > 0 && (p->opt.two_query == 2 || t2 < tl);
+      if (two) {
+        P.n_spairs = K;
+        P.n_inter2_items = (int64_t)K * 2 * (v.groups - gf);
+      } else {
+        n_strips = 0;
+      }
     }
-  }
-  // and for the long subjects (the subject-pair kernels then have no items);
-  // its table follows the short subjects' in the same buffers
-  P.strips2 = p->strips;
-  P.spairs2 = p->spairs + P.n_spairs;
-  P.n_spairs2 = 0;
-  P.n_pair2_items = 0;
-  int64_t n_strips2 = 0;
-  if (packed && n_long > 0 && nq >= 2 && p->opt.two_query_long > 0) {
-    const int32_t K2 = plan_streams_long(p, hb, nq, n_long, n_strips, P.n_spairs, &n_strips2);
-    if (K2 > 0) {
-      P.n_spairs2 = K2;
-      P.n_pair2_items = (int64_t)K2 * ((n_long + PAIR2_GROUP - 1) / PAIR2_GROUP);
-      P.pair_queries = 0;
-      P.n_wide_pairs = 0;
-      P.nq_pair32 = 0;
-      P.nq_pair16 = 0;
-    } else {
-      n_strips2 = 0;
+    if (has_long && nq >= 2 && p->opt.two_query_long > 0) {
+      const int32_t K2 =
+          plan_streams_long(p, hb, nq, n_long, n_strips, P.n_spairs, &n_strips2, &t2);
+      if (K2 > 0 && p->opt.two_query_long == 1) plan_lanes(p, hb, nq, 0, long_pairs, &n_segs, &tl);
+      two_long = K2 > 0 && (p->opt.two_query_long == 2 || t2 < tl);
+      if (two_long) {
+        P.n_spairs2 = K2;
+        P.n_pair2_items = (int64_t)K2 * ((n_long + PAIR2_GROUP - 1) / PAIR2_GROUP);
+        kernels |= K_PAIR2;
+      } else {
+        n_strips2 = 0;
+      }
     }
+    const bool lanes_long = has_long && !two_long, lanes_short = has_short && !two;
+    if (lanes_long || lanes_short) {
+      P.n_lane_items = plan_lanes(p, hb, nq, lanes_long ? 0 : long_pairs,
+                                  lanes_short ? npairs : long_pairs, &n_segs, &tl);
+      P.n_lane_segs = n_segs;
+      p->lane_grid = (int)std::min<int64_t>(P.n_lane_items, p->lane_blocks);
+      kernels |= lanes_short ? K_LANES : K_LANES_LONG;
+      if (lanes_long && lanes_short && p->db->residues > 0)
+        long_share = (double)p->db->cres_h[n_long] / (double)p->db->residues;
+    }
+    if (two) kernels |= K_INTER2;
+    // no score above max_sm per aligned column: without one at the recompute
+    // threshold the int32 kernel has nothing to do
+    const int64_t longest = hb.len[hb.order[0]];
+    if (max_sm * std::min<int64_t>(longest, v.max_len) >= P.sat_threshold) kernels |= K_INT32;
+  } else if (nq > 0 && v.n > 0) {
+    kernels = K_INT32;
   }
-  memcpy(p->qoff_h, hb.off.data(), sizeof(int64_t) * nq);
-  memcpy(p->qlen_h, hb.len.data(), sizeof(int32_t) * nq);
-  memcpy(p->qorder_h, hb.order.data(), sizeof(int32_t) * nq);
-  if (hb.total > 0) memcpy(p->qres_h, hb.res, (size_t)hb.total);
+  // the upload block: parameters, zeroed state, tables
+  size_t at = BLOCK_HEADER;
+  auto put = [&](const void* src, size_t bytes) {
+    uint8_t* dev = p->block + at;
+    if (bytes) memcpy(p->block_h + at, src, bytes);
+    at += block_align(bytes);
+    return dev;
+  };
+  P.qoff = (const int64_t*)put(hb.off.data(), sizeof(int64_t) * nq);
+  P.qlen = (const int32_t*)put(hb.len.data(), sizeof(int32_t) * nq);
+  P.qorder = (const int32_t*)put(hb.order.data(), sizeof(int32_t) * nq);
+  P.lane_segs = (const LaneSeg*)put(p->segs.data(), sizeof(LaneSeg) * P.n_lane_segs);
+  P.spairs = (const int2*)put(p->spairs.data(), sizeof(int2) * (P.n_spairs + P.n_spairs2));
+  P.spairs2 = P.spairs + P.n_spairs;
+  P.strips = P.strips2 = (const int4*)put(p->strips.data(), sizeof(int4) * (n_strips + n_strips2));
+  P.qres = put(hb.res, (size_t)hb.total);
   if (injected_fault("copy"))
     return sw_set_cuda_error(cudaErrorInvalidValue, "query upload (injected fault)");
-  CUDA_TRY(cudaMemcpyAsync(p->qres, p->qres_h, (size_t)std::max<int64_t>(hb.total, 1), cudaMemcpyHostToDevice, s));
-  if (nq > 0) {
-    CUDA_TRY(cudaMemcpyAsync(p->qoff, p->qoff_h, sizeof(int64_t) * nq, cudaMemcpyHostToDevice, s));
-    CUDA_TRY(cudaMemcpyAsync(p->qlen, p->qlen_h, sizeof(int32_t) * nq, cudaMemcpyHostToDevice, s));
-    CUDA_TRY(cudaMemcpyAsync(p->qorder, p->qorder_h, sizeof(int32_t) * 2 * nq, cudaMemcpyHostToDevice, s));
-  }
-  if (P.n_spairs + P.n_spairs2 > 0) {
-    CUDA_TRY(cudaMemcpyAsync(p->strips, p->strips_h, sizeof(int4) * (n_strips + n_strips2),
-                             cudaMemcpyHostToDevice, s));
-    CUDA_TRY(cudaMemcpyAsync(p->spairs, p->spairs_h, sizeof(int2) * (P.n_spairs + P.n_spairs2),
-                             cudaMemcpyHostToDevice, s));
-  }
-  CUDA_TRY(cudaMemcpyAsync(p->params, p->params_h, sizeof(SearchParams), cudaMemcpyHostToDevice, s));
+  CUDA_TRY(cudaMemcpyAsync(p->block, p->block_h, at, cudaMemcpyHostToDevice, s));
   p->stream = s;
   p->gclass = gap_class(P.go, P.ge);
-  CUDA_TRY(run_kernels(p, s));
-  CUDA_TRY(cudaMemcpyAsync(p->state_h, p->state, sizeof(SearchState), cudaMemcpyDeviceToHost, s));
+  p->kernels = kernels;
+  p->long_share = long_share;
+  if (kernels) CUDA_TRY(run_kernels(p, s));
+  memset(p->state_h, 0, sizeof(SearchState));
+  if (kernels & K_INT32)
+    CUDA_TRY(cudaMemcpyAsync(p->state_h, p->state, sizeof(SearchState), cudaMemcpyDeviceToHost, s));
   p->pending = sw_stats{};
   int64_t qsum = hb.total;
   p->pending.cells = qsum * p->db->residues;
-  p->pending.inter_items = P.n_inter_items;
+  p->pending.inter_items = packed && P.n_spairs == 0 ? (int64_t)(v.groups - gf) * nq : 0;
   p->pending.inter2_items = P.n_inter2_items;
   p->pending.pair2_items = P.n_pair2_items;
   p->pending.intra_items = n_long * nq;  // (query, long subject) pairs, packed or int32
   p->pending.inter_cells = qsum * (p->db->residues - p->db->cres_h[n_long]);
-  p->pending.kernels_launched = 6;
+  for (int k = kernels; k; k &= k - 1) p->pending.kernels_launched++;
   return SW_OK;
 }
 
 static void finish_stats(sw_plan* p) {
   p->stats = p->pending;
-  // with overlap_kernels the pair and inter-task kernels both start at ev[0]
-  const bool ov = p->opt.overlap_kernels != 0;
-  if (cudaEventElapsedTime(&p->stats.pair_ms, p->ev[0], p->ev[1]) != cudaSuccess ||
-      cudaEventElapsedTime(&p->stats.search_ms, ov ? p->ev[0] : p->ev[1], p->ev[2]) != cudaSuccess ||
-      cudaEventElapsedTime(&p->stats.recompute_ms, ov ? p->ev_join : p->ev[2], p->ev[3]) !=
-          cudaSuccess) {
-    cudaGetLastError();
-    p->stats.pair_ms = p->stats.search_ms = p->stats.recompute_ms = -1.f;
+  const int set = p->kernels;
+  const bool is_long = set & (K_PAIR2 | K_LANES_LONG), is_short = set & (K_LANES | K_INTER2);
+  const bool both = is_long && is_short;
+  // with overlap_kernels the kernels of both parts start at ev[0]
+  const bool ov = p->opt.overlap_kernels != 0 && both;
+  auto between = [&](cudaEvent_t a, cudaEvent_t b) {
+    float ms = 0.f;
+    if (cudaEventElapsedTime(&ms, a, b) != cudaSuccess) {
+      cudaGetLastError();
+      ms = -1.f;
+    }
+    return ms;
+  };
+  if (both) {
+    p->stats.pair_ms = between(p->ev[0], p->ev[1]);
+    p->stats.search_ms = between(ov ? p->ev[0] : p->ev[1], p->ev[2]);
+  } else if (is_long) {
+    p->stats.pair_ms = between(p->ev[0], p->ev[2]);
+  } else if (is_short) {
+    // one launch for all subjects: its time split by their cells
+    const float ms = between(p->ev[0], p->ev[2]);
+    p->stats.pair_ms = (float)p->long_share * ms;
+    p->stats.search_ms = ms - p->stats.pair_ms;
   }
+  if (set & K_INT32) p->stats.recompute_ms = between(ov ? p->ev_join : p->ev[2], p->ev[3]);
   p->stats.recomputed_pairs = (int64_t)p->state_h->n_flags;
   p->in_flight = false;
 }

@@ -1,5 +1,6 @@
 // device_common.cuh -- device helpers shared by the alignment kernels of
-// libswgb: inter_kernel.cu, intra_kernel.cu, pair_kernel.cu, plain_kernel.cu.
+// libswgb: lane_kernel.cu, inter2q_kernel.cu, pair2q_kernel.cu, intra_kernel.cu,
+// align_kernel.cu, plain_kernel.cu.
 //
 // Every kernel computes Eq. 1-3 of arxiv 2309.09609 (Section II-B) in the
 // shared-gap form

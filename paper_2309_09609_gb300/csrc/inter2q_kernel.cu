@@ -1,7 +1,7 @@
 // inter2q_kernel.cu -- the inter-task kernel of libswgb with two queries per
 // 32-bit word.
 //
-// The packed inter-task kernel (inter_kernel.cu) puts two subjects in the two
+// The lane-group kernel (lane_kernel.cu) puts two subjects in the two
 // 16-bit halves of a word, so each cell's substitution score SM(q_i, d_j)
 // comes from two profile rows (one per subject's residue) and costs one
 // byte-merge instruction per word.  Here each lane owns ONE subject and the

@@ -1,7 +1,7 @@
 // pair2q_kernel.cu -- the packed intra-task kernel of libswgb with two
 // queries per 32-bit word (long subjects).
 //
-// pair_kernel.cu packs two SUBJECTS into the halves of a word, so every word
+// lane_kernel.cu packs two SUBJECTS into the halves of a word, so every word
 // of substitution scores is merged from two profile rows (one byte-permute
 // per word).  Here a warp scores ONE long subject, and the halves hold two
 // query streams (the layout of inter2q_kernel.cu): the word of rows (a_i,

@@ -49,6 +49,16 @@ struct DbView {
   int32_t max_len;       // longest subject
 };
 
+// ---- work of the lane-group kernel (lane_kernel.cu) ---------------------------
+// One segment: a query against the subject pairs [pair0, pair1) of the length
+// order, on groups of lg lanes with pr rows each.  A query of several passes
+// has lg = 32, 32 rows per lane in every pass but the last, and pr in that.
+struct LaneSeg {
+  long long first;  // its first block item
+  int32_t q, lg, pr, passes;
+  int32_t pair0, pair1;
+};
+
 // ---- per-search parameters, read by the kernels from device memory ----------
 // Kept in device memory (not kernel arguments) so that one captured CUDA graph
 // serves every batch: a new search only rewrites this block.
@@ -58,8 +68,6 @@ struct SearchParams {
   const int64_t* qoff;    // [nq]
   const int32_t* qlen;    // [nq]
   const int32_t* qorder;  // [nq] query indices, longest first
-  const int32_t* qpair;   // [nq_pair32 + nq_pair16] query indices for the pair kernels:
-                          // those of pair_kernel<32>, then those of pair_kernel<16>
   int32_t* scores;        // [nq x N] caller order
   // two queries per word (inter2q_kernel.cu): the strip table, per strip
   // (query of half 0, its first row | end bit 31, query of half 1, its first
@@ -67,21 +75,19 @@ struct SearchParams {
   // first strip and strip count
   const int4* strips;
   const int2* spairs;
-  int64_t n_inter2_items; // stream pairs x 2 x inter groups (0: the one-query kernel runs)
+  int64_t n_inter2_items; // stream pairs x 2 x inter groups (0: the lane groups score the short subjects)
   // two queries per word for the long subjects (pair2q_kernel.cu): a strip
   // table of 32-row strips and its stream pairs, in the same format
   const int4* strips2;
   const int2* spairs2;
-  int64_t n_pair2_items;  // stream pairs x groups of PAIR2_GROUP long subjects (0: pair_kernel runs)
+  int64_t n_pair2_items;  // stream pairs x groups of PAIR2_GROUP long subjects (0: the lane groups score them)
+  const LaneSeg* lane_segs;  // lane-group kernel: its segments ...
+  int64_t n_lane_items;      // ... and block items (0: it does not run)
   int64_t n_intra_items;  // n_long x nq  (int32 intra-task items, when the packed path is off)
-  int64_t n_inter_items;  // inter groups x nq  (packed inter-task items)
   int32_t nq;
+  int32_t n_lane_segs;
   int32_t n_spairs;       // stream pairs of the two-query kernel
   int32_t n_spairs2;      // stream pairs of the two-query intra-task kernel
-  int32_t pair_queries;   // nq when the packed path scores the long subjects, else 0
-  int32_t n_wide_pairs;   // subject pairs [0, n_wide_pairs) may go to pair_kernel<32> ...
-  int32_t nq_pair32;      // ... with these queries (qpair[0, nq_pair32)); the narrow
-  int32_t nq_pair16;      // kernel takes them with the others, and every other pair
   int32_t n_long;         // sorted subjects [0, n_long) go to the intra-task kernels
   int32_t g_first;        // first inter-task group (n_long / GROUP)
   int32_t go;             // Go = gap_open + gap_extend  (Eq. 2-3)
@@ -92,13 +98,11 @@ struct SearchParams {
 
 // ---- per-search device state (zeroed before each search) --------------------
 struct SearchState {
-  unsigned long long work;        // next work item (inter-task kernel)
   unsigned long long n_flags;     // saturated pairs appended to the flag list
   unsigned long long recompute;   // next flagged pair (int32 intra-task kernel, per block)
-  unsigned long long pair_work;   // next work item (pair_kernel<16>)
-  unsigned long long pair_work32; // next work item (pair_kernel<32>)
   unsigned long long intra_work;  // next int32 intra-task item (per warp)
   unsigned long long work2;       // next work item (two-query inter-task kernel)
+  unsigned long long lane_work;   // next block item (lane-group kernel)
   unsigned long long pair2_work;  // next work item (two-query intra-task kernel, per block)
   unsigned int status;            // reserved: error bits raised on the device
   unsigned int pad;
@@ -112,10 +116,10 @@ struct Scratch {
   int64_t intra_stride;       // int2 per warp
   int2* flags;                // saturated pairs: (query index, sorted subject index)
   int64_t flag_capacity;
-  uint2* pair_border;         // packed intra-task kernels, per warp: [column] (H, F) words;
-                              // rows [0, pair_rows16) for pair_kernel<16>, the rest for <32>
+  uint2* pair_border;         // lane-group and two-query intra-task kernels, per warp:
+                              // [column] (H, F) words of the pass border
+  int64_t lane_row0;          // the lane-group kernel's first row
   int64_t pair_stride;        // uint2 per warp
-  int64_t pair_rows16;
 };
 
 // ---- gap classes ------------------------------------------------------------------
@@ -136,19 +140,11 @@ inline int gap_class(int go, int ge) {
 
 // ---- kernel launchers -----------------------------------------------------------
 struct KernelConfig {
-  int variant;     // inter: packed rows per thread (16/32); intra: int32 rows per lane (8/16)
-  int cols;        // inter: columns per wavefront (4, or 8 with 32 rows)
+  int variant;     // inter: packed rows per strip (16/24/32); intra: int32 rows per lane (8/16)
   int warps;       // warps per block
   int blocks;      // grid size
   size_t smem;     // dynamic shared memory per block
 };
-
-// Inter-task kernel, packed 16-bit (inter_kernel.cu).
-size_t inter_smem_bytes(int rows, int warps);
-int inter_blocks_per_sm(int rows, int cols, int warps);  // resident blocks per SM, 0 if none
-cudaError_t launch_inter(const KernelConfig& kc, int gclass, const DbView& db,
-                         const SearchParams* params, SearchState* state, const Scratch& scr,
-                         cudaStream_t stream);
 
 // Inter-task kernel with two queries per word (inter2q_kernel.cu), 16, 24 or
 // 32 rows per strip.
@@ -173,14 +169,13 @@ cudaError_t launch_intra(const KernelConfig& kc, const DbView& db, const SearchP
 cudaError_t launch_collect(int blocks, const DbView& db, const SearchParams* params,
                            SearchState* state, const Scratch& scr, cudaStream_t stream);
 
-// Packed intra-task kernel over subject pairs, long subjects (pair_kernel.cu),
-// with 16 or 32 query rows per lane.
-constexpr int PAIR_WARPS = 4;  // warps per block
-int pair_blocks_per_sm(int rows);
-size_t pair_smem_bytes(int rows);
-cudaError_t launch_pairs(int rows, int gclass, int blocks, const DbView& db,
-                         const SearchParams* params, SearchState* state, const Scratch& scr,
-                         cudaStream_t stream);
+// Lane-group kernel, two subjects per word (lane_kernel.cu).  Scratch: one
+// pair_border row per warp.
+constexpr int LANE_WARPS = 4;  // warps per block
+int lane_blocks_per_sm();
+cudaError_t launch_lanes(int gclass, int blocks, const DbView& db, const SearchParams* params,
+                         SearchState* state, const Scratch& scr, cudaStream_t stream);
+
 // Packed intra-task kernel with two queries per word, long subjects
 // (pair2q_kernel.cu): one block of pair2q_warps() warps per SM, one subject
 // per warp, 32-row strips; scratch: the pair_border rows [0, blocks x warps).
@@ -191,15 +186,6 @@ size_t pair2q_smem_bytes();
 int pair2q_blocks_per_sm();
 cudaError_t launch_pair2q(int gclass, int blocks, const DbView& db, const SearchParams* params,
                           SearchState* state, const Scratch& scr, cudaStream_t stream);
-// pair_kernel<32> costs about 0.85 of pair_kernel<16> per cell it computes
-// but pads a query to 1024-row passes instead of 512: a query of m residues
-// goes to the wide kernel when 0.85 * ceil(m / 1024) * 1024 is below
-// ceil(m / 512) * 512, i.e. 17 * ceil(m / 1024) < 10 * ceil(m / 512).
-inline bool pair_wide(int32_t m) {
-  const int64_t a = ((int64_t)m + 1023) / 1024, b = ((int64_t)m + 511) / 512;
-  return m > 0 && 17 * a < 10 * b;
-}
-
 // Plain int32 baseline (Algorithm 1 per cell), one query per launch (plain_kernel.cu).
 int plain_blocks_per_sm();
 cudaError_t launch_plain(int blocks, const DbView& db, const SearchParams* params, int query,
