@@ -19,6 +19,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libswgb.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 SOURCES = ["api.cu", "inter2q_kernel.cu", "pair2q_kernel.cu", "lane_kernel.cu",
+           "lane_class1.cu", "lane_class2.cu",
            "intra_kernel.cu", "plain_kernel.cu",
            "align_kernel.cu", "intpeak.cu", "noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

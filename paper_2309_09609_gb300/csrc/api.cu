@@ -415,7 +415,7 @@ static sw_status fill_scoring(SearchParams& P, int32_t gap_open, int32_t gap_ext
 }
 
 // ---- plan ---------------------------------------------------------------------------------
-constexpr int MAX_SEGS = 3;  // segments of the lane-group kernel per query: one per group size
+constexpr int MAX_SEGS = 8;  // segments of the lane-group kernel per query: one per shape
 
 // The upload block: parameters, state, then the tables, each on a 16-byte boundary.
 static constexpr size_t block_align(size_t bytes) { return (bytes + 15) & ~(size_t)15; }
@@ -425,7 +425,9 @@ static constexpr size_t BLOCK_HEADER = block_align(sizeof(SearchParams)) + block
 // or the lane groups for the long subjects, the lane groups (for the short
 // subjects, or for all in one launch) or the two-query kernel for the short
 // ones, and the int32 kernel.
-enum { K_PAIR2 = 1, K_LANES_LONG = 2, K_LANES = 4, K_INTER2 = 8, K_INT32 = 16, K_SETS = 32 };
+// K_WIDE: the lane groups are launched with room for chains of 16 rows.
+enum { K_PAIR2 = 1, K_LANES_LONG = 2, K_LANES = 4, K_INTER2 = 8, K_INT32 = 16, K_WIDE = 32,
+       K_SETS = 64 };
 
 struct sw_plan {
   sw_db* db = nullptr;
@@ -438,7 +440,7 @@ struct sw_plan {
   int32_t g_first = 0;      // first inter-task group under the cutoff
   int32_t sms = 1;
   int32_t pair2_blocks = 0;   // grid of pair2q_kernel
-  int32_t lane_blocks = 0;    // grid of lane_kernel
+  int32_t lane_blocks[2] = {0, 0};  // grid of lane_kernel: as it is, and wide
   // One device block and its pinned image hold what a search uploads, in one
   // copy: the parameter block, the zeroed state, and the tables that follow
   // (the query arrays, the lane-group segments, the stream pairs, the strip
@@ -582,12 +584,14 @@ extern "C" sw_status sw_plan_create(sw_db* db, int32_t max_queries, int64_t max_
   p->ikc.blocks = dev_sms;
   p->ikc.smem = intra_smem_bytes(o.intra_rows);
   const int64_t WI = (int64_t)p->ikc.blocks * INTRA_WARPS;
-  const int lbps = lane_blocks_per_sm();
-  if (lbps < 1) {
-    plan_free(p);
-    return sw_set_error(SW_ECUDA, "lane-group kernel cannot launch");
+  for (int wide = 0; wide < 2; wide++) {
+    const int lbps = lane_blocks_per_sm(wide != 0);
+    if (lbps < 1) {
+      plan_free(p);
+      return sw_set_error(SW_ECUDA, "lane-group kernel cannot launch");
+    }
+    p->lane_blocks[wide] = dev_sms * lbps;
   }
-  p->lane_blocks = dev_sms * lbps;
   const int p2bps = pair2q_blocks_per_sm();
   if (p2bps < 1) {
     plan_free(p);
@@ -597,7 +601,7 @@ extern "C" sw_status sw_plan_create(sw_db* db, int32_t max_queries, int64_t max_
   // border rows of the two-query intra-task kernel and of the lane-group
   // kernel, which share them unless overlap_kernels runs them side by side
   const int64_t rows2 = (int64_t)p->pair2_blocks * pair2q_warps();
-  const int64_t rowsl = (int64_t)p->lane_blocks * LANE_WARPS;
+  const int64_t rowsl = (int64_t)std::max(p->lane_blocks[0], p->lane_blocks[1]) * LANE_WARPS;
   const int64_t WP = o.overlap_kernels ? rows2 + rowsl : std::max(rows2, rowsl);
   p->scr.lane_row0 = o.overlap_kernels ? rows2 : 0;
 
@@ -677,13 +681,13 @@ static cudaError_t enqueue_kernels(sw_plan* p, cudaStream_t s, bool capturing) {
   // needs a whole SM's shared memory, so it starts on an SM when the blocks
   // there run out of work, and no SM idles in their tails
   const bool is_long = set & (K_PAIR2 | K_LANES_LONG), is_short = set & (K_LANES | K_INTER2);
-  const bool overlap = p->opt.overlap_kernels && is_long && is_short;
+  const bool overlap = p->opt.overlap_kernels && is_long && is_short, wide = set & K_WIDE;
   cudaError_t e = record(p->ev[0], s, capturing);
   if (e == cudaSuccess && overlap) e = cudaEventRecord(p->fork, s);
   if (e == cudaSuccess && (set & K_PAIR2))
     e = launch_pair2q(gc, p->pair2_blocks, v, p->params, p->state, p->scr, s);
   if (e == cudaSuccess && (set & K_LANES_LONG))
-    e = launch_lanes(gc, p->lane_grid, v, p->params, p->state, p->scr, s);
+    e = launch_lanes(gc, wide, p->lane_grid, v, p->params, p->state, p->scr, s);
   cudaStream_t s2 = s;
   if (overlap) {
     s2 = p->side;
@@ -691,7 +695,7 @@ static cudaError_t enqueue_kernels(sw_plan* p, cudaStream_t s, bool capturing) {
   }
   if (e == cudaSuccess && is_long && is_short) e = record(p->ev[1], s, capturing);
   if (e == cudaSuccess && (set & K_LANES))
-    e = launch_lanes(gc, p->lane_grid, v, p->params, p->state, p->scr, s2);
+    e = launch_lanes(gc, wide, p->lane_grid, v, p->params, p->state, p->scr, s2);
   if (e == cudaSuccess && (set & K_INTER2))
     e = launch_inter2q(p->kc2, gc, v, p->params, p->state, p->scr, s2);
   if (e == cudaSuccess) e = record(p->ev[2], s2, capturing);
@@ -709,9 +713,10 @@ static cudaError_t enqueue_kernels(sw_plan* p, cudaStream_t s, bool capturing) {
 
 static cudaError_t run_kernels(sw_plan* p, cudaStream_t s) {
   // one kernel is launched as it is, on a grid of its size
-  const bool single = (p->kernels & (p->kernels - 1)) == 0;
+  const int launches = p->kernels & ~K_WIDE;
+  const bool single = (launches & (launches - 1)) == 0;
   if (!p->opt.use_graph || single) return enqueue_kernels(p, s, false);
-  p->lane_grid = p->lane_blocks;  // a graph serves searches of any size
+  p->lane_grid = p->lane_blocks[(p->kernels & K_WIDE) != 0];  // a graph serves searches of any size
   cudaGraphExec_t& graph = p->graphs[p->gclass][p->kernels];
   if (!graph) {
     cudaStream_t cs;
@@ -944,126 +949,175 @@ static int32_t plan_streams_long(sw_plan* p, const HostBatch& hb, int32_t nq, in
 }
 
 // The lane-group kernel's segments (lane_kernel.cu) for the subject pairs
-// [pair0, pair1): per query up to one per group size.  A (group size, rows)
-// shape costs, per subject pair, passes x (columns + LG) steps of
-// kLaneWordCycles x rows + kLaneStepCycles cycles of a scheduler on LG / 32 of a
-// warp; the cheapest shape is used, except where one item of it would take
-// longer than kLaneTail of the whole search: those subjects (a prefix, longest
-// first) go to a larger group, whose items are shorter.
+// [pair0, pair1): per query up to one per shape.  A shape costs, per subject
+// pair, (columns + LG) steps of kLaneWordCycles x rows + kLaneStepCycles per
+// pass, in cycles of a scheduler on LG / 32 of a warp (serve-sized searches of
+// one query measured 9.3 and 30).  The cheapest shape is used, except where one
+// item of it would take longer than `tail` of the whole search: those subjects
+// (a prefix, longest first) go to a shape with shorter items, a larger group
+// or a chain.  A warp alone on its scheduler takes kLaneRowLatency x rows +
+// kLaneStepLatency cycles a step (the chain of F down the lane's rows, and the
+// shuffle).
 static constexpr double kLaneWordCycles = 9.3, kLaneStepCycles = 30;
-static constexpr double kLaneRowLatency = 14, kLaneStepLatency = 100;
-static constexpr double kLaneTail = 0.5;
+static constexpr double kLaneRowLatency = 14, kLaneStepLatency = 70;
 
 struct LaneCand {
-  int lg, pr, passes;
-  // cycles of one step of every pass: of a scheduler, and of a warp alone
-  double thr() const {
-    return kLaneWordCycles * (32.0 * (passes - 1) + pr) + kLaneStepCycles * passes;
-  }
-  double lat() const {
-    return kLaneRowLatency * (32.0 * (passes - 1) + pr) + kLaneStepLatency * passes;
+  int lg, pr, passes, full, chain, halves;
+  double rows() const { return (double)full * (passes - 1) + pr; }
+  int ramp() const { return halves ? 2 * lg : lg; }
+  // scheduler cycles of one step of every pass
+  double thr() const { return kLaneWordCycles * rows() + kLaneStepCycles * passes; }
+  // cycles of the passes over n columns when `share` warps share a scheduler
+  double item(double n, double share) const {
+    const double deep = halves ? 0.5 * kLaneRowLatency : kLaneRowLatency;
+    if (!chain)
+      return (n + ramp()) * std::max(deep * rows() + kLaneStepLatency * passes, share * thr());
+    const double step = std::max(deep * full + kLaneStepLatency,
+                                 share * (kLaneWordCycles * full + kLaneStepCycles));
+    const double stages = (n + ramp()) / 64 + 1, period = std::max(stages, 8.0);
+    return ((passes - 1) / LANE_WARPS * period + (passes - 1) % LANE_WARPS * 2 + stages) * 64 * step;
   }
 };
 
-static int lane_candidates(int32_t m, LaneCand* c) {
+// The shapes for a query of m residues: 8, 16 and 32 lanes; 32 lanes in halves;
+// chains of 4 to 16 rows per lane (16 only with the wide launch).
+static int lane_candidates(int32_t m, bool wide, LaneCand* c) {
   int n = 0;
+  auto fit = [](int rows, int step) { return std::max(step, (rows + step - 1) / step * step); };
   for (int lg = 8; lg <= 32; lg *= 2) {
     const int passes = lg == 32 ? std::max(1, (m + 1023) / 1024) : 1;
     const int rows = (m - (passes - 1) * 1024 + lg - 1) / lg;  // per lane, last pass
-    if (rows > 32) continue;
-    c[n++] = LaneCand{lg, std::max(4, (rows + 3) / 4 * 4), passes};
+    if (rows <= 32) c[n++] = LaneCand{lg, fit(rows, 4), passes, 32, 0, 0};
+  }
+  if (m <= 24 * 32) c[n++] = LaneCand{32, fit((m + 31) / 32, 8), 1, 32, 0, 1};
+  for (int full : {4, 8, 16}) {
+    if (m <= 32 * full || (full > 8 && !wide)) continue;  // one pass; no room for the profiles
+    const int passes = (m + 32 * full - 1) / (32 * full);
+    if (passes > LANE_WARPS && (full < 8 || (wide && full < 16))) continue;  // a larger one has fewer
+    int pr = fit((m - (passes - 1) * 32 * full + 31) / 32, 4);
+    while (pr & (pr - 1)) pr += 4;  // chains come in 4, 8, 16 and 32 rows
+    c[n++] = LaneCand{32, pr, passes, full, 1, full > 4};
   }
   return n;
 }
 
-static int64_t plan_lanes(sw_plan* p, const HostBatch& hb, int32_t nq, int64_t pair0, int64_t pair1,
-                          int32_t* n_segs, double* cycles) {
+static int64_t plan_lanes_as(sw_plan* p, const HostBatch& hb, int32_t nq, int64_t pair0,
+                             int64_t pair1, bool wide, double tail, int32_t* n_segs,
+                             double* cycles) {
   *n_segs = 0;
   *cycles = 0;
   if (nq <= 0 || pair0 >= pair1) return 0;
   const sw_db* db = p->db;
   const int64_t N = db->view.n;
   auto pair_len = [&](int64_t i) { return (double)db->clen_h[(size_t)(2 * i)]; };
-  const double npairs = (double)(pair1 - pair0);
-  const double cols = 0.5 * (double)(db->cres_h[std::min(N, 2 * pair1)] - db->cres_h[2 * pair0]);
+  auto cols = [&](int64_t a, int64_t b) {  // columns of the pairs [a, b)
+    return 0.5 * (double)(db->cres_h[std::min(N, 2 * b)] - db->cres_h[2 * a]);
+  };
+  // scheduler cycles, and warps, of a shape on the pairs [a, b)
+  auto cost = [&](const LaneCand& x, int64_t a, int64_t b) {
+    return x.thr() * x.lg / 32 * (cols(a, b) + (double)(b - a) * x.ramp());
+  };
+  auto warps_of = [&](const LaneCand& x, int64_t a, int64_t b) {
+    return (double)(b - a) * (x.chain ? std::min(x.passes, LANE_WARPS) : x.lg / 32.0);
+  };
   const double sched = 4.0 * p->sms;
+  const double resident = (double)p->lane_blocks[wide] * LANE_WARPS / sched;
+  auto share_of = [&](double w) { return std::min(resident, std::max(1.0, w / sched)); };
   double total = 0, warps = 0;
   for (int32_t i = 0; i < nq; i++) {
     LaneCand c[MAX_SEGS];
-    const int nc = lane_candidates(hb.len[i], c);
-    double best = 1e300, w = 0;
-    for (int k = 0; k < nc; k++) {
-      const double cost = c[k].thr() * c[k].lg / 32 * (cols + npairs * c[k].lg);
-      if (cost < best) best = cost, w = npairs * c[k].lg / 32;
-    }
-    total += best;
-    warps += w;
+    const int nc = lane_candidates(hb.len[i], wide, c);
+    const LaneCand* best = c;
+    for (int k = 1; k < nc; k++)
+      if (cost(c[k], pair0, pair1) < cost(*best, pair0, pair1)) best = c + k;
+    total += cost(*best, pair0, pair1);
+    warps += warps_of(*best, pair0, pair1);
   }
-  const double t_all = total / sched;
-  const double share = std::min(4.0, std::max(1.0, warps / sched));
-  struct Seg { LaneSeg s; double t; };
-  std::vector<Seg> segs;
+  const double t_all = total / sched, share = share_of(warps);
+  struct Chosen {
+    LaneCand c;
+    LaneSeg s;
+    double t;
+  };
+  std::vector<Chosen> segs;
+  total = warps = 0;
   for (int32_t i = 0; i < nq; i++) {
     const int32_t q = hb.order[i];
     LaneCand c[MAX_SEGS];
-    const int nc = lane_candidates(hb.len[q], c);
-    double cost[MAX_SEGS];
-    int ord[MAX_SEGS];
-    for (int k = 0; k < nc; k++) {
-      cost[k] = c[k].thr() * c[k].lg / 32 * (cols + npairs * c[k].lg);
-      ord[k] = k;
-    }
-    std::sort(ord, ord + nc, [&](int a, int b) { return cost[a] < cost[b]; });
-    auto item = [&](const LaneCand& x, double len) {
-      return (len + x.lg) * std::max(x.lat(), share * x.thr());
-    };
+    const int nc = lane_candidates(hb.len[q], wide, c);
+    std::sort(c, c + nc, [&](const LaneCand& a, const LaneCand& b) {
+      return cost(a, pair0, pair1) < cost(b, pair0, pair1);
+    });
+    // from the dearest shape to the cheapest: each takes the longest pairs
+    // left, as far down as every cheaper one's item is too long and longer
     int64_t at = pair0;
-    // longest subjects first: the shapes from the largest group to the cheapest
     for (int k = nc - 1; k >= 0 && at < pair1; k--) {
-      const LaneCand& x = c[ord[k]];
-      int64_t end = pair1;
-      if (k > 0) {
-        // the subjects for which no cheaper shape is short enough, and this
-        // one is shorter than those
-        int64_t lo = at, hi = pair1;
-        auto wants = [&](int64_t j) {
-          for (int kk = 0; kk < k; kk++) {
-            const double t = item(c[ord[kk]], pair_len(j));
-            if (t <= kLaneTail * t_all || t <= item(x, pair_len(j))) return false;
-          }
-          return true;
-        };
-        while (lo < hi) {
-          const int64_t mid = (lo + hi) / 2;
-          if (wants(mid)) lo = mid + 1; else hi = mid;
+      auto wants = [&](int64_t j) {
+        const double n = pair_len(j), t = c[k].item(n, share);
+        for (int kk = 0; kk < k; kk++) {
+          const double tt = c[kk].item(n, share);
+          if (tt <= tail * t_all || tt <= t) return false;
         }
-        end = lo;
+        return true;
+      };
+      int64_t lo = at, hi = pair1;
+      while (lo < hi) {
+        const int64_t mid = (lo + hi) / 2;
+        if (wants(mid)) lo = mid + 1; else hi = mid;
       }
-      if (end <= at) continue;
-      LaneSeg s{};
-      s.q = q;
-      s.lg = x.lg;
-      s.pr = x.pr;
-      s.passes = x.passes;
-      s.pair0 = (int32_t)at;
-      s.pair1 = (int32_t)end;
-      segs.push_back({s, item(x, pair_len(at))});
-      at = end;
+      if (lo <= at) continue;
+      const LaneSeg s{0, q, c[k].lg, c[k].pr, c[k].passes, c[k].full, c[k].chain, c[k].halves,
+                      (int32_t)at, (int32_t)lo};
+      segs.push_back({c[k], s, 0.0});
+      total += cost(c[k], at, lo);
+      warps += warps_of(c[k], at, lo);
+      at = lo;
     }
   }
-  std::stable_sort(segs.begin(), segs.end(), [](const Seg& a, const Seg& b) { return a.t > b.t; });
+  double longest = 0;
+  for (size_t i = segs.size(); i-- > 0;) {
+    Chosen& x = segs[i];
+    x.t = x.c.item(pair_len(x.s.pair0), share_of(warps));
+    longest = std::max(longest, x.t);
+    // a query's longest subjects go first, however short their shape's items
+    if (i + 1 < segs.size() && segs[i + 1].s.q == x.s.q) x.t = std::max(x.t, segs[i + 1].t);
+  }
+  std::stable_sort(segs.begin(), segs.end(),
+                   [](const Chosen& a, const Chosen& b) { return a.t > b.t; });
   int64_t items = 0;
   for (size_t i = 0; i < segs.size(); i++) {
     LaneSeg& s = p->segs[i];
     s = segs[i].s;
-    *cycles = std::max(*cycles, segs[i].t);
     s.first = items;
-    const int64_t per = LANE_WARPS * 32 / s.lg;
+    const int64_t per = s.chain ? 1 : LANE_WARPS * 32 / s.lg;
     items += (s.pair1 - s.pair0 + per - 1) / per;
   }
-  *cycles = std::max(*cycles, t_all);
+  // the longest item starts first, beside the rest of the work; fewer warps
+  // on a scheduler (wide) hide less latency
+  *cycles = (std::max(longest, total / sched) + 0.2 * std::min(longest, total / sched)) * (wide ? 1.05 : 1);
   *n_segs = (int32_t)segs.size();
   return items;
+}
+
+// The same with the tail limit, and with or without wide chains (*wide), that
+// are expected to end the search soonest.  A large batch takes the middle one:
+// its items are short beside the search.
+static int64_t plan_lanes(sw_plan* p, const HostBatch& hb, int32_t nq, int64_t pair0, int64_t pair1,
+                          int32_t* n_segs, double* cycles, bool* wide) {
+  double tail = 0.5, best = 1e300;
+  *wide = false;
+  if (nq > 0 && nq <= 32) {
+    for (int w = 0; w < (hb.len[hb.order[0]] > 512 ? 2 : 1); w++)
+      for (double t : {0.35, 0.5, 0.7, 1.0, 1.5, 1e9}) {
+        plan_lanes_as(p, hb, nq, pair0, pair1, w != 0, t, n_segs, cycles);
+        if (*cycles < best * 0.999) {
+          best = *cycles;
+          tail = t;
+          *wide = w != 0;
+        }
+      }
+  }
+  return plan_lanes_as(p, hb, nq, pair0, pair1, *wide, tail, n_segs, cycles);
 }
 
 // The stream layout alone, for a given number of stream pairs (host only).
@@ -1151,10 +1205,10 @@ static sw_status plan_enqueue(sw_plan* p, const HostBatch& hb, int32_t nq, int32
     const bool has_long = n_long > 0, has_short = gf < v.groups;
     int32_t n_segs = 0;
     double t2 = 0, tl = 0;
-    bool two = false, two_long = false;
+    bool two = false, two_long = false, wide = false;
     if (has_short && nq >= 2 && p->opt.two_query > 0) {
       const int32_t K = plan_streams(p, hb, nq, gf, &n_strips, &t2);
-      if (K > 0 && p->opt.two_query == 1) plan_lanes(p, hb, nq, long_pairs, npairs, &n_segs, &tl);
+      if (K > 0 && p->opt.two_query == 1) plan_lanes(p, hb, nq, long_pairs, npairs, &n_segs, &tl, &wide);
       two = K > 0 && (p->opt.two_query == 2 || t2 < tl);
       if (two) {
         P.n_spairs = K;
@@ -1166,7 +1220,7 @@ static sw_status plan_enqueue(sw_plan* p, const HostBatch& hb, int32_t nq, int32
     if (has_long && nq >= 2 && p->opt.two_query_long > 0) {
       const int32_t K2 =
           plan_streams_long(p, hb, nq, n_long, n_strips, P.n_spairs, &n_strips2, &t2);
-      if (K2 > 0 && p->opt.two_query_long == 1) plan_lanes(p, hb, nq, 0, long_pairs, &n_segs, &tl);
+      if (K2 > 0 && p->opt.two_query_long == 1) plan_lanes(p, hb, nq, 0, long_pairs, &n_segs, &tl, &wide);
       two_long = K2 > 0 && (p->opt.two_query_long == 2 || t2 < tl);
       if (two_long) {
         P.n_spairs2 = K2;
@@ -1179,10 +1233,10 @@ static sw_status plan_enqueue(sw_plan* p, const HostBatch& hb, int32_t nq, int32
     const bool lanes_long = has_long && !two_long, lanes_short = has_short && !two;
     if (lanes_long || lanes_short) {
       P.n_lane_items = plan_lanes(p, hb, nq, lanes_long ? 0 : long_pairs,
-                                  lanes_short ? npairs : long_pairs, &n_segs, &tl);
+                                  lanes_short ? npairs : long_pairs, &n_segs, &tl, &wide);
       P.n_lane_segs = n_segs;
-      p->lane_grid = (int)std::min<int64_t>(P.n_lane_items, p->lane_blocks);
-      kernels |= lanes_short ? K_LANES : K_LANES_LONG;
+      p->lane_grid = (int)std::min<int64_t>(P.n_lane_items, p->lane_blocks[wide]);
+      kernels |= (lanes_short ? K_LANES : K_LANES_LONG) | (wide ? K_WIDE : 0);
       if (lanes_long && lanes_short && p->db->residues > 0)
         long_share = (double)p->db->cres_h[n_long] / (double)p->db->residues;
     }
@@ -1229,7 +1283,7 @@ static sw_status plan_enqueue(sw_plan* p, const HostBatch& hb, int32_t nq, int32
   p->pending.pair2_items = P.n_pair2_items;
   p->pending.intra_items = n_long * nq;  // (query, long subject) pairs, packed or int32
   p->pending.inter_cells = qsum * (p->db->residues - p->db->cres_h[n_long]);
-  for (int k = kernels; k; k &= k - 1) p->pending.kernels_launched++;
+  for (int k = kernels & ~K_WIDE; k; k &= k - 1) p->pending.kernels_launched++;
   return SW_OK;
 }
 

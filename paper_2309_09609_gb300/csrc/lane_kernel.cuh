@@ -1,0 +1,550 @@
+// lane_kernel.cuh -- packed 16-bit scores of (query, subject pair) items on
+// groups of 8, 16 or 32 lanes.
+//
+// A lane group scores two subjects, adjacent in length order, as the two
+// halves of every word.  Lane k of the group owns PR consecutive query rows in
+// registers and updates column t - k at step t, one whole column of its rows;
+// it takes the (H, F) border of the row above from lane k - 1 by shuffle
+// (Section II-B: intra-task parallelism with neighbour border exchange).  A
+// query of up to LG x PR rows needs no border memory at all; a longer one runs
+// in passes of 32 x PR rows whose border row goes through this warp's scratch.
+//
+// Why lane groups: one warp that sweeps 64 subjects with 32 rows in each lane
+// has the lowest cost per column, but its item takes (query / 32 rows) x
+// (subject columns) x 32 rows one after the other, and a search with few
+// queries has too few of those items for 152 SMs and ends on the longest one.
+// With a group per subject pair an item is 8 to 32 times shorter, so a search
+// of some thousand subjects already fills the chip, and the ends of a large
+// one are short.  What the group costs is the ramp, LG - 1 steps per subject
+// pair, and two shuffles, two residue loads and the profile loads per step of
+// PR words.  Measured on one GB300 (wall time of the search):
+//   1 query of 144 x 2,000 subjects      1.27 -> 0.12 ms
+//   1 query of 375 x 20,000              6.04 -> 0.49 ms
+//   1 query of 375 x 570,000             15.4 -> 10.9 ms
+//   7 queries of 400 x 40,000            15.0 ->  7.2 ms
+// (before: a warp per 64 subjects, and a warp per subject pair above 1,500
+// residues.)
+//
+// An item that would outlast the search (a long subject in a small search, a
+// long query against few subjects) is cut further: into chains, the query's
+// passes on the four warps of a block, each a few stages behind the one above
+// (4 queries x 500 subjects, all of 5,000-35,000 residues: 323 ms with the
+// passes one after the other, 165 with chains of 8 rows per lane and 156 of 16,
+// whose step overhead is spread over twice the words); and each lane's rows
+// into halves one column apart, two independent chains of cells for a warp
+// alone on its scheduler (1 query of 144 x 2,000: 0.100 -> 0.081 ms of kernel
+// time).  Chains of 32 rows measured 188 ms: their profiles leave room for 8
+// warps per SM, too few.
+// The kernel is bound by the ALU pipe: 4.5 operations per word (packed_cell
+// and the merge of the two subjects' profile bytes).
+//
+// Columns left and right of a subject hold the padding code, whose score of
+// -64 leaves H = E = 0 before the first column and raises no S after the last,
+// so no step tests its column.  The lanes of a warp walk in step; the items of
+// a block's warps are neighbours in length order and share one query profile.
+#pragma once
+
+#include "device_common.cuh"
+
+namespace swgb {
+
+constexpr int LANE_ROWS_MAX = 32;
+constexpr int SM_ROW = 28;  // bytes per row of the matrix copy: 25 scores, in whole words
+
+// Dynamic shared memory: one residue ring per warp, then the block's query
+// profile (or, for chained passes, one per warp).  Profile of the 32 lanes'
+// rows, int8, code-major:
+//   rows [VB * v, VB * v + VB) of lane l against code c at
+//   c * 32 * PR + v * 32 * VB + l * VB,   VB = bytes per load,
+// so the lanes of a quarter- or half-warp read distinct banks whatever codes
+// they read.  Ring: per group two blocks of 8 * LG columns, as the byte
+// offsets (code x 32 * PR) of the two subjects' profile rows, 16 bits each;
+// the first 8 columns are repeated after the last, so 8 steps need one wrap.
+constexpr int LANE_PROFILE = NCODES * 32 * LANE_ROWS_MAX;
+constexpr int LANE_RING = 4 * (2 * 256 + 32);  // bytes per warp: 2 * 8 * 32 columns and the repeats
+constexpr int LANE_RINGS = LANE_WARPS * LANE_RING;
+constexpr int LANE_SMEM = LANE_RINGS + LANE_PROFILE;
+constexpr int LANE_SMEM_WIDE = LANE_RINGS + LANE_WARPS * LANE_PROFILE / 2;  // chains of 16 rows
+constexpr int CHAIN_STAGE = 64;  // steps between the block barriers of a chain
+constexpr int CHAIN_LAG = 2;     // stages between the starts of consecutive passes
+
+// 4 x 4 byte transpose: word b of the result holds byte b of a, b, c, d
+__device__ __forceinline__ uint4 transpose4(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  const uint32_t ab0 = prmt(a, b, 0x5140u), ab1 = prmt(a, b, 0x7362u);
+  const uint32_t cd0 = prmt(c, d, 0x5140u), cd1 = prmt(c, d, 0x7362u);
+  return make_uint4(prmt(ab0, cd0, 0x5410u), prmt(ab0, cd0, 0x7632u), prmt(ab1, cd1, 0x5410u),
+                    prmt(ab1, cd1, 0x7632u));
+}
+
+// A lane's PR rows may be cut into NQ quarters (halves) of PR / NQ rows, each one
+// column behind the one above: NQ independent chains of cells per step, for a
+// warp that has its scheduler (nearly) to itself, at NQ times the ramp.
+template <int PR, int NQ>
+struct LaneShape {
+  static constexpr int R = PR / NQ;  // rows per quarter
+  static_assert(R % 4 == 0 && PR <= LANE_ROWS_MAX, "whole 4-row words, at most 32 rows");
+  static constexpr int VB = R % 16 == 0 ? 16 : R % 8 == 0 ? 8 : 4;  // bytes per profile load
+  static constexpr int UNROLL = PR >= 24 ? 2 : 4;                   // steps per loop body
+  static constexpr bool AHEAD = PR <= 24;  // registers allow the next step's profile words
+};
+
+// The profile of rows [row0 + li * PR, ...) of query residues qr[0, m)
+// for lanes li = l % lg.  Four rows and four codes at a time: one word of four
+// scores per row, transposed into one word of four rows per code.
+// Warp `first` of `warps` takes every warps-th row quad.
+template <int PR, int NQ>
+__device__ __forceinline__ void lane_profile_rows(uint8_t* prof, const uint8_t* sm,
+                                                  const uint8_t* __restrict__ qr, int m, int row0,
+                                                  int lg, int first, int warps) {
+  constexpr int VB = LaneShape<PR, NQ>::VB;
+  const int l = threadIdx.x & 31;
+  for (int rq = first; rq < PR / 4; rq += warps) {
+    const int r0 = row0 + (l & (lg - 1)) * PR + 4 * rq;
+    const uint8_t* s[4];
+#pragma unroll
+    for (int b = 0; b < 4; b++) s[b] = sm + (r0 + b < m ? (int)qr[r0 + b] : PAD_CODE) * SM_ROW;
+    uint8_t* dst = prof + (4 * rq / VB) * 32 * VB + l * VB + (4 * rq) % VB;
+#pragma unroll
+    for (int cq = 0; cq < SM_ROW / 4; cq++) {
+      const uint4 w = transpose4(*(const uint32_t*)(s[0] + 4 * cq), *(const uint32_t*)(s[1] + 4 * cq),
+                                 *(const uint32_t*)(s[2] + 4 * cq), *(const uint32_t*)(s[3] + 4 * cq));
+      const uint32_t v[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+      for (int b = 0; b < 4; b++)
+        if (4 * cq + b < NCODES) *(uint32_t*)(dst + (4 * cq + b) * 32 * PR) = v[b];
+    }
+  }
+}
+
+// Profile words of one column of a quarter: four rows to a word, per subject.
+template <int PR, int NQ>
+struct LaneWords {
+  static constexpr int R = LaneShape<PR, NQ>::R, VB = LaneShape<PR, NQ>::VB;
+  uint32_t a[R / 4], b[R / 4];
+
+  // pa, pb: the lane's profile rows of the two codes; q: the quarter
+  __device__ __forceinline__ void load(const uint8_t* pa, const uint8_t* pb, int q) {
+#pragma unroll
+    for (int v = 0; v < R / VB; v++) {
+      const int o = (q * (R / VB) + v) * 32 * VB;
+      if constexpr (VB == 16) {
+        const uint4 x = *(const uint4*)(pa + o), y = *(const uint4*)(pb + o);
+        a[4 * v] = x.x, a[4 * v + 1] = x.y, a[4 * v + 2] = x.z, a[4 * v + 3] = x.w;
+        b[4 * v] = y.x, b[4 * v + 1] = y.y, b[4 * v + 2] = y.z, b[4 * v + 3] = y.w;
+      } else if constexpr (VB == 8) {
+        const uint2 x = *(const uint2*)(pa + o), y = *(const uint2*)(pb + o);
+        a[2 * v] = x.x, a[2 * v + 1] = x.y;
+        b[2 * v] = y.x, b[2 * v + 1] = y.y;
+      } else {
+        a[v] = *(const uint32_t*)(pa + o);
+        b[v] = *(const uint32_t*)(pb + o);
+      }
+    }
+  }
+};
+
+// One column of quarter q's rows; hd: H above and left of its first row, f: F
+// of its first row, then of the row below its last.
+template <int PR, int NQ>
+__device__ __forceinline__ void lane_column(uint32_t (&H)[PR], uint32_t (&E)[PR], int q,
+                                            uint32_t& smax, uint32_t hd, uint32_t& f,
+                                            const LaneWords<PR, NQ>& w, uint32_t GO2,
+                                            uint32_t NGE2) {
+  constexpr int R = LaneShape<PR, NQ>::R;
+  uint32_t xp = 0;
+#pragma unroll
+  for (int i = 0; i < R; i++) {
+    const int r = q * R + i;
+    uint32_t x;
+    const uint32_t h = packed_cell(hd, prmt(w.a[i / 4], w.b[i / 4], sext_pair_sel(i & 3)), E[r], f,
+                                   x, GO2, NGE2);
+    hd = H[r];
+    H[r] = h;
+    if (i & 1)
+      smax = __vimax3_s16x2(smax, xp, x);
+    else
+      xp = x;
+  }
+}
+
+// How a pass meets the one before: alone (the whole query), one after the
+// other on one warp, or chained, on another warp of the block.
+enum { ALONE = 0, SERIAL = 1, CHAINED = 2 };
+
+// All warps of the block have finished the stage.  The warps of a chain meet
+// here from different places of the code, so it is a barrier of its own.
+__device__ __forceinline__ void chain_barrier() {
+  asm volatile("bar.sync 1, %0;" ::"n"(LANE_WARPS * 32) : "memory");
+}
+
+// One pass of the lane's rows over its group's subject pair.  n: columns of
+// the warp's longest subject (uniform over the warp); src: the pair's first
+// 16-byte chunk of 8 + 8 residues, one every 512 bytes, `chunks` of them.
+// Quarter q of lane k updates column t - NQ k - q at step t; it takes what the
+// quarter above (the last one of lane k - 1 for q = 0) left at step t - 1.
+// With several passes LG is 32, hb_in holds the border row below the pass
+// before (unless this is the first) and hb_out takes this pass's (unless it is
+// the last): lane 0 reads column j at most U steps before its step j, lane 31
+// writes it at step j + 32 NQ - 1.  SERIAL: both are one row.  CHAINED: every
+// CHAIN_STAGE steps the block's warps meet at a barrier, and the pass before,
+// on another warp, is CHAIN_LAG stages ahead: the columns up to 64 k + 63 that
+// stage k reads were written by that pass's step 64 k + 126 at the latest, in
+// its stage k + 1, which ended before this stage began.
+template <int PR, int NQ, int MODE>
+__device__ __forceinline__ void lane_sweep(const uint8_t* prof, uint8_t* ring, int lane, int lg,
+                                           int n, const uint4* src, int chunks, const uint2* hb_in,
+                                           uint2* hb_out, bool first, bool last, uint32_t& smax,
+                                           uint32_t GO2, uint32_t NGE2) {
+  constexpr bool PASSES = MODE != ALONE;
+  constexpr int U = LaneShape<PR, NQ>::UNROLL;
+  constexpr bool AHEAD = LaneShape<PR, NQ>::AHEAD;
+  constexpr uint32_t CODE = 32 * PR;  // bytes between the profile rows of two codes
+  const int li = lane & (lg - 1);
+  const int cols = 8 * lg;  // columns per ring block
+  // this group's ring: 2 * cols columns and the repeats, 4 bytes each; the
+  // gap to the next group's keeps the groups' reads on distinct banks
+  uint8_t* gr = ring + (lane / lg) * 4 * (2 * cols + (lg == 8 ? 8 : 16));
+  const uint32_t not0 = li == 0 ? 0u : 1u;
+  const uint8_t* pl = prof + lane * LaneShape<PR, NQ>::VB;
+  uint32_t H[PR], E[PR];
+#pragma unroll
+  for (int r = 0; r < PR; r++) H[r] = E[r] = 0u;  // H(i, 0) = 0; any E(i, 1) <= 0 will do
+  // per quarter: H below its rows one and two steps back, F one step back,
+  // and the profile rows of its column's codes
+  uint32_t hdiag = 0u, h1[NQ], h2[NQ], f1[NQ];
+  const uint8_t *pa[NQ], *pb[NQ];
+#pragma unroll
+  for (int q = 0; q < NQ; q++) {
+    h1[q] = h2[q] = f1[q] = 0u;
+    pa[q] = pb[q] = pl + PAD_CODE * CODE;
+  }
+  const uint4 pad = make_uint4(0x18181818u, 0x18181818u, 0x18181818u, 0x18181818u);
+  static_assert(PAD_CODE == 0x18, "the padding chunk");
+  // this lane's 8 columns of a ring block
+  auto store = [&](int slot, const uint4& v) {
+    uint32_t w[8];
+#pragma unroll
+    for (int c = 0; c < 8; c++) {
+      const uint32_t a = prmt(c < 4 ? v.x : v.y, 0u, 0x4440u + (c & 3));
+      const uint32_t b = prmt(c < 4 ? v.z : v.w, 0u, 0x4440u + (c & 3));
+      w[c] = imad(a, CODE, imad(b, CODE << 16, 0u));
+    }
+    const uint4 lo = make_uint4(w[0], w[1], w[2], w[3]), hi = make_uint4(w[4], w[5], w[6], w[7]);
+    uint4* dst = (uint4*)(gr + 4 * (slot * cols + 8 * li));
+    dst[0] = lo;
+    dst[1] = hi;
+    if (slot == 0 && li == 0) {
+      dst = (uint4*)(gr + 4 * 2 * cols);
+      dst[0] = lo;
+      dst[1] = hi;
+    }
+  };
+  auto load = [&](int b) {
+    const int c = b * lg + li;
+    return c < chunks ? ldg_nc(src + (int64_t)c * 32) : pad;
+  };
+  __syncwarp();
+  store(1, pad);  // the columns left of the first
+  uint4 next = load(0);
+  const int steps = n + NQ * lg - 1;
+  const uint32_t mask = (uint32_t)(4 * (2 * cols - 1));
+  const int span = MODE == CHAINED ? CHAIN_STAGE : cols;
+  int b = 0;
+  for (int t0 = 0; t0 < steps; t0 += span) {
+    if (MODE != CHAINED || (t0 & (cols - 1)) == 0) {
+      __syncwarp();
+      store(b & 1, next);
+      next = load(++b);
+      __syncwarp();
+    }
+    const int tend = min(t0 + span, steps);
+    uint2 bq[U];  // the border of columns t .. t + U - 1
+    if constexpr (PASSES) {
+#pragma unroll
+      for (int u = 0; u < U; u++) bq[u] = hb_in[min(t0 + u, n - 1)];
+    }
+    // the profile words of step t are loaded one step ahead; the last step of
+    // a ring block reads whatever code the slot holds, and is read again here
+    LaneWords<PR, NQ> w[NQ];
+    auto fetch = [&](const uint8_t* rp) {
+      const uint8_t *a = pl + *(const uint16_t*)rp, *b = pl + *(const uint16_t*)(rp + 2);
+      w[0].load(a, b, 0);
+#pragma unroll
+      for (int q = 1; q < NQ; q++) w[q].load(pa[q - 1], pb[q - 1], q);
+    };
+    if constexpr (AHEAD) fetch(gr + ((uint32_t)(4 * (t0 - NQ * li)) & mask));
+#pragma unroll 1
+    for (int t = t0; t < tend; t += U) {
+      const uint8_t* rp = gr + ((uint32_t)(4 * (t - NQ * li)) & mask);
+#pragma unroll
+      for (int u = 0; u < U; u++) {
+        // the row above: lane k - 1's bottom row, H = F = 0 above the matrix
+        uint32_t in_h = imad(__shfl_up_sync(FULL, h1[NQ - 1], 1, lg), not0, 0u);
+        uint32_t in_f = imad(__shfl_up_sync(FULL, f1[NQ - 1], 1, lg), not0, 0u);
+        if constexpr (PASSES) {
+          const uint2 bv = bq[u];
+          bq[u] = hb_in[min(t + u + U, min(tend, n) - 1)];
+          if (li == 0 && !first) {
+            in_h = bv.x;
+            in_f = bv.y;
+          }
+        }
+        if constexpr (!AHEAD) fetch(rp + 4 * u);
+        LaneWords<PR, NQ> now[NQ];
+#pragma unroll
+        for (int q = 0; q < NQ; q++) now[q] = w[q];
+#pragma unroll
+        for (int q = NQ - 1; q > 0; q--) {
+          pa[q] = pa[q - 1];
+          pb[q] = pb[q - 1];
+        }
+        if constexpr (NQ > 1) {
+          pa[0] = pl + *(const uint16_t*)(rp + 4 * u);
+          pb[0] = pl + *(const uint16_t*)(rp + 4 * u + 2);
+        }
+        if constexpr (AHEAD) fetch(rp + 4 * (u + 1));
+        uint32_t nh[NQ], nf[NQ];
+#pragma unroll
+        for (int q = 0; q < NQ; q++) {
+          nf[q] = q == 0 ? in_f : f1[q - 1];
+          lane_column<PR, NQ>(H, E, q, smax, q == 0 ? hdiag : h2[q - 1], nf[q], now[q], GO2, NGE2);
+          nh[q] = H[(q + 1) * (PR / NQ) - 1];
+        }
+        hdiag = in_h;
+#pragma unroll
+        for (int q = 0; q < NQ; q++) {
+          h2[q] = h1[q];
+          h1[q] = nh[q];
+          f1[q] = nf[q];
+        }
+        if constexpr (PASSES) {
+          const int j = t + u - (32 * NQ - 1);
+          if (lane == 31 && !last && j >= 0 && j < n)
+            hb_out[j] = make_uint2(h1[NQ - 1], f1[NQ - 1]);
+        }
+      }
+    }
+    if constexpr (MODE == CHAINED) chain_barrier();
+  }
+}
+
+// S of each subject of the group's pair: recorded, or flagged for the int32
+// recompute when it may have saturated.
+__device__ __forceinline__ void lane_emit(const DbView& db, const SearchParams* __restrict__ P,
+                                          SearchState* st, const Scratch& scr, int q, int pair,
+                                          uint32_t smax) {
+#pragma unroll
+  for (int half = 0; half < 2; half++) {
+    const int sidx = 2 * pair + half;
+    const int orig = db.perm[sidx];
+    if (orig < 0) continue;
+    const int s = (int)(int16_t)(half ? (smax >> 16) : (smax & 0xffffu));
+    if (s >= P->sat_threshold) {
+      const unsigned long long k = atomicAdd(&st->n_flags, 1ull);
+      if ((int64_t)k < scr.flag_capacity)
+        scr.flags[k] = make_int2(q, sidx);
+      else  // the list is full: mark the pair for the host's next recompute round
+        P->scores[(int64_t)q * db.n + orig] = FLAG_SENTINEL;
+    } else {
+      P->scores[(int64_t)q * db.n + orig] = s;
+    }
+  }
+}
+
+// One warp's share of a block item: where its pairs lie.
+struct LanePlace {
+  int lg, n;         // lanes per group; columns of the warp's longest subject
+  const uint4* src;  // this group's subject pair in the interleaved layout
+  int chunks;
+  uint2* hb;         // the warp's border row
+};
+
+// One pass, the rows [row0, row0 + lg x PR) of the query.  `build`: the block
+// does not hold this profile yet (uniform over the block).
+template <int PR, int NQ, int G>
+__device__ __forceinline__ void lane_pass(const SearchParams* __restrict__ P, uint8_t* smem,
+                                          const uint8_t* sm, const uint8_t* __restrict__ qr, int m,
+                                          int row0, bool build, const LanePlace& at, int pass,
+                                          int passes, uint32_t& smax) {
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  uint8_t *ring = smem + wib * LANE_RING, *prof = smem + LANE_RINGS;
+  uint32_t GO2, NGE2;  // (Go, Go), (-Ge, -Ge)
+  gap_words<G>(P, GO2, NGE2);
+  if (build) {
+    __syncthreads();  // every warp is done with the profile before
+    lane_profile_rows<PR, NQ>(prof, sm, qr, m, row0, at.lg, wib, LANE_WARPS);
+    __syncthreads();
+  }
+  if (at.n == 0) return;  // uniform over the warp
+  if (passes == 1)
+    lane_sweep<PR, NQ, ALONE>(prof, ring, lane, at.lg, at.n, at.src, at.chunks, nullptr, nullptr,
+                              true, true, smax, GO2, NGE2);
+  else if constexpr (NQ == 1)
+    lane_sweep<PR, 1, SERIAL>(prof, ring, lane, 32, at.n, at.src, at.chunks, at.hb, at.hb,
+                              pass == 0, pass == passes - 1, smax, GO2, NGE2);
+}
+
+// One pass of a chain, on this warp, with a profile of its own.
+template <int PR, int NQ, int G>
+__device__ __forceinline__ void chain_pass(const SearchParams* __restrict__ P, uint8_t* smem,
+                                           const uint8_t* sm, const uint8_t* __restrict__ qr, int m,
+                                           int row0, int slice, const LanePlace& at,
+                                           const uint2* hb_in, bool first, bool last,
+                                           uint32_t& smax) {
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  uint8_t *ring = smem + wib * LANE_RING, *prof = smem + LANE_RINGS + wib * slice;
+  uint32_t GO2, NGE2;
+  gap_words<G>(P, GO2, NGE2);
+  __syncwarp();
+  lane_profile_rows<PR, NQ>(prof, sm, qr, m, row0, 32, 0, 1);
+  __syncwarp();
+  lane_sweep<PR, NQ, CHAINED>(prof, ring, lane, 32, at.n, at.src, at.chunks, hb_in, at.hb, first,
+                              last, smax, GO2, NGE2);
+}
+
+// A chain: one subject pair on the whole block, for items that would take too
+// long on one warp.  Warp w takes the passes w, w + LANE_WARPS, ...; pass p
+// starts at stage (p / W) * period + (p % W) * CHAIN_LAG with period the larger
+// of a pass's stages and W * CHAIN_LAG, so consecutive passes are at least
+// CHAIN_LAG stages apart, and a warp's next pass starts after its previous one
+// ends and at least W * CHAIN_LAG stages after it started, when the pass that
+// read the border row it will overwrite is further on.  Every warp meets the
+// same number of barriers.
+template <int G>
+__device__ __forceinline__ void lane_chain(const DbView& db, const SearchParams* __restrict__ P,
+                                           SearchState* st, const Scratch& scr, uint8_t* smem,
+                                           const uint8_t* sm, uint32_t* red, const LaneSeg& sg,
+                                           int unit) {
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const int pair = sg.pair0 + unit;
+  uint2* rows = scr.pair_border +
+                (scr.lane_row0 + (int64_t)blockIdx.x * LANE_WARPS) * scr.pair_stride;
+  LanePlace at;
+  at.lg = 32;
+  at.n = db.clen[2 * pair];
+  at.src = (const uint4*)(db.inter + db.goff[pair / 32]) + (pair & 31);
+  at.chunks = db.glen[pair / 32] / CHUNK;
+  at.hb = rows + wib * scr.pair_stride;
+  const uint2* hb_in = rows + (wib + LANE_WARPS - 1) % LANE_WARPS * scr.pair_stride;
+  const int m = P->qlen[sg.q];
+  const uint8_t* __restrict__ qr = P->qres + P->qoff[sg.q];
+  // stages of a pass (at NQ = 2; a pass of fewer steps waits out the rest)
+  const int spass = (at.n + 63 + CHAIN_STAGE - 1) / CHAIN_STAGE;
+  const int period = max(spass, LANE_WARPS * CHAIN_LAG);
+  const int end = (sg.passes - 1) / LANE_WARPS * period +
+                  (sg.passes - 1) % LANE_WARPS * CHAIN_LAG + spass;
+  uint32_t smax = 0u;
+  if (at.n > 0) {  // uniform over the block
+    int g = 0;
+    for (int p = wib; p < sg.passes; p += LANE_WARPS) {
+      for (const int start = p / LANE_WARPS * period + p % LANE_WARPS * CHAIN_LAG; g < start; g++)
+        chain_barrier();
+      const bool last = p == sg.passes - 1;
+      const int pr = last ? sg.pr : sg.full, row0 = p * 32 * sg.full, slice = NCODES * 32 * sg.full;
+      switch (pr) {  // uniform over the warp
+        case 4: chain_pass<4, 1, G>(P, smem, sm, qr, m, row0, slice, at, hb_in, p == 0, last, smax); break;
+        case 8: chain_pass<8, 2, G>(P, smem, sm, qr, m, row0, slice, at, hb_in, p == 0, last, smax); break;
+        default: chain_pass<16, 2, G>(P, smem, sm, qr, m, row0, slice, at, hb_in, p == 0, last, smax); break;
+      }
+      g += pr == 4 ? (at.n + 31 + CHAIN_STAGE - 1) / CHAIN_STAGE : spass;
+    }
+    for (; g < end; g++) chain_barrier();
+  }
+  for (int o = 16; o > 0; o >>= 1) smax = __vmaxs2(smax, __shfl_xor_sync(FULL, smax, o));
+  if (lane == 0) red[wib] = smax;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int w = 1; w < LANE_WARPS; w++) smax = __vmaxs2(smax, red[w]);
+    lane_emit(db, P, st, scr, sg.q, pair, smax);
+  }
+}
+
+// One block item: LANE_WARPS x 32 / lg subject pairs of one segment.
+// `cached` is the segment whose (single-pass) profile the block holds, or -1.
+template <int G>
+__device__ __forceinline__ void lane_item(const DbView& db, const SearchParams* __restrict__ P,
+                                          SearchState* st, const Scratch& scr, uint8_t* smem,
+                                          const uint8_t* sm, const LaneSeg& sg, int seg,
+                                          int& cached, int unit) {
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  LanePlace at;
+  at.lg = sg.lg;
+  const int first = sg.pair0 + (unit * LANE_WARPS + wib) * (32 / sg.lg);  // the warp's first pair
+  const int pair = first + lane / sg.lg;
+  const bool has = pair < sg.pair1;
+  at.n = first < sg.pair1 ? db.clen[2 * first] : 0;
+  const int grp = (has ? pair : 0) / 32;
+  at.src = (const uint4*)(db.inter + db.goff[grp]) + (pair & 31);
+  at.chunks = has ? db.glen[grp] / CHUNK : 0;
+  at.hb = scr.pair_border +
+          (scr.lane_row0 + (int64_t)blockIdx.x * LANE_WARPS + wib) * scr.pair_stride;
+  const int m = P->qlen[sg.q];
+  const uint8_t* __restrict__ qr = P->qres + P->qoff[sg.q];
+  uint32_t smax = 0u;
+  for (int p = 0; p < sg.passes; p++) {
+    // every pass but the last has 32 rows per lane
+    const int pr = p < sg.passes - 1 ? LANE_ROWS_MAX : sg.pr;
+    const int row0 = p * 32 * LANE_ROWS_MAX;
+    const bool build = sg.passes > 1 || cached != seg;
+    switch (sg.halves ? -pr : pr) {  // uniform over the block
+      case 4: lane_pass<4, 1, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
+      case 8: lane_pass<8, 1, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
+      case 12: lane_pass<12, 1, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
+      case 16: lane_pass<16, 1, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
+      case 20: lane_pass<20, 1, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
+      case 24: lane_pass<24, 1, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
+      case 28: lane_pass<28, 1, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
+      case -8: lane_pass<8, 2, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
+      case -16: lane_pass<16, 2, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
+      case -24: lane_pass<24, 2, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
+      default: lane_pass<32, 1, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
+    }
+  }
+  cached = sg.passes > 1 ? -1 : seg;
+  for (int o = sg.lg >> 1; o > 0; o >>= 1) smax = __vmaxs2(smax, __shfl_xor_sync(FULL, smax, o));
+  if (has && (lane & (sg.lg - 1)) == 0) lane_emit(db, P, st, scr, sg.q, pair, smax);
+}
+
+template <int G>
+__global__ void __launch_bounds__(LANE_WARPS * 32, 4)
+lane_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Scratch scr) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  __shared__ __align__(16) uint8_t sm[NCODES * SM_ROW];
+  __shared__ unsigned long long s_item;
+  __shared__ uint32_t red[LANE_WARPS];
+  const long long total = P->n_lane_items;
+  for (int i = threadIdx.x; i < NCODES * SM_ROW; i += blockDim.x)
+    sm[i] = i % SM_ROW < NCODES ? (uint8_t)P->sm[i / SM_ROW * NCODES + i % SM_ROW] : 0;
+  const LaneSeg* __restrict__ segs = P->lane_segs;
+  const int nseg = P->n_lane_segs;
+  int cached = -1;
+  __syncthreads();
+  // The first item of a block is its index: consecutive blocks start on
+  // different SMs, so a search of few items uses every SM (taken from the
+  // counter, they all went to the blocks of the SMs that started first).
+  for (long long it = blockIdx.x; it < total;) {  // uniform over the block
+    int lo = 0, hi = nseg - 1;  // the last segment whose first item is at most `it`
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (segs[mid].first <= it)
+        lo = mid;
+      else
+        hi = mid - 1;
+    }
+    const LaneSeg sg = segs[lo];
+    if (sg.chain) {
+      __syncthreads();  // every warp is done with the profile before
+      lane_chain<G>(db, P, st, scr, smem, sm, red, sg, (int)(it - sg.first));
+      cached = -1;
+    } else {
+      lane_item<G>(db, P, st, scr, smem, sm, sg, lo, cached, (int)(it - sg.first));
+    }
+    __syncthreads();  // the item before is read by all, and its chain is done
+    if (threadIdx.x == 0) s_item = gridDim.x + atomicAdd(&st->lane_work, 1ull);
+    __syncthreads();
+    it = (long long)s_item;
+  }
+}
+
+}  // namespace swgb

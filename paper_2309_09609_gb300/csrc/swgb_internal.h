@@ -52,10 +52,13 @@ struct DbView {
 // ---- work of the lane-group kernel (lane_kernel.cu) ---------------------------
 // One segment: a query against the subject pairs [pair0, pair1) of the length
 // order, on groups of lg lanes with pr rows each.  A query of several passes
-// has lg = 32, 32 rows per lane in every pass but the last, and pr in that.
+// has lg = 32, `full` rows per lane (32, less only in a chain) in every pass
+// but the last, and pr in that.  chain: the passes of a pair run on the warps
+// of a block, one behind the other, instead of one after the other on a warp.
+// halves: each lane's rows in two halves, one column apart (a query of one pass).
 struct LaneSeg {
   long long first;  // its first block item
-  int32_t q, lg, pr, passes;
+  int32_t q, lg, pr, passes, full, chain, halves;
   int32_t pair0, pair1;
 };
 
@@ -172,9 +175,12 @@ cudaError_t launch_collect(int blocks, const DbView& db, const SearchParams* par
 // Lane-group kernel, two subjects per word (lane_kernel.cu).  Scratch: one
 // pair_border row per warp.
 constexpr int LANE_WARPS = 4;  // warps per block
-int lane_blocks_per_sm();
-cudaError_t launch_lanes(int gclass, int blocks, const DbView& db, const SearchParams* params,
-                         SearchState* state, const Scratch& scr, cudaStream_t stream);
+// wide: with the shared memory for chains of more than 8 rows per lane (fewer
+// blocks per SM)
+int lane_blocks_per_sm(bool wide);
+cudaError_t launch_lanes(int gclass, bool wide, int blocks, const DbView& db,
+                         const SearchParams* params, SearchState* state, const Scratch& scr,
+                         cudaStream_t stream);
 
 // Packed intra-task kernel with two queries per word, long subjects
 // (pair2q_kernel.cu): one block of pair2q_warps() warps per SM, one subject
