@@ -705,7 +705,7 @@ static cudaError_t enqueue_kernels(sw_plan* p, cudaStream_t s, bool capturing) {
     if (e == cudaSuccess) e = record(p->ev_join, s, capturing);
   }
   if (set & K_INT32) {
-    if (e == cudaSuccess) e = launch_intra(p->ikc, v, p->params, p->state, p->scr, s);
+    if (e == cudaSuccess) e = launch_intra(p->ikc, (set & ~K_INT32) == 0, v, p->params, p->state, p->scr, s);
     if (e == cudaSuccess) e = record(p->ev[3], s, capturing);
   }
   return e;
@@ -1284,6 +1284,7 @@ static sw_status plan_enqueue(sw_plan* p, const HostBatch& hb, int32_t nq, int32
   p->pending.intra_items = n_long * nq;  // (query, long subject) pairs, packed or int32
   p->pending.inter_cells = qsum * (p->db->residues - p->db->cres_h[n_long]);
   for (int k = kernels & ~K_WIDE; k; k &= k - 1) p->pending.kernels_launched++;
+  if ((kernels & K_INT32) && kernels != K_INT32) p->pending.kernels_launched++;  // both recomputes
   return SW_OK;
 }
 
@@ -1333,7 +1334,7 @@ static cudaError_t overflow_rounds(sw_plan* p, int32_t* rounds) {
   while (nf > (unsigned long long)p->scr.flag_capacity) {
     cudaError_t e = cudaMemsetAsync(p->state, 0, sizeof(SearchState), s);
     if (e == cudaSuccess) e = launch_collect(4 * std::max(sms, 1), p->db->view, p->params, p->state, p->scr, s);
-    if (e == cudaSuccess) e = launch_intra(p->ikc, p->db->view, p->params, p->state, p->scr, s);
+    if (e == cudaSuccess) e = launch_intra(p->ikc, false, p->db->view, p->params, p->state, p->scr, s);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(p->state_h, p->state, sizeof(SearchState), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);

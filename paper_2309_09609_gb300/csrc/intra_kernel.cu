@@ -16,6 +16,18 @@
 //     p - 1, so a flagged pair of two 35,000-residue sequences runs on sixteen
 //     warps instead of one.  Stages end at __syncthreads, which orders each
 //     border write before its read and each read before the next overwrite.
+//
+// Few flagged pairs leave most SMs idle that way, and the search waits for the
+// longest.  Up to RECOMPUTE_PER_CLUSTER of them for every cluster of the grid
+// are therefore scored by recompute_kernel instead: the same schedule over
+// the 128 warps of a cluster of sixteen blocks, with the cluster's barrier
+// between the stages.  More pairs than that fill the chip one block each, and
+// most blocks of a cluster would idle on short queries.  Two pairs of 35,000 x
+// 26,620 residues took 68 ms on a block each, 15.9 on clusters of eight blocks
+// of 16 warps, 11.6 on clusters of sixteen of 8 (two warps to a scheduler) and
+// 9.7 with the codes and profile words loaded ahead of their columns.
+#include <cooperative_groups.h>
+
 #include "device_common.cuh"
 
 namespace swgb {
@@ -27,39 +39,65 @@ struct IntraSlice {
 
 constexpr int LAG = 3;  // stages between the starts of consecutive passes (block items)
 
+// The lane's profile words along its columns, loaded ahead of the cells: the
+// code of column j + 2 and the words of column j + 1 while column j is scored
+// (columns past either end read the last or first code, for lanes that skip
+// them).
+template <int TI>
+struct IntraFeed {
+  const uint8_t* d;     // the subject's codes
+  const uint8_t* prof;  // the lane's profile rows, 32 * TI bytes per code
+  int n, code;
+  uint32_t next[TI / 4];
+
+  __device__ __forceinline__ int at(int j) const { return d[min(max(j, 0), n - 1)]; }
+  __device__ __forceinline__ void words() {
+    const uint8_t* lp = prof + code * 32 * TI;
+    if constexpr (TI == 8) {
+      const uint2 v = *(const uint2*)lp;
+      next[0] = v.x, next[1] = v.y;
+    } else {
+      const uint4 v = *(const uint4*)lp;
+      next[0] = v.x, next[1] = v.y, next[2] = v.z, next[3] = v.w;
+    }
+  }
+  __device__ __forceinline__ void start(int j) {  // the next column is j
+    code = at(j);
+    words();
+    code = at(j + 1);
+  }
+  __device__ __forceinline__ void step(uint32_t (&pw)[TI / 4], int j) {  // column j's words
+#pragma unroll
+    for (int k = 0; k < TI / 4; k++) pw[k] = next[k];
+    words();
+    code = at(j + 2);
+  }
+};
+
 // The TI cells of one lane at one column: (in_h, in_f) are H and F of the row
-// above the lane's first row at this column; lp is the lane's profile row of
-// the column's residue.  Eq. 1-3 in the shared-gap form, int32.
+// above the lane's first row at this column; pw are the lane's profile words
+// of the column's residue.  Eq. 1-3 in the shared-gap form, int32.
 template <int TI>
 __device__ __forceinline__ void intra_cells(int (&Hp)[TI], int (&E)[TI], int& hdiag, int& out_h,
                                             int& out_f, int& S, int in_h, int in_f,
-                                            const uint8_t* lp, int go, int ge) {
-  uint32_t pw[TI / 4];
-  if constexpr (TI == 8) {
-    const uint2 v = *(const uint2*)lp;
-    pw[0] = v.x;
-    pw[1] = v.y;
-  } else {
-    const uint4 v = *(const uint4*)lp;
-    pw[0] = v.x;
-    pw[1] = v.y;
-    pw[2] = v.z;
-    pw[3] = v.w;
-  }
-  int hd = hdiag;
+                                            const uint32_t (&pw)[TI / 4], int go, int ge) {
+  int hd = hdiag, xp = 0;
   hdiag = in_h;
   int f = in_f;
 #pragma unroll
   for (int r = 0; r < TI; r++) {
-    const int w = sext_byte(pw[r / 4], r & 3);
-    const int e = E[r];
-    const int h = __viaddmax_s32_relu(hd, w, max(e, f));  // Eq. 1
+    // as packed_cell: E >= 0 stands for the zero term, S from the diagonal term
+    const int x = hd + sext_byte(pw[r / 4], r & 3);
+    const int h = __vimax3_s32(x, E[r], f);  // Eq. 1
     hd = Hp[r];
     Hp[r] = h;
     const int tt = h - go;
-    E[r] = __viaddmax_s32(e, -ge, tt);  // Eq. 2, next column
-    f = __viaddmax_s32(f, -ge, tt);     // Eq. 3, next row
-    S = max(S, h);
+    E[r] = __viaddmax_s32_relu(E[r], -ge, tt);  // Eq. 2, next column
+    f = __viaddmax_s32(f, -ge, tt);             // Eq. 3, next row
+    if (r & 1)
+      S = __vimax3_s32(S, xp, x);
+    else
+      xp = x;
   }
   out_h = Hp[TI - 1];
   out_f = f;
@@ -70,8 +108,8 @@ __device__ __forceinline__ void intra_start(int (&Hp)[TI], int (&E)[TI], int& hd
                                             int& out_f, int go) {
 #pragma unroll
   for (int r = 0; r < TI; r++) {
-    Hp[r] = 0;   // H(i, 0)
-    E[r] = -go;  // E(i, 1)
+    Hp[r] = 0;  // H(i, 0)
+    E[r] = 0;   // any E(i, 1) <= 0 gives the same H
   }
   hdiag = 0;
   out_h = 0;
@@ -99,7 +137,11 @@ __device__ void intra_warp_item(const DbView& db, const SearchParams* __restrict
     intra_start<TI>(Hp, E, hdiag, out_h, out_f, go);
     const bool last_pass = (p == npass - 1);
     const int steps = n + 31;
+    IntraFeed<TI> feed{d, slice + lane * TI, n};
+    feed.start(-lane);
     for (int t = 0; t < steps; t++) {
+      uint32_t pw[TI / 4];
+      feed.step(pw, t - lane);
       int in_h = __shfl_up_sync(FULL, out_h, 1);
       int in_f = __shfl_up_sync(FULL, out_f, 1);
       const int j = t - lane;
@@ -114,8 +156,7 @@ __device__ void intra_warp_item(const DbView& db, const SearchParams* __restrict
         }
       }
       if (j >= 0 && j < n) {
-        intra_cells<TI>(Hp, E, hdiag, out_h, out_f, S, in_h, in_f, slice + (d[j] * 32 + lane) * TI,
-                        go, ge);
+        intra_cells<TI>(Hp, E, hdiag, out_h, out_f, S, in_h, in_f, pw, go, ge);
         if (lane == 31 && !last_pass) hb[j] = make_int2(out_h, out_f);
       }
     }
@@ -125,19 +166,22 @@ __device__ void intra_warp_item(const DbView& db, const SearchParams* __restrict
   if (lane == 0) emit_score(db, P, q, s, S);
 }
 
-// One (query, subject) pair on the whole block.  Pass p runs on warp
-// p % INTRA_WARPS and starts at stage (p / W) * period + (p % W) * LAG, with
-// period = max(stages of a pass, LAG * W): consecutive passes are LAG stages
-// apart, and a warp's next pass starts after its previous one ends.  Lane 0 of
-// pass p at column j needs the bottom row of pass p - 1 at column j, written
-// by that pass at its step j + 31, i.e. at most two of its stages after the
-// stage holding its step j; LAG = 3 leaves one stage in between, in which the
-// warp fetches the next 32 border values with one coalesced load.
-template <int TI>
-__device__ void intra_block_item(const DbView& db, const SearchParams* __restrict__ P,
-                                 const int8_t* __restrict__ sm, uint8_t* slice, int lane, int wib,
-                                 int2* border, int64_t stride, int* red, int q, int s) {
-  constexpr int W = INTRA_WARPS;
+// One (query, subject) pair on the W warps of a block, or of a cluster of
+// blocks.  Pass p runs on warp p % W and starts at stage (p / W) * period +
+// (p % W) * LAG, with period = max(stages of a pass, LAG * W): consecutive
+// passes are LAG stages apart, and a warp's next pass starts after its
+// previous one ends.  Lane 0 of pass p at column j needs the bottom row of pass
+// p - 1 at column j, written by that pass at its step j + 31, i.e. at most two
+// of its stages after the stage holding its step j; LAG = 3 leaves one stage in
+// between, in which the warp fetches the next 32 border values with one
+// coalesced load.  own: this warp's border row, src: that of the warp before;
+// they go through L2, where the other blocks of a cluster see them.  Returns
+// the block's maximum in thread 0.
+template <int TI, int W, int BLOCK_WARPS, typename Barrier>
+__device__ int intra_block_item(const DbView& db, const SearchParams* __restrict__ P,
+                                const int8_t* __restrict__ sm, uint8_t* slice, int lane, int wib,
+                                int warp, int2* own, const int2* src, int* red, int q, int s,
+                                Barrier barrier) {
   constexpr int ROWS = 32 * TI;
   const int n = db.clen[s];
   const int m = P->qlen[q];
@@ -149,22 +193,20 @@ __device__ void intra_block_item(const DbView& db, const SearchParams* __restric
   const int period = max(spass, LAG * W);
   const int nstages =
       npass > 0 ? ((npass - 1) / W) * period + ((npass - 1) % W) * LAG + spass : 0;
-  int2* own = border + wib * stride;                    // bottom rows of this warp's passes
-  const int2* src = border + ((wib + W - 1) % W) * stride;  // those of the pass before
   const int2 top = make_int2(0, -go);                   // (H(0, j), F(1, j))
   int S = 0;
   int Hp[TI], E[TI], hdiag = 0, out_h = 0, out_f = -go;
   int p = 0;
   int2 bcur = top, bnext = top;  // border of columns 32k + lane and 32(k + 1) + lane
   for (int g = 0; g < nstages; g++) {
-    const int rel = g - wib * LAG;
+    const int rel = g - warp * LAG;
     int k = -1;
     if (rel >= 0) {
       const int r = rel / period;
       const int kk = rel - r * period;
-      if (kk < spass && wib + r * W < npass) {
+      if (kk < spass && warp + r * W < npass) {
         k = kk;
-        p = wib + r * W;
+        p = warp + r * W;
       }
     }
     if (k >= 0) {  // warp-uniform
@@ -173,17 +215,21 @@ __device__ void intra_block_item(const DbView& db, const SearchParams* __restric
         lane_profile<TI>(slice, sm, qr, m, p * ROWS + lane * TI, lane);
         __syncwarp();
         intra_start<TI>(Hp, E, hdiag, out_h, out_f, go);
-        bcur = (p > 0 && lane < n) ? src[lane] : top;
+        bcur = (p > 0 && lane < n) ? __ldcg(src + lane) : top;
       } else {
         bcur = bnext;
       }
       const int jn = 32 * (k + 1) + lane;
-      bnext = (p > 0 && jn < n) ? src[jn] : top;
+      bnext = (p > 0 && jn < n) ? __ldcg(src + jn) : top;
       const bool last_pass = (p == npass - 1);
       const int t0 = 32 * k;
       const int tend = min(t0 + 32, n + 31);
+      IntraFeed<TI> feed{d, slice + lane * TI, n};
+      feed.start(t0 - lane);
 #pragma unroll 4
       for (int t = t0; t < tend; t++) {
+        uint32_t pw[TI / 4];
+        feed.step(pw, t - lane);
         int in_h = __shfl_up_sync(FULL, out_h, 1);
         int in_f = __shfl_up_sync(FULL, out_f, 1);
         const int bh = __shfl_sync(FULL, bcur.x, t - t0);
@@ -194,23 +240,27 @@ __device__ void intra_block_item(const DbView& db, const SearchParams* __restric
         }
         const int j = t - lane;
         if (j >= 0 && j < n) {
-          intra_cells<TI>(Hp, E, hdiag, out_h, out_f, S, in_h, in_f,
-                          slice + (d[j] * 32 + lane) * TI, go, ge);
-          if (lane == 31 && !last_pass) own[j] = make_int2(out_h, out_f);
+          intra_cells<TI>(Hp, E, hdiag, out_h, out_f, S, in_h, in_f, pw, go, ge);
+          if (lane == 31 && !last_pass) __stcg(own + j, make_int2(out_h, out_f));
         }
       }
     }
-    __syncthreads();
+    barrier();
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) S = max(S, __shfl_xor_sync(FULL, S, o));
   if (lane == 0) red[wib] = S;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    int best = 0;
-    for (int w = 0; w < W; w++) best = max(best, red[w]);
-    emit_score(db, P, q, s, best);
-  }
+  int best = 0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < BLOCK_WARPS; w++) best = max(best, red[w]);
+  return best;
+}
+
+// Whether the flagged pairs are few enough for a cluster each.
+__device__ __forceinline__ bool recompute_in_clusters(unsigned long long flagged,
+                                                      unsigned clusters) {
+  return flagged <= (unsigned long long)RECOMPUTE_PER_CLUSTER * clusters;
 }
 
 template <int TI>
@@ -244,6 +294,8 @@ intra_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Scr
   const unsigned long long nf = *(volatile unsigned long long*)&st->n_flags;
   const unsigned long long total =
       nf < (unsigned long long)scr.flag_capacity ? nf : (unsigned long long)scr.flag_capacity;
+  if (recompute_in_clusters(total, gridDim.x / RECOMPUTE_CLUSTER)) return;  // recompute_kernel
+  const int64_t stride = scr.intra_stride;
   for (;;) {
     if (threadIdx.x == 0) s_item = atomicAdd(&st->recompute, 1ull);
     __syncthreads();
@@ -251,7 +303,53 @@ intra_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Scr
     __syncthreads();  // every thread has read s_item before thread 0 rewrites it
     if (it >= total) break;
     const int2 fl = scr.flags[it];
-    intra_block_item<TI>(db, P, sm, slice, lane, wib, border, scr.intra_stride, red, fl.x, fl.y);
+    const int best = intra_block_item<TI, INTRA_WARPS, INTRA_WARPS>(
+        db, P, sm, slice, lane, wib, wib, border + wib * stride,
+        border + (wib + INTRA_WARPS - 1) % INTRA_WARPS * stride, red, fl.x, fl.y,
+        []() { __syncthreads(); });
+    if (threadIdx.x == 0) emit_score(db, P, fl.x, fl.y, best);
+  }
+}
+
+// Few flagged pairs, one cluster each: cluster c takes the pairs c, c +
+// clusters, ...  Every block of a cluster runs the same stages.
+template <int TI>
+__global__ void __cluster_dims__(RECOMPUTE_CLUSTER) __launch_bounds__(RECOMPUTE_WARPS * 32)
+recompute_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Scratch scr) {
+  extern __shared__ __align__(16) uint8_t smem[];
+  __shared__ int red[RECOMPUTE_WARPS];
+  __shared__ int block_best;
+  const unsigned clusters = gridDim.x / RECOMPUTE_CLUSTER;
+  const unsigned long long nf = *(volatile unsigned long long*)&st->n_flags;
+  const unsigned long long total =
+      nf < (unsigned long long)scr.flag_capacity ? nf : (unsigned long long)scr.flag_capacity;
+  if (total == 0 || !recompute_in_clusters(total, clusters)) return;  // uniform over the grid
+  namespace cg = cooperative_groups;
+  cg::cluster_group cluster = cg::this_cluster();
+  constexpr int W = RECOMPUTE_CLUSTER * RECOMPUTE_WARPS;
+  int8_t* sm = (int8_t*)smem;
+  load_matrix(sm, P);
+  __syncthreads();
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const int rank = (int)cluster.block_rank(), warp = rank * RECOMPUTE_WARPS + wib;
+  uint8_t* slice = smem + MATRIX_SMEM + wib * IntraSlice<TI>::BYTES;
+  // the cluster's border rows, one per warp
+  int2* rows = scr.intra_border + ((int64_t)blockIdx.x - rank) * RECOMPUTE_WARPS * scr.intra_stride;
+  int2* own = rows + warp * scr.intra_stride;
+  const int2* src = rows + (warp + W - 1) % W * scr.intra_stride;
+  for (unsigned long long it = blockIdx.x / RECOMPUTE_CLUSTER; it < total; it += clusters) {
+    const int2 fl = scr.flags[it];
+    const int best = intra_block_item<TI, W, RECOMPUTE_WARPS>(db, P, sm, slice, lane, wib, warp, own, src, red, fl.x,
+                                             fl.y, [&]() { cluster.sync(); });
+    if (threadIdx.x == 0) block_best = best;
+    cluster.sync();
+    if (rank == 0 && threadIdx.x == 0) {
+      int score = best;
+      for (int r = 1; r < RECOMPUTE_CLUSTER; r++)
+        score = max(score, *cluster.map_shared_rank(&block_best, r));
+      emit_score(db, P, fl.x, fl.y, score);
+    }
+    cluster.sync();  // block_best is read, and no block leaves before that
   }
 }
 
@@ -288,6 +386,10 @@ static IntraKernel pick_intra(int rows) {
   return nullptr;
 }
 
+static IntraKernel pick_recompute(int rows) {
+  return rows == 8 ? recompute_kernel<8> : recompute_kernel<16>;
+}
+
 size_t intra_smem_bytes(int rows) {
   const int slice = rows == 8 ? IntraSlice<8>::BYTES : IntraSlice<16>::BYTES;
   return (size_t)MATRIX_SMEM + (size_t)INTRA_WARPS * slice;
@@ -297,8 +399,12 @@ int intra_blocks_per_sm(int rows) {
   IntraKernel k = pick_intra(rows);
   if (!k) return 0;
   const size_t smem = intra_smem_bytes(rows);
-  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-      cudaSuccess)
+  for (IntraKernel f : {k, pick_recompute(rows)})
+    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+        cudaSuccess)
+      return 0;
+  if (cudaFuncSetAttribute(pick_recompute(rows), cudaFuncAttributeNonPortableClusterSizeAllowed,
+                           1) != cudaSuccess)
     return 0;
   int nb = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, INTRA_WARPS * 32, smem) !=
@@ -307,11 +413,18 @@ int intra_blocks_per_sm(int rows) {
   return nb;
 }
 
-cudaError_t launch_intra(const KernelConfig& kc, const DbView& db, const SearchParams* params,
-                         SearchState* state, const Scratch& scr, cudaStream_t stream) {
+cudaError_t launch_intra(const KernelConfig& kc, bool items, const DbView& db,
+                         const SearchParams* params, SearchState* state, const Scratch& scr,
+                         cudaStream_t stream) {
   IntraKernel k = pick_intra(kc.variant);
   if (!k) return cudaErrorInvalidValue;
   cudaGetLastError();  // a stale error must not be read as this launch's
+  if (!items && kc.blocks >= RECOMPUTE_CLUSTER) {  // flagged pairs: few of them, or many
+    pick_recompute(kc.variant)<<<kc.blocks / RECOMPUTE_CLUSTER * RECOMPUTE_CLUSTER,
+                                 RECOMPUTE_WARPS * 32, kc.smem, stream>>>(db, params, state, scr);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
   k<<<kc.blocks, INTRA_WARPS * 32, kc.smem, stream>>>(db, params, state, scr);
   return cudaGetLastError();
 }

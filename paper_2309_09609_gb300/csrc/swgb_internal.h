@@ -163,8 +163,13 @@ cudaError_t launch_inter2q(const KernelConfig& kc, int gclass, const DbView& db,
 constexpr int INTRA_WARPS = 16;  // warps per block
 size_t intra_smem_bytes(int rows);
 int intra_blocks_per_sm(int rows);
-cudaError_t launch_intra(const KernelConfig& kc, const DbView& db, const SearchParams* params,
-                         SearchState* state, const Scratch& scr, cudaStream_t stream);
+// items: int32 items, which leave no flagged pairs; otherwise the flagged pairs
+cudaError_t launch_intra(const KernelConfig& kc, bool items, const DbView& db,
+                         const SearchParams* params, SearchState* state, const Scratch& scr,
+                         cudaStream_t stream);
+constexpr int RECOMPUTE_CLUSTER = 16;     // blocks per cluster
+constexpr int RECOMPUTE_WARPS = 8;        // warps per block
+constexpr int RECOMPUTE_PER_CLUSTER = 4;  // at most so many flagged pairs per cluster
 
 // Flag-list overflow (intra_kernel.cu): appends every pair whose score in
 // P->scores is FLAG_SENTINEL to the flag list (up to its capacity, counting

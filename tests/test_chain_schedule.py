@@ -36,3 +36,22 @@ def test_borders_are_written_before_and_read_before_overwritten(passes, n):
         assert start[p] + spass <= end
         if p + W < passes:
             assert start[p] + spass <= start[p + W]
+
+
+@pytest.mark.parametrize("passes", [2, 105, 128, 129, 140])
+@pytest.mark.parametrize("n", [1, 33, 400, 12_500])
+def test_recompute_over_a_cluster(passes, n):
+    """recompute_kernel (csrc/intra_kernel.cu): the stages of 32 steps of the
+    block recompute over the 128 warps of a cluster; a stage's reads fetch the
+    next one's 32 columns."""
+    warps, lag = 128, 3
+    spass = (n + 31 + 31) // 32
+    period = max(spass, lag * warps)
+    start = [p // warps * period + p % warps * lag for p in range(passes)]
+    for p in range(1, passes):
+        for j in range(0, n, 7):
+            read = start[p] + (0 if j < 32 else j // 32 - 1)
+            assert start[p - 1] + (j + 31) // 32 < read
+            if p - 1 + warps < passes:
+                assert read < start[p - 1 + warps] + (j + 31) // 32
+    assert all(start[p] + spass <= start[p + warps] for p in range(passes - warps))
