@@ -87,7 +87,8 @@ __device__ __forceinline__ void intra_cells(int (&Hp)[TI], int (&E)[TI], int& hd
 #pragma unroll
   for (int r = 0; r < TI; r++) {
     // as packed_cell: E >= 0 stands for the zero term, S from the diagonal term
-    const int x = hd + sext_byte(pw[r / 4], r & 3);
+    // (one DP4A picks row r's score from its profile word and adds it)
+    const int x = __dp4a((int)pw[r / 4], 1 << (8 * (r & 3)), hd);
     const int h = __vimax3_s32(x, E[r], f);  // Eq. 1
     hd = Hp[r];
     Hp[r] = h;
