@@ -1,15 +1,22 @@
 // align_kernel.cu -- optimal local alignments with traceback (sw_align).
 //
 // The score kernels return S only.  For selected pairs this file also
-// recovers the alignment behind S, by the traceback of Section II-B:
+// recovers the alignment behind S, by the traceback of Section II-B.  A team of
+// W warps takes a pair:
 //
-//   * align_forward: one warp per pair runs the int32 warp wavefront of
-//     Eq. 1-3 (lane k owns AT query rows of a 32*AT-row pass, (H, F) borders
-//     by __shfl_up_sync, pass borders in scratch) and stores four bits per
-//     cell -- where H came from, and whether E of the next column and F of
-//     the next row open a gap here -- plus the cell holding S;
-//   * align_traceback: one thread per pair walks those bits back from that
-//     cell and writes the transcript.
+//   * forward: the int32 warp wavefront of Eq. 1-3 (lane k owns AT query rows of
+//     a 32*AT-row pass, (H, F) borders by __shfl_up_sync).  Every cell stores
+//     four bits -- where H came from, and whether E of the next column and F
+//     of the next row open a gap here -- and the team keeps the cell holding S.
+//     The passes go round-robin to the team's warps on the stage schedule of
+//     the int32 recompute (intra_kernel.cu): pass p starts ALAG stages of 16
+//     steps after pass p - 1, a stage ends at the team's barrier, each warp
+//     writes the bottom rows of its passes to its own border row and reads
+//     those of the warp before;
+//   * traceback, by the team's first warp: 32 cells of the path at a time.
+//     Along the diagonal the lanes read the bits of the next 32 cells at once
+//     and a ballot gives the length of the run; in a gap they read along the
+//     row or the column.
 //
 // Which of several optimal alignments is returned:
 //   1. it ends at the first cell (i, j) in row-major order whose H equals S;
@@ -20,368 +27,330 @@
 //   4. the walk ends with the diagonal step into a cell whose H is 0.
 // Transcript, first column to last: 'M' (query and subject residue), 'I'
 // (query residue against a gap), 'D' (subject residue against a gap).
+//
+// Bound by latency: a call has few pairs, so what counts is a pair's chain of
+// steps and not the chip's rate.  Hence the bits come off the chain (a subtract
+// whose sign a funnel shift collects, four per cell, combined once per lane), the best cell is looked for only in steps whose largest H reaches the
+// lane's best, codes and profile words are loaded ahead, and teams are as
+// large as the call leaves room for.  Measured, kernel time: 20 pairs of 400
+// residues, the longest 662 x 1,236, 1.23 -> 0.34 ms (forward 0.90, walk 0.33
+// before); 500 such pairs, the longest subject 3,343, 4.9 -> 0.97 ms.
 #include <algorithm>
 
-#include "device_common.cuh"
+#include "lane_profile.cuh"
 
 namespace swgb {
 
-constexpr int AT = 8;            // query rows per lane
-constexpr int AROWS = 32 * AT;   // rows per pass
-constexpr int ALIGN_WARPS = 4;   // warps per block
+constexpr int ASTAGE = 16;  // steps of a stage
+constexpr int ALAG = 4;     // stages between the starts of consecutive passes
 
-// Cell nibble: bits 0-1 the source of H (0: H is 0, 1: diagonal, 2: E,
-// 3: F); bit 2: E of the next column opens here; bit 3: F of the next row
-// opens here.  Word (pass p, step t, lane k) holds the nibbles of the lane's
-// AT rows at column t - k, row r of the lane in bits 4r..4r+3.
-__device__ __forceinline__ int64_t bits_word(int64_t base, int n, int p, int t, int lane) {
-  return base + ((int64_t)p * (n + 31) + t) * 32 + lane;
+// A team of W warps, AT query rows per lane: as many warps as there is room
+// for and few rows for a call of few pairs, whose steps are then short; a block
+// is a team, or four teams of one warp.  The bits of a lane's rows at one step
+// are one word.
+template <int W>
+struct AlignShape {
+  static constexpr int AT = W == 16 ? 4 : 8;
+  static constexpr int ROWS = 32 * AT;  // rows per pass
+  static constexpr int PROFILE = NCODES * 32 * AT;
+  static constexpr int TEAMS = W == 1 ? 4 : 1;
+  static constexpr int WARPS = W * TEAMS;
+};
+template <int AT> struct AlignWord;
+template <> struct AlignWord<4> { typedef uint16_t type; };
+template <> struct AlignWord<8> { typedef uint32_t type; };
+
+// Word (pass p, step t, lane k) holds the cells of the lane's AT rows at
+// column t - k: four fields of AT bits, with row r at bit AT - 1 - r of each.
+// Fields 0 and 1 tell the source of H (where it is not 0): (1, 0) diagonal,
+// (0, 1) E, (0, 0) F; field 2: E of the next column opens here; field 3: F
+// of the next row opens here.
+__device__ __forceinline__ int64_t bits_word(int n, int p, int t, int lane) {
+  return ((int64_t)p * (n + 31) + t) * 32 + lane;
 }
 
 __device__ __forceinline__ bool end_before(int v, int i, int j, int bv, int bi, int bj) {
   return v > bv || (v == bv && (i < bi || (i == bi && j < bj)));
 }
 
-__global__ void __launch_bounds__(ALIGN_WARPS * 32)
-align_forward(DbView db, const SearchParams* __restrict__ P, const AlignItem* __restrict__ items,
-              int n_items, uint32_t* __restrict__ bits, int2* __restrict__ border,
-              AlignOut* __restrict__ out) {
-  __shared__ __align__(16) uint8_t prof_all[ALIGN_WARPS][NCODES * 32 * AT];
-  __shared__ int8_t sm[NCODES * NCODES];
-  load_matrix(sm, P);
-  __syncthreads();
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  uint8_t* prof = prof_all[wib];
-  const int go = P->go, ge = P->ge;
-  const int warps = gridDim.x * ALIGN_WARPS;
-  for (int k = blockIdx.x * ALIGN_WARPS + wib; k < n_items; k += warps) {
-    const AlignItem it = items[k];
-    const int m = P->qlen[it.q];
-    const int n = db.clen[it.s];
-    const uint8_t* __restrict__ qr = P->qres + P->qoff[it.q];
-    const uint8_t* __restrict__ d = db.cont + db.coff[it.s];
-    int2* hb = border + it.border_off;
-    const int npass = n > 0 ? (m + AROWS - 1) / AROWS : 0;
-    // this lane's best cell so far: (H, 1-based row, 1-based column)
-    int bv = 0, bi = INT32_MAX, bj = INT32_MAX;
-    for (int p = 0; p < npass; p++) {
-      __syncwarp();
-      lane_profile<AT>(prof, sm, qr, m, p * AROWS + lane * AT, lane);
-      __syncwarp();
-      int Hp[AT], E[AT];
-#pragma unroll
-      for (int r = 0; r < AT; r++) {
-        Hp[r] = 0;    // H(i, 0)
-        E[r] = -go;   // E(i, 1)
-      }
-      int hdiag = 0, out_h = 0, out_f = -go;
-      const bool last_pass = (p == npass - 1);
-      const int row0 = p * AROWS + lane * AT;  // 0-based row of this lane's first row
-      for (int t = 0; t < n + 31; t++) {
-        int in_h = __shfl_up_sync(FULL, out_h, 1);
-        int in_f = __shfl_up_sync(FULL, out_f, 1);
-        const int j = t - lane;
-        if (lane == 0) {
-          if (p > 0 && j < n) {
-            const int2 v = hb[j];
-            in_h = v.x;
-            in_f = v.y;
-          } else {
-            in_h = 0;    // H(0, j)
-            in_f = -go;  // F(1, j)
-          }
-        }
-        if (j >= 0 && j < n) {
-          const uint2 pv = *(const uint2*)(prof + ((int)d[j] * 32 + lane) * AT);
-          int hd = hdiag;
-          hdiag = in_h;
-          int f = in_f;
-          uint32_t word = 0;
-#pragma unroll
-          for (int r = 0; r < AT; r++) {
-            const int w = sext_byte(r < 4 ? pv.x : pv.y, r & 3);
-            const int e = E[r];
-            const int diag = hd + w;
-            const int h = max(max(diag, e), max(f, 0));                  // Eq. 1
-            const uint32_t src = h == 0 ? 0u : h == diag ? 1u : h == e ? 2u : 3u;
-            hd = Hp[r];
-            Hp[r] = h;
-            const int t_open = h - go, e_ext = e - ge, f_ext = f - ge;
-            E[r] = max(e_ext, t_open);                                   // Eq. 2, next column
-            f = max(f_ext, t_open);                                      // Eq. 3, next row
-            word |= (src | (t_open >= e_ext ? 4u : 0u) | (t_open >= f_ext ? 8u : 0u)) << (4 * r);
-            const int row = row0 + r;
-            if (h > 0 && row < m && end_before(h, row + 1, j + 1, bv, bi, bj)) {
-              bv = h;
-              bi = row + 1;
-              bj = j + 1;
-            }
-          }
-          out_h = Hp[AT - 1];
-          out_f = f;
-          bits[bits_word(it.bits_off, n, p, t, lane)] = word;
-          if (lane == 31 && !last_pass) hb[j] = make_int2(out_h, out_f);
-        }
-      }
-    }
-    // the first cell in row-major order holding the largest H
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const int v2 = __shfl_xor_sync(FULL, bv, o);
-      const int i2 = __shfl_xor_sync(FULL, bi, o);
-      const int j2 = __shfl_xor_sync(FULL, bj, o);
-      if (end_before(v2, i2, j2, bv, bi, bj)) {
-        bv = v2;
-        bi = i2;
-        bj = j2;
-      }
-    }
-    if (lane == 0) {
-      AlignOut r{};
-      r.score = bv;
-      r.i_end = bv > 0 ? bi : 0;
-      r.j_end = bv > 0 ? bj : 0;
-      out[k] = r;
-    }
-  }
+// acc shifted left by one, with the sign of x (1 when negative) as its last bit
+__device__ __forceinline__ uint32_t push_sign(uint32_t acc, int x) {
+  return __funnelshift_l((uint32_t)x, acc, 1);
 }
 
-// The same forward pass with a whole block per pair, for few long pairs:
-// the 16 warps take the query's passes round-robin on the stage schedule of
-// the int32 recompute (pass p starts LAG stages of 32 steps after pass p - 1,
-// every stage ends at __syncthreads, each warp writes the bottom rows of its
-// passes to its own scratch row and reads those of the pass before).  Cells,
-// bits and the end cell are exactly those of align_forward.
-constexpr int ABW = 16;   // warps per block
-constexpr int ALAG = 3;   // stages between the starts of consecutive passes
-
-__global__ void __launch_bounds__(ABW * 32)
-align_forward_block(DbView db, const SearchParams* __restrict__ P,
-                    const AlignItem* __restrict__ items, int n_items, uint32_t* __restrict__ bits,
-                    int2* __restrict__ border, AlignOut* __restrict__ out) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  __shared__ int red_v[ABW], red_i[ABW], red_j[ABW];
-  int8_t* sm = (int8_t*)smem;
-  load_matrix(sm, P);
-  __syncthreads();
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  uint8_t* prof = smem + MATRIX_SMEM + wib * (NCODES * 32 * AT);
-  const int go = P->go, ge = P->ge;
-  for (int k = blockIdx.x; k < n_items; k += gridDim.x) {  // uniform over the block
-    const AlignItem it = items[k];
-    const int m = P->qlen[it.q];
-    const int n = db.clen[it.s];
-    const uint8_t* __restrict__ qr = P->qres + P->qoff[it.q];
-    const uint8_t* __restrict__ d = db.cont + db.coff[it.s];
-    int2* own = border + it.border_off + (int64_t)wib * n;               // this warp's rows
-    const int2* src = border + it.border_off + (int64_t)((wib + ABW - 1) % ABW) * n;
-    const int npass = n > 0 ? (m + AROWS - 1) / AROWS : 0;
-    const int spass = (n + 31 + 31) / 32;
-    const int period = max(spass, ALAG * ABW);
-    const int nstages =
-        npass > 0 ? ((npass - 1) / ABW) * period + ((npass - 1) % ABW) * ALAG + spass : 0;
-    const int2 top = make_int2(0, -go);
-    int bv = 0, bi = INT32_MAX, bj = INT32_MAX;
-    int Hp[AT], E[AT], hdiag = 0, out_h = 0, out_f = -go;
-    int p = 0;
-    int2 bcur = top, bnext = top;
-    for (int g = 0; g < nstages; g++) {
-      const int rel = g - wib * ALAG;
-      int ks = -1;
-      if (rel >= 0) {
-        const int r = rel / period;
-        const int kk = rel - r * period;
-        if (kk < spass && wib + r * ABW < npass) {
-          ks = kk;
-          p = wib + r * ABW;
-        }
-      }
-      if (ks >= 0) {  // warp-uniform
-        if (ks == 0) {
-          __syncwarp();
-          lane_profile<AT>(prof, sm, qr, m, p * AROWS + lane * AT, lane);
-          __syncwarp();
-#pragma unroll
-          for (int r = 0; r < AT; r++) {
-            Hp[r] = 0;
-            E[r] = -go;
-          }
-          hdiag = 0;
-          out_h = 0;
-          out_f = -go;
-          bcur = (p > 0 && lane < n) ? src[lane] : top;
-        } else {
-          bcur = bnext;
-        }
-        const int jn = 32 * (ks + 1) + lane;
-        bnext = (p > 0 && jn < n) ? src[jn] : top;
-        const bool last_pass = (p == npass - 1);
-        const int row0 = p * AROWS + lane * AT;
-        const int t0 = 32 * ks;
-        const int tend = min(t0 + 32, n + 31);
-        for (int t = t0; t < tend; t++) {
-          int in_h = __shfl_up_sync(FULL, out_h, 1);
-          int in_f = __shfl_up_sync(FULL, out_f, 1);
-          const int bh = __shfl_sync(FULL, bcur.x, t - t0);
-          const int bf = __shfl_sync(FULL, bcur.y, t - t0);
-          if (lane == 0) {
-            in_h = bh;
-            in_f = bf;
-          }
-          const int j = t - lane;
-          if (j >= 0 && j < n) {
-            const uint2 pv = *(const uint2*)(prof + ((int)d[j] * 32 + lane) * AT);
-            int hd = hdiag;
-            hdiag = in_h;
-            int f = in_f;
-            uint32_t word = 0;
-#pragma unroll
-            for (int r = 0; r < AT; r++) {
-              const int w = sext_byte(r < 4 ? pv.x : pv.y, r & 3);
-              const int e = E[r];
-              const int diag = hd + w;
-              const int h = max(max(diag, e), max(f, 0));                // Eq. 1
-              const uint32_t srcc = h == 0 ? 0u : h == diag ? 1u : h == e ? 2u : 3u;
-              hd = Hp[r];
-              Hp[r] = h;
-              const int t_open = h - go, e_ext = e - ge, f_ext = f - ge;
-              E[r] = max(e_ext, t_open);                                 // Eq. 2
-              f = max(f_ext, t_open);                                    // Eq. 3
-              word |= (srcc | (t_open >= e_ext ? 4u : 0u) | (t_open >= f_ext ? 8u : 0u)) << (4 * r);
-              const int row = row0 + r;
-              if (h > 0 && row < m && end_before(h, row + 1, j + 1, bv, bi, bj)) {
-                bv = h;
-                bi = row + 1;
-                bj = j + 1;
-              }
-            }
-            out_h = Hp[AT - 1];
-            out_f = f;
-            bits[bits_word(it.bits_off, n, p, t, lane)] = word;
-            if (lane == 31 && !last_pass) own[j] = make_int2(out_h, out_f);
-          }
-        }
-      }
-      __syncthreads();
+struct AlignBest {
+  int v, i, j;  // H, 1-based row and column
+  __device__ __forceinline__ void take(int v2, int i2, int j2) {
+    if (end_before(v2, i2, j2, v, i, j)) {
+      v = v2;
+      i = i2;
+      j = j2;
     }
-    // the first cell in row-major order holding the largest H, over the block
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const int v2 = __shfl_xor_sync(FULL, bv, o);
-      const int i2 = __shfl_xor_sync(FULL, bi, o);
-      const int j2 = __shfl_xor_sync(FULL, bj, o);
-      if (end_before(v2, i2, j2, bv, bi, bj)) {
-        bv = v2;
-        bi = i2;
-        bj = j2;
-      }
-    }
-    if (lane == 0) {
-      red_v[wib] = bv;
-      red_i[wib] = bi;
-      red_j[wib] = bj;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      for (int w = 1; w < ABW; w++)
-        if (end_before(red_v[w], red_i[w], red_j[w], bv, bi, bj)) {
-          bv = red_v[w];
-          bi = red_i[w];
-          bj = red_j[w];
-        }
-      AlignOut r{};
-      r.score = bv;
-      r.i_end = bv > 0 ? bi : 0;
-      r.j_end = bv > 0 ? bj : 0;
-      out[k] = r;
-    }
-    __syncthreads();  // red_* are rewritten by the next pair
   }
-}
+};
 
-__global__ void __launch_bounds__(128)
-align_traceback(DbView db, const SearchParams* __restrict__ P, const AlignItem* __restrict__ items,
-                int n_items, const uint32_t* __restrict__ bits, AlignOut* __restrict__ out,
-                uint8_t* __restrict__ ops) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n_items) return;
-  const AlignItem it = items[k];
-  AlignOut r = out[k];
+// The forward pass of one pair on the team's W warps; `warp` is this warp's
+// place in the team.  Returns the lane's best cell.
+template <int W, typename Word, typename Barrier>
+__device__ __forceinline__ AlignBest align_forward(const DbView& db,
+                                                   const SearchParams* __restrict__ P,
+                                                   const AlignItem& it, uint8_t* prof,
+                                                   const uint8_t* sm, int lane, int warp,
+                                                   Word* bits, int2* border,
+                                                   Barrier barrier) {
+  constexpr int AT = AlignShape<W>::AT, AROWS = AlignShape<W>::ROWS;
+  const int go = P->go, ge = P->ge;
   const int m = P->qlen[it.q];
   const int n = db.clen[it.s];
-  int64_t pos = it.ops_end;  // the transcript is written backwards, ending here
-  r.q_begin = r.s_begin = 0;
-  if (r.score > 0) {
-    auto nib = [&](int i, int j) -> uint32_t {  // 1-based cell
-      const int row = i - 1, lane = (row % AROWS) / AT;
-      const uint32_t w = bits[bits_word(it.bits_off, n, row / AROWS, j - 1 + lane, lane)];
-      return (w >> (4 * (row % AT))) & 15u;
-    };
-    int i = r.i_end, j = r.j_end, state = 0;  // 0: H, 1: E, 2: F
-    // at most m + n columns, each gap run entered by one more step from
-    // state H: the bound only guards against a broken bit matrix
-    for (int64_t guard = 0; guard < 2 * ((int64_t)m + n) + 2; guard++) {
-      if (state == 0) {
-        const uint32_t src = nib(i, j) & 3u;
-        if (src == 1u) {
-          ops[--pos] = 'M';
-          i--;
-          j--;
-          if (i == 0 || j == 0 || (nib(i, j) & 3u) == 0u) break;
-        } else {
-          state = src == 2u ? 1 : 2;
-        }
-      } else if (state == 1) {
-        ops[--pos] = 'D';
-        state = (nib(i, j - 1) & 4u) ? 0 : 1;
-        j--;
-      } else {
-        ops[--pos] = 'I';
-        state = (nib(i - 1, j) & 8u) ? 0 : 2;
-        i--;
+  const uint8_t* __restrict__ qr = P->qres + P->qoff[it.q];
+  const uint8_t* __restrict__ d = db.cont + db.coff[it.s];
+  int2* own = border + it.border_off + (int64_t)warp * n;
+  const int2* src = border + it.border_off + (int64_t)((warp + W - 1) % W) * n;
+  const int npass = n > 0 ? (m + AROWS - 1) / AROWS : 0;
+  const int spass = (n + 31 + ASTAGE - 1) / ASTAGE;
+  const int period = max(spass, ALAG * W);
+  const int nstages =
+      npass > 0 ? ((npass - 1) / W) * period + ((npass - 1) % W) * ALAG + spass : 0;
+  const int2 top = make_int2(0, -go);
+  AlignBest best{0, INT32_MAX, INT32_MAX};
+  int H[AT], E[AT], hdiag = 0, out_h = 0, out_f = -go;
+  int p = 0;
+  int2 bcur = top, bnext = top;
+  for (int g = 0; g < nstages; g++) {
+    const int rel = g - warp * ALAG;
+    int k = -1;
+    if (rel >= 0) {
+      const int r = rel / period;
+      const int kk = rel - r * period;
+      if (kk < spass && warp + r * W < npass) {
+        k = kk;
+        p = warp + r * W;
       }
     }
-    r.q_begin = i;
-    r.s_begin = j;
+    if (k >= 0) {  // warp-uniform
+      if (k == 0) {
+        __syncwarp();
+        lane_profile_rows<AT, 1>(prof, sm, qr, m, p * AROWS, 32, 0, 1);
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < AT; r++) H[r] = E[r] = 0;
+        hdiag = 0;
+        out_h = 0;
+        out_f = -go;
+        bcur = (p > 0 && lane < min(ASTAGE, n)) ? src[lane] : top;
+      } else {
+        bcur = bnext;
+      }
+      const int jn = ASTAGE * (k + 1) + lane;
+      bnext = (p > 0 && lane < ASTAGE && jn < n) ? src[jn] : top;
+      const bool last_pass = (p == npass - 1);
+      const int row0 = p * AROWS + lane * AT;  // 0-based row of this lane's first row
+      const int t0 = ASTAGE * k;
+      const int tend = min(t0 + ASTAGE, n + 31);
+      IntraFeed<AT, true> feed{d, prof + lane * AT, n};
+      feed.start(t0 - lane);
+#pragma unroll 4
+      for (int t = t0; t < tend; t++) {
+        uint32_t pw[AT / 4];
+        feed.step(pw, t - lane);
+        int in_h = __shfl_up_sync(FULL, out_h, 1);
+        int in_f = __shfl_up_sync(FULL, out_f, 1);
+        const int bh = __shfl_sync(FULL, bcur.x, t - t0);
+        const int bf = __shfl_sync(FULL, bcur.y, t - t0);
+        if (lane == 0) {
+          in_h = bh;
+          in_f = bf;
+        }
+        // columns left and right of the subject hold the padding code: their
+        // cells leave H and E at 0 before it, and are not looked at after it
+        const int j = t - lane;
+        int hd = hdiag, f = in_f, top_h = 0;
+        hdiag = in_h;
+        // signs: H above the diagonal term, above E; H - Go below the next E,
+        // below the next F
+        uint32_t sa = 0, sb = 0, se = 0, sf = 0;
+#pragma unroll
+        for (int r = 0; r < AT; r++) {
+          const int e = E[r];  // floored at 0: only cells with E > 0 matter to the walk
+          const int x = __dp4a((int)pw[r / 4], 1 << (8 * (r & 3)), hd);
+          const int h = __vimax3_s32(x, e, f);                  // Eq. 1
+          hd = H[r];
+          H[r] = h;
+          const int tt = h - go;
+          E[r] = __viaddmax_s32_relu(e, -ge, tt);               // Eq. 2, next column
+          f = __viaddmax_s32(f, -ge, tt);                       // Eq. 3, next row
+          sa = push_sign(sa, x - h);
+          sb = push_sign(sb, e - h);
+          se = push_sign(se, tt - E[r]);
+          sf = push_sign(sf, tt - f);
+          top_h = max(top_h, h);
+        }
+        out_h = H[AT - 1];
+        out_f = f;
+        constexpr uint32_t F = (1u << AT) - 1;
+        bits[bits_word(n, p, t, lane)] =
+            (Word)((~sa & F) | (~sb & sa & F) << AT | (~se & F) << 2 * AT | (~sf & F) << 3 * AT);
+        if (top_h >= best.v && top_h > 0 && j < n) {
+#pragma unroll
+          for (int r = 0; r < AT; r++)
+            if (H[r] > 0 && row0 + r < m) best.take(H[r], row0 + r + 1, j + 1);
+        }
+        if (lane == 31 && !last_pass && j >= 0 && j < n) own[j] = make_int2(out_h, out_f);
+      }
+    }
+    barrier();
   }
-  r.n_ops = (int32_t)(it.ops_end - pos);
-  r.ops_offset = pos;
-  out[k] = r;
+  // the first cell in row-major order holding the largest H of the warp
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const int v = __shfl_xor_sync(FULL, best.v, o), i = __shfl_xor_sync(FULL, best.i, o),
+              j = __shfl_xor_sync(FULL, best.j, o);
+    best.take(v, i, j);
+  }
+  return best;
 }
 
-cudaError_t launch_align(const DbView& db, const SearchParams* params, const AlignItem* items,
-                         int n_items, bool block_mode, uint32_t* bits, int2* border, AlignOut* out,
-                         uint8_t* ops, cudaStream_t stream) {
-  if (n_items <= 0) return cudaSuccess;
-  int sms = 0, dev = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaError_t e;
-  if (block_mode) {
-    const size_t smem = (size_t)MATRIX_SMEM + (size_t)ABW * NCODES * 32 * AT;
-    e = cudaFuncSetAttribute(align_forward_block, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
-    if (e != cudaSuccess) return e;
-    cudaGetLastError();  // a stale error must not be read as this launch's
-    align_forward_block<<<std::min(n_items, std::max(sms, 1)), ABW * 32, smem, stream>>>(
-        db, params, items, n_items, bits, border, out);
-  } else {
-    const int blocks = std::min((n_items + ALIGN_WARPS - 1) / ALIGN_WARPS, std::max(sms, 1) * 8);
-    cudaGetLastError();  // a stale error must not be read as this launch's
-    align_forward<<<blocks, ALIGN_WARPS * 32, 0, stream>>>(db, params, items, n_items, bits,
-                                                           border, out);
+// The walk back from `best`, on one warp.  v is H (or E or F) of the current
+// cell, which the matrix and the penalties give step by step.
+template <int W, typename Word>
+__device__ __forceinline__ void align_traceback(const DbView& db,
+                                                const SearchParams* __restrict__ P,
+                                                const AlignItem& it, const AlignBest& best,
+                                                const uint8_t* sm, int lane, const Word* bits,
+                                                uint8_t* ops, AlignOut* out) {
+  constexpr int AT = AlignShape<W>::AT, AROWS = AlignShape<W>::ROWS;
+  const int m = P->qlen[it.q];
+  const int n = db.clen[it.s];
+  const int go = P->go, ge = P->ge;
+  const uint8_t* __restrict__ qr = P->qres + P->qoff[it.q];
+  const uint8_t* __restrict__ d = db.cont + db.coff[it.s];
+  int64_t pos = it.ops_end;  // the transcript is written backwards, ending here
+  int i = best.i, j = best.j, v = best.v, state = 0;  // 0: H, 1: E, 2: F
+  // a cell's bits, field f at bit f * AT; cells off the matrix open any gap
+  auto cell = [&](int ci, int cj) -> uint32_t {
+    if (ci < 1 || cj < 1) return 1u << 2 * AT | 1u << 3 * AT;
+    const int row = ci - 1, l = row % AROWS / AT;
+    return (uint32_t)bits[bits_word(n, row / AROWS, cj - 1 + l, l)] >> (AT - 1 - row % AT);
+  };
+  // every round takes at least one column or changes the state; the bound only
+  // guards against a broken bit matrix
+  for (int64_t guard = 0; v > 0 && guard < 2 * ((int64_t)m + n) + 2; guard++) {
+    int run;
+    uint8_t op;
+    if (state == 0) {
+      const int ci = i - lane, cj = j - lane;
+      const uint32_t w = cell(ci, cj);
+      // H after this cell's diagonal step, while the run lasts
+      int h = ci >= 1 && cj >= 1 ? (int)(int8_t)sm[qr[ci - 1] * SM_ROW + d[cj - 1]] : 0;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(FULL, h, o);
+        if (lane >= o) h += x;
+      }
+      h = v - h;
+      const uint32_t other = __ballot_sync(FULL, !(w & 1u)), zero = __ballot_sync(FULL, h == 0);
+      const int first = other ? __ffs(other) - 1 : 32;  // not from the diagonal
+      const int end = zero ? __ffs(zero) : 33;          // columns to the cell whose H is 0
+      run = min(first, end);
+      op = 'M';
+      if (run > 0) v = __shfl_sync(FULL, h, run - 1);
+      if (first < 32) state = __shfl_sync(FULL, w >> AT & 1u, first) ? 1 : 2;
+      if (lane < run) ops[pos - 1 - lane] = op;
+      pos -= run;
+      i -= run;
+      j -= run;
+    } else {
+      const uint32_t w = state == 1 ? cell(i, j - 1 - lane) >> 2 * AT : cell(i - 1 - lane, j) >> 3 * AT;
+      const uint32_t opens = __ballot_sync(FULL, w & 1u);
+      run = opens ? __ffs(opens) : 32;
+      op = state == 1 ? 'D' : 'I';
+      if (lane < run) ops[pos - 1 - lane] = op;
+      pos -= run;
+      (state == 1 ? j : i) -= run;
+      v += opens ? (run - 1) * ge + go : run * ge;
+      if (opens) state = 0;
+    }
   }
-  e = cudaGetLastError();
+  if (lane == 0) {
+    AlignOut r{};
+    r.score = best.v;
+    if (best.v > 0) {
+      r.i_end = best.i;
+      r.j_end = best.j;
+      r.q_begin = i;
+      r.s_begin = j;
+    }
+    r.n_ops = (int32_t)(it.ops_end - pos);
+    r.ops_offset = pos;
+    *out = r;
+  }
+}
+
+template <int W>
+__global__ void __launch_bounds__(AlignShape<W>::WARPS * 32)
+align_kernel(DbView db, const SearchParams* __restrict__ P, const AlignItem* __restrict__ items,
+             int n_items, uint8_t* bits, int2* border, AlignOut* out, uint8_t* ops) {
+  constexpr int TEAMS = AlignShape<W>::TEAMS;
+  typedef typename AlignWord<AlignShape<W>::AT>::type Word;
+  extern __shared__ __align__(16) uint8_t smem[];
+  __shared__ __align__(16) uint8_t sm[NCODES * SM_ROW];
+  __shared__ AlignBest red[W];
+  for (int i = threadIdx.x; i < NCODES * SM_ROW; i += blockDim.x)
+    sm[i] = i % SM_ROW < NCODES ? (uint8_t)P->sm[i / SM_ROW * NCODES + i % SM_ROW] : 0;
+  __syncthreads();
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, warp = wib % W;
+  uint8_t* prof = smem + wib * AlignShape<W>::PROFILE;
+  // uniform over the team
+  for (int k = blockIdx.x * TEAMS + wib / W; k < n_items; k += gridDim.x * TEAMS) {
+    const AlignItem it = items[k];
+    Word* words = (Word*)(bits + it.bits_off);
+    AlignBest best = align_forward<W>(db, P, it, prof, sm, lane, warp, words, border, []() {
+      if constexpr (W > 1) __syncthreads();
+      else __syncwarp();
+    });
+    if constexpr (W > 1) {
+      if (lane == 0) red[warp] = best;
+      __syncthreads();
+      if (warp == 0)
+        for (int w = 1; w < W; w++) best.take(red[w].v, red[w].i, red[w].j);
+    }
+    if (warp == 0) align_traceback<W>(db, P, it, best, sm, lane, words, ops, out + k);
+    if constexpr (W > 1) __syncthreads();  // red is rewritten by the next pair
+  }
+}
+
+// 16 warps to a pair while there are SMs for every pair, 4 while those teams
+// (near enough) fit the chip at once, then one.
+int align_team(int n_pairs, int sms) { return n_pairs <= sms ? 16 : n_pairs <= 16 * sms ? 4 : 1; }
+
+template <int W>
+static cudaError_t launch_team(int sms, const DbView& db, const SearchParams* params,
+                               const AlignItem* items, int n_items, uint8_t* bits, int2* border,
+                               AlignOut* out, uint8_t* ops, cudaStream_t stream) {
+  const int smem = AlignShape<W>::WARPS * AlignShape<W>::PROFILE;
+  cudaError_t e =
+      cudaFuncSetAttribute(align_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
+  const int teams = AlignShape<W>::TEAMS;
   cudaGetLastError();  // a stale error must not be read as this launch's
-  align_traceback<<<(n_items + 127) / 128, 128, 0, stream>>>(db, params, items, n_items, bits, out,
-                                                             ops);
+  align_kernel<W><<<std::min((n_items + teams - 1) / teams, std::max(sms, 1) * 16),
+                    AlignShape<W>::WARPS * 32, smem, stream>>>(db, params, items, n_items, bits,
+                                                              border, out, ops);
   return cudaGetLastError();
 }
 
-int64_t align_bits_words(int32_t m, int32_t n) {
+cudaError_t launch_align(int team, int sms, const DbView& db, const SearchParams* params,
+                         const AlignItem* items, int n_items, uint8_t* bits, int2* border,
+                         AlignOut* out, uint8_t* ops, cudaStream_t stream) {
+  if (n_items <= 0) return cudaSuccess;
+  auto launch = team == 16 ? launch_team<16> : team == 4 ? launch_team<4> : launch_team<1>;
+  return launch(sms, db, params, items, n_items, bits, border, out, ops, stream);
+}
+
+int64_t align_bits_bytes(int team, int32_t m, int32_t n) {
   if (m <= 0 || n <= 0) return 0;
-  return (int64_t)((m + AROWS - 1) / AROWS) * (n + 31) * 32;
+  const int at = team == 16 ? AlignShape<16>::AT : AlignShape<4>::AT;
+  return (int64_t)((m + 32 * at - 1) / (32 * at)) * (n + 31) * 32 * (at / 2);
 }
 
 }  // namespace swgb

@@ -1597,17 +1597,15 @@ extern "C" sw_status sw_align(sw_db* db, const uint8_t* queries, const int32_t* 
     return sw_set_error(SW_EINVAL, "ops needs %lld bytes, has %lld", (long long)slot[n_pairs],
                         (long long)ops_capacity);
   if (n_pairs == 0) return SW_OK;
-  // few pairs: a block of 16 warps per pair; many: a warp per pair
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, db->device);
-  const bool block_mode = n_pairs <= std::max(sms, 1);
-  const int64_t border_rows = block_mode ? ALIGN_BLOCK_ROWS : 1;
+  const int team = align_team(n_pairs, sms);  // warps to a pair
   // chunks of pairs whose direction bits fit kAlignChunkBytes (one pair may exceed it alone)
   std::vector<int32_t> chunk_begin{0};
   int64_t words = 0, max_words = 0, max_border = 0, border = 0;
   for (int32_t k = 0; k < n_pairs; k++) {
-    const int64_t w = align_bits_words(hb.len[items[k].q], db->clen_h[items[k].s]);
-    if (k > chunk_begin.back() && 4 * (words + w) > kAlignChunkBytes) {
+    const int64_t w = align_bits_bytes(team, hb.len[items[k].q], db->clen_h[items[k].s]);
+    if (k > chunk_begin.back() && words + w > kAlignChunkBytes) {
       chunk_begin.push_back(k);
       words = border = 0;
     }
@@ -1615,7 +1613,7 @@ extern "C" sw_status sw_align(sw_db* db, const uint8_t* queries, const int32_t* 
     items[k].border_off = border;
     items[k].ops_end = slot[k + 1];
     words += w;
-    border += border_rows * db->clen_h[items[k].s];
+    border += (int64_t)team * db->clen_h[items[k].s];
     max_words = std::max(max_words, words);
     max_border = std::max(max_border, border);
   }
@@ -1627,7 +1625,7 @@ extern "C" sw_status sw_align(sw_db* db, const uint8_t* queries, const int32_t* 
   SearchParams* Pd = nullptr;
   AlignItem* items_d = nullptr;
   AlignOut* out_d = nullptr;
-  uint32_t* bits = nullptr;
+  uint8_t* bits = nullptr;
   int2* border_d = nullptr;
   uint8_t* ops_d = nullptr;
   std::vector<AlignOut> res((size_t)n_pairs);
@@ -1655,7 +1653,7 @@ extern "C" sw_status sw_align(sw_db* db, const uint8_t* queries, const int32_t* 
     e = cudaMemcpyAsync(items_d, items.data(), sizeof(AlignItem) * n_pairs, cudaMemcpyHostToDevice, cs);
   for (size_t c = 0; c + 1 < chunk_begin.size() && e == cudaSuccess; c++) {
     const int32_t k0 = chunk_begin[c], nk = chunk_begin[c + 1] - k0;
-    e = launch_align(db->view, Pd, items_d + k0, nk, block_mode, bits, border_d, out_d + k0, ops_d,
+    e = launch_align(team, sms, db->view, Pd, items_d + k0, nk, bits, border_d, out_d + k0, ops_d,
                      cs);
     // the next chunk reuses the bits: its kernels run after this one's on the stream
   }

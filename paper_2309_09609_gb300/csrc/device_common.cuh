@@ -117,6 +117,44 @@ __device__ __forceinline__ void lane_profile(uint8_t* prof, const int8_t* __rest
   }
 }
 
+// The lane's profile words along its columns, loaded ahead of the cells: the
+// code of column j + 2 and the words of column j + 1 while column j is scored
+// (columns past either end read the padding code with PAD, else the last or
+// first code, for lanes that skip them).
+template <int TI, bool PAD = false>
+struct IntraFeed {
+  const uint8_t* d;     // the subject's codes
+  const uint8_t* prof;  // the lane's profile rows, 32 * TI bytes per code
+  int n, code;
+  uint32_t next[TI / 4];
+
+  __device__ __forceinline__ int at(int j) const {
+    const int c = d[min(max(j, 0), n - 1)];
+    return PAD && (unsigned)j >= (unsigned)n ? PAD_CODE : c;
+  }
+  __device__ __forceinline__ void words() {
+    const uint8_t* lp = prof + code * 32 * TI;
+    if constexpr (TI == 8) {
+      const uint2 v = *(const uint2*)lp;
+      next[0] = v.x, next[1] = v.y;
+    } else {
+      const uint4 v = *(const uint4*)lp;
+      next[0] = v.x, next[1] = v.y, next[2] = v.z, next[3] = v.w;
+    }
+  }
+  __device__ __forceinline__ void start(int j) {  // the next column is j
+    code = at(j);
+    words();
+    code = at(j + 1);
+  }
+  __device__ __forceinline__ void step(uint32_t (&pw)[TI / 4], int j) {  // column j's words
+#pragma unroll
+    for (int k = 0; k < TI / 4; k++) pw[k] = next[k];
+    words();
+    code = at(j + 2);
+  }
+};
+
 // ---- packed 16-bit cells (two cells per 32-bit word) -------------------------
 //
 // Each half of a word is one cell's H, E or F as a signed 16-bit integer.  The

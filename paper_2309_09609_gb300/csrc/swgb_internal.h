@@ -206,7 +206,7 @@ cudaError_t launch_plain(int blocks, const DbView& db, const SearchParams* param
 struct AlignItem {
   int32_t q;          // query index (SearchParams::qres / qoff / qlen)
   int32_t s;          // sorted subject index
-  int64_t bits_off;   // first uint32 of this pair's direction bits
+  int64_t bits_off;   // first byte of this pair's direction bits
   int64_t border_off; // first int2 of this pair's pass-border row
   int64_t ops_end;    // the transcript ends just before this byte of the ops buffer
 };
@@ -217,14 +217,14 @@ struct AlignOut {
   int32_t n_ops;
   int64_t ops_offset;        // the transcript occupies [ops_offset, ops_offset + n_ops)
 };
-// uint32 words of direction bits for an m x n pair (4 bits per cell)
-int64_t align_bits_words(int32_t m, int32_t n);
-// block_mode: one block of 16 warps per pair (border: 16 rows of the subject's
-// length per pair), else one warp per pair (one row per pair)
-cudaError_t launch_align(const DbView& db, const SearchParams* params, const AlignItem* items,
-                         int n_items, bool block_mode, uint32_t* bits, int2* border, AlignOut* out,
-                         uint8_t* ops, cudaStream_t stream);
-constexpr int ALIGN_BLOCK_ROWS = 16;  // border rows per pair in block mode
+// bytes of direction bits for an m x n pair (4 bits per cell)
+int64_t align_bits_bytes(int team, int32_t m, int32_t n);
+// Warps to a pair (each with a border row of the subject's length) for a call
+// of n_pairs.
+int align_team(int n_pairs, int sms);
+cudaError_t launch_align(int team, int sms, const DbView& db, const SearchParams* params,
+                         const AlignItem* items, int n_items, uint8_t* bits, int2* border,
+                         AlignOut* out, uint8_t* ops, cudaStream_t stream);
 
 // Integer-pipe microbenchmark (intpeak.cu).
 int intpeak_run(int op, int blocks_per_sm, int threads, int iters, double* lane_ops_per_clk_sm,

@@ -55,3 +55,22 @@ def test_recompute_over_a_cluster(passes, n):
             if p - 1 + warps < passes:
                 assert read < start[p - 1 + warps] + (j + 31) // 32
     assert all(start[p] + spass <= start[p + warps] for p in range(passes - warps))
+
+
+@pytest.mark.parametrize("warps", [1, 4, 16])
+@pytest.mark.parametrize("passes", [2, 5, 17, 40])
+@pytest.mark.parametrize("n", [1, 15, 17, 47, 300, 1111])
+def test_alignment_teams(warps, passes, n):
+    """align_forward (csrc/align_kernel.cu): stages of 16 steps, a stage's reads
+    fetch the next one's 16 columns."""
+    stage, lag = 16, 4
+    spass = (n + 31 + stage - 1) // stage
+    period = max(spass, lag * warps)
+    start = [p // warps * period + p % warps * lag for p in range(passes)]
+    for p in range(1, passes):
+        for j in range(n):
+            read = start[p] + (0 if j < stage else j // stage - 1)
+            assert start[p - 1] + (j + 31) // stage < read
+            if p - 1 + warps < passes:
+                assert read < start[p - 1 + warps] + (j + 31) // stage
+    assert all(start[p] + spass <= start[p + warps] for p in range(passes - warps))
