@@ -274,9 +274,12 @@ typedef struct {
  *   ops: host buffer of ops_capacity bytes; pair k's transcript lies in its
  *        own slot of q_len + s_len bytes (slots back to back in pair order),
  *        at its end.  Needs ops_capacity >= sum over pairs of q_len + s_len.
- * Device memory for the direction bits (4 bits per cell of every pair) is
- * allocated by the call and freed before it returns; pairs are processed in
- * chunks of at most 8 GiB of bits.  Synchronous on the stream.
+ * Of ops only the transcripts are written.
+ * Device memory for the direction bits (4 bits per cell of every pair) and the
+ * call's other buffers is allocated by the call; the database keeps up to
+ * 256 MiB of it (and 16 MiB of pinned memory) for later calls and frees it with
+ * sw_db_destroy.  Pairs are processed in chunks of at most 8 GiB of bits.
+ * Synchronous on the stream.
  * Errors: SW_EINVAL (index out of range, short ops buffer, bad gaps or
  * codes), SW_ENOMEM, SW_ECUDA. */
 sw_status sw_align(sw_db* db, const uint8_t* queries, const int32_t* q_lengths, int32_t n_queries,

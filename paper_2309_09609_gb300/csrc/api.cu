@@ -180,6 +180,46 @@ static void parallel_for(int64_t n, F f) {
 // ---- database -----------------------------------------------------------------------
 static void plan_free(sw_plan* p);
 
+// Buffers of sw_align calls, grown to the largest call so far up to the keep
+// limits: device memory, and pinned memory for what goes up and comes back.
+struct AlignBuffers {
+  uint8_t* dev = nullptr;
+  uint8_t* pinned = nullptr;
+  size_t dev_bytes = 0, pinned_bytes = 0;
+
+  cudaError_t reserve(size_t dev_need, size_t pinned_need) {
+    cudaError_t e = cudaSuccess;
+    if (dev_bytes < dev_need) {
+      cudaFree(dev);
+      dev_bytes = 0;
+      e = cudaMalloc((void**)&dev, dev_need);
+      if (e == cudaSuccess) dev_bytes = dev_need;
+      else dev = nullptr;
+    }
+    if (e == cudaSuccess && pinned_bytes < pinned_need) {
+      cudaFreeHost(pinned);
+      pinned_bytes = 0;
+      e = cudaMallocHost((void**)&pinned, pinned_need);
+      if (e == cudaSuccess) pinned_bytes = pinned_need;
+      else pinned = nullptr;
+    }
+    return e;
+  }
+  // gives back what exceeds the limits (0: everything)
+  void trim(size_t dev_keep, size_t pinned_keep) {
+    if (dev_bytes > dev_keep) {
+      cudaFree(dev);
+      dev = nullptr;
+      dev_bytes = 0;
+    }
+    if (pinned_bytes > pinned_keep) {
+      cudaFreeHost(pinned);
+      pinned = nullptr;
+      pinned_bytes = 0;
+    }
+  }
+};
+
 struct sw_db {
   int device = 0;
   DbView view{};
@@ -199,6 +239,10 @@ struct sw_db {
   // the plan behind sw_search, kept between calls (guarded by oneshot_mu)
   sw_plan* oneshot = nullptr;
   std::mutex oneshot_mu;
+  // sw_align's buffers between calls; a call that finds them in use by another
+  // thread takes its own
+  AlignBuffers align;
+  std::mutex align_mu;
 };
 
 static void db_free(sw_db* db) {
@@ -214,6 +258,7 @@ static void db_free(sw_db* db) {
   cudaFree(db->coff);
   cudaFree(db->clen);
   cudaFree(db->perm);
+  db->align.trim(0, 0);
   cudaSetDevice(cur);
   cudaGetLastError();  // a failed free or device switch leaves no stale error
   delete db;
@@ -1556,6 +1601,8 @@ extern "C" sw_status sw_search_plain(sw_db* db, const uint8_t* queries, const in
 // ---- optimal alignments with traceback ------------------------------------------------------
 // Largest direction-bit buffer of one chunk of pairs (bytes).
 static constexpr int64_t kAlignChunkBytes = 8ll << 30;
+// What a database keeps of a call's buffers, at most.
+static constexpr size_t kAlignKeepDevice = 256u << 20, kAlignKeepPinned = 16u << 20;
 
 extern "C" sw_status sw_align(sw_db* db, const uint8_t* queries, const int32_t* q_lengths,
                               int32_t n_queries, const int32_t* pair_query,
@@ -1619,69 +1666,74 @@ extern "C" sw_status sw_align(sw_db* db, const uint8_t* queries, const int32_t* 
   }
   chunk_begin.push_back(n_pairs);
   cudaStream_t cs = (cudaStream_t)stream;
-  uint8_t* qres = nullptr;
-  int64_t* qoff = nullptr;
-  int32_t* qlen = nullptr;
-  SearchParams* Pd = nullptr;
-  AlignItem* items_d = nullptr;
-  AlignOut* out_d = nullptr;
-  uint8_t* bits = nullptr;
-  int2* border_d = nullptr;
-  uint8_t* ops_d = nullptr;
-  std::vector<AlignOut> res((size_t)n_pairs);
-  cudaError_t e = dalloc(&qres, std::max<int64_t>(hb.total, 1));
-  if (e == cudaSuccess) e = dalloc(&qoff, std::max(n_queries, 1));
-  if (e == cudaSuccess) e = dalloc(&qlen, std::max(n_queries, 1));
-  if (e == cudaSuccess) e = dalloc(&Pd, 1);
-  if (e == cudaSuccess) e = dalloc(&items_d, n_pairs);
-  if (e == cudaSuccess) e = dalloc(&out_d, n_pairs);
-  if (e == cudaSuccess) e = dalloc(&bits, std::max<int64_t>(max_words, 1));
-  if (e == cudaSuccess) e = dalloc(&border_d, std::max<int64_t>(max_border, 1));
-  if (e == cudaSuccess) e = dalloc(&ops_d, std::max<int64_t>(slot[n_pairs], 1));
-  if (e == cudaSuccess && hb.total > 0)
-    e = cudaMemcpyAsync(qres, hb.res, hb.total, cudaMemcpyHostToDevice, cs);
-  if (e == cudaSuccess && n_queries > 0)
-    e = cudaMemcpyAsync(qoff, hb.off.data(), sizeof(int64_t) * n_queries, cudaMemcpyHostToDevice, cs);
-  if (e == cudaSuccess && n_queries > 0)
-    e = cudaMemcpyAsync(qlen, hb.len.data(), sizeof(int32_t) * n_queries, cudaMemcpyHostToDevice, cs);
-  P.qres = qres;
-  P.qoff = qoff;
-  P.qlen = qlen;
-  P.nq = n_queries;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(Pd, &P, sizeof P, cudaMemcpyHostToDevice, cs);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(items_d, items.data(), sizeof(AlignItem) * n_pairs, cudaMemcpyHostToDevice, cs);
+  // One device buffer: what goes up (parameters, items, the query arrays) in
+  // one copy, what comes back (records, transcripts) in one copy, the border
+  // rows and the bits.
+  const size_t up_items = block_align(sizeof(SearchParams));
+  const size_t up_qoff = up_items + block_align(sizeof(AlignItem) * (size_t)n_pairs);
+  const size_t up_qlen = up_qoff + block_align(sizeof(int64_t) * (size_t)n_queries);
+  const size_t up_qres = up_qlen + block_align(sizeof(int32_t) * (size_t)n_queries);
+  const size_t up_bytes = up_qres + block_align((size_t)hb.total);
+  const size_t ops_at = block_align(sizeof(AlignOut) * (size_t)n_pairs);
+  const size_t back_bytes = ops_at + block_align((size_t)slot[n_pairs]);
+  const size_t at_out = up_bytes, at_border = at_out + back_bytes;
+  const size_t at_bits = at_border + block_align(sizeof(int2) * (size_t)max_border);
+  const size_t dev_bytes = at_bits + (size_t)std::max<int64_t>(max_words, 1);
+  std::unique_lock<std::mutex> kept(db->align_mu, std::try_to_lock);
+  AlignBuffers own;
+  AlignBuffers& buf = kept.owns_lock() ? db->align : own;
+  // staged in pinned memory, a very large call's in pageable memory
+  const size_t host_bytes = std::max(up_bytes, back_bytes);
+  const bool pinned = host_bytes <= 4 * kAlignKeepPinned;
+  std::vector<uint8_t> pageable(pinned ? 0 : host_bytes);
+  cudaError_t e = buf.reserve(dev_bytes, pinned ? host_bytes : 0);
+  uint8_t* host = pinned ? buf.pinned : pageable.data();
+  if (e == cudaSuccess) {
+    uint8_t* up = host;
+    P.qoff = (const int64_t*)(buf.dev + up_qoff);
+    P.qlen = (const int32_t*)(buf.dev + up_qlen);
+    P.qres = buf.dev + up_qres;
+    P.nq = n_queries;
+    memcpy(up, &P, sizeof P);
+    memcpy(up + up_items, items.data(), sizeof(AlignItem) * (size_t)n_pairs);
+    if (n_queries > 0) {
+      memcpy(up + up_qoff, hb.off.data(), sizeof(int64_t) * (size_t)n_queries);
+      memcpy(up + up_qlen, hb.len.data(), sizeof(int32_t) * (size_t)n_queries);
+    }
+    if (hb.total > 0) memcpy(up + up_qres, hb.res, (size_t)hb.total);
+    e = cudaMemcpyAsync(buf.dev, up, up_bytes, cudaMemcpyHostToDevice, cs);
+  }
+  const AlignItem* items_d = (const AlignItem*)(buf.dev + up_items);
+  AlignOut* out_d = (AlignOut*)(buf.dev + at_out);
   for (size_t c = 0; c + 1 < chunk_begin.size() && e == cudaSuccess; c++) {
     const int32_t k0 = chunk_begin[c], nk = chunk_begin[c + 1] - k0;
-    e = launch_align(team, sms, db->view, Pd, items_d + k0, nk, bits, border_d, out_d + k0, ops_d,
-                     cs);
-    // the next chunk reuses the bits: its kernels run after this one's on the stream
+    e = launch_align(team, sms, db->view, (const SearchParams*)buf.dev, items_d + k0, nk,
+                     buf.dev + at_bits, (int2*)(buf.dev + at_border), out_d + k0,
+                     buf.dev + at_out + ops_at, cs);
+    // the next chunk reuses the bits: its kernel runs after this one's on the stream
   }
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(res.data(), out_d, sizeof(AlignOut) * n_pairs, cudaMemcpyDeviceToHost, cs);
-  if (e == cudaSuccess && slot[n_pairs] > 0)
-    e = cudaMemcpyAsync(ops, ops_d, (size_t)slot[n_pairs], cudaMemcpyDeviceToHost, cs);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(cs);
-  cudaFree(qres);
-  cudaFree(qoff);
-  cudaFree(qlen);
-  cudaFree(Pd);
-  cudaFree(items_d);
-  cudaFree(out_d);
-  cudaFree(bits);
-  cudaFree(border_d);
-  cudaFree(ops_d);
-  if (e != cudaSuccess) return sw_set_cuda_error(e, "sw_align");
-  for (int32_t k = 0; k < n_pairs; k++) {
-    const AlignOut& r = res[k];
-    out[k].score = r.score;
-    out[k].q_begin = r.q_begin;
-    out[k].q_end = r.score > 0 ? r.i_end : 0;
-    out[k].s_begin = r.s_begin;
-    out[k].s_end = r.score > 0 ? r.j_end : 0;
-    out[k].n_ops = r.n_ops;
-    out[k].ops_offset = r.ops_offset;
+    e = cudaMemcpyAsync(host, buf.dev + at_out, back_bytes, cudaMemcpyDeviceToHost, cs);
+  if (e == cudaSuccess)
+    e = cudaStreamSynchronize(cs);
+  else
+    cudaStreamSynchronize(cs);  // nothing queued may outlive the buffers
+  if (e == cudaSuccess) {
+    const AlignOut* res = (const AlignOut*)host;
+    for (int32_t k = 0; k < n_pairs; k++) {
+      const AlignOut& r = res[k];
+      out[k].score = r.score;
+      out[k].q_begin = r.q_begin;
+      out[k].q_end = r.score > 0 ? r.i_end : 0;
+      out[k].s_begin = r.s_begin;
+      out[k].s_end = r.score > 0 ? r.j_end : 0;
+      out[k].n_ops = r.n_ops;
+      out[k].ops_offset = r.ops_offset;
+      if (r.n_ops > 0) memcpy(ops + r.ops_offset, host + ops_at + r.ops_offset, (size_t)r.n_ops);
+    }
   }
+  buf.trim(kept.owns_lock() ? kAlignKeepDevice : 0, kept.owns_lock() ? kAlignKeepPinned : 0);
+  if (e != cudaSuccess) return sw_set_cuda_error(e, "sw_align");
   return SW_OK;
 }
 

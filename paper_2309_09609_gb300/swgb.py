@@ -50,6 +50,9 @@ class Alignment(ctypes.Structure):
                 ("ops_offset", ctypes.c_int64)]
 
 
+_ALIGNMENT = np.dtype([(name, np.dtype(t)) for name, t in Alignment._fields_])   # its records
+
+
 class Stats(ctypes.Structure):
     _fields_ = [("cells", ctypes.c_int64), ("inter_items", ctypes.c_int64),
                 ("intra_items", ctypes.c_int64), ("recomputed_pairs", ctypes.c_int64),
@@ -316,21 +319,19 @@ class Database:
             raise SwError(SW_EINVAL, "pair_query out of range")
         if ps.size and (ps.min() < 0 or ps.max() >= self.n):
             raise SwError(SW_EINVAL, "pair_subject out of range")
-        need = int(sum(int(lens[a]) for a in pq)) + int(self.subject_lengths()[ps].sum()) \
-            if pq.size else 0
-        ops = np.zeros(max(need, 1), dtype=np.uint8)
+        need = int(lens[pq].sum(dtype=np.int64)) + \
+            int(self.subject_lengths()[ps].sum(dtype=np.int64)) if pq.size else 0
+        ops = np.empty(max(need, 1), dtype=np.uint8)   # only the transcripts are written, and read
         out = (Alignment * max(pq.size, 1))()
         m = _matrix(matrix)
         _check(lib().sw_align(self._h, _ptr(q), _ptr(ql), nq, _ptr(pq), _ptr(ps), pq.size,
                               gap_open, gap_extend, _ptr(m), out, _ptr(ops), ops.size,
                               _stream(stream)))
-        res = []
-        for k in range(pq.size):
-            r = out[k]
-            res.append({"score": r.score, "q_begin": r.q_begin, "q_end": r.q_end,
-                        "s_begin": r.s_begin, "s_end": r.s_end,
-                        "ops": ops[r.ops_offset:r.ops_offset + r.n_ops].tobytes().decode()})
-        return res
+        text = memoryview(ops)
+        return [{"score": score, "q_begin": qb, "q_end": qe, "s_begin": sb, "s_end": se,
+                 "ops": str(text[at:at + n], "ascii")}
+                for score, qb, qe, sb, se, n, at in
+                np.frombuffer(out, dtype=_ALIGNMENT, count=pq.size).tolist()]
 
     def plan(self, max_queries: int, max_query_residues: int, **opts) -> "Plan":
         return Plan(self, max_queries, max_query_residues, options(**opts))
