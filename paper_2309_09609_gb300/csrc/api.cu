@@ -995,30 +995,30 @@ static int32_t plan_streams_long(sw_plan* p, const HostBatch& hb, int32_t nq, in
 
 // The lane-group kernel's segments (lane_kernel.cu) for the subject pairs
 // [pair0, pair1): per query up to one per shape.  A shape costs, per subject
-// pair, (columns + LG) steps of kLaneWordCycles x rows + kLaneStepCycles per
-// pass, in cycles of a scheduler on LG / 32 of a warp (serve-sized searches of
-// one query measured 9.3 and 30).  The cheapest shape is used, except where one
-// item of it would take longer than `tail` of the whole search: those subjects
-// (a prefix, longest first) go to a shape with shorter items, a larger group
-// or a chain.  A warp alone on its scheduler takes kLaneRowLatency x rows +
-// kLaneStepLatency cycles a step (the chain of F down the lane's rows, and the
-// shuffle).
-static constexpr double kLaneWordCycles = 9.3, kLaneStepCycles = 30;
-static constexpr double kLaneRowLatency = 14, kLaneStepLatency = 70;
-
+// pair, (columns + ramp) steps of every pass on LG / 32 of a warp.  The cheapest
+// shape is used, except where one item of it would take longer than `tail` of
+// the whole search: those subjects (a prefix, longest first) go to a shape
+// with shorter items, a larger group, halves or a chain.
+// Measured cycles of a step with PR rows per lane: of a scheduler with four
+// warps, 98, 185, 273 and 366 for 8, 16, 24 and 32 rows, 94 and 262 for 8 and
+// 24 rows in halves, 69 and 107 for 4 and 8 rows in a chain; of a warp alone,
+// 158, 284, 403 and 559, in halves 108 and 280, in a chain 132 and 148.
 struct LaneCand {
   int lg, pr, passes, full, chain, halves;
-  double rows() const { return (double)full * (passes - 1) + pr; }
   int ramp() const { return halves ? 2 * lg : lg; }
+  double busy(int rows) const {  // scheduler cycles of a step
+    return ((halves ? 10.5 : 11.1) * rows + 9) * (chain ? 1.18 : 1.0);
+  }
+  double alone(int rows) const {  // cycles of a step on a scheduler of its own
+    return (halves ? 10.7 * rows + 22 : 16.0 * rows + 30) + (chain ? 38 : 0);
+  }
   // scheduler cycles of one step of every pass
-  double thr() const { return kLaneWordCycles * rows() + kLaneStepCycles * passes; }
+  double thr() const { return (passes - 1) * busy(full) + busy(pr); }
   // cycles of the passes over n columns when `share` warps share a scheduler
   double item(double n, double share) const {
-    const double deep = halves ? 0.5 * kLaneRowLatency : kLaneRowLatency;
     if (!chain)
-      return (n + ramp()) * std::max(deep * rows() + kLaneStepLatency * passes, share * thr());
-    const double step = std::max(deep * full + kLaneStepLatency,
-                                 share * (kLaneWordCycles * full + kLaneStepCycles));
+      return (n + ramp()) * std::max((passes - 1) * alone(full) + alone(pr), share * thr());
+    const double step = std::max(alone(full), share * busy(full));
     const double stages = (n + ramp()) / 64 + 1, period = std::max(stages, 8.0);
     return ((passes - 1) / LANE_WARPS * period + (passes - 1) % LANE_WARPS * 2 + stages) * 64 * step;
   }
@@ -1046,123 +1046,132 @@ static int lane_candidates(int32_t m, bool wide, LaneCand* c) {
   return n;
 }
 
-static int64_t plan_lanes_as(sw_plan* p, const HostBatch& hb, int32_t nq, int64_t pair0,
-                             int64_t pair1, bool wide, double tail, int32_t* n_segs,
-                             double* cycles) {
+// The segments for the subject pairs [pair0, pair1), without and with wide
+// chains: the ones expected to end the search soonest.  *cycles is that time,
+// *wide tells whether they need the wide launch.  The length order is cut at
+// pair0 + 0, 1, 2, 4, 8, ...; a piece takes the cheapest shape whose item is at
+// most `tail` of the search for its longest pair, or the shape with the
+// shortest item, and a few values of `tail` are tried (one for a large batch,
+// whose items are short beside the search).
+static int64_t plan_lanes(sw_plan* p, const HostBatch& hb, int32_t nq, int64_t pair0, int64_t pair1,
+                          int32_t* n_segs, double* cycles, bool* wide) {
   *n_segs = 0;
   *cycles = 0;
+  *wide = false;
   if (nq <= 0 || pair0 >= pair1) return 0;
   const sw_db* db = p->db;
   const int64_t N = db->view.n;
-  auto pair_len = [&](int64_t i) { return (double)db->clen_h[(size_t)(2 * i)]; };
-  auto cols = [&](int64_t a, int64_t b) {  // columns of the pairs [a, b)
-    return 0.5 * (double)(db->cres_h[std::min(N, 2 * b)] - db->cres_h[2 * a]);
-  };
-  // scheduler cycles, and warps, of a shape on the pairs [a, b)
-  auto cost = [&](const LaneCand& x, int64_t a, int64_t b) {
-    return x.thr() * x.lg / 32 * (cols(a, b) + (double)(b - a) * x.ramp());
-  };
-  auto warps_of = [&](const LaneCand& x, int64_t a, int64_t b) {
-    return (double)(b - a) * (x.chain ? std::min(x.passes, LANE_WARPS) : x.lg / 32.0);
-  };
-  const double sched = 4.0 * p->sms;
-  const double resident = (double)p->lane_blocks[wide] * LANE_WARPS / sched;
-  auto share_of = [&](double w) { return std::min(resident, std::max(1.0, w / sched)); };
-  double total = 0, warps = 0;
-  for (int32_t i = 0; i < nq; i++) {
-    LaneCand c[MAX_SEGS];
-    const int nc = lane_candidates(hb.len[i], wide, c);
-    const LaneCand* best = c;
-    for (int k = 1; k < nc; k++)
-      if (cost(c[k], pair0, pair1) < cost(*best, pair0, pair1)) best = c + k;
-    total += cost(*best, pair0, pair1);
-    warps += warps_of(*best, pair0, pair1);
+  int64_t cut[66];
+  int cuts = 0;
+  for (int64_t at = 0; at < pair1 - pair0; at = at ? 2 * at : 1) cut[cuts++] = pair0 + at;
+  cut[cuts] = pair1;
+  double cols[65], len[65], all_cols = 0;  // columns of each piece, its longest subject
+  for (int i = 0; i < cuts; i++) {
+    cols[i] = 0.5 * (double)(db->cres_h[std::min(N, 2 * cut[i + 1])] - db->cres_h[2 * cut[i]]);
+    len[i] = (double)db->clen_h[(size_t)(2 * cut[i])];
+    all_cols += cols[i];
   }
-  const double t_all = total / sched, share = share_of(warps);
-  struct Chosen {
+  const double npairs = (double)(pair1 - pair0), sched = 4.0 * p->sms;
+  // scheduler cycles, and warps, of a shape on `n` pairs of `c` columns
+  auto cost = [](const LaneCand& x, double c, double n) {
+    return x.thr() * x.lg / 32 * (c + n * x.ramp());
+  };
+  auto warps_of = [](const LaneCand& x, double n) {
+    return n * (x.chain ? std::min(x.passes, LANE_WARPS) : x.lg / 32.0);
+  };
+  struct Query {
+    LaneCand c[MAX_SEGS];
+    int nc;
+  };
+  struct Piece {
     LaneCand c;
     LaneSeg s;
     double t;
   };
-  std::vector<Chosen> segs;
-  total = warps = 0;
-  for (int32_t i = 0; i < nq; i++) {
-    const int32_t q = hb.order[i];
-    LaneCand c[MAX_SEGS];
-    const int nc = lane_candidates(hb.len[q], wide, c);
-    std::sort(c, c + nc, [&](const LaneCand& a, const LaneCand& b) {
-      return cost(a, pair0, pair1) < cost(b, pair0, pair1);
-    });
-    // from the dearest shape to the cheapest: each takes the longest pairs
-    // left, as far down as every cheaper one's item is too long and longer
-    int64_t at = pair0;
-    for (int k = nc - 1; k >= 0 && at < pair1; k--) {
-      auto wants = [&](int64_t j) {
-        const double n = pair_len(j), t = c[k].item(n, share);
-        for (int kk = 0; kk < k; kk++) {
-          const double tt = c[kk].item(n, share);
-          if (tt <= tail * t_all || tt <= t) return false;
+  std::vector<Query> qs((size_t)nq);
+  std::vector<double> times;
+  std::vector<Piece> pieces, best_pieces;
+  double best = 1e300;
+  const bool large = nq > 32;
+  for (int w = 0; w < (!large && hb.len[hb.order[0]] > 512 ? 2 : 1); w++) {
+    const double resident = (double)p->lane_blocks[w] * LANE_WARPS / sched;
+    auto share_of = [&](double warps) { return std::min(resident, std::max(1.0, warps / sched)); };
+    double total = 0, warps = 0;
+    for (int32_t i = 0; i < nq; i++) {
+      Query& q = qs[i];
+      q.nc = lane_candidates(hb.len[hb.order[i]], w != 0, q.c);
+      std::sort(q.c, q.c + q.nc, [&](const LaneCand& a, const LaneCand& b) {
+        return cost(a, all_cols, npairs) < cost(b, all_cols, npairs);
+      });
+      total += cost(q.c[0], all_cols, npairs);
+      warps += warps_of(q.c[0], npairs);
+    }
+    const double t_all = total / sched, share = share_of(warps);
+    // the time of an item of each shape on each piece
+    times.resize((size_t)nq * cuts * MAX_SEGS);
+    for (int32_t i = 0; i < nq; i++)
+      for (int k = 0; k < cuts; k++)
+        for (int c = 0; c < qs[i].nc; c++)
+          times[((size_t)i * cuts + k) * MAX_SEGS + c] = qs[i].c[c].item(len[k], share);
+    for (double tail : {1e9, 1.2, 0.8, 0.5, 0.35}) {
+      if (large && tail != 0.5) continue;
+      pieces.clear();
+      total = warps = 0;
+      for (int32_t i = 0; i < nq; i++) {
+        int last = -1;
+        size_t first = pieces.size();
+        for (int k = 0; k < cuts; k++) {
+          const double* t = &times[((size_t)i * cuts + k) * MAX_SEGS];
+          int c = 0;
+          while (c < qs[i].nc && t[c] > tail * t_all) c++;
+          if (c == qs[i].nc) c = (int)(std::min_element(t, t + qs[i].nc) - t);
+          if (c != last && pieces.size() - first == MAX_SEGS) c = last;  // room for no more
+          const LaneCand& x = qs[i].c[c];
+          if (c == last) {
+            pieces.back().s.pair1 = (int32_t)cut[k + 1];
+          } else {
+            const LaneSeg sg{0, hb.order[i], x.lg, x.pr, x.passes, x.full, x.chain, x.halves,
+                             (int32_t)cut[k], (int32_t)cut[k + 1]};
+            pieces.push_back({x, sg, len[k]});
+          }
+          last = c;
+          total += cost(x, cols[k], (double)(cut[k + 1] - cut[k]));
+          warps += warps_of(x, (double)(cut[k + 1] - cut[k]));
         }
-        return true;
-      };
-      int64_t lo = at, hi = pair1;
-      while (lo < hi) {
-        const int64_t mid = (lo + hi) / 2;
-        if (wants(mid)) lo = mid + 1; else hi = mid;
       }
-      if (lo <= at) continue;
-      const LaneSeg s{0, q, c[k].lg, c[k].pr, c[k].passes, c[k].full, c[k].chain, c[k].halves,
-                      (int32_t)at, (int32_t)lo};
-      segs.push_back({c[k], s, 0.0});
-      total += cost(c[k], at, lo);
-      warps += warps_of(c[k], at, lo);
-      at = lo;
+      double longest = 0;
+      for (size_t i = pieces.size(); i-- > 0;) {
+        Piece& x = pieces[i];
+        x.t = x.c.item(x.t, share_of(warps));
+        longest = std::max(longest, x.t);
+        // a query's longest subjects go first, however short their shape's items
+        if (i + 1 < pieces.size() && pieces[i + 1].s.q == x.s.q) x.t = std::max(x.t, pieces[i + 1].t);
+      }
+      // the longest item starts first, beside the rest of the work; fewer
+      // warps on a scheduler (wide) hide less latency
+      const double t = (std::max(longest, total / sched) + 0.2 * std::min(longest, total / sched)) *
+                       (w ? 1.05 : 1.0);
+      if (t < 0.999 * best) {
+        best = t;
+        best_pieces = pieces;
+        *wide = w != 0;
+      }
+      if (longest < 0.3 * total / sched) break;  // shorter items cannot help
     }
   }
-  double longest = 0;
-  for (size_t i = segs.size(); i-- > 0;) {
-    Chosen& x = segs[i];
-    x.t = x.c.item(pair_len(x.s.pair0), share_of(warps));
-    longest = std::max(longest, x.t);
-    // a query's longest subjects go first, however short their shape's items
-    if (i + 1 < segs.size() && segs[i + 1].s.q == x.s.q) x.t = std::max(x.t, segs[i + 1].t);
-  }
-  std::stable_sort(segs.begin(), segs.end(),
-                   [](const Chosen& a, const Chosen& b) { return a.t > b.t; });
+  std::stable_sort(best_pieces.begin(), best_pieces.end(),
+                   [](const Piece& a, const Piece& b) { return a.t > b.t; });
   int64_t items = 0;
-  for (size_t i = 0; i < segs.size(); i++) {
-    LaneSeg& s = p->segs[i];
-    s = segs[i].s;
-    s.first = items;
-    const int64_t per = s.chain ? 1 : LANE_WARPS * 32 / s.lg;
-    items += (s.pair1 - s.pair0 + per - 1) / per;
+  for (size_t i = 0; i < best_pieces.size(); i++) {
+    LaneSeg& sg = p->segs[i];
+    sg = best_pieces[i].s;
+    sg.first = items;
+    const int64_t per = sg.chain ? 1 : LANE_WARPS * 32 / sg.lg;
+    items += (sg.pair1 - sg.pair0 + per - 1) / per;
   }
-  // the longest item starts first, beside the rest of the work; fewer warps
-  // on a scheduler (wide) hide less latency
-  *cycles = (std::max(longest, total / sched) + 0.2 * std::min(longest, total / sched)) * (wide ? 1.05 : 1);
-  *n_segs = (int32_t)segs.size();
+  *cycles = best;
+  *n_segs = (int32_t)best_pieces.size();
   return items;
-}
-
-// The same with the tail limit, and with or without wide chains (*wide), that
-// are expected to end the search soonest.  A large batch takes the middle one:
-// its items are short beside the search.
-static int64_t plan_lanes(sw_plan* p, const HostBatch& hb, int32_t nq, int64_t pair0, int64_t pair1,
-                          int32_t* n_segs, double* cycles, bool* wide) {
-  double tail = 0.5, best = 1e300;
-  *wide = false;
-  if (nq > 0 && nq <= 32) {
-    for (int w = 0; w < (hb.len[hb.order[0]] > 512 ? 2 : 1); w++)
-      for (double t : {0.35, 0.5, 0.7, 1.0, 1.5, 1e9}) {
-        plan_lanes_as(p, hb, nq, pair0, pair1, w != 0, t, n_segs, cycles);
-        if (*cycles < best * 0.999) {
-          best = *cycles;
-          tail = t;
-          *wide = w != 0;
-        }
-      }
-  }
-  return plan_lanes_as(p, hb, nq, pair0, pair1, *wide, tail, n_segs, cycles);
 }
 
 // The stream layout alone, for a given number of stream pairs (host only).

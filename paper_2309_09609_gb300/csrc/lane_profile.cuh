@@ -31,7 +31,7 @@ struct LaneShape {
   static constexpr int R = PR / NQ;  // rows per quarter
   static_assert(R % 4 == 0 && PR <= LANE_ROWS_MAX, "whole 4-row words, at most 32 rows");
   static constexpr int VB = R % 16 == 0 ? 16 : R % 8 == 0 ? 8 : 4;  // bytes per profile load
-  static constexpr int UNROLL = PR >= 24 ? 2 : 4;                   // steps per loop body
+  static constexpr int UNROLL = 4;                                  // steps per loop body
   static constexpr bool AHEAD = PR <= 24;  // registers allow the next step's profile words
 };
 
