@@ -845,20 +845,22 @@ static void balance_pair(std::vector<int32_t>& a, std::vector<int32_t>& b, int64
 // each to the stream with the fewest strips so far (each query padded to
 // whole strips of T rows, at least one), pairs streams 2k and 2k + 1 and
 // balances each pair's two streams (balance_pair).
-// Unless fixed_K > 0, K is the smallest power of two, at most nq / 2, for
-// which the largest work item -- the longest column set (len_max) against
-// the longest stream pair -- is at most `share` of one worker's share of the
-// search (len_sum columns against every stream pair, over `workers`): fewer,
-// longer streams pad less (a stream pair is as long as its longer stream,
-// and the fewer queries a pair holds the less evenly its two streams
-// split), but an item longer than a worker's share finishes late; items run
-// longest first, so the last ones are short.  Writes the strip table (per strip: the
-// query of each half, its first row | end bit 31; query -1 for an empty
-// half) to tab and per stream pair (first strip, counted from first_strip,
-// strips) to pairs.  Returns K, or 0 when the table would exceed cap strips;
-// *n_strips is the table's length.
+// Unless fixed_K > 0, K is the power of two, at most nq / 2, for which the
+// search is expected to end first.  Fewer, longer streams pad less (a stream
+// pair is as long as its longer stream, in units of `unit` strips, and the
+// fewer queries a pair holds the less evenly its two streams split), but an
+// item is as long as its stream pair: the longest one -- the longest column
+// set (len_max) against the longest pair -- takes `len_max x strips`, and the
+// whole search len_sum columns against every pair over `workers`.  Items run
+// longest first, so a longest item well within the search costs little: kTail
+// of its length (20 queries of 144-5,478 x 100,000 subjects took 126.3, 129.4
+// and 135.9 ms with 2, 4 and 8 pairs, 96 of 50-2,000 402, 395 and 395 with 2, 4
+// and 8).  Writes the strip table (per strip: the query of each half, its
+// first row | end bit 31; query -1 for an empty half) to tab and per stream
+// pair (first strip, counted from first_strip, strips) to pairs.  Returns K, or
+// 0 when the table would exceed cap strips; *n_strips is the table's length.
 static int32_t deal_streams(const HostBatch& hb, int32_t nq, int T, int32_t fixed_K,
-                            double workers, double share, double len_max, double len_sum,
+                            double workers, int unit, double len_max, double len_sum,
                             int4* tab, int2* pairs, int64_t first_strip, int64_t cap,
                             int64_t* n_strips) {
   *n_strips = 0;
@@ -881,18 +883,28 @@ static int32_t deal_streams(const HostBatch& hb, int32_t nq, int T, int32_t fixe
       balance_pair(streams[2 * k], streams[2 * k + 1], load[2 * k], load[2 * k + 1], strips_of);
   };
   auto pair_strips = [&](int32_t k) { return std::max(load[2 * k], load[2 * k + 1]); };
+  constexpr double kTail = 0.045;
   int32_t K = fixed_K > 0 ? std::min(fixed_K, nq / 2) : 1;
-  deal(K);
-  while (fixed_K == 0 && 2 * K <= nq / 2) {
-    int64_t smax = 0, ssum = 0;
-    for (int32_t k = 0; k < K; k++) {
-      smax = std::max(smax, pair_strips(k));
-      ssum += pair_strips(k);
+  if (fixed_K == 0) {
+    double best = 1e300;
+    for (int32_t k2 = 1; k2 <= nq / 2; k2 *= 2) {
+      deal(k2);
+      int64_t smax = 0, ssum = 0;
+      for (int32_t k = 0; k < k2; k++) {
+        const int64_t S = (pair_strips(k) + unit - 1) / unit * unit;
+        smax = std::max(smax, S);
+        ssum += S;
+      }
+      const double all = len_sum * (double)ssum / workers, longest = len_max * (double)smax;
+      const double t = std::max(all, longest) + kTail * std::min(all, longest);
+      if (t < best) {
+        best = t;
+        K = k2;
+      }
+      if (longest < 0.2 * all) break;  // more pairs only pad more
     }
-    if (len_max * (double)smax <= share * len_sum * (double)ssum / workers) break;
-    K *= 2;
-    deal(K);
   }
+  deal(K);
   int64_t total = 0;
   for (int32_t k = 0; k < K; k++) total += pair_strips(k);
   if (total > cap) return 0;
@@ -948,7 +960,7 @@ static int32_t plan_streams(sw_plan* p, const HostBatch& hb, int32_t nq, int32_t
   for (int32_t g = g_first; g < v.groups; g++) glen_sum += p->db->glen_h[g];
   const double glen_max = g_first < v.groups ? p->db->glen_h[g_first] : 0.0;
   const int32_t K = deal_streams(hb, nq, T, p->opt.two_query_pairs,
-                                 (double)p->kc2.blocks * p->kc2.warps, 0.35, glen_max, glen_sum,
+                                 (double)p->kc2.blocks * p->kc2.warps, 1, glen_max, 2 * glen_sum,
                                  p->strips.data(), p->spairs.data(), 0,
                                  (int64_t)p->strips.size(), n_strips);
   int64_t longest = 0;
@@ -960,10 +972,7 @@ static int32_t plan_streams(sw_plan* p, const HostBatch& hb, int32_t nq, int32_t
 
 // The long subjects' two-query layout (pair2q_kernel.cu), its table placed
 // after the short subjects' (first_strip, first_pair): items are (stream
-// pair, group of PAIR2_GROUP long subjects), the workers its blocks, and the
-// largest item may be one worker's share (on the paper-shaped search's long
-// subjects, 1, 2, 4 and 8 stream pairs took 45.4, 35.6, 40.0 and 44.2 ms;
-// the rule picks 2 there, and 1 on the long-sequence workload).  Returns the
+// pair, group of PAIR2_GROUP long subjects), the workers its blocks.  Returns the
 // number of stream pairs, and in *cycles what the layout is expected to take:
 // the passes' steps of 32 words, three warps to a scheduler, over as many
 // rounds of blocks as the items need, or the longest item.
@@ -977,7 +986,7 @@ static int32_t plan_streams_long(sw_plan* p, const HostBatch& hb, int32_t nq, in
   double len_sum = 0;
   for (int64_t s = 0; s < n_long; s += PAIR2_GROUP) len_sum += clen[s];
   const int32_t K = deal_streams(hb, nq, PAIR2_STRIP, p->opt.two_query_pairs,
-                                 (double)p->pair2_blocks, 1.0, clen[0],
+                                 (double)p->pair2_blocks, 32, clen[0],
                                  len_sum, p->strips.data() + first_strip,
                                  p->spairs.data() + first_pair, first_strip,
                                  (int64_t)p->strips.size() - first_strip, n_strips);
@@ -1199,7 +1208,7 @@ extern "C" sw_status sw_query_streams(const int32_t* q_lengths, int32_t n_querie
   for (int32_t i = 0; i < n_queries; i++) bound += std::max<int64_t>(1, (hb.len[i] + rows - 1) / rows);
   std::vector<int4> tab((size_t)std::min(strip_capacity, bound));
   std::vector<int2> pr((size_t)n_pairs);
-  const int32_t K = deal_streams(hb, n_queries, rows, n_pairs, 1.0, 1.0, 0.0, 0.0, tab.data(),
+  const int32_t K = deal_streams(hb, n_queries, rows, n_pairs, 1.0, 1, 0.0, 0.0, tab.data(),
                                  pr.data(), 0, strip_capacity, n_strips);
   if (K == 0) return sw_set_error(SW_EBUSY, "the strip table exceeds %lld strips",
                                   (long long)strip_capacity);
