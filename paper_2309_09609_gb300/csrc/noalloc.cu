@@ -14,18 +14,23 @@
 // The kernel scores each pair on one warp, in int32: lane k owns PR consecutive
 // query rows, takes the (H, F) border of the row above from lane k - 1 by
 // shuffle and walks one column a step, as in lane_kernel.cuh.  PR follows the
-// query's length, so a query of up to 1,024 residues needs no border memory
-// and any number of warps may run; a longer one goes in passes of 1,024 rows
-// whose border rows lie in the array, on the blocks that have rows there.  A
-// block takes a query and a few subjects, builds one profile in shared memory
-// for its warps, and they share the subjects out as they finish.
+// query's length, so a query of up to 1,024 residues needs no border memory.
+// A block takes a query and a few subjects, builds one profile in shared
+// memory for its warps, and they share the subjects out as they finish.
+//
+// A longer query, and a query of over 256 residues against a subject of over
+// 1,024, goes first and as a chain: passes of 256 rows on the block's four
+// warps, each two stages of 64 columns behind the one above, borders through
+// rings in shared memory, and from the fourth warp to the first one's next pass
+// through a row of the array.  One warp would take 1.2 ms for 1,024 x 4,096.
 //
 // Bound by the ALU pipe at 3.5 operations per cell: one DP4A adds a row's
 // score, picked from the four in a profile word, to the diagonal (a PRMT and an
 // add took the ALU pipe twice; in a loop of independent cells 7.9 cycles per
 // warp and scheduler, against 9.1 for the earlier update).  16 queries of 400 x
-// 2,000 subjects: 12.5 -> 2.5 ms (before: 512 warps on the whole chip, 256-row passes
-// through the border rows, codes loaded at the step that used them).
+// 2,000 subjects: 12.5 -> 2.3 ms, 2.8 without the chains (before: 512 warps on the
+// whole chip, 256-row passes through the border rows, codes loaded at the step
+// that used them).
 #include <mutex>
 
 #include "lane_profile.cuh"
@@ -35,11 +40,16 @@ namespace {
 
 constexpr int NA_MAX_LEN = 4096;         // longest subject accepted
 constexpr int NA_WARPS = 4;              // warps per block
-constexpr int NA_ROW_BLOCKS = 128;       // blocks with border rows
+constexpr int NA_ROWS = 512;             // border rows: blocks that may run chains
 constexpr int NA_HEADER = 32;            // int2 slots (256 bytes) for the counters and status
-constexpr size_t NA_SCRATCH =
-    NA_HEADER + (size_t)NA_ROW_BLOCKS * NA_WARPS * NA_MAX_LEN;  // int2: ~16 MiB
-constexpr int NA_PASS = 32 * LANE_ROWS_MAX;  // query rows of a pass
+constexpr size_t NA_SCRATCH = NA_HEADER + (size_t)NA_ROWS * NA_MAX_LEN;  // int2: ~16 MiB
+constexpr int NA_ALONE = 32 * LANE_ROWS_MAX;  // longest query on one warp
+constexpr int NA_CHAIN_PR = 8;                // rows per lane in a chain
+constexpr int NA_CHAIN_PASS = 32 * NA_CHAIN_PR;
+constexpr int NA_CHAIN_LEN = 1024;            // longest subject that is not one
+constexpr int NA_STAGE = 64;                  // steps between a chain's barriers
+constexpr int NA_LAG = 2;                     // stages between consecutive passes
+constexpr int NA_EDGE = 256;                  // columns of a border ring
 constexpr int NA_COLS = 256;                 // columns per ring block: 8 per lane
 constexpr unsigned NA_BAD_LENGTH = 1u, NA_BAD_CODE = 2u;
 
@@ -58,16 +68,36 @@ struct NaArgs {
   const int32_t *qlen, *slen;
   int32_t* scores;
   int nq, ns, go, ge;
-  int chunk;  // subjects per block item
+  // subjects per block item: of the chains, and of the other pairs, whose
+  // items are large for the subjects [0, split) and small, and last, for the
+  // rest: a block's warps share a large one out evenly, and small ones end
+  // the call evenly
+  int chain, large, small, split;
+};
+
+// The warps of a chain meet here from different places of the code.
+__device__ __forceinline__ void na_chain_barrier() {
+  asm volatile("bar.sync 1, %0;" ::"n"(NA_WARPS * 32) : "memory");
+}
+
+// Where a chain's pass takes the border row above it and leaves its own: rings
+// of NA_EDGE columns, or a whole row (mask -1).  A ring's reader is NA_LAG
+// stages behind its writer, which is then at most 64 * 2 + 32 columns ahead.
+struct NaEdges {
+  const int2* in;
+  int2* out;
+  int in_mask, out_mask;
+  bool first, last;
 };
 
 // One pass of a pair, on a warp: n > 0 columns, the lane's PR rows of the
-// profile.  hb: the border row of a query of several passes (PASSES), as in
-// lane_sweep; bad is set when a subject code is outside the alphabet.
-template <int PR, bool PASSES>
+// profile; bad is set when a subject code is outside the alphabet.  CHAIN: the
+// passes of the pair run on the block's warps, which meet at a barrier every
+// NA_STAGE steps.
+template <int PR, bool CHAIN>
 __device__ __forceinline__ void na_sweep(const uint8_t* prof, uint16_t* ring, int lane, int n,
-                                         const uint8_t* __restrict__ d, int2* hb, bool first,
-                                         bool last, int& S, int& bad, int go, int ge) {
+                                         const uint8_t* __restrict__ d, const NaEdges& ed, int& S,
+                                         int& bad, int go, int ge) {
   using Shape = LaneShape<PR, 1>;
   constexpr int VB = Shape::VB, U = Shape::UNROLL;
   const uint8_t* pl = prof + lane * VB;
@@ -114,16 +144,19 @@ __device__ __forceinline__ void na_sweep(const uint8_t* prof, uint16_t* ring, in
   uint2 next = load(0);
   const int steps = n + 31;
   int b = 0;
-  for (int t0 = 0; t0 < steps; t0 += NA_COLS) {
-    __syncwarp();
-    store(b & 1, next);
-    next = load(++b);
-    __syncwarp();
-    const int tend = min(t0 + NA_COLS, steps);
+  constexpr int SPAN = CHAIN ? NA_STAGE : NA_COLS;
+  for (int t0 = 0; t0 < steps; t0 += SPAN) {
+    if (!CHAIN || t0 % NA_COLS == 0) {
+      __syncwarp();
+      store(b & 1, next);
+      next = load(++b);
+      __syncwarp();
+    }
+    const int tend = min(t0 + SPAN, steps);
     int2 bq[U];  // the border of columns t .. t + U - 1
-    if constexpr (PASSES) {
+    if constexpr (CHAIN) {
 #pragma unroll
-      for (int u = 0; u < U; u++) bq[u] = hb[min(t0 + u, n - 1)];
+      for (int u = 0; u < U; u++) bq[u] = ed.in[min(t0 + u, n - 1) & ed.in_mask];
     }
 #pragma unroll 1
     for (int t = t0; t < tend; t += U) {
@@ -132,10 +165,10 @@ __device__ __forceinline__ void na_sweep(const uint8_t* prof, uint16_t* ring, in
       for (int u = 0; u < U; u++) {
         int in_h = __shfl_up_sync(FULL, out_h, 1) * not0;  // H = F = 0 above the matrix
         int in_f = __shfl_up_sync(FULL, out_f, 1) * not0;
-        if constexpr (PASSES) {
+        if constexpr (CHAIN) {
           const int2 bv = bq[u];
-          bq[u] = hb[min(t + u + U, n - 1)];
-          if (lane == 0 && !first) {
+          bq[u] = ed.in[min(t + u + U, min(tend, n) - 1) & ed.in_mask];
+          if (lane == 0 && !ed.first) {
             in_h = bv.x;
             in_f = bv.y;
           }
@@ -173,43 +206,45 @@ __device__ __forceinline__ void na_sweep(const uint8_t* prof, uint16_t* ring, in
         hdiag = in_h;
         out_h = H[PR - 1];
         out_f = f;
-        if constexpr (PASSES) {
+        if constexpr (CHAIN) {
           const int j = t + u - 31;
-          if (lane == 31 && !last && j >= 0 && j < n) hb[j] = make_int2(out_h, out_f);
+          if (lane == 31 && !ed.last && j >= 0 && j < n)
+            ed.out[j & ed.out_mask] = make_int2(out_h, out_f);
         }
       }
     }
+    if constexpr (CHAIN) na_chain_barrier();
   }
 }
 
-template <bool PASSES>
-__device__ __forceinline__ void na_pass(int pr, const uint8_t* prof, uint16_t* ring, int lane,
-                                        int n, const uint8_t* d, int2* hb, bool first, bool last,
-                                        int& S, int& bad, int go, int ge) {
+__device__ __forceinline__ void na_alone(int pr, const uint8_t* prof, uint16_t* ring, int lane,
+                                         int n, const uint8_t* d, int& S, int& bad, int go,
+                                         int ge) {
+  const NaEdges none{nullptr, nullptr, 0, 0, true, true};
   switch (pr) {  // uniform over the block
-    case 4: na_sweep<4, PASSES>(prof, ring, lane, n, d, hb, first, last, S, bad, go, ge); break;
-    case 8: na_sweep<8, PASSES>(prof, ring, lane, n, d, hb, first, last, S, bad, go, ge); break;
-    case 12: na_sweep<12, PASSES>(prof, ring, lane, n, d, hb, first, last, S, bad, go, ge); break;
-    case 16: na_sweep<16, PASSES>(prof, ring, lane, n, d, hb, first, last, S, bad, go, ge); break;
-    case 20: na_sweep<20, PASSES>(prof, ring, lane, n, d, hb, first, last, S, bad, go, ge); break;
-    case 24: na_sweep<24, PASSES>(prof, ring, lane, n, d, hb, first, last, S, bad, go, ge); break;
-    case 28: na_sweep<28, PASSES>(prof, ring, lane, n, d, hb, first, last, S, bad, go, ge); break;
-    default: na_sweep<32, PASSES>(prof, ring, lane, n, d, hb, first, last, S, bad, go, ge); break;
+    case 4: na_sweep<4, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
+    case 8: na_sweep<8, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
+    case 12: na_sweep<12, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
+    case 16: na_sweep<16, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
+    case 20: na_sweep<20, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
+    case 24: na_sweep<24, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
+    case 28: na_sweep<28, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
+    default: na_sweep<32, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
   }
 }
 
-// The profile of rows [row0, row0 + 32 * pr), by the whole block.
+// The profile of a query of up to 32 * pr rows, by the whole block.
 __device__ __forceinline__ void na_profile(int pr, uint8_t* prof, const uint8_t* sm,
-                                           const uint8_t* qr, int m, int row0, int wib) {
+                                           const uint8_t* qr, int m, int wib) {
   switch (pr) {
-    case 4: lane_profile_rows<4, 1>(prof, sm, qr, m, row0, 32, wib, NA_WARPS); break;
-    case 8: lane_profile_rows<8, 1>(prof, sm, qr, m, row0, 32, wib, NA_WARPS); break;
-    case 12: lane_profile_rows<12, 1>(prof, sm, qr, m, row0, 32, wib, NA_WARPS); break;
-    case 16: lane_profile_rows<16, 1>(prof, sm, qr, m, row0, 32, wib, NA_WARPS); break;
-    case 20: lane_profile_rows<20, 1>(prof, sm, qr, m, row0, 32, wib, NA_WARPS); break;
-    case 24: lane_profile_rows<24, 1>(prof, sm, qr, m, row0, 32, wib, NA_WARPS); break;
-    case 28: lane_profile_rows<28, 1>(prof, sm, qr, m, row0, 32, wib, NA_WARPS); break;
-    default: lane_profile_rows<32, 1>(prof, sm, qr, m, row0, 32, wib, NA_WARPS); break;
+    case 4: lane_profile_rows<4, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
+    case 8: lane_profile_rows<8, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
+    case 12: lane_profile_rows<12, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
+    case 16: lane_profile_rows<16, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
+    case 20: lane_profile_rows<20, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
+    case 24: lane_profile_rows<24, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
+    case 28: lane_profile_rows<28, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
+    default: lane_profile_rows<32, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
   }
 }
 
@@ -219,29 +254,70 @@ __device__ __forceinline__ int na_warp_max(int S) {
   return S;
 }
 
+// Pairs that run as chains.
+__device__ __forceinline__ bool na_is_chain(int m, int n) {
+  return m > NA_ALONE || (m > NA_CHAIN_PASS && n > NA_CHAIN_LEN);
+}
+
+// One pair on the block's warps, n > 0.  Pass p runs on warp p % NA_WARPS from
+// stage (p / W) * period + (p % W) * NA_LAG on, with a period that leaves a
+// ring's reader time to finish before its writer's next pass.  Returns this
+// lane's S; every warp meets the same number of barriers.
+__device__ __forceinline__ int na_chain(uint8_t* prof, uint16_t* ring, int2 (*edges)[NA_EDGE],
+                                        int2* row, const uint8_t* sm, const uint8_t* qr, int m,
+                                        const uint8_t* d, int n, int lane, int wib, int& bad,
+                                        int go, int ge) {
+  constexpr int W = NA_WARPS;
+  const int passes = (m + NA_CHAIN_PASS - 1) / NA_CHAIN_PASS;
+  const int spass = (n + 31 + NA_STAGE - 1) / NA_STAGE;
+  const int period = max(spass + NA_LAG, W * NA_LAG);
+  const int end = (passes - 1) / W * period + (passes - 1) % W * NA_LAG + spass;
+  uint8_t* mine = prof + wib * NCODES * NA_CHAIN_PASS;
+  NaEdges ed;
+  ed.in = wib == 0 ? row : edges[wib - 1];
+  ed.in_mask = wib == 0 ? -1 : NA_EDGE - 1;
+  ed.out = wib == W - 1 ? row : edges[wib];
+  ed.out_mask = wib == W - 1 ? -1 : NA_EDGE - 1;
+  int S = 0, g = 0;
+  for (int p = wib; p < passes; p += W) {
+    for (const int start = p / W * period + p % W * NA_LAG; g < start; g++) na_chain_barrier();
+    ed.first = p == 0;
+    ed.last = p == passes - 1;
+    __syncwarp();
+    lane_profile_rows<NA_CHAIN_PR, 1>(mine, sm, qr, m, p * NA_CHAIN_PASS, 32, 0, 1);
+    __syncwarp();
+    na_sweep<NA_CHAIN_PR, true>(mine, ring, lane, n, d, ed, S, bad, go, ge);
+    g += spass;
+  }
+  for (; g < end; g++) na_chain_barrier();
+  return S;
+}
+
 __global__ void __launch_bounds__(NA_WARPS * 32, 4)
 noalloc_kernel(NaArgs a, NaMatrix mat, int2* scratch) {
   __shared__ __align__(16) uint8_t prof[NCODES * 32 * LANE_ROWS_MAX];
   __shared__ __align__(16) uint16_t ring_all[NA_WARPS][2 * NA_COLS + 8];
+  __shared__ __align__(16) int2 edges[NA_WARPS - 1][NA_EDGE];
   __shared__ __align__(16) uint8_t sm[NCODES * SM_ROW];
   __shared__ unsigned long long s_item;
-  __shared__ int s_subject, s_qbad;
+  __shared__ int s_subject, s_qbad, red_s[NA_WARPS], red_bad[NA_WARPS];
   for (int i = threadIdx.x; i < NCODES * SM_ROW; i += blockDim.x)
     sm[i] = i % SM_ROW < NCODES ? (uint8_t)mat.sm[i / SM_ROW * NCODES + i % SM_ROW] : 0;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   uint16_t* ring = ring_all[wib];
   unsigned int* status = (unsigned int*)(scratch + 1);
-  const int chunks = (a.ns - 1) / a.chunk + 1;  // per query
-  const long long total = (long long)a.nq * chunks;
-  const bool rows = blockIdx.x < NA_ROW_BLOCKS;
-  int2* hb = scratch + NA_HEADER + (size_t)(rows ? blockIdx.x * NA_WARPS + wib : 0) * NA_MAX_LEN;
-  // round 0: the queries of several passes, on the blocks with border rows;
-  // round 1: the others, on all blocks
+  const int n_large = a.split / a.large, n_small = (a.ns - a.split + a.small - 1) / a.small;
+  const int n_chain = (a.ns - 1) / a.chain + 1;  // items per query
+  const bool rows = blockIdx.x < NA_ROWS;
+  int2* row = scratch + NA_HEADER + (size_t)(rows ? blockIdx.x : 0) * NA_MAX_LEN;
+  // round 0: the chains, on the blocks with a border row; round 1: the other
+  // pairs, and the refused ones, on all blocks
   for (int round = rows ? 0 : 1; round < 2; round++) {
     unsigned long long* counter = (unsigned long long*)scratch + (round == 0 ? 0 : 2);
-    int cached = -1;  // the query whose single-pass profile the block holds
+    const long long total = (long long)a.nq * (round == 0 ? n_chain : n_large + n_small);
+    int checked = -1, cached = -1;  // the query scanned for bad codes, and that of the profile
     // a block's first item is its index, so few items spread over the SMs
-    const unsigned starters = round == 0 ? min(gridDim.x, (unsigned)NA_ROW_BLOCKS) : gridDim.x;
+    const unsigned starters = round == 0 ? min(gridDim.x, (unsigned)NA_ROWS) : gridDim.x;
     for (bool start = true;; start = false) {
       __syncthreads();  // the item before is done with the shared words
       if (threadIdx.x == 0) {
@@ -251,64 +327,93 @@ noalloc_kernel(NaArgs a, NaMatrix mat, int2* scratch) {
       __syncthreads();
       const long long it = (long long)s_item;
       if (it >= total) break;  // uniform over the block
-      const int q = (int)(it / chunks), s0 = (int)(it % chunks) * a.chunk;
-      const int cnt = min(a.chunk, a.ns - s0);
+      int q, s0, cnt;
+      if (round == 0) {
+        q = (int)(it / n_chain), s0 = (int)(it % n_chain) * a.chain;
+        cnt = min(a.chain, a.ns - s0);
+      } else if (it < (long long)a.nq * n_large) {
+        q = (int)(it / n_large), s0 = (int)(it % n_large) * a.large;
+        cnt = a.large;
+      } else {
+        const long long i = it - (long long)a.nq * n_large;
+        q = (int)(i / n_small), s0 = a.split + (int)(i % n_small) * a.small;
+        cnt = min(a.small, a.ns - s0);
+      }
       const int m = a.qlen[q];
-      if ((m > NA_PASS) != (round == 0)) continue;
       // a negative length, or residues to read from a NULL buffer
       const bool q_ok = m >= 0 && (m == 0 || a.qres);
+      if (round == 0 && (!q_ok || m <= NA_CHAIN_PASS)) continue;  // no chain with this query
       const uint8_t* qr = a.qres + (q_ok && m > 0 ? a.qoff[q] : 0);
-      const int passes = q_ok && m > 0 ? (m + NA_PASS - 1) / NA_PASS : 0;
-      const int last_rows = m - (passes - 1) * NA_PASS;
-      const int pr = max(1, ((last_rows + 31) / 32 + 3) / 4) * 4;  // of the last pass
-      if (passes > 0 && cached != q) {
+      const int pr = max(1, (min(m, NA_ALONE) + 127) / 128) * 4;  // of a query on one warp
+      // a subject length that may be scored
+      auto valid = [&](int n) { return q_ok && n >= 0 && n <= NA_MAX_LEN && (n == 0 || a.sres); };
+      if (q_ok && m > 0 && checked != q) {
         if (threadIdx.x == 0) s_qbad = 0;
         __syncthreads();
         int bad = 0;
         for (int i = threadIdx.x; i < m; i += blockDim.x) bad |= qr[i] >= ALPHA;
         if (bad) s_qbad = 1;  // every writer writes 1
-        if (passes == 1) {
-          na_profile(pr, prof, sm, qr, m, 0, wib);
-          cached = q;
-        }
         __syncthreads();
+        checked = q;
       }
-      const bool qbad = passes > 0 && s_qbad;
-      // the warps take the chunk's subjects one by one; with several passes, in
-      // step, since they share each pass's profile
-      for (int k = wib;; k += NA_WARPS) {
-        if (passes <= 1) {
-          if (lane == 0) k = atomicAdd(&s_subject, 1);
-          k = __shfl_sync(FULL, k, 0);
-          if (k >= cnt) break;
-        } else if (k - wib >= cnt) {
-          break;  // uniform over the block
-        }
-        const int s = s0 + min(k, cnt - 1);
-        const int n = a.slen[s];
-        // refused, with nothing read or written: a bad length on either side
-        const bool ok = k < cnt && q_ok && n >= 0 && n <= NA_MAX_LEN && (n == 0 || a.sres);
-        if (k < cnt && !ok && lane == 0) atomicOr(status, NA_BAD_LENGTH);
-        const uint8_t* d = a.sres + (ok && n > 0 ? a.soff[s] : 0);
-        int S = 0, bad = 0;
-        if (passes == 1) {
-          if (ok && n > 0)
-            na_pass<false>(pr, prof, ring, lane, n, d, nullptr, true, true, S, bad, a.go, a.ge);
-        } else {
-          for (int p = 0; p < passes; p++) {
-            const int rows_p = p < passes - 1 ? LANE_ROWS_MAX : pr;
-            __syncthreads();  // every warp is done with the profile before
-            na_profile(rows_p, prof, sm, qr, m, p * NA_PASS, wib);
+      const bool qbad = q_ok && m > 0 && s_qbad;
+      if (round == 0) {
+        for (int k0 = 0; k0 < cnt; k0 += 32) {
+          const int nk = k0 + lane < cnt ? a.slen[s0 + k0 + lane] : -1;
+          unsigned todo = __ballot_sync(FULL, nk > 0 && valid(nk) && na_is_chain(m, nk));
+          for (; todo; todo &= todo - 1) {  // uniform over the block
+            const int k = __ffs(todo) - 1, s = s0 + k0 + k;
+            const int n = __shfl_sync(FULL, nk, k);
+            int bad = 0;
+            const int S = na_warp_max(na_chain(prof, ring, edges, row, sm, qr, m,
+                                               a.sres + a.soff[s], n, lane, wib, bad, a.go, a.ge));
+            bad = __any_sync(FULL, bad);
+            if (lane == 0) {
+              red_s[wib] = S;
+              red_bad[wib] = bad;
+            }
             __syncthreads();
-            if (ok && n > 0)
-              na_pass<true>(rows_p, prof, ring, lane, n, d, hb, p == 0, p == passes - 1, S, bad,
-                            a.go, a.ge);
+            if (threadIdx.x == 0) {
+              int best = red_s[0];
+              for (int w = 1; w < NA_WARPS; w++) {
+                best = max(best, red_s[w]);
+                bad |= red_bad[w];
+              }
+              // a code outside the alphabet on either side: no score
+              if (bad || qbad)
+                atomicOr(status, NA_BAD_CODE);
+              else
+                a.scores[(long long)q * a.ns + s] = best;
+            }
+            __syncthreads();  // the next pair rewrites the shared words
           }
         }
-        if (!ok) continue;
-        // a code outside the alphabet on either side: the pair gets no score
-        bad = __any_sync(FULL, bad) || (qbad && n > 0);
-        S = na_warp_max(S);
+        continue;
+      }
+      if (q_ok && m > 0 && m <= NA_ALONE && cached != q) {
+        na_profile(pr, prof, sm, qr, m, wib);
+        cached = q;
+        __syncthreads();
+      }
+      // the warps take the chunk's subjects one by one
+      for (;;) {
+        int k = 0;
+        if (lane == 0) k = atomicAdd(&s_subject, 1);
+        k = __shfl_sync(FULL, k, 0);
+        if (k >= cnt) break;
+        const int s = s0 + k, n = a.slen[s];
+        if (!valid(n)) {  // refused, with nothing read or written
+          if (lane == 0) atomicOr(status, NA_BAD_LENGTH);
+          continue;
+        }
+        if (n > 0 && na_is_chain(m, n)) continue;  // scored in round 0
+        int S = 0, bad = 0;
+        if (m > 0 && n > 0) {
+          na_alone(pr, prof, ring, lane, n, a.sres + a.soff[s], S, bad, a.go, a.ge);
+          // a code outside the alphabet on either side: the pair gets no score
+          bad = __any_sync(FULL, bad) || qbad;
+          S = na_warp_max(S);
+        }
         if (lane == 0) {
           if (bad)
             atomicOr(status, NA_BAD_CODE);
@@ -410,11 +515,18 @@ extern "C" sw_status sw_search_pairs_noalloc(const uint8_t* queries, const int64
   // the counters and the status word must start at zero on every call
   CUDA_TRY(cudaMemsetAsync(scratch, 0, NA_HEADER * sizeof(int2), s));
   NaArgs a{queries, subjects, q_offsets, s_offsets, q_lengths, s_lengths, scores, n_queries,
-           n_subjects, gap_open + gap_extend, gap_extend, 0};
-  // subjects per block item: about eight items per block, and between one
-  // subject per warp and 64 (a profile is built per item)
-  const int64_t per = (int64_t)n_queries * n_subjects / ((int64_t)na.blocks * 8);
-  a.chunk = (int)(per < NA_WARPS ? NA_WARPS : per > 64 ? 64 : (per + NA_WARPS - 1) / NA_WARPS * NA_WARPS);
+           n_subjects, gap_open + gap_extend, gap_extend, 0, 0, 0, 0};
+  // large items for three quarters of the subjects, at least four to a block;
+  // small ones of a subject per warp
+  const int64_t pairs = (int64_t)n_queries * n_subjects;
+  auto items = [&](int64_t per_block, int lo, int hi) {
+    const int64_t c = pairs / (per_block * na.blocks);
+    return (int)(c < lo ? lo : c > hi ? hi : c);
+  };
+  a.chain = items(64, 1, 32);
+  a.small = items(64, NA_WARPS, 16);
+  a.large = items(4, NA_WARPS, 64);
+  a.split = (int)((int64_t)n_subjects * 3 / 4 / a.large) * a.large;
   noalloc_kernel<<<na.blocks, NA_WARPS * 32, 0, s>>>(a, mat, scratch);
   CUDA_TRY(cudaGetLastError());
   unsigned int status = 0;

@@ -74,3 +74,29 @@ def test_alignment_teams(warps, passes, n):
             if p - 1 + warps < passes:
                 assert read < start[p - 1 + warps] + (j + 31) // stage
     assert all(start[p] + spass <= start[p + warps] for p in range(passes - warps))
+
+
+@pytest.mark.parametrize("passes", [2, 4, 5, 9, 17])
+@pytest.mark.parametrize("n", [1, 33, 250, 353, 417, 1025, 1100])
+def test_caller_memory_chains(passes, n):
+    """na_chain (csrc/noalloc.cu): borders through rings of 256 columns between
+    neighbouring warps, through a whole row from the last warp to the first."""
+    ring = 256
+    spass = (n + 31 + STAGE - 1) // STAGE
+    period = max(spass + LAG, W * LAG)
+    start = [p // W * period + p % W * LAG for p in range(passes)]
+
+    def write(p, j):
+        return start[p] + (j + 31) // STAGE
+
+    for p in range(1, passes):
+        for j in range(n):
+            read = start[p] + j // STAGE
+            assert write(p - 1, j) < read
+            overwrites = [write(p - 1 + W, j)] if p - 1 + W < passes else []
+            if p % W:                                    # a ring: the same slot, later columns
+                overwrites += [write(p - 1, k) for k in range(j + ring, n, ring)]
+                if p - 1 + W < passes:
+                    overwrites += [write(p - 1 + W, k) for k in range(j % ring, n, ring)]
+            assert all(read < o for o in overwrites)
+    assert all(start[p] + spass <= start[p + W] for p in range(passes - W))
