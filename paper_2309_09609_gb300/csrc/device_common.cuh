@@ -134,7 +134,10 @@ struct IntraFeed {
   }
   __device__ __forceinline__ void words() {
     const uint8_t* lp = prof + code * 32 * TI;
-    if constexpr (TI == 8) {
+    static_assert(TI == 4 || TI == 8 || TI == 16, "rows per lane");
+    if constexpr (TI == 4) {
+      next[0] = *(const uint32_t*)lp;
+    } else if constexpr (TI == 8) {
       const uint2 v = *(const uint2*)lp;
       next[0] = v.x, next[1] = v.y;
     } else {
