@@ -275,9 +275,10 @@ typedef struct {
  *        own slot of q_len + s_len bytes (slots back to back in pair order),
  *        at its end.  Needs ops_capacity >= sum over pairs of q_len + s_len.
  * Of ops only the transcripts are written.
- * Device memory for the direction bits (4 bits per cell of every pair) and the
+ * Device memory for the cells (2 bytes per cell of every pair while that is at
+ * most 1 GiB and no score can exceed 32767, else 4 bits per cell) and the
  * call's other buffers is allocated by the call; the database keeps up to
- * 256 MiB of it (and 16 MiB of pinned memory) for later calls and frees it with
+ * 512 MiB of it (and 16 MiB of pinned memory) for later calls and frees it with
  * sw_db_destroy.  Pairs are processed in chunks of at most 8 GiB of bits.
  * Synchronous on the stream.
  * Errors: SW_EINVAL (index out of range, short ops buffer, bad gaps or

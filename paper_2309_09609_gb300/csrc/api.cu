@@ -1617,10 +1617,15 @@ extern "C" sw_status sw_search_plain(sw_db* db, const uint8_t* queries, const in
 }
 
 // ---- optimal alignments with traceback ------------------------------------------------------
-// Largest direction-bit buffer of one chunk of pairs (bytes).
+// Largest buffer of cells of one chunk of pairs (bytes).
 static constexpr int64_t kAlignChunkBytes = 8ll << 30;
+// A call's cells with H kept, at most (bytes, two to a cell): larger calls are
+// bound by the chip's rate, where four bits cost no more (20 pairs of 5,000 x
+// 5,000, just below: 5.0 ms with bits, 4.1 with H).
+static constexpr int64_t kAlignKeepH = 1ll << 30;
+static constexpr int32_t kAlignKeepHColumns = 65000;  // a cell's step in 16 bits
 // What a database keeps of a call's buffers, at most.
-static constexpr size_t kAlignKeepDevice = 256u << 20, kAlignKeepPinned = 16u << 20;
+static constexpr size_t kAlignKeepDevice = 512u << 20, kAlignKeepPinned = 16u << 20;
 
 extern "C" sw_status sw_align(sw_db* db, const uint8_t* queries, const int32_t* q_lengths,
                               int32_t n_queries, const int32_t* pair_query,
@@ -1639,7 +1644,8 @@ extern "C" sw_status sw_align(sw_db* db, const uint8_t* queries, const int32_t* 
   SearchParams P;
   memset(&P, 0, sizeof P);
   bool packed_ok;
-  st = fill_scoring(P, gap_open, gap_extend, matrix, &packed_ok);
+  int max_sm = 0;
+  st = fill_scoring(P, gap_open, gap_extend, matrix, &packed_ok, &max_sm);
   if (st != SW_OK) return st;
   const int64_t N = db->view.n;
   // per pair: sorted subject, sizes, and its transcript slot
@@ -1665,11 +1671,21 @@ extern "C" sw_status sw_align(sw_db* db, const uint8_t* queries, const int32_t* 
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, db->device);
   const int team = align_team(n_pairs, sms);  // warps to a pair
-  // chunks of pairs whose direction bits fit kAlignChunkBytes (one pair may exceed it alone)
+  // H of every cell is kept where 16 bits hold it and the cells are few, else
+  // four direction bits
+  bool keep_h = P.go <= INT16_MAX;
+  int64_t cell_bytes = 0;
+  for (int32_t k = 0; k < n_pairs && keep_h; k++) {
+    const int32_t m = hb.len[items[k].q], n = db->clen_h[items[k].s];
+    cell_bytes += align_bits_bytes(team, true, m, n);
+    keep_h = cell_bytes <= kAlignKeepH && (int64_t)max_sm * std::min(m, n) <= INT16_MAX &&
+             n <= kAlignKeepHColumns;
+  }
+  // chunks of pairs whose cells fit kAlignChunkBytes (one pair may exceed it alone)
   std::vector<int32_t> chunk_begin{0};
   int64_t words = 0, max_words = 0, max_border = 0, border = 0;
   for (int32_t k = 0; k < n_pairs; k++) {
-    const int64_t w = align_bits_bytes(team, hb.len[items[k].q], db->clen_h[items[k].s]);
+    const int64_t w = align_bits_bytes(team, keep_h, hb.len[items[k].q], db->clen_h[items[k].s]);
     if (k > chunk_begin.back() && words + w > kAlignChunkBytes) {
       chunk_begin.push_back(k);
       words = border = 0;
@@ -1678,7 +1694,7 @@ extern "C" sw_status sw_align(sw_db* db, const uint8_t* queries, const int32_t* 
     items[k].border_off = border;
     items[k].ops_end = slot[k + 1];
     words += w;
-    border += (int64_t)team * db->clen_h[items[k].s];
+    border += align_border_ints(team, db->clen_h[items[k].s]);
     max_words = std::max(max_words, words);
     max_border = std::max(max_border, border);
   }
@@ -1686,7 +1702,7 @@ extern "C" sw_status sw_align(sw_db* db, const uint8_t* queries, const int32_t* 
   cudaStream_t cs = (cudaStream_t)stream;
   // One device buffer: what goes up (parameters, items, the query arrays) in
   // one copy, what comes back (records, transcripts) in one copy, the border
-  // rows and the bits.
+  // rows and the cells.
   const size_t up_items = block_align(sizeof(SearchParams));
   const size_t up_qoff = up_items + block_align(sizeof(AlignItem) * (size_t)n_pairs);
   const size_t up_qlen = up_qoff + block_align(sizeof(int64_t) * (size_t)n_queries);
@@ -1725,10 +1741,10 @@ extern "C" sw_status sw_align(sw_db* db, const uint8_t* queries, const int32_t* 
   AlignOut* out_d = (AlignOut*)(buf.dev + at_out);
   for (size_t c = 0; c + 1 < chunk_begin.size() && e == cudaSuccess; c++) {
     const int32_t k0 = chunk_begin[c], nk = chunk_begin[c + 1] - k0;
-    e = launch_align(team, sms, db->view, (const SearchParams*)buf.dev, items_d + k0, nk,
+    e = launch_align(team, keep_h, sms, db->view, (const SearchParams*)buf.dev, items_d + k0, nk,
                      buf.dev + at_bits, (int2*)(buf.dev + at_border), out_d + k0,
                      buf.dev + at_out + ops_at, cs);
-    // the next chunk reuses the bits: its kernel runs after this one's on the stream
+    // the next chunk reuses the cells: its kernel runs after this one's on the stream
   }
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(host, buf.dev + at_out, back_bytes, cudaMemcpyDeviceToHost, cs);

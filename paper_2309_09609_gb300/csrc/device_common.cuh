@@ -43,10 +43,6 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
 __device__ __forceinline__ constexpr uint32_t sext_pair_sel(int k) {
   return (uint32_t)(k | ((8 | k) << 4) | ((4 + k) << 8) | ((12 + k) << 12));
 }
-// int8 byte k of w, sign-extended to int32
-__device__ __forceinline__ int sext_byte(uint32_t w, int k) {
-  return (int)prmt(w, 0u, (uint32_t)(k | ((8 | k) << 4) | ((8 | k) << 8) | ((8 | k) << 12)));
-}
 
 __device__ __forceinline__ uint4 ldg_nc(const uint4* p) {
   uint4 v;
@@ -119,9 +115,9 @@ __device__ __forceinline__ void lane_profile(uint8_t* prof, const int8_t* __rest
 
 // The lane's profile words along its columns, loaded ahead of the cells: the
 // code of column j + 2 and the words of column j + 1 while column j is scored
-// (columns past either end read the padding code with PAD, else the last or
-// first code, for lanes that skip them).
-template <int TI, bool PAD = false>
+// (columns past either end read the first or last code, for lanes that skip
+// them).
+template <int TI>
 struct IntraFeed {
   const uint8_t* d;     // the subject's codes
   const uint8_t* prof;  // the lane's profile rows, 32 * TI bytes per code
@@ -129,15 +125,12 @@ struct IntraFeed {
   uint32_t next[TI / 4];
 
   __device__ __forceinline__ int at(int j) const {
-    const int c = d[min(max(j, 0), n - 1)];
-    return PAD && (unsigned)j >= (unsigned)n ? PAD_CODE : c;
+    return d[min(max(j, 0), n - 1)];
   }
   __device__ __forceinline__ void words() {
     const uint8_t* lp = prof + code * 32 * TI;
-    static_assert(TI == 4 || TI == 8 || TI == 16, "rows per lane");
-    if constexpr (TI == 4) {
-      next[0] = *(const uint32_t*)lp;
-    } else if constexpr (TI == 8) {
+    static_assert(TI == 8 || TI == 16, "rows per lane");
+    if constexpr (TI == 8) {
       const uint2 v = *(const uint2*)lp;
       next[0] = v.x, next[1] = v.y;
     } else {

@@ -217,12 +217,14 @@ struct AlignOut {
   int32_t n_ops;
   int64_t ops_offset;        // the transcript occupies [ops_offset, ops_offset + n_ops)
 };
-// bytes of direction bits for an m x n pair (4 bits per cell)
-int64_t align_bits_bytes(int team, int32_t m, int32_t n);
+// int2 of an n-column pair's border rows, one per warp of the team
+int64_t align_border_ints(int team, int32_t n);
+// bytes of an m x n pair's cells: H in 16 bits (keep_h) or 4 direction bits
+int64_t align_bits_bytes(int team, bool keep_h, int32_t m, int32_t n);
 // Warps to a pair (each with a border row of the subject's length) for a call
 // of n_pairs.
 int align_team(int n_pairs, int sms);
-cudaError_t launch_align(int team, int sms, const DbView& db, const SearchParams* params,
+cudaError_t launch_align(int team, bool keep_h, int sms, const DbView& db, const SearchParams* params,
                          const AlignItem* items, int n_items, uint8_t* bits, int2* border,
                          AlignOut* out, uint8_t* ops, cudaStream_t stream);
 

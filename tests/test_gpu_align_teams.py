@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("pairs", [9, 600, 2700])
-@pytest.mark.parametrize("gaps", [(10, 2), (0, 1)])
+@pytest.mark.parametrize("gaps", [(10, 2), (0, 1), (3, 0)])
 def test_every_team_size(pairs, gaps):
     nvbuild.build()
     rng = np.random.default_rng(pairs)
@@ -33,3 +33,23 @@ def test_every_team_size(pairs, gaps):
         if (a, b) not in want:
             want[a, b] = oracle.align(seqs[a], seqs[b], *gaps)
         assert got[k] == want[a, b], (a, b)
+
+
+@pytest.mark.parametrize("top", [6, 127])
+def test_scores_below_and_above_16_bits(top):
+    # with an entry of 127 a pair of 420 could exceed 32767, so the call stores
+    # direction bits; with 6 it stores H
+    nvbuild.build()
+    rng = np.random.default_rng(top)
+    m = rng.integers(-6, 3, size=(24, 24)).astype(np.int8)
+    np.fill_diagonal(m, top)
+    base = seqset(rng, [420]).seq(0)
+    seqs = [base, np.delete(base, np.arange(100, 140)), np.delete(synth.mutate(rng, base, 0.2), [7]),
+            seqset(rng, [300]).seq(0)]
+    ss = synth.SeqSet(np.concatenate(seqs), np.array([s.size for s in seqs], np.int32))
+    pq, ps = np.repeat(np.arange(4), 4), np.tile(np.arange(4), 4)
+    for repeat, gaps in ((1, (9, 1)), (1, (0, 0)), (1, (40000, 3)), (40, (5, 0)), (160, (11, 1))):
+        a, b = np.tile(pq, repeat), np.tile(ps, repeat)
+        got = swgb.Database.from_seqset(ss).align(ss.res, ss.lens, a, b, *gaps, m)
+        want = [oracle.align(seqs[q], seqs[s], *gaps, m.astype(np.int32)) for q, s in zip(pq, ps)]
+        assert got == want * repeat
