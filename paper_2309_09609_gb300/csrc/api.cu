@@ -653,8 +653,9 @@ extern "C" sw_status sw_plan_create(sw_db* db, int32_t max_queries, int64_t max_
   cudaError_t e = injected_fault("alloc") ? cudaErrorMemoryAllocation : cudaSuccess;
   p->scr.inter_stride_vec = (int64_t)(L_inter / CHUNK) * 4 * 32;
   p->scr.intra_stride = std::max(v.max_len, 1);
-  // (+4: the two-query pair kernel loads its border 4 columns ahead)
-  p->scr.pair_stride = std::max(v.max_len, 1) + 4;
+  // (the lane kernel's rows start 64 columns before the first and end 4 after
+  // the last; the two-query pair kernel loads its border 4 columns ahead)
+  p->scr.pair_stride = std::max(v.max_len, 1) + 72;
   p->scr.flag_capacity = o.flag_capacity > 0
                             ? (int64_t)o.flag_capacity
                             : std::min<int64_t>((int64_t)max_queries * std::max<int64_t>(v.n, 1),
@@ -1010,16 +1011,16 @@ static int32_t plan_streams_long(sw_plan* p, const HostBatch& hb, int32_t nq, in
 // with shorter items, a larger group, halves or a chain.
 // Measured cycles of a step with PR rows per lane: of a scheduler with four
 // warps, 98, 185, 273 and 366 for 8, 16, 24 and 32 rows, 94 and 262 for 8 and
-// 24 rows in halves, 69 and 107 for 4 and 8 rows in a chain; of a warp alone,
-// 158, 284, 403 and 559, in halves 108 and 280, in a chain 132 and 148.
+// 24 rows in halves, 65 and 102 for 4 and 8 rows in a chain; of a warp alone,
+// 158, 284, 403 and 559, in halves 108 and 280, in a chain 118 and 123.
 struct LaneCand {
   int lg, pr, passes, full, chain, halves;
   int ramp() const { return halves ? 2 * lg : lg; }
   double busy(int rows) const {  // scheduler cycles of a step
-    return ((halves ? 10.5 : 11.1) * rows + 9) * (chain ? 1.18 : 1.0);
+    return ((halves ? 10.5 : 11.1) * rows + 9) * (chain ? 1.1 : 1.0);
   }
   double alone(int rows) const {  // cycles of a step on a scheduler of its own
-    return (halves ? 10.7 * rows + 22 : 16.0 * rows + 30) + (chain ? 38 : 0);
+    return (halves ? 10.7 * rows + 22 : 16.0 * rows + 30) + (chain ? 18 : 0);
   }
   // scheduler cycles of one step of every pass
   double thr() const { return (passes - 1) * busy(full) + busy(pr); }
@@ -1028,8 +1029,9 @@ struct LaneCand {
     if (!chain)
       return (n + ramp()) * std::max((passes - 1) * alone(full) + alone(pr), share * thr());
     const double step = std::max(alone(full), share * busy(full));
-    const double stages = (n + ramp()) / 64 + 1, period = std::max(stages, 8.0);
-    return ((passes - 1) / LANE_WARPS * period + (passes - 1) % LANE_WARPS * 2 + stages) * 64 * step;
+    const double lag = full == 4 ? 3 : 4;
+    const double stages = (n + ramp()) / 32 + 1, period = std::max(stages, LANE_WARPS * lag);
+    return ((passes - 1) / LANE_WARPS * period + (passes - 1) % LANE_WARPS * lag + stages) * 32 * step;
   }
 };
 

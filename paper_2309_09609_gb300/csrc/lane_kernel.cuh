@@ -57,8 +57,19 @@ constexpr int LANE_RING = 4 * (2 * 256 + 32);  // bytes per warp: 2 * 8 * 32 col
 constexpr int LANE_RINGS = LANE_WARPS * LANE_RING;
 constexpr int LANE_SMEM = LANE_RINGS + LANE_PROFILE;
 constexpr int LANE_SMEM_WIDE = LANE_RINGS + LANE_WARPS * LANE_PROFILE / 2;  // chains of 16 rows
-constexpr int CHAIN_STAGE = 64;  // steps between the block barriers of a chain
-constexpr int CHAIN_LAG = 2;     // stages between the starts of consecutive passes
+constexpr int EDGE_STAGE = 32;  // steps of a stage: a chain's block barriers lie between
+constexpr int EDGE_PAD = 64;    // a border row holds column j at EDGE_PAD + j
+// Stages between the starts of a chain's consecutive passes of `full` rows per
+// lane (4, or 8 and 16 in halves).
+__host__ __device__ __forceinline__ constexpr int chain_lag(int full) { return full == 4 ? 3 : 4; }
+// Stages of a pass of pr rows per lane over n columns.
+__host__ __device__ __forceinline__ constexpr int chain_stages(int pr, int n) {
+  return (n + (pr == 4 ? 31 : 63) + EDGE_STAGE - 1) / EDGE_STAGE;
+}
+// A warp's stage of border columns, and what its last steps read ahead.
+struct LaneEdge {
+  uint2 col[EDGE_STAGE + 4];
+};
 
 // Profile words of one column of a quarter: four rows to a word, per subject.
 template <int PR, int NQ>
@@ -128,16 +139,21 @@ __device__ __forceinline__ void chain_barrier() {
 // quarter above (the last one of lane k - 1 for q = 0) left at step t - 1.
 // With several passes LG is 32, hb_in holds the border row below the pass
 // before (unless this is the first) and hb_out takes this pass's (unless it is
-// the last): lane 0 reads column j at most U steps before its step j, lane 31
-// writes it at step j + 32 NQ - 1.  SERIAL: both are one row.  CHAINED: every
-// CHAIN_STAGE steps the block's warps meet at a barrier, and the pass before,
-// on another warp, is CHAIN_LAG stages ahead: the columns up to 64 k + 63 that
-// stage k reads were written by that pass's step 64 k + 126 at the latest, in
-// its stage k + 1, which ended before this stage began.
+// the last): lane 31 writes column j at step j + 32 NQ - 1.  The steps go by
+// stages of EDGE_STAGE columns, which the warp fetches a stage ahead and keeps
+// in `edge`; a column goes to lane 0 in the rotation that takes the lanes'
+// edges one lane down, as lane 31's.  SERIAL: hb_in and hb_out are one row.
+// CHAINED: after every stage the block's warps meet at a barrier, and the pass
+// before, on another warp, is chain_lag stages ahead: the columns up to 32 k +
+// 63 that stage k fetches were written by that pass's step 32 k + 62 + 32 NQ at
+// the latest, in its stage k + 1 + NQ, which ended before this stage began.
+// (With each step fetching its own border column 4 steps ahead and testing it,
+// a chain's step took 124 cycles for 4 rows on a scheduler of its own and 279
+// with four warps, 143 and 437 for 8 rows; now 118 and 261, 123 and 409.)
 template <int PR, int NQ, int MODE>
 __device__ __forceinline__ void lane_sweep(const uint8_t* prof, uint8_t* ring, int lane, int lg,
-                                           int n, const uint4* src, int chunks, const uint2* hb_in,
-                                           uint2* hb_out, bool first, bool last, uint32_t& smax,
+                                           int n, const uint4* src, int chunks, LaneEdge* edge,
+                                           const uint2* hb_in, uint2* hb_out, bool first, bool last, uint32_t& smax,
                                            uint32_t GO2, uint32_t NGE2) {
   constexpr bool PASSES = MODE != ALONE;
   constexpr int U = LaneShape<PR, NQ>::UNROLL;
@@ -192,10 +208,18 @@ __device__ __forceinline__ void lane_sweep(const uint8_t* prof, uint8_t* ring, i
   uint4 next = load(0);
   const int steps = n + NQ * lg - 1;
   const uint32_t mask = (uint32_t)(4 * (2 * cols - 1));
-  const int span = MODE == CHAINED ? CHAIN_STAGE : cols;
+  const int span = PASSES ? EDGE_STAGE : cols;
+  // columns past the end are zeros, like those above the first pass
+  auto border = [&](int c) {
+    return !first && c < n ? hb_in[EDGE_PAD + c] : make_uint2(0u, 0u);
+  };
+  uint2 edge_next;
+  if constexpr (PASSES) edge_next = border(lane);
+  const int from = (lane + 31) & 31;
+  const bool keep = lane == 31 && !last;
   int b = 0;
   for (int t0 = 0; t0 < steps; t0 += span) {
-    if (MODE != CHAINED || (t0 & (cols - 1)) == 0) {
+    if (!PASSES || (t0 & (cols - 1)) == 0) {
       __syncwarp();
       store(b & 1, next);
       next = load(++b);
@@ -204,8 +228,13 @@ __device__ __forceinline__ void lane_sweep(const uint8_t* prof, uint8_t* ring, i
     const int tend = min(t0 + span, steps);
     uint2 bq[U];  // the border of columns t .. t + U - 1
     if constexpr (PASSES) {
+      static_assert(U <= 4, "columns read ahead");
+      __syncwarp();
+      edge->col[lane] = edge_next;
+      edge_next = border(t0 + EDGE_STAGE + lane);
+      __syncwarp();
 #pragma unroll
-      for (int u = 0; u < U; u++) bq[u] = hb_in[min(t0 + u, n - 1)];
+      for (int u = 0; u < U; u++) bq[u] = edge->col[u];
     }
     // the profile words of step t are loaded one step ahead; the last step of
     // a ring block reads whatever code the slot holds, and is read again here
@@ -223,15 +252,14 @@ __device__ __forceinline__ void lane_sweep(const uint8_t* prof, uint8_t* ring, i
 #pragma unroll
       for (int u = 0; u < U; u++) {
         // the row above: lane k - 1's bottom row, H = F = 0 above the matrix
-        uint32_t in_h = imad(__shfl_up_sync(FULL, h1[NQ - 1], 1, lg), not0, 0u);
-        uint32_t in_f = imad(__shfl_up_sync(FULL, f1[NQ - 1], 1, lg), not0, 0u);
+        uint32_t in_h, in_f;
         if constexpr (PASSES) {
-          const uint2 bv = bq[u];
-          bq[u] = hb_in[min(t + u + U, min(tend, n) - 1)];
-          if (li == 0 && !first) {
-            in_h = bv.x;
-            in_f = bv.y;
-          }
+          in_h = __shfl_sync(FULL, lane == 31 ? bq[u].x : h1[NQ - 1], from);
+          in_f = __shfl_sync(FULL, lane == 31 ? bq[u].y : f1[NQ - 1], from);
+          bq[u] = edge->col[t - t0 + u + U];
+        } else {
+          in_h = imad(__shfl_up_sync(FULL, h1[NQ - 1], 1, lg), not0, 0u);
+          in_f = imad(__shfl_up_sync(FULL, f1[NQ - 1], 1, lg), not0, 0u);
         }
         if constexpr (!AHEAD) fetch(rp + 4 * u);
         LaneWords<PR, NQ> now[NQ];
@@ -262,9 +290,7 @@ __device__ __forceinline__ void lane_sweep(const uint8_t* prof, uint8_t* ring, i
           f1[q] = nf[q];
         }
         if constexpr (PASSES) {
-          const int j = t + u - (32 * NQ - 1);
-          if (lane == 31 && !last && j >= 0 && j < n)
-            hb_out[j] = make_uint2(h1[NQ - 1], f1[NQ - 1]);
+          if (keep) hb_out[EDGE_PAD - (32 * NQ - 1) + t + u] = make_uint2(h1[NQ - 1], f1[NQ - 1]);
         }
       }
     }
@@ -300,6 +326,7 @@ struct LanePlace {
   int lg, n;         // lanes per group; columns of the warp's longest subject
   const uint4* src;  // this group's subject pair in the interleaved layout
   int chunks;
+  LaneEdge* edge;    // the warp's
   uint2* hb;         // the warp's border row
 };
 
@@ -322,10 +349,10 @@ __device__ __forceinline__ void lane_pass(const SearchParams* __restrict__ P, ui
   if (at.n == 0) return;  // uniform over the warp
   if (passes == 1)
     lane_sweep<PR, NQ, ALONE>(prof, ring, lane, at.lg, at.n, at.src, at.chunks, nullptr, nullptr,
-                              true, true, smax, GO2, NGE2);
+                              nullptr, true, true, smax, GO2, NGE2);
   else if constexpr (NQ == 1)
-    lane_sweep<PR, 1, SERIAL>(prof, ring, lane, 32, at.n, at.src, at.chunks, at.hb, at.hb,
-                              pass == 0, pass == passes - 1, smax, GO2, NGE2);
+    lane_sweep<PR, 1, SERIAL>(prof, ring, lane, 32, at.n, at.src, at.chunks, at.edge, at.hb,
+                              at.hb, pass == 0, pass == passes - 1, smax, GO2, NGE2);
 }
 
 // One pass of a chain, on this warp, with a profile of its own.
@@ -342,23 +369,23 @@ __device__ __forceinline__ void chain_pass(const SearchParams* __restrict__ P, u
   __syncwarp();
   lane_profile_rows<PR, NQ>(prof, sm, qr, m, row0, 32, 0, 1);
   __syncwarp();
-  lane_sweep<PR, NQ, CHAINED>(prof, ring, lane, 32, at.n, at.src, at.chunks, hb_in, at.hb, first,
-                              last, smax, GO2, NGE2);
+  lane_sweep<PR, NQ, CHAINED>(prof, ring, lane, 32, at.n, at.src, at.chunks, at.edge, hb_in, at.hb,
+                              first, last, smax, GO2, NGE2);
 }
 
 // A chain: one subject pair on the whole block, for items that would take too
 // long on one warp.  Warp w takes the passes w, w + LANE_WARPS, ...; pass p
-// starts at stage (p / W) * period + (p % W) * CHAIN_LAG with period the larger
-// of a pass's stages and W * CHAIN_LAG, so consecutive passes are at least
-// CHAIN_LAG stages apart, and a warp's next pass starts after its previous one
-// ends and at least W * CHAIN_LAG stages after it started, when the pass that
+// starts at stage (p / W) * period + (p % W) * lag with period the larger of a
+// pass's stages and W * lag (lag = chain_lag), so consecutive passes are at least
+// lag stages apart, and a warp's next pass starts after its previous one ends
+// and at least W * lag stages after it started, when the pass that
 // read the border row it will overwrite is further on.  Every warp meets the
 // same number of barriers.
 template <int G>
 __device__ __forceinline__ void lane_chain(const DbView& db, const SearchParams* __restrict__ P,
                                            SearchState* st, const Scratch& scr, uint8_t* smem,
                                            const uint8_t* sm, uint32_t* red, const LaneSeg& sg,
-                                           int unit) {
+                                           LaneEdge* edge, int unit) {
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int pair = sg.pair0 + unit;
   uint2* rows = scr.pair_border +
@@ -368,20 +395,20 @@ __device__ __forceinline__ void lane_chain(const DbView& db, const SearchParams*
   at.n = db.clen[2 * pair];
   at.src = (const uint4*)(db.inter + db.goff[pair / 32]) + (pair & 31);
   at.chunks = db.glen[pair / 32] / CHUNK;
+  at.edge = edge + wib;
   at.hb = rows + wib * scr.pair_stride;
   const uint2* hb_in = rows + (wib + LANE_WARPS - 1) % LANE_WARPS * scr.pair_stride;
   const int m = P->qlen[sg.q];
   const uint8_t* __restrict__ qr = P->qres + P->qoff[sg.q];
-  // stages of a pass (at NQ = 2; a pass of fewer steps waits out the rest)
-  const int spass = (at.n + 63 + CHAIN_STAGE - 1) / CHAIN_STAGE;
-  const int period = max(spass, LANE_WARPS * CHAIN_LAG);
-  const int end = (sg.passes - 1) / LANE_WARPS * period +
-                  (sg.passes - 1) % LANE_WARPS * CHAIN_LAG + spass;
+  // stages of a pass of `full` rows (one of fewer steps waits out the rest)
+  const int lag = chain_lag(sg.full), spass = chain_stages(sg.full, at.n);
+  const int period = max(spass, LANE_WARPS * lag);
+  const int end = (sg.passes - 1) / LANE_WARPS * period + (sg.passes - 1) % LANE_WARPS * lag + spass;
   uint32_t smax = 0u;
   if (at.n > 0) {  // uniform over the block
     int g = 0;
     for (int p = wib; p < sg.passes; p += LANE_WARPS) {
-      for (const int start = p / LANE_WARPS * period + p % LANE_WARPS * CHAIN_LAG; g < start; g++)
+      for (const int start = p / LANE_WARPS * period + p % LANE_WARPS * lag; g < start; g++)
         chain_barrier();
       const bool last = p == sg.passes - 1;
       const int pr = last ? sg.pr : sg.full, row0 = p * 32 * sg.full, slice = NCODES * 32 * sg.full;
@@ -390,7 +417,7 @@ __device__ __forceinline__ void lane_chain(const DbView& db, const SearchParams*
         case 8: chain_pass<8, 2, G>(P, smem, sm, qr, m, row0, slice, at, hb_in, p == 0, last, smax); break;
         default: chain_pass<16, 2, G>(P, smem, sm, qr, m, row0, slice, at, hb_in, p == 0, last, smax); break;
       }
-      g += pr == 4 ? (at.n + 31 + CHAIN_STAGE - 1) / CHAIN_STAGE : spass;
+      g += chain_stages(pr, at.n);
     }
     for (; g < end; g++) chain_barrier();
   }
@@ -410,7 +437,7 @@ template <int G>
 __device__ __forceinline__ void lane_item(const DbView& db, const SearchParams* __restrict__ P,
                                           SearchState* st, const Scratch& scr, uint8_t* smem,
                                           const uint8_t* sm, const LaneSeg& sg, int seg,
-                                          int& cached, int unit) {
+                                          int& cached, LaneEdge* edge, int unit) {
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   LanePlace at;
   at.lg = sg.lg;
@@ -421,6 +448,7 @@ __device__ __forceinline__ void lane_item(const DbView& db, const SearchParams* 
   const int grp = (has ? pair : 0) / 32;
   at.src = (const uint4*)(db.inter + db.goff[grp]) + (pair & 31);
   at.chunks = has ? db.glen[grp] / CHUNK : 0;
+  at.edge = edge + wib;
   at.hb = scr.pair_border +
           (scr.lane_row0 + (int64_t)blockIdx.x * LANE_WARPS + wib) * scr.pair_stride;
   const int m = P->qlen[sg.q];
@@ -456,6 +484,7 @@ lane_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Scra
   extern __shared__ __align__(16) uint8_t smem[];
   __shared__ __align__(16) uint8_t sm[NCODES * SM_ROW];
   __shared__ unsigned long long s_item;
+  __shared__ LaneEdge edge[LANE_WARPS];
   __shared__ uint32_t red[LANE_WARPS];
   const long long total = P->n_lane_items;
   for (int i = threadIdx.x; i < NCODES * SM_ROW; i += blockDim.x)
@@ -479,10 +508,10 @@ lane_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Scra
     const LaneSeg sg = segs[lo];
     if (sg.chain) {
       __syncthreads();  // every warp is done with the profile before
-      lane_chain<G>(db, P, st, scr, smem, sm, red, sg, (int)(it - sg.first));
+      lane_chain<G>(db, P, st, scr, smem, sm, red, sg, edge, (int)(it - sg.first));
       cached = -1;
     } else {
-      lane_item<G>(db, P, st, scr, smem, sm, sg, lo, cached, (int)(it - sg.first));
+      lane_item<G>(db, P, st, scr, smem, sm, sg, lo, cached, edge, (int)(it - sg.first));
     }
     __syncthreads();  // the item before is read by all, and its chain is done
     if (threadIdx.x == 0) s_item = gridDim.x + atomicAdd(&st->lane_work, 1ull);

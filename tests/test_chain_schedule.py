@@ -1,39 +1,41 @@
-"""The stage schedule of a chain (lane_chain in csrc/lane_kernel.cu): the passes
-of a subject pair on the warps of a block, with a barrier every 64 steps.
+"""The stage schedule of a chain (lane_chain in csrc/lane_kernel.cuh): the
+passes of a subject pair on the warps of a block, with a barrier every 32 steps.
 
-Restated here: every border column is written in an earlier stage than the
-one that reads it (the next pass reads a stage's columns within that stage), it
-is read before the warp's next pass overwrites it, a warp's passes do not
-overlap, and every warp meets the same number of barriers.  Passes of 4 rows per
-lane write a column 31 steps after reading it, the others 63 (`skews`).
+Restated here: every border column is written in an earlier stage than the one
+that fetches it (stage k fetches the columns of stage k + 1, the first also its
+own), it is read before the warp's next pass overwrites it, a warp's passes do
+not overlap, and every warp meets the same number of barriers.  Passes of 4 rows
+per lane write a column 31 steps after reading it, the others 63 (`skew`).
 """
-import itertools
-
 import pytest
 
-W, LAG, STAGE = 4, 2, 64
+W, STAGE = 4, 32
 
 
 @pytest.mark.parametrize("passes", [2, 3, 4, 5, 8, 9, 26])
 @pytest.mark.parametrize("n", [1, 30, 33, 64, 97, 200, 417, 449, 513, 2000])
-def test_borders_are_written_before_and_read_before_overwritten(passes, n):
-    spass = (n + 63 + STAGE - 1) // STAGE
-    period = max(spass, W * LAG)
-    start = [p // W * period + p % W * LAG for p in range(passes)]
+@pytest.mark.parametrize("full,last", [(4, 4), (8, 4), (8, 8), (16, 4), (16, 16)])
+def test_borders_are_written_before_and_read_before_overwritten(passes, n, full, last):
+    rows = [full] * (passes - 1) + [last]
+    lag = 3 if full == 4 else 4
+
+    def stages(pr):
+        return (n + (31 if pr == 4 else 63) + STAGE - 1) // STAGE
+
+    spass = stages(full)
+    period = max(spass, W * lag)
+    start = [p // W * period + p % W * lag for p in range(passes)]
     end = start[-1] + spass
-    # every pass but the last has one number of rows, the last may have fewer
-    for skews in itertools.product((31, 63), (31, 63)):
-        skew = [skews[0]] * (passes - 1) + [skews[1]]
-        for p in range(1, passes):
-            for j in range(n):
-                read = start[p] + j // STAGE
-                assert start[p - 1] + (j + skew[p - 1]) // STAGE < read
-                if p - 1 + W < passes:
-                    assert read < start[p - 1 + W] + (j + skew[p - 1 + W]) // STAGE
-        for p in range(passes):
-            assert (n + skew[p] + STAGE - 1) // STAGE <= spass
+    skew = [31 if pr == 4 else 63 for pr in rows]
+    for p in range(1, passes):
+        for j in range(n):
+            read = start[p] + max(j // STAGE - 1, 0)
+            assert start[p - 1] + (j + skew[p - 1]) // STAGE < read
+            if p - 1 + W < passes:
+                assert read < start[p - 1 + W] + (j + skew[p - 1 + W]) // STAGE
     for p in range(passes):
-        assert start[p] + spass <= end
+        own = stages(rows[p])
+        assert own <= spass and start[p] + own <= end
         if p + W < passes:
             assert start[p] + spass <= start[p + W]
 
@@ -81,7 +83,7 @@ def test_alignment_teams(warps, passes, n):
 def test_caller_memory_chains(passes, n):
     """na_chain (csrc/noalloc.cu): borders through rings of 256 columns between
     neighbouring warps, through a whole row from the last warp to the first."""
-    ring = 256
+    ring, STAGE, LAG = 256, 64, 2
     spass = (n + 31 + STAGE - 1) // STAGE
     period = max(spass + LAG, W * LAG)
     start = [p // W * period + p % W * LAG for p in range(passes)]
