@@ -1015,6 +1015,7 @@ static int32_t plan_streams_long(sw_plan* p, const HostBatch& hb, int32_t nq, in
 // 158, 284, 403 and 559, in halves 108 and 280, in a chain 118 and 123.
 struct LaneCand {
   int lg, pr, passes, full, chain, halves;
+  int tail = 1;  // passes of pr rows at the end, the others of `full`
   int ramp() const { return halves ? 2 * lg : lg; }
   double busy(int rows) const {  // scheduler cycles of a step
     return ((halves ? 10.5 : 11.1) * rows + 9) * (chain ? 1.1 : 1.0);
@@ -1023,7 +1024,7 @@ struct LaneCand {
     return (halves ? 10.7 * rows + 22 : 16.0 * rows + 30) + (chain ? 18 : 0);
   }
   // scheduler cycles of one step of every pass
-  double thr() const { return (passes - 1) * busy(full) + busy(pr); }
+  double thr() const { return (passes - tail) * busy(full) + tail * busy(pr); }
   // cycles of the passes over n columns when `share` warps share a scheduler
   double item(double n, double share) const {
     if (!chain)
@@ -1031,12 +1032,16 @@ struct LaneCand {
     const double step = std::max(alone(full), share * busy(full));
     const double lag = full == 4 ? 3 : 4;
     const double stages = (n + ramp()) / 32 + 1, period = std::max(stages, LANE_WARPS * lag);
+    if (tail > 1)
+      return ((passes - tail) / LANE_WARPS * period * step +
+              ((tail - 1) * lag + stages) * std::max(alone(pr), share * busy(pr))) * 32;
     return ((passes - 1) / LANE_WARPS * period + (passes - 1) % LANE_WARPS * lag + stages) * 32 * step;
   }
 };
 
 // The shapes for a query of m residues: 8, 16 and 32 lanes; 32 lanes in halves;
 // chains of 4 to 16 rows per lane (16 only with the wide launch).
+static constexpr int MAX_SHAPES = 12;
 static int lane_candidates(int32_t m, bool wide, LaneCand* c) {
   int n = 0;
   auto fit = [](int rows, int step) { return std::max(step, (rows + step - 1) / step * step); };
@@ -1053,6 +1058,14 @@ static int lane_candidates(int32_t m, bool wide, LaneCand* c) {
     int pr = fit((m - (passes - 1) * 32 * full + 31) / 32, 4);
     while (pr & (pr - 1)) pr += 4;  // chains come in 4, 8, 16 and 32 rows
     c[n++] = LaneCand{32, pr, passes, full, 1, full > 4};
+    // The passes after the last whole round of the block's warps leave some of
+    // them idle: the same rows as up to a round of passes of fewer rows each.
+    const int heads = m / (32 * full * LANE_WARPS) * LANE_WARPS, rest = m - heads * 32 * full;
+    if (heads == 0 || rest == 0) continue;
+    pr = 4;
+    while (32 * pr * LANE_WARPS < rest) pr *= 2;
+    const int tail = (rest + 32 * pr - 1) / (32 * pr);
+    if (pr < full && tail > 1) c[n++] = LaneCand{32, pr, heads + tail, full, 1, 1, tail};
   }
   return n;
 }
@@ -1091,7 +1104,7 @@ static int64_t plan_lanes(sw_plan* p, const HostBatch& hb, int32_t nq, int64_t p
     return n * (x.chain ? std::min(x.passes, LANE_WARPS) : x.lg / 32.0);
   };
   struct Query {
-    LaneCand c[MAX_SEGS];
+    LaneCand c[MAX_SHAPES];
     int nc;
   };
   struct Piece {
@@ -1119,11 +1132,11 @@ static int64_t plan_lanes(sw_plan* p, const HostBatch& hb, int32_t nq, int64_t p
     }
     const double t_all = total / sched, share = share_of(warps);
     // the time of an item of each shape on each piece
-    times.resize((size_t)nq * cuts * MAX_SEGS);
+    times.resize((size_t)nq * cuts * MAX_SHAPES);
     for (int32_t i = 0; i < nq; i++)
       for (int k = 0; k < cuts; k++)
         for (int c = 0; c < qs[i].nc; c++)
-          times[((size_t)i * cuts + k) * MAX_SEGS + c] = qs[i].c[c].item(len[k], share);
+          times[((size_t)i * cuts + k) * MAX_SHAPES + c] = qs[i].c[c].item(len[k], share);
     for (double tail : {1e9, 1.2, 0.8, 0.5, 0.35}) {
       if (large && tail != 0.5) continue;
       pieces.clear();
@@ -1132,7 +1145,7 @@ static int64_t plan_lanes(sw_plan* p, const HostBatch& hb, int32_t nq, int64_t p
         int last = -1;
         size_t first = pieces.size();
         for (int k = 0; k < cuts; k++) {
-          const double* t = &times[((size_t)i * cuts + k) * MAX_SEGS];
+          const double* t = &times[((size_t)i * cuts + k) * MAX_SHAPES];
           int c = 0;
           while (c < qs[i].nc && t[c] > tail * t_all) c++;
           if (c == qs[i].nc) c = (int)(std::min_element(t, t + qs[i].nc) - t);
@@ -1141,7 +1154,7 @@ static int64_t plan_lanes(sw_plan* p, const HostBatch& hb, int32_t nq, int64_t p
           if (c == last) {
             pieces.back().s.pair1 = (int32_t)cut[k + 1];
           } else {
-            const LaneSeg sg{0, hb.order[i], x.lg, x.pr, x.passes, x.full, x.chain, x.halves,
+            const LaneSeg sg{0, hb.order[i], x.lg, x.pr, x.passes, x.tail, x.full, x.chain, x.halves,
                              (int32_t)cut[k], (int32_t)cut[k + 1]};
             pieces.push_back({x, sg, len[k]});
           }

@@ -411,7 +411,9 @@ __device__ __forceinline__ void lane_chain(const DbView& db, const SearchParams*
       for (const int start = p / LANE_WARPS * period + p % LANE_WARPS * lag; g < start; g++)
         chain_barrier();
       const bool last = p == sg.passes - 1;
-      const int pr = last ? sg.pr : sg.full, row0 = p * 32 * sg.full, slice = NCODES * 32 * sg.full;
+      const int heads = sg.passes - sg.tail, slice = NCODES * 32 * sg.full;
+      const int pr = p < heads ? sg.full : sg.pr;
+      const int row0 = 32 * (p < heads ? p * sg.full : heads * sg.full + (p - heads) * sg.pr);
       switch (pr) {  // uniform over the warp
         case 4: chain_pass<4, 1, G>(P, smem, sm, qr, m, row0, slice, at, hb_in, p == 0, last, smax); break;
         case 8: chain_pass<8, 2, G>(P, smem, sm, qr, m, row0, slice, at, hb_in, p == 0, last, smax); break;

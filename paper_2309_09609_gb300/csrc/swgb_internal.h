@@ -53,12 +53,13 @@ struct DbView {
 // One segment: a query against the subject pairs [pair0, pair1) of the length
 // order, on groups of lg lanes with pr rows each.  A query of several passes
 // has lg = 32, `full` rows per lane (32, less only in a chain) in every pass
-// but the last, and pr in that.  chain: the passes of a pair run on the warps
-// of a block, one behind the other, instead of one after the other on a warp.
+// but the last `tail` (1, more only in a chain), and pr in those.  chain: the
+// passes of a pair run on the warps of a block, one behind the other, instead
+// of one after the other on a warp.
 // halves: each lane's rows in two halves, one column apart (a query of one pass).
 struct LaneSeg {
   long long first;  // its first block item
-  int32_t q, lg, pr, passes, full, chain, halves;
+  int32_t q, lg, pr, passes, tail, full, chain, halves;
   int32_t pair0, pair1;
 };
 

@@ -14,9 +14,12 @@ W, STAGE = 4, 32
 
 @pytest.mark.parametrize("passes", [2, 3, 4, 5, 8, 9, 26])
 @pytest.mark.parametrize("n", [1, 30, 33, 64, 97, 200, 417, 449, 513, 2000])
-@pytest.mark.parametrize("full,last", [(4, 4), (8, 4), (8, 8), (16, 4), (16, 16)])
-def test_borders_are_written_before_and_read_before_overwritten(passes, n, full, last):
-    rows = [full] * (passes - 1) + [last]
+@pytest.mark.parametrize("full,last,tail", [(4, 4, 1), (8, 4, 1), (8, 8, 1), (16, 4, 1), (16, 16, 1),
+                                            (8, 4, 3), (16, 8, 4), (16, 4, 2)])
+def test_borders_are_written_before_and_read_before_overwritten(passes, n, full, last, tail):
+    rows = [full] * (passes - tail) + [last] * tail
+    if len(rows) > passes:
+        return
     lag = 3 if full == 4 else 4
 
     def stages(pr):

@@ -51,3 +51,12 @@ def test_saturated_pairs_in_one_and_in_several_passes():
     p = swgb.Database.from_seqset(db).plan(len(q), q.total, two_query=0, two_query_long=0)
     assert (p.search(q.res, q.lens, 10, 2, m) == want).all()
     assert p.stats()["recomputed_pairs"] >= 2
+
+
+@pytest.mark.parametrize("m", [1153, 1500, 1537, 2200, 2305, 2948, 3073, 4200])
+def test_chains_that_end_in_passes_of_fewer_rows(m):
+    rng = np.random.default_rng(m)
+    db = seqset(rng, [3000, 1, 33, 64, 257, 900, 2999, 0, 31, 1500, 2048, 7, 1100], alpha=24)
+    q = seqset(rng, [m], alpha=24)
+    got = swgb.Database.from_seqset(db).plan(1, m).search(q.res, q.lens, 10, 2)
+    assert (got == oracle_all(q, db, 10, 2)).all()
