@@ -952,9 +952,11 @@ static int32_t deal_streams(const HostBatch& hb, int32_t nq, int T, int32_t fixe
 // The short subjects' two-query layout (inter2q_kernel.cu): items are
 // (stream pair, half of a 64-subject group), the workers its warps.  Returns
 // the number of stream pairs, and in *cycles what the layout is expected to
-// take, in SM cycles: kQ2WordCycles per word row and scheduler, or, when one
-// item outlasts that, the longest item, whose warp shares its scheduler with
-// one other.
+// take, in SM cycles: the larger of kQ2WordCycles per word row and scheduler
+// and the longest item, whose warp shares its scheduler with one other, and a
+// part of the smaller for the search's end (the larger alone took this kernel
+// for 3 queries of 400 x 222,000: 27.3 ms, the lane groups 20.1; 5 of 400 x
+// 71,000: 11.4 and 9.1).
 static constexpr double kQ2WordCycles = 9.4, kQ2ItemCycles = 19;
 static int32_t plan_streams(sw_plan* p, const HostBatch& hb, int32_t nq, int32_t g_first,
                             int64_t* n_strips, double* cycles) {
@@ -969,8 +971,9 @@ static int32_t plan_streams(sw_plan* p, const HostBatch& hb, int32_t nq, int32_t
                                  (int64_t)p->strips.size(), n_strips);
   int64_t longest = 0;
   for (int32_t k = 0; k < K; k++) longest = std::max<int64_t>(longest, p->spairs[(size_t)k].y);
-  *cycles = std::max(kQ2WordCycles * (double)(*n_strips * T) * 2 * glen_sum / (4.0 * p->sms),
-                     kQ2ItemCycles * (double)(longest * T) * glen_max);
+  const double all = kQ2WordCycles * (double)(*n_strips * T) * 2 * glen_sum / (4.0 * p->sms);
+  const double item = kQ2ItemCycles * (double)(longest * T) * glen_max;
+  *cycles = std::max(all, item) + 0.2 * std::min(all, item);  // as for the lane groups
   return K;
 }
 
