@@ -1054,7 +1054,7 @@ static int lane_candidates(int32_t m, bool wide, LaneCand* c) {
   for (int lg = 8; lg <= 32; lg *= 2) {
     const int passes = lg == 32 ? std::max(1, (m + 1023) / 1024) : 1;
     const int rows = (m - (passes - 1) * 1024 + lg - 1) / lg;  // per lane, last pass
-    if (rows <= 32) c[n++] = LaneCand{lg, fit(rows, 4), passes, 32, 0, 0};
+    if (rows <= 32) c[n++] = LaneCand{lg, std::max(4, fit(rows, passes > 1 ? 4 : 2)), passes, 32, 0, 0};
   }
   if (m <= 24 * 32) c[n++] = LaneCand{32, fit((m + 31) / 32, 8), 1, 32, 0, 1};
   for (int full : {4, 8, 16}) {
@@ -1087,7 +1087,7 @@ static int lane_candidates(int32_t m, bool wide, LaneCand* c) {
 // well (4 queries of 10,000-37,000 residues x 500 subjects of up to 35,000,
 // where passes one after the other looked short beside the few warps that they
 // are: 201 -> 140 ms), and the pieces of a few queries as segments of their own
-// (7 queries of 400 x 40,000, whose shorter subjects no longer start before
+// (7 queries of 140-600 x 40,000, whose shorter subjects no longer start before
 // another query's long ones: 7.2 -> 6.75 ms).
 static int64_t plan_lanes(sw_plan* p, const HostBatch& hb, int32_t nq, int64_t pair0, int64_t pair1,
                           int32_t* n_segs, double* cycles, bool* wide) {

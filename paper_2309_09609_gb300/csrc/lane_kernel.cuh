@@ -19,9 +19,9 @@
 // pair, and two shuffles, two residue loads and the profile loads per step of
 // PR words.  Measured on one GB300 (wall time of the search):
 //   1 query of 144 x 2,000 subjects      1.27 -> 0.12 ms
-//   1 query of 375 x 20,000              6.04 -> 0.49 ms
+//   1 query of 375 x 20,000              6.04 -> 0.46 ms
 //   1 query of 375 x 570,000             15.4 -> 10.9 ms
-//   7 queries of 400 x 40,000            15.0 ->  7.2 ms
+//   7 queries of 140-600 x 40,000        15.0 ->  6.5 ms
 // (before: a warp per 64 subjects, and a warp per subject pair above 1,500
 // residues.)
 //
@@ -38,6 +38,12 @@
 // The kernel is bound by the ALU pipe: 4.5 operations per word (packed_cell
 // and the merge of the two subjects' profile bytes).
 //
+// Rows per lane come in steps of 2 where a group holds the whole query, of 4 in
+// passes: 3 queries of 66 residues x 549,000 subjects 11.8 ms with steps of 4
+// throughout, 10.1 so (80 rows swept instead of 96); 7 queries of 140-600 x
+// 40,000 6.75 and 6.5.  Passes in steps of 2 as well measured 1 to 3% less for
+// those and 3% more for the rest, by the size of the kernel.
+//
 // Columns left and right of a subject hold the padding code, whose score of
 // -64 leaves H = E = 0 before the first column and raises no S after the last,
 // so no step tests its column.  The lanes of a warp walk in step; the items of
@@ -49,8 +55,9 @@
 namespace swgb {
 
 // Dynamic shared memory: one residue ring per warp, then the block's query
-// profile (lane_profile.cuh; for chained passes, one per warp).  Ring: per group two blocks of 8 * LG columns, as the byte
-// offsets (code x 32 * PR) of the two subjects' profile rows, 16 bits each;
+// profile (lane_profile.cuh; for chained passes, one per warp).  Ring: per
+// group two blocks of 8 * LG columns, as the byte
+// offsets (code x 32 * PW) of the two subjects' profile rows, 16 bits each;
 // the first 8 columns are repeated after the last, so 8 steps need one wrap.
 constexpr int LANE_PROFILE = NCODES * 32 * LANE_ROWS_MAX;
 constexpr int LANE_RING = 4 * (2 * 256 + 32);  // bytes per warp: 2 * 8 * 32 columns and the repeats
@@ -74,14 +81,14 @@ struct LaneEdge {
 // Profile words of one column of a quarter: four rows to a word, per subject.
 template <int PR, int NQ>
 struct LaneWords {
-  static constexpr int R = LaneShape<PR, NQ>::R, VB = LaneShape<PR, NQ>::VB;
-  uint32_t a[R / 4], b[R / 4];
+  static constexpr int RW = LaneShape<PR, NQ>::RW, VB = LaneShape<PR, NQ>::VB;
+  uint32_t a[RW], b[RW];
 
   // pa, pb: the lane's profile rows of the two codes; q: the quarter
   __device__ __forceinline__ void load(const uint8_t* pa, const uint8_t* pb, int q) {
 #pragma unroll
-    for (int v = 0; v < R / VB; v++) {
-      const int o = (q * (R / VB) + v) * 32 * VB;
+    for (int v = 0; v < 4 * RW / VB; v++) {
+      const int o = (q * (4 * RW / VB) + v) * 32 * VB;
       if constexpr (VB == 16) {
         const uint4 x = *(const uint4*)(pa + o), y = *(const uint4*)(pb + o);
         a[4 * v] = x.x, a[4 * v + 1] = x.y, a[4 * v + 2] = x.z, a[4 * v + 3] = x.w;
@@ -158,7 +165,7 @@ __device__ __forceinline__ void lane_sweep(const uint8_t* prof, uint8_t* ring, i
   constexpr bool PASSES = MODE != ALONE;
   constexpr int U = LaneShape<PR, NQ>::UNROLL;
   constexpr bool AHEAD = LaneShape<PR, NQ>::AHEAD;
-  constexpr uint32_t CODE = 32 * PR;  // bytes between the profile rows of two codes
+  constexpr uint32_t CODE = 32 * LaneShape<PR, NQ>::PW;  // bytes between the profile rows of two codes
   const int li = lane & (lg - 1);
   const int cols = 8 * lg;  // columns per ring block
   // this group's ring: 2 * cols columns and the repeats, 4 bytes each; the
@@ -350,7 +357,7 @@ __device__ __forceinline__ void lane_pass(const SearchParams* __restrict__ P, ui
   if (passes == 1)
     lane_sweep<PR, NQ, ALONE>(prof, ring, lane, at.lg, at.n, at.src, at.chunks, nullptr, nullptr,
                               nullptr, true, true, smax, GO2, NGE2);
-  else if constexpr (NQ == 1)
+  else if constexpr (NQ == 1 && PR % 4 == 0)  // as the planner cuts a query of several passes
     lane_sweep<PR, 1, SERIAL>(prof, ring, lane, 32, at.n, at.src, at.chunks, at.edge, at.hb,
                               at.hb, pass == 0, pass == passes - 1, smax, GO2, NGE2);
 }
@@ -463,12 +470,19 @@ __device__ __forceinline__ void lane_item(const DbView& db, const SearchParams* 
     const bool build = sg.passes > 1 || cached != seg;
     switch (sg.halves ? -pr : pr) {  // uniform over the block
       case 4: lane_pass<4, 1, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
+      case 6: lane_pass<6, 1, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
       case 8: lane_pass<8, 1, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
+      case 10: lane_pass<10, 1, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
       case 12: lane_pass<12, 1, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
+      case 14: lane_pass<14, 1, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
       case 16: lane_pass<16, 1, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
+      case 18: lane_pass<18, 1, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
       case 20: lane_pass<20, 1, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
+      case 22: lane_pass<22, 1, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
       case 24: lane_pass<24, 1, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
+      case 26: lane_pass<26, 1, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
       case 28: lane_pass<28, 1, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
+      case 30: lane_pass<30, 1, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
       case -8: lane_pass<8, 2, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
       case -16: lane_pass<16, 2, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;
       case -24: lane_pass<24, 2, G>(P, smem, sm, qr, m, row0, build, at, p, sg.passes, smax); break;

@@ -1,9 +1,10 @@
 // lane_profile.cuh -- the int8 query profile of kernels whose lanes own
 // consecutive query rows (lane_kernel.cuh, noalloc.cu).
 //
-// Profile of 32 lanes with PR rows each, code-major:
+// Profile of 32 lanes with PR rows each (PW bytes: PR in whole words),
+// code-major:
 //   rows [VB * v, VB * v + VB) of lane l against code c at
-//   c * 32 * PR + v * 32 * VB + l * VB,   VB = bytes per load,
+//   c * 32 * PW + v * 32 * VB + l * VB,   VB = bytes per load,
 // so the lanes of a quarter- or half-warp read distinct banks whatever codes
 // they read.
 #pragma once
@@ -29,8 +30,10 @@ __device__ __forceinline__ uint4 transpose4(uint32_t a, uint32_t b, uint32_t c, 
 template <int PR, int NQ>
 struct LaneShape {
   static constexpr int R = PR / NQ;  // rows per quarter
-  static_assert(R % 4 == 0 && PR <= LANE_ROWS_MAX, "whole 4-row words, at most 32 rows");
-  static constexpr int VB = R % 16 == 0 ? 16 : R % 8 == 0 ? 8 : 4;  // bytes per profile load
+  static constexpr int RW = (R + 3) / 4;  // their profile words
+  static constexpr int PW = 4 * RW * NQ;  // profile bytes per lane and code
+  static_assert(R % (NQ == 1 ? 2 : 4) == 0 && PW <= LANE_ROWS_MAX, "pairs of rows, at most 32");
+  static constexpr int VB = RW % 4 == 0 ? 16 : RW % 2 == 0 ? 8 : 4;  // bytes per profile load
   static constexpr int UNROLL = 4;                                  // steps per loop body
   static constexpr bool AHEAD = PR <= 24;  // registers allow the next step's profile words
 };
@@ -43,9 +46,11 @@ template <int PR, int NQ>
 __device__ __forceinline__ void lane_profile_rows(uint8_t* prof, const uint8_t* sm,
                                                   const uint8_t* __restrict__ qr, int m, int row0,
                                                   int lg, int first, int warps) {
-  constexpr int VB = LaneShape<PR, NQ>::VB;
+  constexpr int VB = LaneShape<PR, NQ>::VB, PW = LaneShape<PR, NQ>::PW;
   const int l = threadIdx.x & 31;
-  for (int rq = first; rq < PR / 4; rq += warps) {
+  // (of PR = 4 k + 2 rows, the last word's upper half is the next lane's rows
+  // and is not used)
+  for (int rq = first; rq < PW / 4; rq += warps) {
     const int r0 = row0 + (l & (lg - 1)) * PR + 4 * rq;
     const uint8_t* s[4];
 #pragma unroll
@@ -58,7 +63,7 @@ __device__ __forceinline__ void lane_profile_rows(uint8_t* prof, const uint8_t* 
       const uint32_t v[4] = {w.x, w.y, w.z, w.w};
 #pragma unroll
       for (int b = 0; b < 4; b++)
-        if (4 * cq + b < NCODES) *(uint32_t*)(dst + (4 * cq + b) * 32 * PR) = v[b];
+        if (4 * cq + b < NCODES) *(uint32_t*)(dst + (4 * cq + b) * 32 * PW) = v[b];
     }
   }
 }

@@ -60,3 +60,13 @@ def test_chains_that_end_in_passes_of_fewer_rows(m):
     q = seqset(rng, [m], alpha=24)
     got = swgb.Database.from_seqset(db).plan(1, m).search(q.res, q.lens, 10, 2)
     assert (got == oracle_all(q, db, 10, 2)).all()
+
+
+def test_query_lengths_at_the_edges_of_odd_pairs_of_rows():
+    rng = np.random.default_rng(8)
+    db = seqset(rng, list(rng.integers(0, 500, size=301)), alpha=24)
+    q = seqset(rng, [47, 48, 49, 79, 80, 81, 111, 112, 113, 144, 176, 208, 239, 240, 241, 288, 289,
+                     352, 416, 417, 480, 481, 576, 704, 705, 832, 960, 961], alpha=24)
+    d = swgb.Database.from_seqset(db)
+    got = d.plan(len(q), q.total, two_query=0, two_query_long=0).search(q.res, q.lens, 10, 2)
+    assert (got == oracle_all(q, db, 10, 2)).all()
