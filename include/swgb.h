@@ -170,7 +170,7 @@ typedef struct {
  * max_query_residues residues in total, on the database's device.  The
  * device memory a search needs is allocated here, once: the query buffers,
  * the per-warp border scratch of each kernel (a fixed amount for the device
- * and database, about 2.2 GB on a GB300 for a database whose longest subject
+ * and database, about 1.9 GB on a GB300 for a database whose longest subject
  * has 35,000 residues, independent of the queries), the saturated-pair list
  * (opt.flag_capacity entries of 8 bytes, 8 MiB by default) and the work
  * counters.  One more buffer, max_queries x subjects int32, is allocated by
@@ -279,7 +279,7 @@ typedef struct {
  * most 1 GiB and no score can exceed 32767, else 4 bits per cell) and the
  * call's other buffers is allocated by the call; the database keeps up to
  * 512 MiB of it (and 16 MiB of pinned memory) for later calls and frees it with
- * sw_db_destroy.  Pairs are processed in chunks of at most 8 GiB of bits.
+ * sw_db_destroy.  Pairs are processed in chunks of at most 8 GiB of cells.
  * Synchronous on the stream.
  * Errors: SW_EINVAL (index out of range, short ops buffer, bad gaps or
  * codes), SW_ENOMEM, SW_ECUDA. */
@@ -308,7 +308,7 @@ sw_status sw_align(sw_db* db, const uint8_t* queries, const int32_t* q_lengths, 
  * Every device buffer must belong to the current device (or be managed
  * memory); the call checks this before any launch.
  * Same gap convention and the same scores as sw_search.  The kernel's
- * scratch (one border row per warp, a work counter, a status word) is a
+ * scratch (512 border rows, a work counter, a status word) is a
  * file-scope device array of ~16 MiB that every GPU loading the library holds
  * until the process exits; the counter and status are cleared at the start of
  * every call.  The first call on a device looks the array's address up on
@@ -354,8 +354,8 @@ sw_status sw_query_streams(const int32_t* q_lengths, int32_t n_queries, int32_t 
  * measured instead of looked up).  op selects an instruction kind (0 iadd,
  * 1 imax, 2 viaddmax_s32, 3 viaddmax_s16x2, 4 viaddmax_s16x2_relu,
  * 5 vimax3_s16x2, 6 vmaxs2, 7 vsub2, 8 vaddss2, 9 prmt, 10 packed cell pair,
- * 11 packed cell pair + prmt, 12 int32 cell, 13 imad, 14 the biased packed
- * cell pair of the search kernel, 15 vadd4, 16 vmaxu4, 17 vmaxs4, 18 vaddus4,
+ * 11 packed cell pair + prmt, 12 int32 cell, 13 imad, 14 a packed cell
+ * pair biased by Go, 15 vadd4, 16 vmaxu4, 17 vmaxs4, 18 vaddus4,
  * 19 vsubus4, 20 an unsigned biased 8x4 cell update of four cells, 10 ops);
  * results (host memory):
  * out[0] lane-operations per SM clock, out[1] SM clock in MHz, out[2] seconds. */

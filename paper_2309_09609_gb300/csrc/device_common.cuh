@@ -16,8 +16,9 @@
 // names instruction reordering and narrower integers; the packed kernels do
 // both).
 //
-// Threads wait on one another only at __syncwarp / __syncthreads; the only
-// interaction between blocks is an atomic work counter, so nothing can spin.
+// Threads wait on one another only at __syncwarp and at barriers of a block or
+// of a cluster; the only other interaction between blocks is an atomic work
+// counter, so nothing can spin.
 #pragma once
 
 #include <stdint.h>

@@ -6,7 +6,7 @@
 // must not allocate once it is serving (so memory use stays fixed and no call
 // can fail with out-of-memory), or code that is not permitted to call
 // cudaMalloc at all.  This entry point takes the caller's device buffers for
-// inputs and outputs and keeps its scratch -- one (H, F) border row per warp,
+// inputs and outputs and keeps its scratch -- (H, F) border rows for 512 blocks,
 // a work counter and a status word -- in the file-scope array below, whose
 // size is fixed at build time.  Every GPU that loads the library holds that
 // array until the process exits.

@@ -7,8 +7,9 @@ The options (all of which change speed only, never a score):
   height compiled with the gap penalties as constants (on the batched
   workload a tuner that tried 24 rows on its 8-query sample picked them, and
   the full batch then ran 7% slower);
-* the one-query inter-task kernel's rows per thread (32, 16), columns per
-  wavefront with 32 rows (8, 4) and warps per block (8, 4);
+* rows per thread (32, 16), columns per wavefront with 32 rows (8, 4) and
+  warps per block (8, 4), which the library accepts and checks; its kernels
+  take their shapes from the plan's cost model, so these now time alike;
 * the inter/intra length cutoff (1500, 3000, 7000, none) and the rows per
   lane of the int32 intra-task kernel (8, 16).
 
@@ -26,8 +27,8 @@ database signature, the sample's query length profile and the gap penalties.
 One shape serves the whole batch: the search is one persistent launch per
 kernel over every (query, subject-group) item, so its kernels run one
 configuration.  What does differ per length bucket is decided per item by
-the plan itself: which subjects go to the pair kernels (the cutoff), which
-pair-kernel width a query takes, and how queries are dealt to query
+the plan itself: which subjects go to the long-subject kernel (the cutoff),
+which lane-group shapes a query takes, and how queries are dealt to query
 streams.
 """
 from __future__ import annotations
