@@ -53,3 +53,15 @@ def test_scores_below_and_above_16_bits(top):
         got = swgb.Database.from_seqset(ss).align(ss.res, ss.lens, a, b, *gaps, m)
         want = [oracle.align(seqs[q], seqs[s], *gaps, m.astype(np.int32)) for q, s in zip(pq, ps)]
         assert got == want * repeat
+
+
+@pytest.mark.parametrize("n", [64_999, 65_000, 65_001, 66_000])
+def test_subjects_around_the_longest_whose_steps_fit_16_bits(n):
+    nvbuild.build()
+    rng = np.random.default_rng(n)
+    q = seqset(rng, [90])
+    s = seqset(rng, [n]).seq(0).copy()
+    s[n - 70:n - 10] = q.seq(0)[20:80]   # the best alignment ends near the last column
+    ss = synth.SeqSet(s, np.array([n], np.int32))
+    got = swgb.Database.from_seqset(ss).align(q.res, q.lens, [0], [0], 10, 2)
+    assert got[0] == oracle.align(q.seq(0), s, 10, 2)
