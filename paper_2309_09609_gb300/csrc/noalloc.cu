@@ -28,9 +28,10 @@
 // score, picked from the four in a profile word, to the diagonal (a PRMT and an
 // add took the ALU pipe twice; in a loop of independent cells 7.9 cycles per
 // warp and scheduler, against 9.1 for the earlier update).  16 queries of 400 x
-// 2,000 subjects: 12.5 -> 2.3 ms, 2.8 without the chains (before: 512 warps on the
+// 2,000 subjects: 12.5 -> 2.2 ms, 2.8 without the chains (before: 512 warps on the
 // whole chip, 256-row passes through the border rows, codes loaded at the step
-// that used them).
+// that used them).  Rows per lane come in steps of 2: 2.05 -> 1.96 ms and 2.23 ->
+// 2.13 against steps of 4.
 #include <mutex>
 
 #include "lane_profile.cuh"
@@ -99,7 +100,7 @@ __device__ __forceinline__ void na_sweep(const uint8_t* prof, uint16_t* ring, in
                                          const uint8_t* __restrict__ d, const NaEdges& ed, int& S,
                                          int& bad, int go, int ge) {
   using Shape = LaneShape<PR, 1>;
-  constexpr int VB = Shape::VB, U = Shape::UNROLL;
+  constexpr int VB = Shape::VB, U = Shape::UNROLL, PW = Shape::PW;
   const uint8_t* pl = prof + lane * VB;
   const int not0 = lane == 0 ? 0 : 1;
   int H[PR], E[PR];
@@ -132,8 +133,8 @@ __device__ __forceinline__ void na_sweep(const uint8_t* prof, uint16_t* ring, in
 #pragma unroll
     for (int i = 0; i < 4; i++) {
       const uint32_t x = i < 2 ? v.x : v.y;
-      w[i] = ((x >> (16 * (i & 1))) & 0xffu) * (32 * PR) +
-             (((x >> (16 * (i & 1) + 8)) & 0xffu) * (32 * PR) << 16);
+      w[i] = ((x >> (16 * (i & 1))) & 0xffu) * (32 * PW) +
+             (((x >> (16 * (i & 1) + 8)) & 0xffu) * (32 * PW) << 16);
     }
     const uint4 o = make_uint4(w[0], w[1], w[2], w[3]);
     *(uint4*)(ring + slot * NA_COLS + 8 * lane) = o;
@@ -174,9 +175,9 @@ __device__ __forceinline__ void na_sweep(const uint8_t* prof, uint16_t* ring, in
           }
         }
         const uint8_t* pp = pl + rp[u];
-        uint32_t w[PR / 4];
+        uint32_t w[PW / 4];
 #pragma unroll
-        for (int v = 0; v < PR / VB; v++) {
+        for (int v = 0; v < PW / VB; v++) {
           if constexpr (VB == 16) {
             const uint4 x = *(const uint4*)(pp + v * 32 * VB);
             w[4 * v] = x.x, w[4 * v + 1] = x.y, w[4 * v + 2] = x.z, w[4 * v + 3] = x.w;
@@ -223,12 +224,19 @@ __device__ __forceinline__ void na_alone(int pr, const uint8_t* prof, uint16_t* 
   const NaEdges none{nullptr, nullptr, 0, 0, true, true};
   switch (pr) {  // uniform over the block
     case 4: na_sweep<4, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
+    case 6: na_sweep<6, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
     case 8: na_sweep<8, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
+    case 10: na_sweep<10, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
     case 12: na_sweep<12, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
+    case 14: na_sweep<14, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
     case 16: na_sweep<16, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
+    case 18: na_sweep<18, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
     case 20: na_sweep<20, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
+    case 22: na_sweep<22, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
     case 24: na_sweep<24, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
+    case 26: na_sweep<26, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
     case 28: na_sweep<28, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
+    case 30: na_sweep<30, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
     default: na_sweep<32, false>(prof, ring, lane, n, d, none, S, bad, go, ge); break;
   }
 }
@@ -238,12 +246,19 @@ __device__ __forceinline__ void na_profile(int pr, uint8_t* prof, const uint8_t*
                                            const uint8_t* qr, int m, int wib) {
   switch (pr) {
     case 4: lane_profile_rows<4, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
+    case 6: lane_profile_rows<6, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
     case 8: lane_profile_rows<8, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
+    case 10: lane_profile_rows<10, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
     case 12: lane_profile_rows<12, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
+    case 14: lane_profile_rows<14, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
     case 16: lane_profile_rows<16, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
+    case 18: lane_profile_rows<18, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
     case 20: lane_profile_rows<20, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
+    case 22: lane_profile_rows<22, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
     case 24: lane_profile_rows<24, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
+    case 26: lane_profile_rows<26, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
     case 28: lane_profile_rows<28, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
+    case 30: lane_profile_rows<30, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
     default: lane_profile_rows<32, 1>(prof, sm, qr, m, 0, 32, wib, NA_WARPS); break;
   }
 }
@@ -344,7 +359,7 @@ noalloc_kernel(NaArgs a, NaMatrix mat, int2* scratch) {
       const bool q_ok = m >= 0 && (m == 0 || a.qres);
       if (round == 0 && (!q_ok || m <= NA_CHAIN_PASS)) continue;  // no chain with this query
       const uint8_t* qr = a.qres + (q_ok && m > 0 ? a.qoff[q] : 0);
-      const int pr = max(1, (min(m, NA_ALONE) + 127) / 128) * 4;  // of a query on one warp
+      const int pr = max(4, (min(m, NA_ALONE) + 63) / 64 * 2);  // of a query on one warp
       // a subject length that may be scored
       auto valid = [&](int n) { return q_ok && n >= 0 && n <= NA_MAX_LEN && (n == 0 || a.sres); };
       if (q_ok && m > 0 && checked != q) {

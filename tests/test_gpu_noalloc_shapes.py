@@ -32,3 +32,20 @@ def test_edges(gaps, subjects):
     want = oracle_all(q, db, *gaps)
     got = out.cpu().numpy()
     assert (got == want).all(), np.argwhere(got != want)[:5]
+
+
+def test_query_lengths_at_the_edges_of_odd_pairs_of_rows():
+    torch = pytest.importorskip("torch")
+    nvbuild.build()
+    rng = np.random.default_rng(11)
+    db = seqset(rng, [255, 300, 1, 33] + list(rng.integers(0, 500, size=60)), alpha=24)
+    q = seqset(rng, [191, 192, 193, 319, 320, 321, 448, 449, 576, 577, 704, 705, 832, 833, 960, 961],
+               alpha=24)
+
+    def dev(a):
+        return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+    out = torch.full((len(q), len(db)), -7, dtype=torch.int32, device="cuda")
+    swgb.search_pairs_noalloc(dev(q.res), dev(q.offs), dev(q.lens), dev(db.res), dev(db.offs),
+                              dev(db.lens), out, 10, 2)
+    assert (out.cpu().numpy() == oracle_all(q, db, 10, 2)).all()
