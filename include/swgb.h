@@ -120,8 +120,9 @@ typedef struct {
   int32_t two_query;         /* scoring of the short subjects with two queries per 32-bit word
                                 against one subject per lane (no per-cell byte merge, 3.5
                                 instead of 4.5 ALU operations per word): 0 never, 1 when the
-                                plan's cost model expects it to be faster than the lane groups
-                                (default), 2 whenever a search has at least two queries */
+                                plan's cost model expects it to be faster than two subjects
+                                per word (default), 2 whenever a search has at least two
+                                queries */
   int32_t two_query_rows;    /* query rows per strip of that kernel: 16, 24 or 32 (default) */
   int32_t two_query_pairs;   /* stream pairs of the two-query layouts, inter- and intra-task
                                 (0: the plan's choice, per layout; otherwise at most
@@ -160,7 +161,8 @@ typedef struct {
   int32_t pad_;
   int64_t inter_cells;       /* cells of the short subjects */
   int64_t inter2_items;      /* (stream pair, half group) items of the two-query inter-task
-                                kernel; 0 when the lane groups scored the short subjects */
+                                kernel; 0 when two subjects per word scored the short
+                                subjects */
   int64_t pair2_items;       /* (stream pair, group of 12 long subjects) items of the two-query
                                 intra-task kernel; 0 when the lane groups scored the long
                                 subjects */
@@ -190,8 +192,10 @@ void sw_plan_destroy(sw_plan* plan);
  * others against one subject per lane, over (pair of query streams, half of a
  * group of 64 subjects) items -- or with two subjects per word on groups of 8
  * to 32 lanes, over (query, subject pairs) items; both parts go in one launch
- * when both take the latter.  opt.two_query_long and opt.two_query with a cost
- * model choose per search; a single query always takes the lane groups.  Last
+ * when both take the latter.  The others may also go two subjects per lane over
+ * (query, group of 64 subjects) items, which is faster for subjects of a few
+ * tens of residues.  opt.two_query_long and opt.two_query with a cost model
+ * choose per search; a single query never takes two queries per word.  Last
  * the int32 intra-task kernel recomputes every pair whose 16-bit score may
  * have saturated (one block per pair; more saturated pairs than
  * opt.flag_capacity are recomputed in further rounds before the call returns);

@@ -224,6 +224,7 @@ struct sw_db {
   int device = 0;
   DbView view{};
   std::vector<int32_t> glen_h;   // padded group lengths (host copy)
+  std::vector<int64_t> gcol_h;   // [G + 1] padded columns of groups [0, g)
   std::vector<int32_t> clen_h;   // sorted lengths (host copy)
   std::vector<int64_t> cres_h;   // [N + 1] residues of sorted subjects [0, s)
   std::vector<int32_t> sorted_of_h;  // caller index -> sorted index
@@ -358,6 +359,8 @@ extern "C" sw_status sw_db_create(const uint8_t* residues, const int32_t* length
   db->view.n = N;
   db->view.groups = G;
   db->view.max_len = max_len;
+  db->gcol_h.assign((size_t)G + 1, 0);
+  for (int32_t g = 0; g < G; g++) db->gcol_h[g + 1] = db->gcol_h[g] + glen[g];
   db->glen_h = std::move(glen);
   db->cres_h.assign((size_t)N + 1, 0);
   for (int64_t s = 0; s < N; s++) db->cres_h[s + 1] = db->cres_h[s] + clen[s];
@@ -470,11 +473,11 @@ static constexpr size_t BLOCK_HEADER = block_align(sizeof(SearchParams)) + block
 
 // The kernels of one search (bits of sw_plan::kernels): the two-query kernel
 // or the lane groups for the long subjects, the lane groups (for the short
-// subjects, or for all in one launch) or the two-query kernel for the short
-// ones, and the int32 kernel.
+// subjects, or for all in one launch) or one of the inter-task kernels for the
+// short ones, and the int32 kernel.
 // K_WIDE: the lane groups are launched with room for chains of 16 rows.
-enum { K_PAIR2 = 1, K_LANES_LONG = 2, K_LANES = 4, K_INTER2 = 8, K_INT32 = 16, K_WIDE = 32,
-       K_SETS = 64 };
+enum { K_PAIR2 = 1, K_LANES_LONG = 2, K_LANES = 4, K_INTER2 = 8, K_INTER = 16, K_INT32 = 32,
+       K_WIDE = 64, K_SETS = 128 };
 
 struct sw_plan {
   sw_db* db = nullptr;
@@ -487,6 +490,7 @@ struct sw_plan {
   int32_t g_first = 0;      // first inter-task group under the cutoff
   int32_t sms = 1;
   int32_t pair2_blocks = 0;   // grid of pair2q_kernel
+  int32_t inter_blocks = 0;   // grid of inter_kernel
   int32_t lane_blocks[2] = {0, 0};  // grid of lane_kernel: as it is, and wide
   // One device block and its pinned image hold what a search uploads, in one
   // copy: the parameter block, the zeroed state, and the tables that follow
@@ -619,7 +623,15 @@ extern "C" sw_status sw_plan_create(sw_db* db, int32_t max_queries, int64_t max_
   p->kc2.warps = warps2;
   p->kc2.blocks = dev_sms * bps2;
   p->kc2.smem = inter2q_smem_bytes(o.two_query_rows, warps2);
-  const int64_t W = (int64_t)p->kc2.blocks * p->kc2.warps;
+  const int ibps = inter_blocks_per_sm();
+  if (ibps < 1) {
+    plan_free(p);
+    return sw_set_error(SW_ECUDA, "inter-task kernel cannot launch");
+  }
+  p->inter_blocks = dev_sms * ibps;
+  // border rows of the inter-task kernels, of which a search launches one
+  const int64_t W = std::max((int64_t)p->kc2.blocks * p->kc2.warps,
+                             (int64_t)p->inter_blocks * inter_warps());
   // one block of INTRA_WARPS per SM: enough for the int32 items, and the
   // border scratch (one subject-length row per warp) stays bounded
   if (intra_blocks_per_sm(o.intra_rows) < 1) {
@@ -729,7 +741,7 @@ static cudaError_t enqueue_kernels(sw_plan* p, cudaStream_t s, bool capturing) {
   // overlap_kernels issues the latter on a second stream: one of its blocks
   // needs a whole SM's shared memory, so it starts on an SM when the blocks
   // there run out of work, and no SM idles in their tails
-  const bool is_long = set & (K_PAIR2 | K_LANES_LONG), is_short = set & (K_LANES | K_INTER2);
+  const bool is_long = set & (K_PAIR2 | K_LANES_LONG), is_short = set & (K_LANES | K_INTER2 | K_INTER);
   const bool overlap = p->opt.overlap_kernels && is_long && is_short, wide = set & K_WIDE;
   cudaError_t e = record(p->ev[0], s, capturing);
   if (e == cudaSuccess && overlap) e = cudaEventRecord(p->fork, s);
@@ -747,6 +759,8 @@ static cudaError_t enqueue_kernels(sw_plan* p, cudaStream_t s, bool capturing) {
     e = launch_lanes(gc, wide, p->lane_grid, v, p->params, p->state, p->scr, s2);
   if (e == cudaSuccess && (set & K_INTER2))
     e = launch_inter2q(p->kc2, gc, v, p->params, p->state, p->scr, s2);
+  if (e == cudaSuccess && (set & K_INTER))
+    e = launch_inter(gc, p->inter_blocks, v, p->params, p->state, p->scr, s2);
   if (e == cudaSuccess) e = record(p->ev[2], s2, capturing);
   if (overlap) {
     if (e == cudaSuccess) e = cudaEventRecord(p->join, s2);
@@ -956,14 +970,15 @@ static int32_t deal_streams(const HostBatch& hb, int32_t nq, int T, int32_t fixe
 // and the longest item, whose warp shares its scheduler with one other, and a
 // part of the smaller for the search's end (the larger alone took this kernel
 // for 3 queries of 400 x 222,000: 27.3 ms, the lane groups 20.1; 5 of 400 x
-// 71,000: 11.4 and 9.1).
-static constexpr double kQ2WordCycles = 9.4, kQ2ItemCycles = 19;
+// 71,000: 11.4 and 9.1).  A strip costs kQ2StripCycles more, its profile and its
+// ends, whatever its columns: 20 queries of 375 x 570,000 subjects of 5-15 residues
+// take 12.2 ms, of which the words alone would be 6.8.
+static constexpr double kQ2WordCycles = 9.4, kQ2ItemCycles = 19, kQ2StripCycles = 3000;
 static int32_t plan_streams(sw_plan* p, const HostBatch& hb, int32_t nq, int32_t g_first,
                             int64_t* n_strips, double* cycles) {
   const int T = p->kc2.variant;
   const DbView& v = p->db->view;
-  double glen_sum = 0;
-  for (int32_t g = g_first; g < v.groups; g++) glen_sum += p->db->glen_h[g];
+  const double glen_sum = (double)(p->db->gcol_h[v.groups] - p->db->gcol_h[g_first]);
   const double glen_max = g_first < v.groups ? p->db->glen_h[g_first] : 0.0;
   const int32_t K = deal_streams(hb, nq, T, p->opt.two_query_pairs,
                                  (double)p->kc2.blocks * p->kc2.warps, 1, glen_max, 2 * glen_sum,
@@ -971,8 +986,10 @@ static int32_t plan_streams(sw_plan* p, const HostBatch& hb, int32_t nq, int32_t
                                  (int64_t)p->strips.size(), n_strips);
   int64_t longest = 0;
   for (int32_t k = 0; k < K; k++) longest = std::max<int64_t>(longest, p->spairs[(size_t)k].y);
-  const double all = kQ2WordCycles * (double)(*n_strips * T) * 2 * glen_sum / (4.0 * p->sms);
-  const double item = kQ2ItemCycles * (double)(longest * T) * glen_max;
+  const double all = (double)*n_strips * 2 *
+                     (kQ2WordCycles * T * glen_sum + kQ2StripCycles * (v.groups - g_first)) /
+                     (4.0 * p->sms);
+  const double item = (double)longest * (kQ2ItemCycles * T * glen_max + 2 * kQ2StripCycles);
   *cycles = std::max(all, item) + 0.2 * std::min(all, item);  // as for the lane groups
   return K;
 }
@@ -1007,6 +1024,24 @@ static int32_t plan_streams_long(sw_plan* p, const HostBatch& hb, int32_t nq, in
   }
   *cycles = std::max(total / p->sms, longest);
   return K;
+}
+
+// The short subjects on the two-subject inter-task kernel (inter_kernel.cu):
+// items are (query, group of 64), the workers its warps, two to a scheduler.
+// Returns what it is expected to take, in SM cycles, as plan_streams does.
+// Fitted to 1 to 20 queries of 144-5,478 residues x 100,000 to 570,000 subjects of
+// 5-15 to 250-350 residues: within 8% of the time measured above 0.4 ms.
+static constexpr double kIWordCycles = 10.5, kIStripCycles = 1000, kIItemCycles = 18;
+static double plan_groups(const sw_plan* p, const HostBatch& hb, int32_t nq, int32_t g_first) {
+  const sw_db* db = p->db;
+  const int32_t G = db->view.groups;
+  double strips = 0;
+  for (int32_t i = 0; i < nq; i++) strips += (hb.len[i] + 31) / 32;
+  const double longest = (double)((hb.len[hb.order[0]] + 31) / 32);
+  const double all = strips * (kIWordCycles * 32 * (double)(db->gcol_h[G] - db->gcol_h[g_first]) +
+                               kIStripCycles * (G - g_first)) / (4.0 * p->sms);
+  const double item = longest * (kIItemCycles * 32 * db->glen_h[g_first] + 2 * kIStripCycles);
+  return std::max(all, item) + 0.2 * std::min(all, item);
 }
 
 // The lane-group kernel's segments (lane_kernel.cu) for the subject pairs
@@ -1074,6 +1109,21 @@ static int lane_candidates(int32_t m, bool wide, LaneCand* c) {
     if (pr < full && tail > 1) c[n++] = LaneCand{32, pr, heads + tail, full, 1, 1, tail};
   }
   return n;
+}
+
+// What the lane groups take for these subject pairs at the least: the cheapest
+// shapes, with every scheduler busy to the end.
+static double lanes_floor(const sw_plan* p, const HostBatch& hb, int32_t nq, int64_t pair0,
+                          int64_t pair1) {
+  const sw_db* db = p->db;
+  const double cols =
+      0.5 * (double)(db->cres_h[std::min(db->view.n, 2 * pair1)] - db->cres_h[2 * pair0]);
+  double cycles = 0;
+  for (int32_t i = 0; i < nq; i++) {
+    const int32_t m = hb.len[i], lg = m <= 256 ? 8 : m <= 512 ? 16 : 32;
+    cycles += 11.1 / 32 * m * (cols + (double)(pair1 - pair0) * lg);
+  }
+  return cycles / (4.0 * p->sms);
 }
 
 // The segments for the subject pairs [pair0, pair1), without and with wide
@@ -1292,7 +1342,7 @@ static sw_status plan_enqueue(sw_plan* p, const HostBatch& hb, int32_t nq, int32
   P.g_first = gf;
   P.n_intra_items = packed ? 0 : n_long * nq;
   P.n_spairs = P.n_spairs2 = 0;
-  P.n_inter2_items = P.n_pair2_items = P.n_lane_items = 0;
+  P.n_inter_items = P.n_inter2_items = P.n_pair2_items = P.n_lane_items = 0;
   P.n_lane_segs = 0;
   int64_t n_strips = 0, n_strips2 = 0;
   int kernels = 0;
@@ -1301,16 +1351,27 @@ static sw_status plan_enqueue(sw_plan* p, const HostBatch& hb, int32_t nq, int32
     // Each part of the subjects -- the long ones, above the cutoff, and the
     // short ones -- goes to a two-query kernel or to the lane groups, whichever
     // is expected to finish it first (options two_query and two_query_long: 0
-    // never two queries, 2 always with two or more queries).
+    // never two queries, 2 always with two or more queries).  Short subjects go
+    // to the two-subject inter-task kernel where it is expected to beat both, the
+    // lane groups by a tenth: theirs may be one launch for all subjects, whose
+    // end is shorter than that of two.
     const int64_t npairs = (v.n + 1) / 2, long_pairs = std::min(npairs, (n_long + 1) / 2);
     const bool has_long = n_long > 0, has_short = gf < v.groups;
     int32_t n_segs = 0;
     double t2 = 0, tl = 0;
-    bool two = false, two_long = false, wide = false;
-    if (has_short && nq >= 2 && p->opt.two_query > 0) {
-      const int32_t K = plan_streams(p, hb, nq, gf, &n_strips, &t2);
-      if (K > 0 && p->opt.two_query == 1) plan_lanes(p, hb, nq, long_pairs, npairs, &n_segs, &tl, &wide);
-      two = K > 0 && (p->opt.two_query == 2 || t2 < tl);
+    bool two = false, two_long = false, wide = false, groups = false;
+    if (has_short) {
+      int32_t K = 0;
+      if (nq >= 2 && p->opt.two_query > 0) K = plan_streams(p, hb, nq, gf, &n_strips, &t2);
+      if (K > 0 && p->opt.two_query == 2) {
+        two = true;
+      } else {
+        const double t1 = plan_groups(p, hb, nq, gf);
+        groups = t1 < 0.95 * lanes_floor(p, hb, nq, long_pairs, npairs);
+        if (K > 0 || groups) plan_lanes(p, hb, nq, long_pairs, npairs, &n_segs, &tl, &wide);
+        two = K > 0 && t2 < tl && !(groups && t1 < t2);
+        groups = groups && !two && t1 < 0.9 * tl;
+      }
       if (two) {
         P.n_spairs = K;
         P.n_inter2_items = (int64_t)K * 2 * (v.groups - gf);
@@ -1331,7 +1392,7 @@ static sw_status plan_enqueue(sw_plan* p, const HostBatch& hb, int32_t nq, int32
         n_strips2 = 0;
       }
     }
-    const bool lanes_long = has_long && !two_long, lanes_short = has_short && !two;
+    const bool lanes_long = has_long && !two_long, lanes_short = has_short && !two && !groups;
     if (lanes_long || lanes_short) {
       P.n_lane_items = plan_lanes(p, hb, nq, lanes_long ? 0 : long_pairs,
                                   lanes_short ? npairs : long_pairs, &n_segs, &tl, &wide);
@@ -1342,6 +1403,10 @@ static sw_status plan_enqueue(sw_plan* p, const HostBatch& hb, int32_t nq, int32
         long_share = (double)p->db->cres_h[n_long] / (double)p->db->residues;
     }
     if (two) kernels |= K_INTER2;
+    if (groups) {
+      P.n_inter_items = (int64_t)(v.groups - gf) * nq;
+      kernels |= K_INTER;
+    }
     // no score above max_sm per aligned column: without one at the recompute
     // threshold the int32 kernel has nothing to do
     const int64_t longest = hb.len[hb.order[0]];
@@ -1392,7 +1457,7 @@ static sw_status plan_enqueue(sw_plan* p, const HostBatch& hb, int32_t nq, int32
 static void finish_stats(sw_plan* p) {
   p->stats = p->pending;
   const int set = p->kernels;
-  const bool is_long = set & (K_PAIR2 | K_LANES_LONG), is_short = set & (K_LANES | K_INTER2);
+  const bool is_long = set & (K_PAIR2 | K_LANES_LONG), is_short = set & (K_LANES | K_INTER2 | K_INTER);
   const bool both = is_long && is_short;
   // with overlap_kernels the kernels of both parts start at ev[0]
   const bool ov = p->opt.overlap_kernels != 0 && both;

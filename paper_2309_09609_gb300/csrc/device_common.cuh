@@ -1,5 +1,5 @@
 // device_common.cuh -- device helpers shared by the alignment kernels of
-// libswgb: lane_kernel.cu, inter2q_kernel.cu, pair2q_kernel.cu, intra_kernel.cu,
+// libswgb: lane_kernel.cu, inter_kernel.cu, inter2q_kernel.cu, pair2q_kernel.cu, intra_kernel.cu,
 // align_kernel.cu, plain_kernel.cu.
 //
 // Every kernel computes Eq. 1-3 of arxiv 2309.09609 (Section II-B) in the
@@ -71,6 +71,29 @@ __device__ __forceinline__ void emit_score(const DbView& db, const SearchParams*
                                            int q, int s, int score) {
   const int orig = db.perm[s];
   if (orig >= 0) P->scores[(int64_t)q * db.n + orig] = score;
+}
+
+// S of each subject of a pair (the halves of smax): recorded, or flagged for the
+// int32 recompute when it may have saturated.
+__device__ __forceinline__ void emit_pair(const DbView& db, const SearchParams* __restrict__ P,
+                                          SearchState* st, const Scratch& scr, int q, int pair,
+                                          uint32_t smax) {
+#pragma unroll
+  for (int half = 0; half < 2; half++) {
+    const int sidx = 2 * pair + half;
+    const int orig = db.perm[sidx];
+    if (orig < 0) continue;
+    const int s = (int)(int16_t)(half ? (smax >> 16) : (smax & 0xffffu));
+    if (s >= P->sat_threshold) {
+      const unsigned long long k = atomicAdd(&st->n_flags, 1ull);
+      if ((int64_t)k < scr.flag_capacity)
+        scr.flags[k] = make_int2(q, sidx);
+      else  // the list is full: mark the pair for the host's next recompute round
+        P->scores[(int64_t)q * db.n + orig] = FLAG_SENTINEL;
+    } else {
+      P->scores[(int64_t)q * db.n + orig] = s;
+    }
+  }
 }
 
 // SM into shared memory (every thread of the block takes part; the caller syncs)

@@ -305,29 +305,6 @@ __device__ __forceinline__ void lane_sweep(const uint8_t* prof, uint8_t* ring, i
   }
 }
 
-// S of each subject of the group's pair: recorded, or flagged for the int32
-// recompute when it may have saturated.
-__device__ __forceinline__ void lane_emit(const DbView& db, const SearchParams* __restrict__ P,
-                                          SearchState* st, const Scratch& scr, int q, int pair,
-                                          uint32_t smax) {
-#pragma unroll
-  for (int half = 0; half < 2; half++) {
-    const int sidx = 2 * pair + half;
-    const int orig = db.perm[sidx];
-    if (orig < 0) continue;
-    const int s = (int)(int16_t)(half ? (smax >> 16) : (smax & 0xffffu));
-    if (s >= P->sat_threshold) {
-      const unsigned long long k = atomicAdd(&st->n_flags, 1ull);
-      if ((int64_t)k < scr.flag_capacity)
-        scr.flags[k] = make_int2(q, sidx);
-      else  // the list is full: mark the pair for the host's next recompute round
-        P->scores[(int64_t)q * db.n + orig] = FLAG_SENTINEL;
-    } else {
-      P->scores[(int64_t)q * db.n + orig] = s;
-    }
-  }
-}
-
 // One warp's share of a block item: where its pairs lie.
 struct LanePlace {
   int lg, n;         // lanes per group; columns of the warp's longest subject
@@ -436,7 +413,7 @@ __device__ __forceinline__ void lane_chain(const DbView& db, const SearchParams*
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int w = 1; w < LANE_WARPS; w++) smax = __vmaxs2(smax, red[w]);
-    lane_emit(db, P, st, scr, sg.q, pair, smax);
+    emit_pair(db, P, st, scr, sg.q, pair, smax);
   }
 }
 
@@ -491,7 +468,7 @@ __device__ __forceinline__ void lane_item(const DbView& db, const SearchParams* 
   }
   cached = sg.passes > 1 ? -1 : seg;
   for (int o = sg.lg >> 1; o > 0; o >>= 1) smax = __vmaxs2(smax, __shfl_xor_sync(FULL, smax, o));
-  if (has && (lane & (sg.lg - 1)) == 0) lane_emit(db, P, st, scr, sg.q, pair, smax);
+  if (has && (lane & (sg.lg - 1)) == 0) emit_pair(db, P, st, scr, sg.q, pair, smax);
 }
 
 template <int G>

@@ -79,7 +79,8 @@ struct SearchParams {
   // first strip and strip count
   const int4* strips;
   const int2* spairs;
-  int64_t n_inter2_items; // stream pairs x 2 x inter groups (0: the lane groups score the short subjects)
+  int64_t n_inter2_items; // stream pairs x 2 x inter groups (0: it does not run)
+  int64_t n_inter_items;  // (query, inter group) items of inter_kernel.cu (0: it does not run)
   // two queries per word for the long subjects (pair2q_kernel.cu): a strip
   // table of 32-row strips and its stream pairs, in the same format
   const int4* strips2;
@@ -106,6 +107,7 @@ struct SearchState {
   unsigned long long recompute;   // next flagged pair (int32 intra-task kernel, per block)
   unsigned long long intra_work;  // next int32 intra-task item (per warp)
   unsigned long long work2;       // next work item (two-query inter-task kernel)
+  unsigned long long inter_work;  // next work item (two-subject inter-task kernel)
   unsigned long long lane_work;   // next block item (lane-group kernel)
   unsigned long long pair2_work;  // next work item (two-query intra-task kernel, per block)
   unsigned int status;            // reserved: error bits raised on the device
@@ -158,6 +160,13 @@ int inter2q_blocks_per_sm(int rows, int warps);  // resident blocks per SM, 0 if
 cudaError_t launch_inter2q(const KernelConfig& kc, int gclass, const DbView& db,
                            const SearchParams* params, SearchState* state, const Scratch& scr,
                            cudaStream_t stream);
+
+// Inter-task kernel with two subjects per word (inter_kernel.cu), for short
+// subjects.  Scratch: one inter_border row per warp.
+int inter_warps();  // warps per block
+int inter_blocks_per_sm();
+cudaError_t launch_inter(int gclass, int blocks, const DbView& db, const SearchParams* params,
+                         SearchState* state, const Scratch& scr, cudaStream_t stream);
 
 // Int32 intra-task kernel (intra_kernel.cu): int32 items one warp each, then
 // flagged pairs one block each.  Scratch: one border row per warp.
