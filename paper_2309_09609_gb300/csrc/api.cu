@@ -21,6 +21,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 #include <mutex>
 #include <numeric>
 #include <thread>
@@ -886,16 +887,22 @@ static int32_t deal_streams(const HostBatch& hb, int32_t nq, int T, int32_t fixe
   for (int32_t i = 0; i < nq; i++) strips_of[i] = std::max<int64_t>(1, (hb.len[i] + T - 1) / T);
   std::vector<std::vector<int32_t>> streams;
   std::vector<int64_t> load;
+  // the streams as a heap, the shortest (of equals the first) on top
+  std::vector<std::pair<int64_t, int32_t>> heap;
   auto deal = [&](int32_t K) {
-    streams.assign((size_t)2 * K, {});
+    streams.resize((size_t)2 * K);
+    for (auto& s : streams) s.clear();
     load.assign((size_t)2 * K, 0);
+    heap.resize((size_t)2 * K);
+    for (int32_t t = 0; t < 2 * K; t++) heap[(size_t)t] = {0, t};
     for (int32_t i = 0; i < nq; i++) {
       const int32_t q = hb.order[i];
-      size_t best = 0;
-      for (size_t t = 1; t < load.size(); t++)
-        if (load[t] < load[best]) best = t;
-      streams[best].push_back(q);
-      load[best] += strips_of[q];
+      std::pop_heap(heap.begin(), heap.end(), std::greater<>());
+      auto& top = heap.back();
+      streams[(size_t)top.second].push_back(q);
+      top.first += strips_of[q];
+      load[(size_t)top.second] = top.first;
+      std::push_heap(heap.begin(), heap.end(), std::greater<>());
     }
     for (int32_t k = 0; k < K; k++)
       balance_pair(streams[2 * k], streams[2 * k + 1], load[2 * k], load[2 * k + 1], strips_of);
@@ -1166,6 +1173,7 @@ static int64_t plan_lanes(sw_plan* p, const HostBatch& hb, int32_t nq, int64_t p
     return n * (x.chain ? std::min(x.passes, LANE_WARPS) : x.lg / 32.0);
   };
   struct Query {
+    int32_t m, n;  // its length, how many there are
     LaneCand c[MAX_SHAPES];
     int nc;
   };
@@ -1174,7 +1182,15 @@ static int64_t plan_lanes(sw_plan* p, const HostBatch& hb, int32_t nq, int64_t p
     LaneSeg s;
     double t;
   };
-  std::vector<Query> qs((size_t)nq);
+  // queries of one length, neighbours in the order, are planned once
+  std::vector<Query> qs;
+  std::vector<int32_t> kind((size_t)nq);
+  for (int32_t i = 0; i < nq; i++) {
+    const int32_t m = hb.len[hb.order[i]];
+    if (i == 0 || m != qs.back().m) qs.push_back(Query{m, 0});
+    qs.back().n++;
+    kind[(size_t)i] = (int32_t)qs.size() - 1;
+  }
   std::vector<double> times;
   std::vector<Piece> pieces, best_pieces;
   double best = 1e300, best_total = 0;
@@ -1183,14 +1199,13 @@ static int64_t plan_lanes(sw_plan* p, const HostBatch& hb, int32_t nq, int64_t p
     const double resident = (double)p->lane_blocks[w] * LANE_WARPS / sched;
     auto share_of = [&](double warps) { return std::min(resident, std::max(1.0, warps / sched)); };
     double total = 0, warps = 0;
-    for (int32_t i = 0; i < nq; i++) {
-      Query& q = qs[i];
-      q.nc = lane_candidates(hb.len[hb.order[i]], w != 0, q.c);
+    for (Query& q : qs) {
+      q.nc = lane_candidates(q.m, w != 0, q.c);
       std::sort(q.c, q.c + q.nc, [&](const LaneCand& a, const LaneCand& b) {
         return cost(a, all_cols, npairs) < cost(b, all_cols, npairs);
       });
-      total += cost(q.c[0], all_cols, npairs);
-      warps += warps_of(q.c[0], npairs);
+      total += q.n * cost(q.c[0], all_cols, npairs);
+      warps += q.n * warps_of(q.c[0], npairs);
     }
     const double t_all = total / sched;
     // an item's time is judged beside as many warps as the cheapest shapes
@@ -1199,26 +1214,28 @@ static int64_t plan_lanes(sw_plan* p, const HostBatch& hb, int32_t nq, int64_t p
     for (int f = 0; f < (!large && shares[0] < 0.9 * resident ? 2 : 1); f++) {
       const double share = shares[f];
       // the time of an item of each shape on each piece
-      times.resize((size_t)nq * cuts * MAX_SHAPES);
-      for (int32_t i = 0; i < nq; i++)
+      times.resize(qs.size() * cuts * MAX_SHAPES);
+      for (size_t i = 0; i < qs.size(); i++)
         for (int k = 0; k < cuts; k++)
           for (int c = 0; c < qs[i].nc; c++)
-            times[((size_t)i * cuts + k) * MAX_SHAPES + c] = qs[i].c[c].item(len[k], share);
+            times[(i * cuts + k) * MAX_SHAPES + c] = qs[i].c[c].item(len[k], share);
       for (double tail : {1e9, 1.2, 0.8, 0.5, 0.35}) {
         if (large && tail != 0.5) continue;
         pieces.clear();
         total = warps = 0;
         for (int32_t i = 0; i < nq; i++) {
+          const size_t qk = (size_t)kind[(size_t)i];
+          const Query& q = qs[qk];
           int last = -1;
           size_t first = pieces.size();
           for (int k = 0; k < cuts; k++) {
-            const double* t = &times[((size_t)i * cuts + k) * MAX_SHAPES];
+            const double* t = &times[(qk * cuts + k) * MAX_SHAPES];
             int c = 0;
-            while (c < qs[i].nc && t[c] > tail * t_all) c++;
-            if (c == qs[i].nc) c = (int)(std::min_element(t, t + qs[i].nc) - t);
+            while (c < q.nc && t[c] > tail * t_all) c++;
+            if (c == q.nc) c = (int)(std::min_element(t, t + q.nc) - t);
             const bool room = pieces.size() - first < (size_t)(large ? MAX_SEGS : MAX_SEGS_FEW);
             if (c != last && last >= 0 && !room) c = last;
-            const LaneCand& x = qs[i].c[c];
+            const LaneCand& x = q.c[c];
             // of a few queries, much shorter subjects are a segment of their own,
             // which may come after the longer items of other queries
             if (c == last && (large || !room || len[k] > 0.6 * pieces.back().t)) {
