@@ -22,7 +22,9 @@
 #include <cstdlib>
 #include <cstring>
 #include <functional>
+#include <memory>
 #include <mutex>
+#include <new>
 #include <numeric>
 #include <thread>
 #include <vector>
@@ -465,8 +467,35 @@ static sw_status fill_scoring(SearchParams& P, int32_t gap_open, int32_t gap_ext
 
 // ---- plan ---------------------------------------------------------------------------------
 // segments of the lane-group kernel per query: at most one per shape in a
-// large batch, more in a batch of few queries
-constexpr int MAX_SEGS = 8, MAX_SEGS_FEW = 24, FEW_QUERIES = 32;
+// large batch, more in a batch of few queries, and two in one of so many that
+// no item is long beside the search
+constexpr int MAX_SEGS = 8, MAX_SEGS_FEW = 24, MAX_SEGS_MANY = 2;
+constexpr int FEW_QUERIES = 32, MANY_QUERIES = 4096;
+static constexpr int max_segs(int32_t nq) {
+  return nq <= FEW_QUERIES ? MAX_SEGS_FEW : nq <= MANY_QUERIES ? MAX_SEGS : MAX_SEGS_MANY;
+}
+// the most segments of any batch of up to max_queries queries
+static constexpr size_t seg_capacity(int32_t max_queries) {
+  const size_t few = (size_t)MAX_SEGS_FEW * std::min(max_queries, FEW_QUERIES);
+  const size_t large = (size_t)MAX_SEGS * std::min(max_queries, MANY_QUERIES);
+  return std::max(std::max(few, large), (size_t)MAX_SEGS_MANY * max_queries);
+}
+
+// An array of a size known once, its elements not initialised: what is never
+// used of a plan of large capacity costs no page.
+template <typename T>
+struct Table {
+  std::unique_ptr<T[]> items;
+  size_t count = 0;
+  bool reserve(size_t n) {
+    items.reset(n <= (size_t)PTRDIFF_MAX / sizeof(T) ? new (std::nothrow) T[n] : nullptr);
+    count = items ? n : 0;
+    return items != nullptr;
+  }
+  size_t size() const { return count; }
+  T* data() const { return items.get(); }
+  T& operator[](size_t i) const { return items[i]; }
+};
 
 // The upload block: parameters, state, then the tables, each on a 16-byte boundary.
 static constexpr size_t block_align(size_t bytes) { return (bytes + 15) & ~(size_t)15; }
@@ -504,9 +533,9 @@ struct sw_plan {
   SearchState* state = nullptr;     // in block
   SearchState* state_h = nullptr;   // pinned: the state a search left
   // the tables while a search is planned
-  std::vector<int4> strips;         // strip tables of the two-query kernels
-  std::vector<int2> spairs;         // their stream pairs
-  std::vector<LaneSeg> segs;
+  Table<int4> strips;               // strip tables of the two-query kernels
+  Table<int2> spairs;               // their stream pairs
+  Table<LaneSeg> segs;
   int32_t* scores_dev = nullptr;  // used when the caller's scores live on the host:
                                   // allocated by the first such search
   cudaStream_t stream = nullptr;  // the stream of the search in flight
@@ -592,7 +621,8 @@ extern "C" sw_status sw_plan_create(sw_db* db, int32_t max_queries, int64_t max_
     return sw_set_error(SW_EINVAL, "two_query_long must be 0, 1 or 2");
   CUDA_TRY(cudaSetDevice(db->device));
 
-  sw_plan* p = new sw_plan();
+  sw_plan* p = new (std::nothrow) sw_plan();
+  if (!p) return sw_set_error(SW_ENOMEM, "sw_plan_create: out of host memory");
   p->db = db;
   p->device = db->device;
   p->opt = o;
@@ -679,10 +709,13 @@ extern "C" sw_status sw_plan_create(sw_db* db, int32_t max_queries, int64_t max_
   // strip, and the intra-task kernel's, 32): every query padded to whole
   // strips (at least one), and as many empty halves at most; stream pairs:
   // one per two queries at most, per table
-  p->strips.resize((size_t)(2 * (max_query_residues / 16 + 2 * (int64_t)max_queries) + 16));
-  p->spairs.resize((size_t)(2 * (max_queries / 2 + 1)));
-  p->segs.resize((size_t)MAX_SEGS * max_queries +
-                 (size_t)(MAX_SEGS_FEW - MAX_SEGS) * std::min(max_queries, FEW_QUERIES));
+  if (!p->strips.reserve(2 * ((size_t)max_query_residues / 16 + 2 * (size_t)max_queries) + 16) ||
+      !p->spairs.reserve(2 * ((size_t)max_queries / 2 + 1)) ||
+      !p->segs.reserve(seg_capacity(max_queries))) {
+    plan_free(p);
+    return sw_set_error(SW_ENOMEM, "sw_plan_create: out of host memory for %d queries of %lld residues",
+                        max_queries, (long long)max_query_residues);
+  }
   p->block_bytes = BLOCK_HEADER + block_align((size_t)max_queries * sizeof(int64_t)) +
                    2 * block_align((size_t)max_queries * sizeof(int32_t)) +
                    block_align(p->segs.size() * sizeof(LaneSeg)) +
@@ -710,7 +743,7 @@ extern "C" sw_status sw_plan_create(sw_db* db, int32_t max_queries, int64_t max_
   }
   p->params = (SearchParams*)p->block;
   p->state = (SearchState*)(p->block + block_align(sizeof(SearchParams)));
-  memset(p->block_h, 0, p->block_bytes);
+  memset(p->block_h, 0, BLOCK_HEADER);
   memset(p->state_h, 0, sizeof(SearchState));
   *out = p;
   return SW_OK;
@@ -1233,7 +1266,7 @@ static int64_t plan_lanes(sw_plan* p, const HostBatch& hb, int32_t nq, int64_t p
             int c = 0;
             while (c < q.nc && t[c] > tail * t_all) c++;
             if (c == q.nc) c = (int)(std::min_element(t, t + q.nc) - t);
-            const bool room = pieces.size() - first < (size_t)(large ? MAX_SEGS : MAX_SEGS_FEW);
+            const bool room = pieces.size() - first < (size_t)max_segs(nq);
             if (c != last && last >= 0 && !room) c = last;
             const LaneCand& x = q.c[c];
             // of a few queries, much shorter subjects are a segment of their own,
