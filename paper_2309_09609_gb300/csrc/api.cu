@@ -128,10 +128,11 @@ extern "C" void sw_options_default(sw_options* opt) {
 
 // ---- small helpers ----------------------------------------------------------------
 // Host-side fault injection for tests: with SWGB_FAULT=alloc the device
-// allocations of sw_db_create and sw_plan_create report out-of-memory, and
-// with SWGB_FAULT=copy the first copy of a search reports a failed copy, so
-// the error paths run without a device fault.  Read at every call; unset, it
-// changes nothing.
+// allocations of sw_db_create and sw_plan_create report out-of-memory, with
+// SWGB_FAULT=copy the first copy of a search reports a failed copy, and with
+// SWGB_FAULT=clusters a plan is made as on a device that has no room for a
+// cluster of the recompute, so these paths run without a device fault.  Read
+// at every call; unset, it changes nothing.
 static bool injected_fault(const char* what) {
   const char* f = getenv("SWGB_FAULT");
   return f && strcmp(f, what) == 0;
@@ -515,6 +516,7 @@ struct sw_plan {
   sw_options opt{};
   KernelConfig kc2{};       // inter-task kernel, two queries per word
   KernelConfig ikc{};       // int32 intra-task kernel
+  int32_t clusters = 0;     // clusters of its recompute of few flagged pairs
   int32_t max_queries = 0;
   int64_t max_residues = 0;
   int32_t g_first = 0;      // first inter-task group under the cutoff
@@ -673,6 +675,7 @@ extern "C" sw_status sw_plan_create(sw_db* db, int32_t max_queries, int64_t max_
   p->ikc.warps = INTRA_WARPS;
   p->ikc.blocks = dev_sms;
   p->ikc.smem = intra_smem_bytes(o.intra_rows);
+  p->clusters = injected_fault("clusters") ? 0 : recompute_clusters(o.intra_rows, p->ikc.blocks);
   const int64_t WI = (int64_t)p->ikc.blocks * INTRA_WARPS;
   for (int wide = 0; wide < 2; wide++) {
     const int lbps = lane_blocks_per_sm(wide != 0);
@@ -802,7 +805,7 @@ static cudaError_t enqueue_kernels(sw_plan* p, cudaStream_t s, bool capturing) {
     if (e == cudaSuccess) e = record(p->ev_join, s, capturing);
   }
   if (set & K_INT32) {
-    if (e == cudaSuccess) e = launch_intra(p->ikc, (set & ~K_INT32) == 0, v, p->params, p->state, p->scr, s);
+    if (e == cudaSuccess) e = launch_intra(p->ikc, p->clusters, (set & ~K_INT32) == 0, v, p->params, p->state, p->scr, s);
     if (e == cudaSuccess) e = record(p->ev[3], s, capturing);
   }
   return e;
@@ -1500,7 +1503,8 @@ static sw_status plan_enqueue(sw_plan* p, const HostBatch& hb, int32_t nq, int32
   p->pending.intra_items = n_long * nq;  // (query, long subject) pairs, packed or int32
   p->pending.inter_cells = qsum * (p->db->residues - p->db->cres_h[n_long]);
   for (int k = kernels & ~K_WIDE; k; k &= k - 1) p->pending.kernels_launched++;
-  if ((kernels & K_INT32) && kernels != K_INT32) p->pending.kernels_launched++;  // both recomputes
+  if ((kernels & K_INT32) && kernels != K_INT32 && p->clusters > 0)
+    p->pending.kernels_launched++;  // both recomputes
   return SW_OK;
 }
 
@@ -1550,7 +1554,7 @@ static cudaError_t overflow_rounds(sw_plan* p, int32_t* rounds) {
   while (nf > (unsigned long long)p->scr.flag_capacity) {
     cudaError_t e = cudaMemsetAsync(p->state, 0, sizeof(SearchState), s);
     if (e == cudaSuccess) e = launch_collect(4 * std::max(sms, 1), p->db->view, p->params, p->state, p->scr, s);
-    if (e == cudaSuccess) e = launch_intra(p->ikc, false, p->db->view, p->params, p->state, p->scr, s);
+    if (e == cudaSuccess) e = launch_intra(p->ikc, p->clusters, false, p->db->view, p->params, p->state, p->scr, s);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(p->state_h, p->state, sizeof(SearchState), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);

@@ -223,7 +223,8 @@ __device__ int intra_block_item(const DbView& db, const SearchParams* __restrict
   return best;
 }
 
-// Whether the flagged pairs are few enough for a cluster each.
+// Whether the flagged pairs go to clusters (uniform over the grid; `clusters` 0:
+// never).
 __device__ __forceinline__ bool recompute_in_clusters(unsigned long long flagged,
                                                       unsigned clusters) {
   return flagged <= (unsigned long long)RECOMPUTE_PER_CLUSTER * clusters;
@@ -231,7 +232,8 @@ __device__ __forceinline__ bool recompute_in_clusters(unsigned long long flagged
 
 template <int TI>
 __global__ void __launch_bounds__(INTRA_WARPS * 32)
-intra_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Scratch scr) {
+intra_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Scratch scr,
+             unsigned clusters) {
   extern __shared__ __align__(16) uint8_t smem[];
   __shared__ unsigned long long s_item;
   __shared__ int red[INTRA_WARPS];
@@ -260,7 +262,7 @@ intra_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Scr
   const unsigned long long nf = *(volatile unsigned long long*)&st->n_flags;
   const unsigned long long total =
       nf < (unsigned long long)scr.flag_capacity ? nf : (unsigned long long)scr.flag_capacity;
-  if (recompute_in_clusters(total, gridDim.x / RECOMPUTE_CLUSTER)) return;  // recompute_kernel
+  if (total == 0 || recompute_in_clusters(total, clusters)) return;  // recompute_kernel
   const int64_t stride = scr.intra_stride;
   for (;;) {
     if (threadIdx.x == 0) s_item = atomicAdd(&st->recompute, 1ull);
@@ -281,11 +283,11 @@ intra_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Scr
 // clusters, ...  Every block of a cluster runs the same stages.
 template <int TI>
 __global__ void __cluster_dims__(RECOMPUTE_CLUSTER) __launch_bounds__(RECOMPUTE_WARPS * 32)
-recompute_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Scratch scr) {
+recompute_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Scratch scr,
+                 unsigned clusters) {
   extern __shared__ __align__(16) uint8_t smem[];
   __shared__ int red[RECOMPUTE_WARPS];
   __shared__ int block_best;
-  const unsigned clusters = gridDim.x / RECOMPUTE_CLUSTER;
   const unsigned long long nf = *(volatile unsigned long long*)&st->n_flags;
   const unsigned long long total =
       nf < (unsigned long long)scr.flag_capacity ? nf : (unsigned long long)scr.flag_capacity;
@@ -344,7 +346,7 @@ cudaError_t launch_collect(int blocks, const DbView& db, const SearchParams* par
   return cudaGetLastError();
 }
 
-typedef void (*IntraKernel)(DbView, const SearchParams*, SearchState*, Scratch);
+typedef void (*IntraKernel)(DbView, const SearchParams*, SearchState*, Scratch, unsigned);
 
 static IntraKernel pick_intra(int rows) {
   if (rows == 8) return intra_kernel<8>;
@@ -356,42 +358,69 @@ static IntraKernel pick_recompute(int rows) {
   return rows == 8 ? recompute_kernel<8> : recompute_kernel<16>;
 }
 
-size_t intra_smem_bytes(int rows) {
+static size_t slices_bytes(int rows, int warps) {
   const int slice = rows == 8 ? IntraSlice<8>::BYTES : IntraSlice<16>::BYTES;
-  return (size_t)MATRIX_SMEM + (size_t)INTRA_WARPS * slice;
+  return (size_t)MATRIX_SMEM + (size_t)warps * slice;
 }
+
+static size_t recompute_smem_bytes(int rows) { return slices_bytes(rows, RECOMPUTE_WARPS); }
+
+size_t intra_smem_bytes(int rows) { return slices_bytes(rows, INTRA_WARPS); }
 
 int intra_blocks_per_sm(int rows) {
   IntraKernel k = pick_intra(rows);
   if (!k) return 0;
   const size_t smem = intra_smem_bytes(rows);
-  for (IntraKernel f : {k, pick_recompute(rows)})
-    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
-      return 0;
-  if (cudaFuncSetAttribute(pick_recompute(rows), cudaFuncAttributeNonPortableClusterSizeAllowed,
-                           1) != cudaSuccess)
-    return 0;
   int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, INTRA_WARPS * 32, smem) !=
-      cudaSuccess)
+  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
+          cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, INTRA_WARPS * 32, smem) !=
+          cudaSuccess) {
+    cudaGetLastError();
     return 0;
+  }
   return nb;
 }
 
-cudaError_t launch_intra(const KernelConfig& kc, bool items, const DbView& db,
+int recompute_clusters(int rows, int blocks) {
+  const int most = blocks / RECOMPUTE_CLUSTER;
+  if (most < 1) return 0;
+  IntraKernel k = pick_recompute(rows);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(RECOMPUTE_CLUSTER);
+  cfg.blockDim = dim3(RECOMPUTE_WARPS * 32);
+  cfg.dynamicSmemBytes = recompute_smem_bytes(rows);
+  cudaLaunchAttribute shape{};
+  shape.id = cudaLaunchAttributeClusterDimension;
+  shape.val.clusterDim.x = RECOMPUTE_CLUSTER;
+  shape.val.clusterDim.y = shape.val.clusterDim.z = 1;
+  cfg.attrs = &shape;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)cfg.dynamicSmemBytes) != cudaSuccess ||
+      cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n < most ? n : most;
+}
+
+cudaError_t launch_intra(const KernelConfig& kc, int clusters, bool items, const DbView& db,
                          const SearchParams* params, SearchState* state, const Scratch& scr,
                          cudaStream_t stream) {
   IntraKernel k = pick_intra(kc.variant);
   if (!k) return cudaErrorInvalidValue;
   cudaGetLastError();  // a stale error must not be read as this launch's
-  if (!items && kc.blocks >= RECOMPUTE_CLUSTER) {  // flagged pairs: few of them, or many
-    pick_recompute(kc.variant)<<<kc.blocks / RECOMPUTE_CLUSTER * RECOMPUTE_CLUSTER,
-                                 RECOMPUTE_WARPS * 32, kc.smem, stream>>>(db, params, state, scr);
+  if (!items && clusters > 0) {  // flagged pairs: few of them, or many
+    pick_recompute(kc.variant)<<<clusters * RECOMPUTE_CLUSTER, RECOMPUTE_WARPS * 32,
+                                 recompute_smem_bytes(kc.variant), stream>>>(
+        db, params, state, scr, (unsigned)clusters);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  k<<<kc.blocks, INTRA_WARPS * 32, kc.smem, stream>>>(db, params, state, scr);
+  k<<<kc.blocks, INTRA_WARPS * 32, kc.smem, stream>>>(db, params, state, scr, (unsigned)clusters);
   return cudaGetLastError();
 }
 

@@ -173,8 +173,12 @@ cudaError_t launch_inter(int gclass, int blocks, const DbView& db, const SearchP
 constexpr int INTRA_WARPS = 16;  // warps per block
 size_t intra_smem_bytes(int rows);
 int intra_blocks_per_sm(int rows);
-// items: int32 items, which leave no flagged pairs; otherwise the flagged pairs
-cudaError_t launch_intra(const KernelConfig& kc, bool items, const DbView& db,
+// Clusters of RECOMPUTE_CLUSTER blocks that fit the device at once (0: none, or
+// no room for one), at most blocks / RECOMPUTE_CLUSTER.
+int recompute_clusters(int rows, int blocks);
+// items: int32 items, which leave no flagged pairs; otherwise the flagged pairs,
+// on `clusters` clusters (0: none, a block each) or a block each
+cudaError_t launch_intra(const KernelConfig& kc, int clusters, bool items, const DbView& db,
                          const SearchParams* params, SearchState* state, const Scratch& scr,
                          cudaStream_t stream);
 constexpr int RECOMPUTE_CLUSTER = 16;     // blocks per cluster
