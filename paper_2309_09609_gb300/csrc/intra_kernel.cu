@@ -18,11 +18,11 @@
 //     border write before its read and each read before the next overwrite.
 //
 // Few flagged pairs leave most SMs idle that way, and the search waits for the
-// longest.  Up to RECOMPUTE_PER_CLUSTER of them for every cluster of the grid
-// are therefore scored by recompute_kernel instead: the same schedule over
-// the 128 warps of a cluster of sixteen blocks, with the cluster's barrier
-// between the stages.  More pairs than that fill the chip one block each, and
-// most blocks of a cluster would idle on short queries.  Two pairs of 35,000 x
+// longest.  They are therefore scored by recompute_kernel where that ends
+// first: the same schedule over the 128 warps of a cluster of sixteen blocks,
+// with the cluster's barrier between the stages.  Many pairs fill the chip one
+// block each, and a query of few passes leaves most blocks of a cluster idle,
+// which takes its pairs in turn (recompute_in_clusters).  Two pairs of 35,000 x
 // 26,620 residues took 68 ms on a block each, 15.9 on clusters of eight blocks
 // of 16 warps, 11.6 on clusters of sixteen of 8 (two warps to a scheduler) and
 // 9.7 with the codes and profile words loaded ahead of their columns.
@@ -132,6 +132,15 @@ __device__ void intra_warp_item(const DbView& db, const SearchParams* __restrict
   if (lane == 0) emit_score(db, P, q, s, S);
 }
 
+// Stages of a pair's passes on W warps.
+template <int TI>
+__device__ __forceinline__ int pair_stages(int m, int n, int W) {
+  const int npass = n > 0 ? (m + 32 * TI - 1) / (32 * TI) : 0;
+  const int spass = (n + 31 + 31) / 32;  // of one pass (n + 31 steps)
+  if (npass == 0) return 0;
+  return (npass - 1) / W * max(spass, LAG * W) + (npass - 1) % W * LAG + spass;
+}
+
 // One (query, subject) pair on the W warps of a block, or of a cluster of
 // blocks.  Pass p runs on warp p % W and starts at stage (p / W) * period +
 // (p % W) * LAG, with period = max(stages of a pass, LAG * W): consecutive
@@ -157,8 +166,7 @@ __device__ int intra_block_item(const DbView& db, const SearchParams* __restrict
   const int npass = n > 0 ? (m + ROWS - 1) / ROWS : 0;
   const int spass = (n + 31 + 31) / 32;  // stages of one pass (n + 31 steps)
   const int period = max(spass, LAG * W);
-  const int nstages =
-      npass > 0 ? ((npass - 1) / W) * period + ((npass - 1) % W) * LAG + spass : 0;
+  const int nstages = pair_stages<TI>(m, n, W);
   const int2 top = make_int2(0, -go);                   // (H(0, j), F(1, j))
   int S = 0;
   int Hp[TI], E[TI], hdiag = 0, out_h = 0, out_f = -go;
@@ -223,11 +231,40 @@ __device__ int intra_block_item(const DbView& db, const SearchParams* __restrict
   return best;
 }
 
-// Whether the flagged pairs go to clusters (uniform over the grid; `clusters` 0:
-// never).
-__device__ __forceinline__ bool recompute_in_clusters(unsigned long long flagged,
+// Whether the flagged pairs go to clusters (`clusters` 0: never): if the stages of
+// the cluster that has most end before those of the longest pair on a block.
+// Every warp of either kernel gets the same answer from the same list.
+// Measured, microseconds a stage: 8.0 on a block of 16 busy warps, 6.4 on a
+// cluster, 8.6 where its SMs hold a second one's blocks (8 pairs at a time, with
+// 9 clusters); here in fifths.  Milliseconds for pairs of 3,100 residues, of 8,000 and of 16,000,
+// with clusters and without: 4 pairs 0.84 and 0.94, 2.2 and 4.4, 4.4 and 16.7; 10
+// pairs 1.79 and 0.94, 4.7 and 4.4, 9.5 and 16.7; 36 pairs 4.2 and 0.95, 11.6 and
+// 4.4, 23.3 and 16.8 (all of which had gone to clusters).
+template <int TI>
+__device__ __forceinline__ bool recompute_in_clusters(const DbView& db,
+                                                      const SearchParams* __restrict__ P,
+                                                      const Scratch& scr, unsigned long long flagged,
                                                       unsigned clusters) {
-  return flagged <= (unsigned long long)RECOMPUTE_PER_CLUSTER * clusters;
+  if (flagged == 0 || flagged > (unsigned long long)RECOMPUTE_PER_CLUSTER * clusters) return false;
+  long long most = 0, block = 0;
+  for (unsigned c = threadIdx.x & 31; c < clusters; c += 32) {
+    long long mine = 0;
+    for (unsigned it = c; it < (unsigned)flagged; it += clusters) {
+      const int2 fl = scr.flags[it];
+      const int m = P->qlen[fl.x], n = db.clen[fl.y];
+      const unsigned left = (unsigned)flagged - (it - c);  // pairs of this turn and the next ones
+      mine += (long long)pair_stages<TI>(m, n, RECOMPUTE_CLUSTER * RECOMPUTE_WARPS) *
+              (4 * left > 3 * clusters ? 43 : 32);
+      block = max(block, 40ll * pair_stages<TI>(m, n, INTRA_WARPS));
+    }
+    most = max(most, mine);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    most = max(most, __shfl_xor_sync(FULL, most, o));
+    block = max(block, __shfl_xor_sync(FULL, block, o));
+  }
+  return most < block;
 }
 
 template <int TI>
@@ -262,7 +299,7 @@ intra_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st, Scr
   const unsigned long long nf = *(volatile unsigned long long*)&st->n_flags;
   const unsigned long long total =
       nf < (unsigned long long)scr.flag_capacity ? nf : (unsigned long long)scr.flag_capacity;
-  if (total == 0 || recompute_in_clusters(total, clusters)) return;  // recompute_kernel
+  if (total == 0 || recompute_in_clusters<TI>(db, P, scr, total, clusters)) return;  // recompute_kernel
   const int64_t stride = scr.intra_stride;
   for (;;) {
     if (threadIdx.x == 0) s_item = atomicAdd(&st->recompute, 1ull);
@@ -291,7 +328,7 @@ recompute_kernel(DbView db, const SearchParams* __restrict__ P, SearchState* st,
   const unsigned long long nf = *(volatile unsigned long long*)&st->n_flags;
   const unsigned long long total =
       nf < (unsigned long long)scr.flag_capacity ? nf : (unsigned long long)scr.flag_capacity;
-  if (total == 0 || !recompute_in_clusters(total, clusters)) return;  // uniform over the grid
+  if (!recompute_in_clusters<TI>(db, P, scr, total, clusters)) return;  // uniform over the grid
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   constexpr int W = RECOMPUTE_CLUSTER * RECOMPUTE_WARPS;
