@@ -1,0 +1,36 @@
+"""sw_align's buffers: calls whose inputs or results are too large for the pinned
+memory that the database keeps, calls that find too little device memory to keep H
+of every cell, and device memory kept for later calls given back to a plan."""
+import numpy as np
+import pytest
+
+from helpers import seqset
+import oracle
+from paper_2309_09609_gb300 import build as nvbuild
+from paper_2309_09609_gb300 import swgb
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    nvbuild.build()
+    swgb.lib()
+
+
+@pytest.mark.parametrize("queries,long", [(10, 0), (42_000, 0), (10, 600), (42_000, 600)])
+def test_inputs_and_results_beyond_the_pinned_memory(queries, long):
+    # 16 MiB: 42,000 queries of 400 go up beyond it, 600 slots of 35,400 come back
+    rng = np.random.default_rng(queries + long)
+    q = seqset(rng, [400] * queries)
+    s = seqset(rng, [35_000, 90, 0, 300])
+    d = swgb.Database.from_seqset(s)
+    pq = np.concatenate([np.arange(10), np.full(long, 3)])
+    ps = np.concatenate([np.arange(10) % 4, np.zeros(long, int)])
+    want = {}
+    for _ in range(2):
+        got = d.align(q.res, q.lens, pq, ps)
+        for a, b, g in zip(pq.tolist(), ps.tolist(), got):
+            if (a, b) not in want:
+                want[a, b] = oracle.align(q.seq(a), s.seq(b), 10, 2)
+            assert g == want[a, b], (a, b)
