@@ -1839,23 +1839,29 @@ extern "C" sw_status sw_align(sw_db* db, const uint8_t* queries, const int32_t* 
              n <= kAlignKeepHColumns;
   }
   // chunks of pairs whose cells fit kAlignChunkBytes (one pair may exceed it alone)
-  std::vector<int32_t> chunk_begin{0};
-  int64_t words = 0, max_words = 0, max_border = 0, border = 0;
-  for (int32_t k = 0; k < n_pairs; k++) {
-    const int64_t w = align_bits_bytes(team, keep_h, hb.len[items[k].q], db->clen_h[items[k].s]);
-    if (k > chunk_begin.back() && words + w > kAlignChunkBytes) {
-      chunk_begin.push_back(k);
-      words = border = 0;
+  std::vector<int32_t> chunk_begin;
+  int64_t max_words = 0, max_border = 0;
+  auto chunk = [&]() {
+    chunk_begin.assign(1, 0);
+    max_words = max_border = 0;
+    int64_t words = 0, border = 0;
+    for (int32_t k = 0; k < n_pairs; k++) {
+      const int64_t w = align_bits_bytes(team, keep_h, hb.len[items[k].q], db->clen_h[items[k].s]);
+      if (k > chunk_begin.back() && words + w > kAlignChunkBytes) {
+        chunk_begin.push_back(k);
+        words = border = 0;
+      }
+      items[k].bits_off = words;
+      items[k].border_off = border;
+      items[k].ops_end = slot[k + 1];
+      words += w;
+      border += align_border_ints(team, db->clen_h[items[k].s]);
+      max_words = std::max(max_words, words);
+      max_border = std::max(max_border, border);
     }
-    items[k].bits_off = words;
-    items[k].border_off = border;
-    items[k].ops_end = slot[k + 1];
-    words += w;
-    border += align_border_ints(team, db->clen_h[items[k].s]);
-    max_words = std::max(max_words, words);
-    max_border = std::max(max_border, border);
-  }
-  chunk_begin.push_back(n_pairs);
+    chunk_begin.push_back(n_pairs);
+  };
+  chunk();
   cudaStream_t cs = (cudaStream_t)stream;
   // One device buffer: what goes up (parameters, items, the query arrays) in
   // one copy, what comes back (records, transcripts) in one copy, the border
@@ -1868,8 +1874,11 @@ extern "C" sw_status sw_align(sw_db* db, const uint8_t* queries, const int32_t* 
   const size_t ops_at = block_align(sizeof(AlignOut) * (size_t)n_pairs);
   const size_t back_bytes = ops_at + block_align((size_t)slot[n_pairs]);
   const size_t at_out = up_bytes, at_border = at_out + back_bytes;
-  const size_t at_bits = at_border + block_align(sizeof(int2) * (size_t)max_border);
-  const size_t dev_bytes = at_bits + (size_t)std::max<int64_t>(max_words, 1);
+  size_t at_bits = 0;
+  auto dev_bytes = [&]() {
+    at_bits = at_border + block_align(sizeof(int2) * (size_t)max_border);
+    return at_bits + (size_t)std::max<int64_t>(max_words, 1);
+  };
   std::unique_lock<std::mutex> kept(db->align_mu, std::try_to_lock);
   AlignBuffers own;
   AlignBuffers& buf = kept.owns_lock() ? db->align : own;
@@ -1883,7 +1892,14 @@ extern "C" sw_status sw_align(sw_db* db, const uint8_t* queries, const int32_t* 
     pageable.reset(new (std::nothrow) uint8_t[back_bytes]);
     if (!pageable) return sw_set_error(SW_ENOMEM, "sw_align: out of host memory");
   }
-  cudaError_t e = buf.reserve(dev_bytes, std::max(pin_up ? up_bytes : 0, pin_back ? back_bytes : 0));
+  const size_t pin_bytes = std::max(pin_up ? up_bytes : 0, pin_back ? back_bytes : 0);
+  cudaError_t e = buf.reserve(dev_bytes(), pin_bytes);
+  if (e == cudaErrorMemoryAllocation && keep_h) {
+    cudaGetLastError();  // no room for H of every cell: a quarter of that for bits
+    keep_h = false;
+    chunk();
+    e = buf.reserve(dev_bytes(), pin_bytes);
+  }
   uint8_t* host = pin_back ? buf.pinned : pageable.get();
   if (e == cudaSuccess) {
     P.qoff = (const int64_t*)(buf.dev + up_qoff);

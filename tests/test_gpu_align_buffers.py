@@ -34,3 +34,30 @@ def test_inputs_and_results_beyond_the_pinned_memory(queries, long):
             if (a, b) not in want:
                 want[a, b] = oracle.align(q.seq(a), s.seq(b), 10, 2)
             assert g == want[a, b], (a, b)
+
+
+def leave_free(torch, nbytes):
+    """Takes device memory until about nbytes are free; returns what holds it."""
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    return torch.empty(free - nbytes, dtype=torch.uint8, device="cuda")
+
+
+def test_direction_bits_where_memory_for_h_is_short():
+    # H of these cells takes 618 MiB, their bits 155
+    torch = pytest.importorskip("torch")
+    rng = np.random.default_rng(5)
+    q = seqset(rng, [2900] * 3)
+    s = seqset(rng, [35_000] * 3)
+    d = swgb.Database.from_seqset(s)
+    args = (q.res, q.lens, [0, 1, 2], [2, 0, 1])
+    want = d.align(*args)
+    d.align(*args, 40_000, 3)                # penalties beyond 16 bits: bits, and their kernel loaded
+    held = leave_free(torch, 400 << 20)
+    try:
+        got = d.align(*args)
+    finally:
+        del held
+        torch.cuda.empty_cache()
+    assert got == want
