@@ -281,10 +281,11 @@ typedef struct {
  * Of ops only the transcripts are written.
  * Device memory for the cells (2 bytes per cell of every pair while that is at
  * most 1 GiB and no score can exceed 32767, else 4 bits per cell) and the
- * call's other buffers is allocated by the call; the database keeps up to
- * 512 MiB of it (and 16 MiB of pinned memory) for later calls and frees it with
- * sw_db_destroy.  Pairs are processed in chunks of at most 8 GiB of cells.
- * Synchronous on the stream.
+ * call's other buffers is allocated by the call (bits as well where there is
+ * too little for 2 bytes); the database keeps up to 512 MiB of it (and 16 MiB of
+ * pinned memory) for later calls, gives it back when another allocation for this
+ * database fails, and frees it with sw_db_destroy.  Pairs are processed in chunks
+ * of at most 8 GiB of cells.  Synchronous on the stream.
  * Errors: SW_EINVAL (index out of range, short ops buffer, bad gaps or
  * codes), SW_ENOMEM, SW_ECUDA. */
 sw_status sw_align(sw_db* db, const uint8_t* queries, const int32_t* q_lengths, int32_t n_queries,

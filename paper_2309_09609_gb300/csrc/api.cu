@@ -269,6 +269,19 @@ static void db_free(sw_db* db) {
   delete db;
 }
 
+// Device memory for a call or a plan of the database.  What sw_align keeps for
+// its next call gives way to it.
+template <typename T>
+static cudaError_t db_alloc(sw_db* db, T** p, size_t count) {
+  cudaError_t e = dalloc(p, count);
+  if (e != cudaErrorMemoryAllocation) return e;
+  std::unique_lock<std::mutex> kept(db->align_mu, std::try_to_lock);
+  if (!kept.owns_lock() || !db->align.dev) return e;  // in use, or nothing there
+  cudaGetLastError();
+  db->align.trim(0, SIZE_MAX);
+  return dalloc(p, count);
+}
+
 extern "C" sw_status sw_db_create(const uint8_t* residues, const int32_t* lengths,
                                   int64_t n_subjects, int device, sw_db** out) {
   sw_clear_error();
@@ -725,11 +738,11 @@ extern "C" sw_status sw_plan_create(sw_db* db, int32_t max_queries, int64_t max_
                    block_align(p->spairs.size() * sizeof(int2)) +
                    block_align(p->strips.size() * sizeof(int4)) +
                    block_align((size_t)std::max<int64_t>(max_query_residues, 1));
-  if (e == cudaSuccess) e = dalloc(&p->scr.pair_border, (size_t)(WP * p->scr.pair_stride));
-  if (e == cudaSuccess) e = dalloc(&p->block, p->block_bytes);
-  if (e == cudaSuccess) e = dalloc(&p->scr.inter_border, (size_t)(W * std::max<int64_t>(p->scr.inter_stride_vec, 1)));
-  if (e == cudaSuccess) e = dalloc(&p->scr.intra_border, (size_t)(WI * p->scr.intra_stride));
-  if (e == cudaSuccess) e = dalloc(&p->scr.flags, (size_t)p->scr.flag_capacity);
+  if (e == cudaSuccess) e = db_alloc(db, &p->scr.pair_border, (size_t)(WP * p->scr.pair_stride));
+  if (e == cudaSuccess) e = db_alloc(db, &p->block, p->block_bytes);
+  if (e == cudaSuccess) e = db_alloc(db, &p->scr.inter_border, (size_t)(W * std::max<int64_t>(p->scr.inter_stride_vec, 1)));
+  if (e == cudaSuccess) e = db_alloc(db, &p->scr.intra_border, (size_t)(WI * p->scr.intra_stride));
+  if (e == cudaSuccess) e = db_alloc(db, &p->scr.flags, (size_t)p->scr.flag_capacity);
   if (e == cudaSuccess) e = cudaMallocHost((void**)&p->block_h, p->block_bytes);
   if (e == cudaSuccess) e = cudaMallocHost((void**)&p->state_h, sizeof(SearchState));
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->done, cudaEventDisableTiming);
@@ -1591,8 +1604,8 @@ extern "C" sw_status sw_plan_search(sw_plan* plan, const uint8_t* queries, const
     // scores for a host buffer are staged on the device: the first such
     // search allocates the plan's staging buffer
     cudaError_t ea = injected_fault("alloc") ? cudaErrorMemoryAllocation
-                                             : dalloc(&plan->scores_dev,
-                                                      (size_t)plan->max_queries * std::max<int64_t>(N, 1));
+                                             : db_alloc(plan->db, &plan->scores_dev,
+                                                        (size_t)plan->max_queries * std::max<int64_t>(N, 1));
     if (ea != cudaSuccess) {
       plan->scores_dev = nullptr;
       return sw_set_cuda_error(ea, "sw_plan_search: host-order scores buffer");
@@ -1736,13 +1749,13 @@ extern "C" sw_status sw_search_plain(sw_db* db, const uint8_t* queries, const in
   int32_t *qlen = nullptr, *sc = nullptr;
   int2* border = nullptr;
   SearchParams* Pd = nullptr;
-  cudaError_t e = dalloc(&qres, hb.total);
-  if (e == cudaSuccess) e = dalloc(&qoff, n_queries);
-  if (e == cudaSuccess) e = dalloc(&qlen, n_queries);
-  if (e == cudaSuccess) e = dalloc(&boff_d, grid);
-  if (e == cudaSuccess) e = dalloc(&border, btotal);
-  if (e == cudaSuccess) e = dalloc(&Pd, 1);
-  if (e == cudaSuccess && !dev_out) e = dalloc(&sc, (size_t)n_queries * N);
+  cudaError_t e = db_alloc(db, &qres, hb.total);
+  if (e == cudaSuccess) e = db_alloc(db, &qoff, n_queries);
+  if (e == cudaSuccess) e = db_alloc(db, &qlen, n_queries);
+  if (e == cudaSuccess) e = db_alloc(db, &boff_d, grid);
+  if (e == cudaSuccess) e = db_alloc(db, &border, btotal);
+  if (e == cudaSuccess) e = db_alloc(db, &Pd, 1);
+  if (e == cudaSuccess && !dev_out) e = db_alloc(db, &sc, (size_t)n_queries * N);
   if (e == cudaSuccess && hb.total > 0)
     e = cudaMemcpyAsync(qres, hb.res, hb.total, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)

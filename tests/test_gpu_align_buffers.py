@@ -61,3 +61,38 @@ def test_direction_bits_where_memory_for_h_is_short():
         del held
         torch.cuda.empty_cache()
     assert got == want
+
+
+def test_memory_kept_for_alignments_gives_way_to_a_plan_and_a_search():
+    # the two pairs' 412 MiB stay with the database; a plan, then a host-order
+    # scores buffer, finds 200 MiB less than it needs outside of them
+    torch = pytest.importorskip("torch")
+    rng = np.random.default_rng(6)
+    q = seqset(rng, [2900] * 2)
+    s = seqset(rng, [35_000] * 2 + [40] * 70_000)
+    d = swgb.Database.from_seqset(s)
+
+    def used_by(make):
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        kept = make()
+        return before - torch.cuda.mem_get_info()[0], kept
+
+    need, plan = used_by(lambda: d.plan(1200, 20_000))
+    scores, want = used_by(lambda: plan.search(q.res[:90], np.array([90], np.int32)))
+    assert scores > 300 << 20
+    plan.close()
+    pairs = (q.res, q.lens, [0, 1], [1, 0])
+    aligned = d.align(*pairs)
+    for extra in (-(200 << 20), scores - (200 << 20)):
+        d.align(*pairs)
+        held = leave_free(torch, need + extra)
+        try:
+            plan = d.plan(1200, 20_000)
+            if extra > 0:
+                assert (plan.search(q.res[:90], np.array([90], np.int32)) == want).all()
+        finally:
+            del held
+            torch.cuda.empty_cache()
+        plan.close()
+    assert d.align(*pairs) == aligned
