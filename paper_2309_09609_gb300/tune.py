@@ -8,8 +8,9 @@ The options (all of which change speed only, never a score):
   workload a tuner that tried 24 rows on its 8-query sample picked them, and
   the full batch then ran 7% slower);
 * rows per thread (32, 16), columns per wavefront with 32 rows (8, 4) and
-  warps per block (8, 4), which the library accepts and checks; its kernels
-  take their shapes from the plan's cost model, so these now time alike;
+  warps per block (8, 4) keep their defaults: the library accepts and checks
+  them, but its kernels take their shapes from the plan's cost model, so a
+  timing could only pick among repeats of itself (``timed``);
 * the inter/intra length cutoff (1500, 3000, 7000, none) and the rows per
   lane of the int32 intra-task kernel (8, 16).
 
@@ -17,7 +18,7 @@ The search is a coordinate descent from the defaults: for each option in
 turn every alternative value is timed with the others at their best so far,
 and the best is kept; a second pass repeats this, and stops early once a
 pass changes nothing.  No option set is timed twice.  On the batched-uneven
-workload that is 15-20 searches of the sample instead of the 90 of the full
+workload that is 8 searches of the sample instead of the 16 of the full
 product.  Each candidate runs a plan over a length-stratified sample of the
 batch's queries against the whole resident database and is timed by the
 plan's own CUDA events around all of its kernels (pair, inter-task and
@@ -72,6 +73,15 @@ def space(db, n_queries: int) -> dict:
 def valid(opt: dict) -> bool:
     """Eight columns per wavefront need 32 rows per thread."""
     return not (opt.get("rows_per_thread") == 16 and opt.get("inter_columns") == 8)
+
+
+#: options that the library checks and that choose no code
+WITHOUT_EFFECT = ("rows_per_thread", "inter_columns", "warps_per_block")
+
+
+def timed(sp: dict) -> dict:
+    """The options of a space that can change a search's time."""
+    return {k: v for k, v in sp.items() if k not in WITHOUT_EFFECT}
 
 
 def descend(sp: dict, measure, passes: int = 2):
@@ -172,7 +182,9 @@ def tune(db: swgb.Database, queries, gap_open: int = 10, gap_extend: int = 2,
         plan.close()
         return best
 
-    best_opt, timings = descend(space(db, len(sample)), measure, passes)
+    sp = space(db, len(sample))
+    best_opt, timings = descend(timed(sp), measure, passes)
+    best_opt = {k: best_opt.get(k, v[0]) for k, v in sp.items()}
     if cache:
         with _lock:
             os.makedirs(os.path.dirname(cache), exist_ok=True)
