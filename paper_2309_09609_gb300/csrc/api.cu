@@ -473,7 +473,6 @@ static sw_status fill_scoring(SearchParams& P, int32_t gap_open, int32_t gap_ext
   P.go = gap_open + gap_extend;
   P.ge = gap_extend;
   P.sat_threshold = S16_LIMIT - maxsm - P.go;
-  P.init_border = make_uint4(0u, 0u, 0u, 0u);
   *packed_ok = (P.go + P.ge) <= kPackedMaxGap;
   if (max_sm) *max_sm = maxsm;
   return SW_OK;
@@ -1028,8 +1027,9 @@ static int32_t deal_streams(const HostBatch& hb, int32_t nq, int T, int32_t fixe
 // for 3 queries of 400 x 222,000: 27.3 ms, the lane groups 20.1; 5 of 400 x
 // 71,000: 11.4 and 9.1).  A strip costs kQ2StripCycles more, its profile and its
 // ends, whatever its columns: 20 queries of 375 x 570,000 subjects of 5-15 residues
-// take 12.2 ms, of which the words alone would be 6.8.
-static constexpr double kQ2WordCycles = 9.4, kQ2ItemCycles = 19, kQ2StripCycles = 3000;
+// take 11.9 ms, of which the words alone would be 6.5.  (2 to 20 queries of
+// 300-2,000 x 20,000 to 570,000 subjects: within 8% of the time measured.)
+static constexpr double kQ2WordCycles = 9.0, kQ2ItemCycles = 16.5, kQ2StripCycles = 3000;
 static int32_t plan_streams(sw_plan* p, const HostBatch& hb, int32_t nq, int32_t g_first,
                             int64_t* n_strips, double* cycles) {
   const int T = p->kc2.variant;
@@ -1047,6 +1047,15 @@ static int32_t plan_streams(sw_plan* p, const HostBatch& hb, int32_t nq, int32_t
                      (4.0 * p->sms);
   const double item = (double)longest * (kQ2ItemCycles * T * glen_max + 2 * kQ2StripCycles);
   *cycles = std::max(all, item) + 0.2 * std::min(all, item);  // as for the lane groups
+  // Items of about one length end in whole rounds: of the first r W + 1 some warp
+  // takes r + 1 (32 queries of 12,234 x 3,345 subjects of 89, 1.4 items per warp:
+  // 21.8 ms, two subjects per word 19.3).
+  const int64_t W = (int64_t)p->kc2.blocks * p->kc2.warps;
+  for (int64_t r = 1; r < 8 && K > 0 && r * W < (int64_t)K * 2 * (v.groups - g_first); r++) {
+    const double L = p->db->glen_h[(size_t)(g_first + r * W / K / 2)];
+    *cycles = std::max(*cycles, (double)(r + 1) * (double)*n_strips / K *
+                                    (kQ2ItemCycles * T * L + 2 * kQ2StripCycles));
+  }
   return K;
 }
 
@@ -1138,7 +1147,11 @@ struct LaneCand {
 
 // The shapes for a query of m residues: 8, 16 and 32 lanes; 32 lanes in halves;
 // chains of 4 to 16 rows per lane (16 only with the wide launch).
+// A block item costs kLaneItemCycles on each of its schedulers beside its steps,
+// which counts where subjects are short (185 queries of 71 x 31,600 subjects of 11,
+// 183,000 items: 2.05 ms, 1.33 without this term).
 static constexpr int MAX_SHAPES = 12;
+static constexpr double kLaneItemCycles = 800;
 static int lane_candidates(int32_t m, bool wide, LaneCand* c) {
   int n = 0;
   auto fit = [](int rows, int step) { return std::max(step, (rows + step - 1) / step * step); };
@@ -1177,7 +1190,8 @@ static double lanes_floor(const sw_plan* p, const HostBatch& hb, int32_t nq, int
   double cycles = 0;
   for (int32_t i = 0; i < nq; i++) {
     const int32_t m = hb.len[i], lg = m <= 256 ? 8 : m <= 512 ? 16 : 32;
-    cycles += 11.1 / 32 * m * (cols + (double)(pair1 - pair0) * lg);
+    cycles += 11.1 / 32 * m * (cols + (double)(pair1 - pair0) * lg) +
+              (double)(pair1 - pair0) * lg / 32 * kLaneItemCycles;
   }
   return cycles / (4.0 * p->sms);
 }
@@ -1324,15 +1338,17 @@ static int64_t plan_lanes(sw_plan* p, const HostBatch& hb, int32_t nq, int64_t p
   }
   std::stable_sort(best_pieces.begin(), best_pieces.end(),
                    [](const Piece& a, const Piece& b) { return a.t > b.t; });
-  int64_t items = 0;
+  int64_t items = 0, on_warps = 0;  // all, and those that are no chains
   for (size_t i = 0; i < best_pieces.size(); i++) {
     LaneSeg& sg = p->segs[i];
     sg = best_pieces[i].s;
     sg.first = items;
     const int64_t per = sg.chain ? 1 : LANE_WARPS * 32 / sg.lg;
-    items += (sg.pair1 - sg.pair0 + per - 1) / per;
+    const int64_t n = (sg.pair1 - sg.pair0 + per - 1) / per;
+    items += n;
+    if (!sg.chain) on_warps += n;
   }
-  *cycles = best;
+  *cycles = best + kLaneItemCycles * 4 * (double)on_warps / sched;
   *n_segs = (int32_t)best_pieces.size();
   return items;
 }

@@ -18,8 +18,8 @@
 // half 1 stream 1's.  A strip table gives, per strip, each half's query and
 // first row and whether the strip is that query's last: there the half's
 // score S is emitted (or flagged for the int32 recompute) and reset, and the
-// strip's bottom row is stored as the empty row above the matrix (H = 0,
-// F = -Go) for the next query of that half.
+// strip's bottom row is stored as the empty row above the matrix (H = F = 0)
+// for the next query of that half.
 //
 // Item = (stream pair, half of a 64-subject group): lane l scores subject
 // 2l + h of the group in the interleaved layout of the database.  One
@@ -218,30 +218,32 @@ __device__ void q2_item(const DbView& db, const SearchParams* __restrict__ P, Se
     // keep-mask of the bottom row: the halves whose query ends here store
     // the empty row above the next query instead (H = F = 0)
     const uint32_t keep = (enda ? 0u : 0x0000ffffu) | (endb ? 0u : 0xffff0000u);
-    // staging ring as in the packed inter-task kernel; the first strip's
-    // border is the row above the matrix, copied from the parameter block
-    const uint4* bsrc = s == 0 ? (const uint4*)&P->init_border : bd;
-    const int bstep = s == 0 ? 0 : 32;
+    // Staging ring of Q2RING chunks, copied with cp.async Q2RING - 1 chunks ahead
+    // (commit group c = chunk c).  A slot is refilled only after the registers
+    // read from it were consumed.  The first strip's border, H = F = 0 above
+    // the matrix, is written to the slots once: copied chunk by chunk from one
+    // word in global memory, every warp of the chip asked one slice of L2 for
+    // it, and a first strip took eight times as long as any other.
+    if (s == 0) {
 #pragma unroll
-    for (int j = 0; j < Q2RING - 1; j++) {
-      if (j < nch) {
+      for (int q = 0; q < 4 * Q2RING; q++) bring[q * 32] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    auto stage = [&](int j) {
+      if (s > 0) {  // uniform
 #pragma unroll
         for (int q = 0; q < 4; q++)
-          cp_async16(bring + ((j % Q2RING) * 4 + q) * 32, bsrc + (j * 4 + q) * bstep);
-        cp_async8(rring + (j % Q2RING) * 32, res + j * 64);
+          cp_async16(bring + ((j % Q2RING) * 4 + q) * 32, bd + (j * 4 + q) * 32);
       }
+      cp_async8(rring + (j % Q2RING) * 32, res + j * 64);
+    };
+#pragma unroll
+    for (int j = 0; j < Q2RING - 1; j++) {
+      if (j < nch) stage(j);
       cp_async_commit();
     }
 #pragma unroll 1
     for (int c = 0; c < nch; c++) {
-      const int cn = c + Q2RING - 1;
-      if (cn < nch) {
-        const int sl = cn % Q2RING;
-#pragma unroll
-        for (int q = 0; q < 4; q++)
-          cp_async16(bring + (sl * 4 + q) * 32, bsrc + (cn * 4 + q) * bstep);
-        cp_async8(rring + sl * 32, res + cn * 64);
-      }
+      if (c + Q2RING - 1 < nch) stage(c + Q2RING - 1);
       cp_async_commit();
       cp_async_wait<Q2RING - 1>();  // chunk c has landed
       const int slot = c % Q2RING;

@@ -67,7 +67,6 @@ struct LaneSeg {
 // Kept in device memory (not kernel arguments) so that one captured CUDA graph
 // serves every batch: a new search only rewrites this block.
 struct SearchParams {
-  uint4 init_border;      // packed (H, F) of the row above the matrix: zeros
   const uint8_t* qres;    // concatenated query codes
   const int64_t* qoff;    // [nq]
   const int32_t* qlen;    // [nq]

@@ -33,6 +33,24 @@ def test_many_short_subjects_cost_as_much_per_residue_as_longer_ones():
     assert ms[0] < 2.2 * ms[1], ms
 
 
+def test_two_query_streams_of_few_strips():
+    # where most strips are a stream's first, whose border all warps fetched from
+    # one word of L2: 3 times the time of the other layouts; and the same scores
+    rng = np.random.default_rng(2)
+    q, db = seqset(rng, [91] * 75), seqset(rng, [35] * 2071)
+    d = swgb.Database.from_seqset(db)
+    want = oracle_all(q, db)
+    ms = []
+    for two_query in (0, 2):
+        p = d.plan(75, q.total, two_query=two_query)
+        best = 1e9
+        for _ in range(9):
+            assert (p.search(q.res, q.lens) == want).all()
+            best = min(best, p.stats()["search_ms"])
+        ms.append(best)
+    assert ms[1] < 2 * ms[0], ms
+
+
 @pytest.mark.parametrize("gaps", [(10, 2), (11, 1), (6, 3)])
 def test_scores_at_the_edges_of_strips_and_chunks(gaps):
     rng = np.random.default_rng(gaps[0])
