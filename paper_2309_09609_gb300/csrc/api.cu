@@ -1018,6 +1018,22 @@ static int32_t deal_streams(const HostBatch& hb, int32_t nq, int T, int32_t fixe
   return K;
 }
 
+// The fewest strips that stream pairs of these queries can have, in all and in the
+// longest pair.
+struct StreamFloor {
+  int64_t strips, longest;
+};
+static StreamFloor stream_floor(const HostBatch& hb, int32_t nq, int T) {
+  StreamFloor f{0, 0};
+  for (int32_t i = 0; i < nq; i++) {
+    const int64_t s = std::max<int64_t>(1, (hb.len[i] + T - 1) / T);
+    f.strips += s;
+    f.longest = std::max(f.longest, s);
+  }
+  f.strips = (f.strips + 1) / 2;
+  return f;
+}
+
 // The short subjects' two-query layout (inter2q_kernel.cu): items are
 // (stream pair, half of a 64-subject group), the workers its warps.  Returns
 // the number of stream pairs, and in *cycles what the layout is expected to
@@ -1025,28 +1041,37 @@ static int32_t deal_streams(const HostBatch& hb, int32_t nq, int T, int32_t fixe
 // and the longest item, whose warp shares its scheduler with one other, and a
 // part of the smaller for the search's end (the larger alone took this kernel
 // for 3 queries of 400 x 222,000: 27.3 ms, the lane groups 20.1; 5 of 400 x
-// 71,000: 11.4 and 9.1).  A strip costs kQ2StripCycles more, its profile and its
+// 71,000: 11.4 and 9.1).  Returns 0, without dealing, when no deal could take
+// less than `limit` (a small search's streams: 14 queries x 4 subjects took
+// longer to deal than to score).  A strip costs kQ2StripCycles more, its profile and its
 // ends, whatever its columns: 20 queries of 375 x 570,000 subjects of 5-15 residues
 // take 11.9 ms, of which the words alone would be 6.5.  (2 to 20 queries of
 // 300-2,000 x 20,000 to 570,000 subjects: within 8% of the time measured.)
 static constexpr double kQ2WordCycles = 9.0, kQ2ItemCycles = 16.5, kQ2StripCycles = 3000;
 static int32_t plan_streams(sw_plan* p, const HostBatch& hb, int32_t nq, int32_t g_first,
-                            int64_t* n_strips, double* cycles) {
+                            double limit, int64_t* n_strips, double* cycles) {
   const int T = p->kc2.variant;
   const DbView& v = p->db->view;
+  *n_strips = 0;
   const double glen_sum = (double)(p->db->gcol_h[v.groups] - p->db->gcol_h[g_first]);
   const double glen_max = g_first < v.groups ? p->db->glen_h[g_first] : 0.0;
+  // scheduler cycles of a strip of every half group, and those of the longest
+  // group's on a warp
+  const double strip = 2 * (kQ2WordCycles * T * glen_sum + kQ2StripCycles * (v.groups - g_first)) /
+                       (4.0 * p->sms);
+  const double item_strip = kQ2ItemCycles * T * glen_max + 2 * kQ2StripCycles;
+  auto end_of = [](double all, double item) {  // as for the lane groups
+    return std::max(all, item) + 0.2 * std::min(all, item);
+  };
+  const StreamFloor least = stream_floor(hb, nq, T);
+  if (end_of((double)least.strips * strip, (double)least.longest * item_strip) >= limit) return 0;
   const int32_t K = deal_streams(hb, nq, T, p->opt.two_query_pairs,
                                  (double)p->kc2.blocks * p->kc2.warps, 1, glen_max, 2 * glen_sum,
                                  p->strips.data(), p->spairs.data(), 0,
                                  (int64_t)p->strips.size(), n_strips);
   int64_t longest = 0;
   for (int32_t k = 0; k < K; k++) longest = std::max<int64_t>(longest, p->spairs[(size_t)k].y);
-  const double all = (double)*n_strips * 2 *
-                     (kQ2WordCycles * T * glen_sum + kQ2StripCycles * (v.groups - g_first)) /
-                     (4.0 * p->sms);
-  const double item = (double)longest * (kQ2ItemCycles * T * glen_max + 2 * kQ2StripCycles);
-  *cycles = std::max(all, item) + 0.2 * std::min(all, item);  // as for the lane groups
+  *cycles = end_of((double)*n_strips * strip, (double)longest * item_strip);
   // Items of about one length end in whole rounds: of the first r W + 1 some warp
   // takes r + 1 (32 queries of 12,234 x 3,345 subjects of 89, 1.4 items per warp:
   // 21.8 ms, two subjects per word 19.3).
@@ -1067,25 +1092,30 @@ static int32_t plan_streams(sw_plan* p, const HostBatch& hb, int32_t nq, int32_t
 // rounds of blocks as the items need, or the longest item.
 static constexpr double kP2WordCycles = 8.9;
 static int32_t plan_streams_long(sw_plan* p, const HostBatch& hb, int32_t nq, int64_t n_long,
-                                 int64_t first_strip, int32_t first_pair, int64_t* n_strips,
-                                 double* cycles) {
+                                 int64_t first_strip, int32_t first_pair, double limit,
+                                 int64_t* n_strips, double* cycles) {
   *n_strips = 0;
   if (nq < 2 || n_long <= 0) return 0;
   const int32_t* clen = p->db->clen_h.data();
   double len_sum = 0;
   for (int64_t s = 0; s < n_long; s += PAIR2_GROUP) len_sum += clen[s];
+  const double groups = (double)((n_long + PAIR2_GROUP - 1) / PAIR2_GROUP);
+  const double step = 3 * 32 * kP2WordCycles;  // cycles per step of a block's three warps
+  const double all_steps = step * (len_sum + 127 * groups), item_steps = step * ((double)clen[0] + 127);
+  const StreamFloor least = stream_floor(hb, nq, PAIR2_STRIP);
+  if (std::max((double)((least.strips + 31) / 32) * all_steps / p->sms,
+               (double)((least.longest + 31) / 32) * item_steps) >= limit)
+    return 0;
   const int32_t K = deal_streams(hb, nq, PAIR2_STRIP, p->opt.two_query_pairs,
                                  (double)p->pair2_blocks, 32, clen[0],
                                  len_sum, p->strips.data() + first_strip,
                                  p->spairs.data() + first_pair, first_strip,
                                  (int64_t)p->strips.size() - first_strip, n_strips);
-  const double groups = (double)((n_long + PAIR2_GROUP - 1) / PAIR2_GROUP);
-  const double step = 3 * 32 * kP2WordCycles;  // cycles per step of a block's three warps
   double total = 0, longest = 0;
   for (int32_t k = 0; k < K; k++) {
     const double passes = (double)((p->spairs[(size_t)(first_pair + k)].y + 31) / 32);
-    total += passes * step * (len_sum + 127 * groups);
-    longest = std::max(longest, passes * step * ((double)clen[0] + 127));
+    total += passes * all_steps;
+    longest = std::max(longest, passes * item_steps);
   }
   *cycles = std::max(total / p->sms, longest);
   return K;
@@ -1439,20 +1469,34 @@ static sw_status plan_enqueue(sw_plan* p, const HostBatch& hb, int32_t nq, int32
     // end is shorter than that of two.
     const int64_t npairs = (v.n + 1) / 2, long_pairs = std::min(npairs, (n_long + 1) / 2);
     const bool has_long = n_long > 0, has_short = gf < v.groups;
-    int32_t n_segs = 0;
-    double t2 = 0, tl = 0;
+    double t2 = 0;
     bool two = false, two_long = false, wide = false, groups = false;
+    // the lane groups' segments for a range of subject pairs, planned once while
+    // the range stays the same
+    int32_t n_segs = 0;
+    int64_t lane_items = 0, planned0 = -1, planned1 = -1;
+    double tl = 0;
+    auto lanes = [&](int64_t pair0, int64_t pair1) {
+      if (pair0 != planned0 || pair1 != planned1)
+        lane_items = plan_lanes(p, hb, nq, pair0, pair1, &n_segs, &tl, &wide);
+      planned0 = pair0;
+      planned1 = pair1;
+      return tl;
+    };
     if (has_short) {
+      const bool may = nq >= 2 && p->opt.two_query > 0;
       int32_t K = 0;
-      if (nq >= 2 && p->opt.two_query > 0) K = plan_streams(p, hb, nq, gf, &n_strips, &t2);
-      if (K > 0 && p->opt.two_query == 2) {
-        two = true;
-      } else {
+      if (may && p->opt.two_query == 2) {
+        K = plan_streams(p, hb, nq, gf, 1e300, &n_strips, &t2);
+        two = K > 0;
+      }
+      if (!two) {
         const double t1 = plan_groups(p, hb, nq, gf);
         groups = t1 < 0.95 * lanes_floor(p, hb, nq, long_pairs, npairs);
-        if (K > 0 || groups) plan_lanes(p, hb, nq, long_pairs, npairs, &n_segs, &tl, &wide);
-        two = K > 0 && t2 < tl && !(groups && t1 < t2);
-        groups = groups && !two && t1 < 0.9 * tl;
+        const double t = may || groups ? lanes(long_pairs, npairs) : 0;
+        if (may && p->opt.two_query == 1) K = plan_streams(p, hb, nq, gf, t, &n_strips, &t2);
+        two = K > 0 && t2 < t && !(groups && t1 < t2);
+        groups = groups && !two && t1 < 0.9 * t;
       }
       if (two) {
         P.n_spairs = K;
@@ -1462,10 +1506,10 @@ static sw_status plan_enqueue(sw_plan* p, const HostBatch& hb, int32_t nq, int32
       }
     }
     if (has_long && nq >= 2 && p->opt.two_query_long > 0) {
+      const double t = p->opt.two_query_long == 1 ? lanes(0, long_pairs) : 1e300;
       const int32_t K2 =
-          plan_streams_long(p, hb, nq, n_long, n_strips, P.n_spairs, &n_strips2, &t2);
-      if (K2 > 0 && p->opt.two_query_long == 1) plan_lanes(p, hb, nq, 0, long_pairs, &n_segs, &tl, &wide);
-      two_long = K2 > 0 && (p->opt.two_query_long == 2 || t2 < tl);
+          plan_streams_long(p, hb, nq, n_long, n_strips, P.n_spairs, t, &n_strips2, &t2);
+      two_long = K2 > 0 && t2 < t;
       if (two_long) {
         P.n_spairs2 = K2;
         P.n_pair2_items = (int64_t)K2 * ((n_long + PAIR2_GROUP - 1) / PAIR2_GROUP);
@@ -1476,8 +1520,8 @@ static sw_status plan_enqueue(sw_plan* p, const HostBatch& hb, int32_t nq, int32
     }
     const bool lanes_long = has_long && !two_long, lanes_short = has_short && !two && !groups;
     if (lanes_long || lanes_short) {
-      P.n_lane_items = plan_lanes(p, hb, nq, lanes_long ? 0 : long_pairs,
-                                  lanes_short ? npairs : long_pairs, &n_segs, &tl, &wide);
+      lanes(lanes_long ? 0 : long_pairs, lanes_short ? npairs : long_pairs);
+      P.n_lane_items = lane_items;
       P.n_lane_segs = n_segs;
       p->lane_grid = (int)std::min<int64_t>(P.n_lane_items, p->lane_blocks[wide]);
       kernels |= (lanes_short ? K_LANES : K_LANES_LONG) | (wide ? K_WIDE : 0);
