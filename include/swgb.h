@@ -197,8 +197,9 @@ void sw_plan_destroy(sw_plan* plan);
  * tens of residues.  opt.two_query_long and opt.two_query with a cost model
  * choose per search; a single query never takes two queries per word.  Last
  * the int32 intra-task kernel recomputes every pair whose 16-bit score may
- * have saturated (one block per pair; more saturated pairs than
- * opt.flag_capacity are recomputed in further rounds before the call returns);
+ * have saturated (a block per pair, or a cluster of blocks for few long ones;
+ * more saturated pairs than opt.flag_capacity are recomputed in further rounds
+ * before the call returns);
  * it is left out when the lengths and the matrix allow no such score.  With
  * gap penalties too large for 16 bits, or opt.force_int32, every pair goes to
  * the int32 kernel instead (one warp per pair).  The packed kernels are
@@ -313,9 +314,9 @@ sw_status sw_align(sw_db* db, const uint8_t* queries, const int32_t* q_lengths, 
  * Every device buffer must belong to the current device (or be managed
  * memory); the call checks this before any launch.
  * Same gap convention and the same scores as sw_search.  The kernel's
- * scratch (512 border rows, a work counter, a status word) is a
+ * scratch (512 border rows, two work counters, a status word) is a
  * file-scope device array of ~16 MiB that every GPU loading the library holds
- * until the process exits; the counter and status are cleared at the start of
+ * until the process exits; the counters and status are cleared at the start of
  * every call.  The first call on a device looks the array's address up on
  * that device (the device must be current); make that first call before any
  * stream capture.  All calls share the one array, so calls whose work

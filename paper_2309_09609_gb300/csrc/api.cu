@@ -1,9 +1,10 @@
 // api.cu -- host side of libswgb: the C ABI of include/swgb.h.
 //
 //   * sw_db_create: sorts subjects by length and builds the two device
-//     layouts (interleaved groups of 64 for the inter-task kernel, contiguous
-//     for the intra-task kernel); the split of the database by length into a
-//     short (inter-task) and long (intra-task) part follows Section III-A.
+//     layouts (interleaved groups of 64 for the inter-task kernels and the
+//     lane groups, contiguous for the others); the split of the database by
+//     length into a short (inter-task) and long (intra-task) part follows
+//     Section III-A.
 //   * sw_plan_*: a reusable search context.  Its device memory is allocated
 //     once (the host-order scores buffer at the first search that needs it);
 //     per search one block is copied (parameters, zeroed counters, queries and
@@ -1196,7 +1197,7 @@ static int lane_candidates(int32_t m, bool wide, LaneCand* c) {
     const int passes = (m + 32 * full - 1) / (32 * full);
     if (passes > LANE_WARPS && (full < 8 || (wide && full < 16))) continue;  // a larger one has fewer
     int pr = fit((m - (passes - 1) * 32 * full + 31) / 32, 4);
-    while (pr & (pr - 1)) pr += 4;  // chains come in 4, 8, 16 and 32 rows
+    while (pr & (pr - 1)) pr += 4;  // chains come in 4, 8 and 16 rows
     c[n++] = LaneCand{32, pr, passes, full, 1, full > 4};
     // The passes after the last whole round of the block's warps leave some of
     // them idle: the same rows as up to a round of passes of fewer rows each.

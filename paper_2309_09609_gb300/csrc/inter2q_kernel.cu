@@ -1,8 +1,8 @@
 // inter2q_kernel.cu -- the inter-task kernel of libswgb with two queries per
 // 32-bit word.
 //
-// The lane-group kernel (lane_kernel.cu) puts two subjects in the two
-// 16-bit halves of a word, so each cell's substitution score SM(q_i, d_j)
+// The lane-group kernel (lane_kernel.cu) and inter_kernel.cu put two subjects
+// in the two 16-bit halves of a word, so each cell's substitution score SM(q_i, d_j)
 // comes from two profile rows (one per subject's residue) and costs one
 // byte-merge instruction per word.  Here each lane owns ONE subject and the
 // two halves hold two different queries: the word of query rows (a_i, b_i)

@@ -23,7 +23,8 @@
 //   1 query of 375 x 570,000             15.4 -> 10.9 ms
 //   7 queries of 140-600 x 40,000        15.0 ->  6.5 ms
 // (before: a warp per 64 subjects, and a warp per subject pair above 1,500
-// residues.)
+// residues.)  For many subjects of a few tens of residues the ramp is most of an
+// item, and a warp per 64 of them is the faster one (inter_kernel.cu).
 //
 // An item that would outlast the search (a long subject in a small search, a
 // long query against few subjects) is cut further: into chains, the query's

@@ -18,8 +18,8 @@
 // The strips of a pass are 32 consecutive entries of the strip table (query,
 // first row, end bit per half), so a query boundary may fall between any two
 // lanes (or passes).  A lane whose strip starts a query in a half replaces
-// that half of its top border by the empty row above the matrix (H = 0,
-// F = -Go).  At the end of a pass the warp takes, per half, a segmented
+// that half of its top border by the empty row above the matrix (H = F = 0).
+// At the end of a pass the warp takes, per half, a segmented
 // maximum of S over the lanes of each query (with the maximum carried from
 // the previous pass), and the lane holding a query's last strip emits the
 // score.
