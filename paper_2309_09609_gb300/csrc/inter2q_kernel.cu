@@ -221,19 +221,14 @@ __device__ void q2_item(const DbView& db, const SearchParams* __restrict__ P, Se
     // Staging ring of Q2RING chunks, copied with cp.async Q2RING - 1 chunks ahead
     // (commit group c = chunk c).  A slot is refilled only after the registers
     // read from it were consumed.  The first strip's border, H = F = 0 above
-    // the matrix, is written to the slots once: copied chunk by chunk from one
+    // the matrix, is filled in without a read: copied chunk by chunk from one
     // word in global memory, every warp of the chip asked one slice of L2 for
     // it, and a first strip took eight times as long as any other.
-    if (s == 0) {
-#pragma unroll
-      for (int q = 0; q < 4 * Q2RING; q++) bring[q * 32] = make_uint4(0u, 0u, 0u, 0u);
-    }
+    const int bytes = s == 0 ? 0 : 16;
     auto stage = [&](int j) {
-      if (s > 0) {  // uniform
 #pragma unroll
-        for (int q = 0; q < 4; q++)
-          cp_async16(bring + ((j % Q2RING) * 4 + q) * 32, bd + (j * 4 + q) * 32);
-      }
+      for (int q = 0; q < 4; q++)
+        cp_async16_or_zeros(bring + ((j % Q2RING) * 4 + q) * 32, bd + (j * 4 + q) * 32, bytes);
       cp_async8(rring + (j % Q2RING) * 32, res + j * 64);
     };
 #pragma unroll

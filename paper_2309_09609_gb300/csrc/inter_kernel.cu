@@ -165,19 +165,14 @@ __device__ void inter_item(const DbView& db, const SearchParams* __restrict__ P,
     // Staging ring of I_RING chunks, copied with cp.async I_RING - 1 chunks ahead
     // (commit group c = chunk c).  A slot is refilled only after the registers
     // read from it were consumed.  The first strip's border, H = F = 0 above
-    // the matrix, is written to the slots once (copied chunk by chunk from one
+    // the matrix, is filled in without a read (copied chunk by chunk from one
     // word in global memory, every warp of the chip asked one slice of L2 for
     // it: one query of 375 x 200,000 subjects of 250-350 took 5.8 ms, now 3.5).
-    if (s == 0) {
-#pragma unroll
-      for (int k = 0; k < 4 * I_RING; k++) bring[k * 32] = make_uint4(0u, 0u, 0u, 0u);
-    }
+    const int bytes = s == 0 ? 0 : 16;
     auto stage = [&](int j) {
-      if (s > 0) {  // uniform
 #pragma unroll
-        for (int k = 0; k < 4; k++)
-          cp_async16(bring + ((j % I_RING) * 4 + k) * 32, bd + (j * 4 + k) * 32);
-      }
+      for (int k = 0; k < 4; k++)
+        cp_async16_or_zeros(bring + ((j % I_RING) * 4 + k) * 32, bd + (j * 4 + k) * 32, bytes);
       cp_async16(rring + (j % I_RING) * 32, res + j * 32);
     };
 #pragma unroll
