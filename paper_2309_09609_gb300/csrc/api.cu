@@ -1043,11 +1043,11 @@ static StreamFloor stream_floor(const HostBatch& hb, int32_t nq, int T) {
 // part of the smaller for the search's end (the larger alone took this kernel
 // for 3 queries of 400 x 222,000: 27.3 ms, the lane groups 20.1; 5 of 400 x
 // 71,000: 11.4 and 9.1).  Returns 0, without dealing, when no deal could take
-// less than `limit` (a small search's streams: 14 queries x 4 subjects took
-// longer to deal than to score).  A strip costs kQ2StripCycles more, its profile and its
-// ends, whatever its columns: 20 queries of 375 x 570,000 subjects of 5-15 residues
-// take 11.9 ms, of which the words alone would be 6.5.  (2 to 20 queries of
-// 300-2,000 x 20,000 to 570,000 subjects: within 8% of the time measured.)
+// less than `limit` (14 queries took longer to deal than to score against 4
+// subjects).  A strip costs kQ2StripCycles beside its words, for its profile and
+// its ends: 20 queries of 375 x 570,000 subjects of 5-15 residues take 11.9 ms,
+// of which the words alone would be 6.5.  (2 to 20 queries of 300-2,000 x 20,000
+// to 570,000 subjects: within 8% of the time measured.)
 static constexpr double kQ2WordCycles = 9.0, kQ2ItemCycles = 16.5, kQ2StripCycles = 3000;
 static int32_t plan_streams(sw_plan* p, const HostBatch& hb, int32_t nq, int32_t g_first,
                             double limit, int64_t* n_strips, double* cycles) {
@@ -1176,13 +1176,14 @@ struct LaneCand {
   }
 };
 
-// The shapes for a query of m residues: 8, 16 and 32 lanes; 32 lanes in halves;
-// chains of 4 to 16 rows per lane (16 only with the wide launch).
 // A block item costs kLaneItemCycles on each of its schedulers beside its steps,
 // which counts where subjects are short (185 queries of 71 x 31,600 subjects of 11,
-// 183,000 items: 2.05 ms, 1.33 without this term).
-static constexpr int MAX_SHAPES = 12;
+// 183,000 items: 2.05 ms, estimated at 1.33 without this term, 1.79 with it).
 static constexpr double kLaneItemCycles = 800;
+
+// The shapes for a query of m residues: 8, 16 and 32 lanes; 32 lanes in halves;
+// chains of 4 to 16 rows per lane (16 only with the wide launch).
+static constexpr int MAX_SHAPES = 12;
 static int lane_candidates(int32_t m, bool wide, LaneCand* c) {
   int n = 0;
   auto fit = [](int rows, int step) { return std::max(step, (rows + step - 1) / step * step); };
